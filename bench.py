@@ -61,17 +61,14 @@ def sha_of(path):
 
 
 def ntt_kernels_sha():
-    """Hash of the source of the per-ring NTT phase kernels: ntt.cu without its marked
-    several-ring sections (kernels and launcher, which those phase kernels do not use) and without
-    its marked host launcher and autotuner (which pick and time the kernels, changing none)."""
-    with open(os.path.join(ROOT, "paper_2207_04620_gb300", "csrc", "ntt.cu")) as f:
-        src = f.read()
+    """Hash of the source of the per-ring NTT phase kernels: ntt_impl.cuh without its marked
+    several-ring section (kernels that those phase kernels do not use) and the fold arithmetic."""
+    src = ""
+    for name in ("ntt_impl.cuh", "modfold.cuh"):
+        with open(os.path.join(ROOT, "paper_2207_04620_gb300", "csrc", name)) as f:
+            src += f.read()
     src = re.sub(r"// ---- several rings in one launch.*?// ---- end of the several-ring kernels\n\n", "", src,
                  flags=re.S)
-    src = re.sub(r"// ---- several rings: launcher\n.*?// ---- end of the several-ring launcher\n\n", "", src,
-                 flags=re.S)
-    src = re.sub(r"// ---- autotuner[^\n]*\n.*?// ---- end of the autotuner\n\n", "", src, flags=re.S)
-    src = re.sub(r"// ---- launcher[^\n]*\n.*?// ---- end of the launcher\n\n", "", src, flags=re.S)
     return hashlib.sha256(src.encode()).hexdigest()[:16]
 
 

@@ -726,9 +726,7 @@ hx_status hx_ntt_multi(const hx_ntt_job *jobs, int n_jobs, int inverse, void *st
         dev = j.ctx->device;
         NttJob &J = v[i];
         J.data = j.data;
-        J.primes = j.ctx->t.primes;
-        J.tw_fwd = j.ctx->t.tw_fwd;
-        J.tw_inv = j.ctx->t.tw_inv;
+        set_ntt_tables(J, j.ctx->t);
         J.log_n = j.ctx->log_n;
         J.n_rows = j.n_polys * j.n_limbs;
         J.n_limbs = j.n_limbs;

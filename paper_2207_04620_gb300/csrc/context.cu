@@ -1,5 +1,6 @@
 // Context construction: primes, roots, twiddles and the RNS conversion tables
 // of hybrid key switching and rescaling, all resident in HBM.
+#include <algorithm>
 #include <cstring>
 
 #include "runtime.h"
@@ -61,6 +62,58 @@ unsigned bitrev(unsigned x, int bits)
         r = (r << 1) | (x & 1);
         x >>= 1;
     }
+    return r;
+}
+
+// Whether fold arithmetic holds for prime q of b bits (modfold.cuh): on a unit u >= 2^b with folded
+// values within 17/16 u and products within 25/16 u, sums up to 127/16 u stay inside 63 bits and
+// the final reduction lands in [-2^(b-1), 2^b + 2^(b-1)) after one fold, or after two (*refold).
+bool fold_bounds(uint64_t q, int *bits, int *refold)
+{
+    int b = 0;
+    while (b < 64 && (q >> b)) b++;
+    *bits = b;
+    if (b < 33 || b > 60) return false;
+    const u128 B = (u128)1 << b, d = B - q;
+    if (d >= (1u << 26)) return false;
+    auto folded = [&](u128 v) { return B + ((v >> b) + 1) * d; };  // bound of fold(v) for |v| <= v
+    const u128 product = B + B / 2 + (d << 31);
+    u128 u = std::max(B, (16 * product + kFoldProduct - 1) / kFoldProduct), limit = 0;
+    for (int i = 0; i < 3; i++) {  // the unit also covers what a fold at the limit leaves
+        limit = u * kFoldLimit / 16 + 1;
+        u = std::max(u, (16 * folded(limit) + kFoldSettled - 1) / kFoldSettled);
+    }
+    limit = u * kFoldLimit / 16 + 1;
+    if (limit >= ((u128)1 << 63) - ((u128)1 << 32) || 16 * folded(limit) > kFoldSettled * u) return false;
+    const u128 once = folded(limit), twice = folded(once);
+    *refold = once - B > B / 2;
+    return (*refold ? twice : once) - B <= B / 2;
+}
+
+// w mod q as a fold constant: centred w and 2^32 w, split at bit c = b - 32 into a signed 32-bit
+// head and a centred tail
+int4 fold_constant(uint64_t w, uint64_t q, int b)
+{
+    const int c = b - 32;
+    auto split = [&](uint64_t x, int *head, int *tail) {
+        int64_t v = x > q / 2 ? (int64_t)x - (int64_t)q : (int64_t)x;
+        for (int k = 0; k < 2; k++) {
+            int64_t t = v & (((int64_t)1 << c) - 1);
+            if (t >= ((int64_t)1 << (c - 1))) t -= (int64_t)1 << c;
+            const int64_t h = (v - t) >> c;
+            *head = (int)h;
+            *tail = (int)t;
+            if (h == (int64_t)*head) return;
+            v -= q;  // rounding the tail up pushed the head to 2^31: the other representative
+        }
+    };
+    // 2^32 w mod q without a division: 2^32 w = 2^b t + l
+    const u128 x = (u128)w << 32;
+    const uint64_t t = (uint64_t)(x >> b), d = (uint64_t)(((u128)1 << b) - q);
+    const u128 y = (x & (((u128)1 << b) - 1)) + (u128)t * d;
+    int4 r;
+    split(w, &r.x, &r.z);
+    split((uint64_t)(y % q), &r.y, &r.w);
     return r;
 }
 
@@ -127,6 +180,31 @@ void build_context(hx_context &c, const hx_params &p)
         }
         P.n_inv_w1 = hmul(P.n_inv, twi[(size_t)i * N + 1].x, q);
         P.n_inv_w1_sh = shoup_companion(P.n_inv_w1, q);
+    }
+
+    // fold arithmetic, where every prime allows it
+    std::vector<FoldPrime> fold(n_all);
+    std::vector<int4> ftwf, ftwi;
+    bool all_fold = true;
+    std::vector<int> fold_bits(n_all);
+    for (int i = 0; i < n_all; i++) all_fold = fold_bounds(c.primes[i], &fold_bits[i], &fold[i].refold) && all_fold;
+    if (all_fold) {
+        ftwf.resize((size_t)n_all * N);
+        ftwi.resize((size_t)n_all * N);
+        for (int i = 0; i < n_all; i++) {
+            const uint64_t q = c.primes[i];
+            const int b = fold_bits[i];
+            fold[i].q = q;
+            fold[i].c = b - 32;
+            fold[i].d = (int)(((uint64_t)1 << b) - q);
+            fold[i].mask = (1 << (b - 32)) - 1;
+            fold[i].n_inv = fold_constant(c.h_primes[i].n_inv, q, b);
+            fold[i].n_inv_w1 = fold_constant(c.h_primes[i].n_inv_w1, q, b);
+            for (int k = 0; k < N; k++) {
+                ftwf[(size_t)i * N + k] = fold_constant(twf[(size_t)i * N + k].x, q, b);
+                ftwi[(size_t)i * N + k] = fold_constant(twi[(size_t)i * N + k].x, q, b);
+            }
+        }
     }
 
     // ModUp tables, by (limbs, digit)
@@ -283,6 +361,11 @@ void build_context(hx_context &c, const hx_params &p)
     c.t.primes = upload(c.h_primes);
     c.t.tw_fwd = upload(twf);
     c.t.tw_inv = upload(twi);
+    if (all_fold) {
+        c.t.fold = upload(fold);
+        c.t.ftw_fwd = upload(ftwf);
+        c.t.ftw_inv = upload(ftwi);
+    }
     c.t.modup = upload(c.h_modup);
     c.t.moddown = upload(c.h_moddown);
     c.t.rescale = upload(c.h_rescale);
@@ -353,6 +436,9 @@ void destroy_context(hx_context &c)
     cudaFree(c.t.primes);
     cudaFree(c.t.tw_fwd);
     cudaFree(c.t.tw_inv);
+    cudaFree(c.t.fold);
+    cudaFree(c.t.ftw_fwd);
+    cudaFree(c.t.ftw_inv);
     cudaFree(c.t.modup);
     cudaFree(c.t.moddown);
     cudaFree(c.t.relin_rs);

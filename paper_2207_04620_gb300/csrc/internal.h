@@ -11,6 +11,7 @@
 
 #include "../../include/hx.h"
 #include "modarith.cuh"
+#include "modfold.cuh"
 
 namespace hx {
 
@@ -110,6 +111,10 @@ struct DeviceTables {
     PrimeConst *primes = nullptr;   // [n_all]
     ulonglong2 *tw_fwd = nullptr;   // [n_all][N] (psi^brv(k), Shoup)
     ulonglong2 *tw_inv = nullptr;   // [n_all][N] (psi^-brv(k), Shoup)
+    // the same for fold arithmetic; null unless every prime of the chain allows it
+    FoldPrime *fold = nullptr;      // [n_all]
+    int4 *ftw_fwd = nullptr;        // [n_all][N] psi^brv(k)
+    int4 *ftw_inv = nullptr;        // [n_all][N] psi^-brv(k)
     ConvTable *modup = nullptr;     // [(n_q+1) * dnum] by (limbs, digit)
     ModDownTable *moddown = nullptr;// [n_q+1] by limbs
     RescaleTable *rescale = nullptr;// [n_q+1] by limbs
@@ -153,6 +158,8 @@ struct NttJob {
     uint64_t *data;
     const PrimeConst *primes;
     const ulonglong2 *tw_fwd, *tw_inv;
+    const FoldPrime *fold;            // null: the ring has no fold tables
+    const int4 *ftw_fwd, *ftw_inv;
     int log_n, n_rows, n_limbs;
     int tile0_cols, tile0_rows;  // filled by the launcher
     int16_t prime[64];
@@ -254,8 +261,19 @@ void launch_moddown_jobs(cudaStream_t s, const ModDownJob *jobs, int n_jobs, lon
 // the NTT over several rings in two steps: tile offsets of every job (host), then the two phase
 // launches over a job table already on the device
 void plan_ntt_jobs(std::vector<NttJob> &jobs, int *tiles_cols, int *tiles_rows);
-void launch_ntt_jobs(cudaStream_t s, const NttJob *jobs, int n_jobs, int tiles_cols, int tiles_rows, bool inverse,
-                     int n_sm, std::atomic<uint64_t> *launches);
+// fold: every job's ring has fold tables
+void launch_ntt_jobs(cudaStream_t s, const NttJob *jobs, int n_jobs, int tiles_cols, int tiles_rows, bool fold,
+                     bool inverse, int n_sm, std::atomic<uint64_t> *launches);
+// the tables of a context that its NTT jobs carry
+inline void set_ntt_tables(NttJob &j, const DeviceTables &t)
+{
+    j.primes = t.primes;
+    j.tw_fwd = t.tw_fwd;
+    j.tw_inv = t.tw_inv;
+    j.fold = t.fold;
+    j.ftw_fwd = t.ftw_fwd;
+    j.ftw_inv = t.ftw_inv;
+}
 void launch_lintrans_mac(const LaunchCtx &c, const MacArgs &a, int B, int limbs, int n_terms);
 // two hoisted rotations selected by a mask in the extended basis (see kernels.cu)
 void launch_key_ip_mux(const LaunchCtx &c, View out, const uint64_t *D, const uint64_t *dnt, size_t dnt_bstride,

@@ -1,0 +1,82 @@
+// Modular products for primes just below a power of two: q = 2^b - d with 33 <= b <= 60 and a
+// small d (the chain takes the largest primes below 2^b, so d is a few hundred multiples of 2N).
+//
+// A constant w (a twiddle) is held as four 32-bit numbers: the centred residues of w and of
+// 2^32 w, each split at bit c = b - 32 into a signed 32-bit head and a centred tail of c bits.
+// For a signed 64-bit y = 2^32 yh + yl (yl signed), w y = yl w + yh (2^32 w) mod q is
+//
+//     2^c (yl w_head + yh v_head) + (yl w_tail + yh v_tail),      v = 2^32 w mod q
+//
+// four 32x32 -> 64-bit multiply-adds with no carries between them.  The split at b - 32 makes
+// the first sum's high word the quotient by 2^b as it stands (2^c times 2^32): with
+// A = 2^32 t + a, 2^c A = 2^b t + 2^c a = d t + 2^c a mod q, one more multiply-add.  Five in all,
+// against ten multiplications of a Shoup product (y w - floor(y w' / 2^64) q).  The result is
+// signed: |r| <= 1.5 2^b + 2^31 d.
+//
+// Values stay signed and unreduced through several butterflies; fold() brings one back to
+// about [0, 2^b) with one multiply-add: v = 2^b h + l = l + d h.  FoldBounds (host) proves for a
+// prime that no sum leaves 64 bits and how many folds the final reduction takes; chains with a
+// prime outside its range use the Shoup kernels.
+#pragma once
+#include <cstdint>
+
+namespace hx {
+
+struct FoldPrime {
+    uint64_t q;
+    int c;         // b - 32
+    int d;         // 2^b - q
+    int mask;      // 2^c - 1: the high word's bits below 2^b
+    int refold;    // != 0: the final reduction folds twice
+    int4 n_inv;    // N^-1 mod q as a constant
+    int4 n_inv_w1; // N^-1 * psi^-brv(1) mod q: the last inverse stage's twiddle with N^-1 folded in
+};
+
+// bounds in sixteenths of the unit u of a prime (u >= 2^b): a folded value, a product, the limit
+constexpr int kFoldSettled = 17, kFoldProduct = 25, kFoldLimit = 127;
+
+#ifdef __CUDACC__
+__device__ __forceinline__ int64_t mad_wide(int a, int b, int64_t c)
+{
+    int64_t r;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ int64_t mul_wide(int a, int b)
+{
+    int64_t r;
+    asm("mul.wide.s32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
+    return r;
+}
+
+// y w mod q, |result| <= 1.5 2^b + 2^31 d, for |y| < 2^63 - 2^32
+__device__ __forceinline__ int64_t fold_mul(int64_t y, const int4 w, const FoldPrime &P)
+{
+    const int yl = (int)y, yh = (int)(y >> 32) + (int)((unsigned)yl >> 31);
+    const int64_t A = mad_wide(yh, w.y, mul_wide(yl, w.x));
+    int64_t B = mad_wide(yh, w.w, mul_wide(yl, w.z));
+    B = mad_wide((int)(A >> 32), P.d, B);
+    return B + (int64_t)((uint64_t)(uint32_t)A << P.c);
+}
+
+// v mod q within 2^b + (|v| / 2^b + 1) d, negative by at most the second term
+__device__ __forceinline__ int64_t fold(int64_t v, const FoldPrime &P)
+{
+    const int vh = (int)(v >> 32);
+    const int64_t l = (int64_t)(((uint64_t)(uint32_t)(vh & P.mask) << 32) | (uint32_t)v);
+    return mad_wide(vh >> P.c, P.d, l);
+}
+
+// v mod q in [0, q)
+__device__ __forceinline__ uint64_t fold_finish(int64_t v, const FoldPrime &P)
+{
+    v = fold(v, P);
+    if (P.refold) v = fold(v, P);
+    const int64_t q = (int64_t)P.q;
+    if (v < 0) v += q;
+    else if (v >= q) v -= q;
+    return (uint64_t)v;
+}
+#endif
+
+} // namespace hx
