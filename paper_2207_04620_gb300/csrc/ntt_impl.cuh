@@ -23,6 +23,7 @@ struct ArithShoup {
     typedef PrimeConst Prime;
     typedef ulonglong2 Tw;
     static constexpr bool kTracked = false;
+    static constexpr int kThreadsPerSm = 768;  // at most 85 registers a thread
     static __device__ __forceinline__ void ct(uint64_t &x, uint64_t &y, const Tw w, const Prime &P)
     {
         const uint64_t two_q = 2 * P.q;
@@ -56,10 +57,6 @@ struct ArithShoup {
     {
         return csub(csub(v, 2 * P.q), P.q);
     }
-    static __device__ __forceinline__ uint64_t times_n_inv(uint64_t v, const Prime &P)
-    {
-        return shoup(v, P.n_inv, P.n_inv_sh, P.q);
-    }
     static const Prime *primes(const DeviceTables &t) { return t.primes; }
     static const Tw *twiddles(const DeviceTables &t, bool inv) { return inv ? t.tw_inv : t.tw_fwd; }
     static __device__ __forceinline__ const Prime *job_primes(const NttJob &J) { return J.primes; }
@@ -74,11 +71,13 @@ struct ArithShoup {
 // so a radix-16 pass of the forward transform folds none of its 64 sums and the inverse one a few.
 //
 // The butterflies set the transform's time, so this is where it was won: 1600 limbs of N = 2^14
-// took 332 us forward and 348 us inverse with Shoup butterflies and take 261 and 269 us.
+// take 215 us forward and 223 us inverse against 274 and 283 with Shoup butterflies in the same
+// tiles (8.5e11 butterflies/s; the five multiply-adds alone allow 2.0e12).
 struct ArithFold {
     typedef FoldPrime Prime;
     typedef int4 Tw;
     static constexpr bool kTracked = true;
+    static constexpr int kThreadsPerSm = 1024;  // at most 64 registers a thread
     static __device__ __forceinline__ void ct(uint64_t &x, uint64_t &y, const Tw w, const Prime &P)
     {
         const uint64_t t = (uint64_t)fold_mul((int64_t)y, w, P), a = x;
@@ -99,10 +98,6 @@ struct ArithFold {
     }
     static __device__ __forceinline__ uint64_t settle(uint64_t v, const Prime &P) { return (uint64_t)fold((int64_t)v, P); }
     static __device__ __forceinline__ uint64_t finish(uint64_t v, const Prime &P) { return fold_finish((int64_t)v, P); }
-    static __device__ __forceinline__ uint64_t times_n_inv(uint64_t v, const Prime &P)
-    {
-        return fold_finish(fold_mul((int64_t)v, P.n_inv, P), P);
-    }
     static const Prime *primes(const DeviceTables &t) { return t.fold; }
     static const Tw *twiddles(const DeviceTables &t, bool inv) { return inv ? t.ftw_inv : t.ftw_fwd; }
     static __device__ __forceinline__ const Prime *job_primes(const NttJob &J) { return J.fold; }
@@ -124,6 +119,21 @@ namespace {
 // back.  Global stage of local stage s is g0 + s; the twiddle of a butterfly
 // at global stage G on global element j is tw[2^G + (j >> (log N - G))].
 
+// two adjacent twiddles, 32-byte aligned (their tables are)
+template <class Tw> __device__ __forceinline__ void load_pair(const Tw *p, Tw &a, Tw &b)
+{
+    static_assert(sizeof(Tw) == 16, "16-byte twiddles");
+    union {
+        uint64_t w[4];
+        Tw t[2];
+    } u;
+    asm("ld.global.nc.v4.u64 {%0, %1, %2, %3}, [%4];"
+        : "=l"(u.w[0]), "=l"(u.w[1]), "=l"(u.w[2]), "=l"(u.w[3])
+        : "l"(p));
+    a = u.t[0];
+    b = u.t[1];
+}
+
 // R stages in registers.  IN: the inputs' bound in sixteenths (tracked arithmetic).  A forward sum
 // x +- w y only bounds x: y may reach the limit.  An inverse sum folds the larger operand first
 // where it would pass the limit.  SCALE: the inverse's stage 0 applies N^-1 and finishes.
@@ -140,10 +150,14 @@ __device__ __forceinline__ void ntt_stages(uint64_t (&v)[1 << R], const typename
         const int vv = INV ? R - 1 - step : step;
         const int s = S0 + vv, half = RR >> (vv + 1);
         const int tbase = (1 << (g0 + s)) + (blk << s) + (hi << vv);
+        typename A::Tw ws[2];
 #pragma unroll
         for (int gl = 0; gl < (1 << vv); gl++) {
             const bool scale = SCALE && vv == 0;
-            const typename A::Tw w = scale ? typename A::Tw() : tw[tbase + gl];
+            if (scale) ws[0] = typename A::Tw();
+            else if (vv == 0) ws[0] = tw[tbase];  // from the second stage of a pass on, pairs (32 bytes, aligned)
+            else if (gl % 2 == 0) load_pair(tw + tbase + gl, ws[0], ws[1]);
+            const typename A::Tw w = ws[gl % 2];
 #pragma unroll
             for (int j = 0; j < half; j++) {
                 const int ix = gl * 2 * half + j, iy = ix + half;
@@ -172,61 +186,6 @@ __device__ __forceinline__ void ntt_stages(uint64_t (&v)[1 << R], const typename
     }
 }
 
-// One register pass in place in shared memory.  SETTLE: leave folded values (every pass but the
-// last, whose results go through finish())
-template <class A, int L, int R, int S0, bool INV, bool KFAST, bool PAD, int IN, bool SETTLE = true>
-__device__ __forceinline__ void ntt_pass(uint64_t *sh, int n_sub, int sk, int se,
-                                         const typename A::Tw *__restrict__ tw, int g0, int blk0, int blk_step,
-                                         const typename A::Prime &P, int nthr)
-{
-    constexpr int M = 1 << L, RR = 1 << R, TL = M >> (S0 + R), ITEMS = M >> R;
-    for (int w = threadIdx.x; w < ITEMS * n_sub; w += nthr) {
-        const int k = KFAST ? w % n_sub : w / ITEMS;
-        const int u = KFAST ? w / n_sub : w % ITEMS;
-        const int hi = u / TL, lo = u % TL;
-        const int base = hi * TL * RR + lo;
-        const int blk = blk0 + k * blk_step;
-        uint64_t v[RR];
-#pragma unroll
-        for (int m = 0; m < RR; m++) {
-            const int e = base + m * TL;
-            v[m] = sh[k * sk + e * se + (PAD ? 2 * (e >> 4) : 0)];
-        }
-        ntt_stages<A, R, S0, INV, IN>(v, tw, g0, blk, hi, P);
-#pragma unroll
-        for (int m = 0; m < RR; m++) {
-            const int e = base + m * TL;
-            sh[k * sk + e * se + (PAD ? 2 * (e >> 4) : 0)] = SETTLE ? A::settle(v[m], P) : v[m];
-        }
-    }
-}
-
-// The column phase's last register pass, its results stored straight to global memory (word e
-// of column k at dst + e*N2 + k): consecutive threads hold consecutive columns, so each warp
-// store covers whole COLS-word row segments and the phase needs no shared-memory round trip
-// for its output.  Forward: outputs stay lazy for the row phase.  Inverse: the pass
-// ends with stage 0, whose butterfly also applies N^-1 -- x' = (x+y) N^-1 and
-// y' = (x-y) psi^-brv(1) N^-1, one product each instead of a butterfly product and two
-// scalings -- and the outputs are fully reduced.
-template <class A, int LOGM, int R, int S0, int COLS, bool INV>
-__device__ __forceinline__ void ntt_pass_out(const uint64_t *sh, const typename A::Tw *__restrict__ tw,
-                                             const typename A::Prime &P, uint64_t *dst, int N2, int nthr)
-{
-    constexpr int M = 1 << LOGM, RR = 1 << R, TL = M >> (S0 + R), ITEMS = M >> R;
-    for (int w = threadIdx.x; w < ITEMS * COLS; w += nthr) {
-        const int k = w % COLS, u = w / COLS;
-        const int hi = u / TL, lo = u % TL;
-        const int base = hi * TL * RR + lo;
-        uint64_t v[RR];
-#pragma unroll
-        for (int m = 0; m < RR; m++) v[m] = sh[k + (base + m * TL) * COLS];
-        static_assert(!INV || S0 == 0, "the inverse output pass must end with stage 0");
-        ntt_stages<A, R, S0, INV, kFoldSettled, INV>(v, tw, 0, 0, hi, P);
-#pragma unroll
-        for (int m = 0; m < RR; m++) dst[(size_t)(base + m * TL) * N2 + k] = INV ? v[m] : A::settle(v[m], P);
-    }
-}
-
 // bounds of a transform's inputs in sixteenths (tracked arithmetic): below 4q forward, 2q inverse,
 // as the Shoup butterflies take them
 constexpr int kFwdIn = 64, kInvIn = 32;
@@ -237,21 +196,147 @@ template <int L, bool ALT = false> struct Split {
     static constexpr int R2 = L - R1;
 };
 
-// Asynchronous global->shared copies (cp.async): the next tile streams in while
-// the current one is transformed.
-__device__ __forceinline__ void cp_async8(void *smem, const void *gmem)
+// Where a tile's element e of sub-transform k lies, in its global rows and in shared memory, and
+// which sub-transform and butterfly group a work item w has.
+//
+// Columns: W adjacent columns, element e in row e; consecutive threads on consecutive columns, so
+// a warp moves whole 128-byte row segments and meets no bank twice.
+template <int L, int W, bool ALT> struct ColTile {
+    static constexpr bool kRows = false;
+    static constexpr int WORDS = (1 << L) * W;
+    int n2;
+    __device__ __forceinline__ static int sub(int w, int) { return w % W; }
+    __device__ __forceinline__ static int group(int w, int) { return w / W; }
+    __device__ __forceinline__ size_t global(int e, int k) const { return (size_t)e * n2 + k; }
+    __device__ __forceinline__ static int shared(int e, int k) { return e * W + k; }
+};
+// Rows: W contiguous blocks of M words.  The first pass of the stages takes elements 2^R2 apart
+// (runs of 2^R2 threads on consecutive words), the second 2^R2 consecutive ones; one spare word
+// per 2^R2 and a block stride of 2^R2 mod 16 words keep both on distinct banks.
+template <int L, int W, bool ALT> struct RowTile {
+    static constexpr bool kRows = true;
+    static constexpr int M = 1 << L, R2 = Split<L, ALT>::R2, RUN = 1 << R2;
+    static constexpr int DATA = M + (M >> R2), SK = DATA + ((RUN - DATA) % 16 + 16) % 16, WORDS = SK * W;
+    __device__ __forceinline__ static int sub(int w, int items) { return w / items; }
+    __device__ __forceinline__ static int group(int w, int items) { return w % items; }
+    __device__ __forceinline__ size_t global(int e, int k) const { return (size_t)k * M + e; }
+    __device__ __forceinline__ static int shared(int e, int k) { return k * SK + e + (e >> R2); }
+};
+
+// 32-byte global accesses (sm_100 and later), for 32-byte aligned addresses
+__device__ __forceinline__ void ld_global_32(const uint64_t *p, uint64_t &a, uint64_t &b, uint64_t &c, uint64_t &d)
 {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem));
+    asm volatile("ld.global.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p));
 }
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
+__device__ __forceinline__ void st_global_32(uint64_t *p, uint64_t a, uint64_t b, uint64_t c, uint64_t d)
 {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem));
+    asm volatile("st.global.v4.u64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-__device__ __forceinline__ void cp_async_wait_all_but_one() { asm volatile("cp.async.wait_group 1;\n" ::); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::); }
+
+// RR elements of a butterfly group, TL apart, from or to global memory; consecutive ones (TL = 1)
+// of a row in 16-byte pieces, or in 32-byte ones where the caller found the rows aligned (wide)
+template <class Tile, int RR, int TL>
+__device__ __forceinline__ void load_group(uint64_t (&v)[RR], const uint64_t *src, const Tile &t, int base, int k, bool wide)
+{
+    if (Tile::kRows && TL == 1) {
+        const uint64_t *p = src + t.global(base, k);
+        if (wide) {
+#pragma unroll
+            for (int m = 0; m < RR; m += 4) ld_global_32(p + m, v[m], v[m + 1], v[m + 2], v[m + 3]);
+        } else {
+#pragma unroll
+            for (int m = 0; m < RR; m += 2) {
+                const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(p + m);
+                v[m] = x.x;
+                v[m + 1] = x.y;
+            }
+        }
+    } else {
+#pragma unroll
+        for (int m = 0; m < RR; m++) v[m] = src[t.global(base + m * TL, k)];
+    }
+}
+template <class Tile, int RR, int TL>
+__device__ __forceinline__ void store_group(const uint64_t (&v)[RR], uint64_t *dst, const Tile &t, int base, int k, bool wide)
+{
+    if (Tile::kRows && TL == 1) {
+        uint64_t *p = dst + t.global(base, k);
+        if (wide) {
+#pragma unroll
+            for (int m = 0; m < RR; m += 4) st_global_32(p + m, v[m], v[m + 1], v[m + 2], v[m + 3]);
+        } else {
+#pragma unroll
+            for (int m = 0; m < RR; m += 2)
+                *reinterpret_cast<ulonglong2 *>(p + m) = make_ulonglong2(v[m], v[m + 1]);
+        }
+    } else {
+#pragma unroll
+        for (int m = 0; m < RR; m++) dst[t.global(base + m * TL, k)] = v[m];
+    }
+}
+
+// A phase's two register passes over one tile with one shared-memory exchange: the first pass
+// takes its elements straight from global memory, the second stores its results straight there.
+// No tile is staged ahead: a block holds its tile once (16 or 19 KB at width 16), so eight blocks
+// of 128 threads share an SM and cover each other's loads.
+//
+// Forward: columns leave lazy (folded) values for the row phase, rows finish.  Inverse: rows leave
+// lazy values; the column phase ends with stage 0, whose butterfly also applies N^-1 --
+// x' = (x+y) N^-1 and y' = (x-y) psi^-brv(1) N^-1, one product each instead of a butterfly product
+// and two scalings -- and finishes.
+template <class A, class Tile, int L, int R, int S0, bool INV, bool FIRST, int IN>
+__device__ __forceinline__ void ntt_pass(uint64_t *sh, const uint64_t *src, uint64_t *dst, const Tile &tile, int n_sub,
+                                         const typename A::Tw *__restrict__ tw, int g0, int blk0, int blk_step,
+                                         const typename A::Prime &P, int nthr, bool wide)
+{
+    constexpr int M = 1 << L, RR = 1 << R, TL = M >> (S0 + R), ITEMS = M >> R;
+    constexpr bool kScale = INV && !FIRST && !Tile::kRows;  // the pass that applies N^-1
+    for (int w = threadIdx.x; w < ITEMS * n_sub; w += nthr) {
+        const int k = Tile::sub(w, ITEMS), u = Tile::group(w, ITEMS);
+        const int hi = u / TL, lo = u % TL;
+        const int base = hi * TL * RR + lo;
+        uint64_t v[RR];
+        if (FIRST) {
+            load_group<Tile, RR, TL>(v, src, tile, base, k, wide);
+        } else {
+#pragma unroll
+            for (int m = 0; m < RR; m++) v[m] = sh[Tile::shared(base + m * TL, k)];
+        }
+        ntt_stages<A, R, S0, INV, IN, kScale>(v, tw, g0, blk0 + k * blk_step, hi, P);
+        if (!kScale) {
+#pragma unroll
+            for (int m = 0; m < RR; m++)
+                v[m] = (!INV && !FIRST && Tile::kRows) ? A::finish(v[m], P) : A::settle(v[m], P);
+        }
+        if (FIRST) {
+#pragma unroll
+            for (int m = 0; m < RR; m++) sh[Tile::shared(base + m * TL, k)] = v[m];
+        } else {
+            store_group<Tile, RR, TL>(v, dst, tile, base, k, wide);
+        }
+    }
+}
+
+// one tile of a phase: src and dst at its first word (they may be the same)
+template <class A, class Tile, int L, int W, bool INV, bool ALT>
+__device__ __forceinline__ void ntt_tile(uint64_t *sh, const uint64_t *src, uint64_t *dst, const Tile &tile,
+                                         const typename A::Tw *__restrict__ tw, int g0, int blk0,
+                                         const typename A::Prime &P, int nthr, bool wide)
+{
+    constexpr int R1 = Split<L, ALT>::R1, R2 = Split<L, ALT>::R2;
+    constexpr int step = Tile::kRows ? 1 : 0;  // rows: every sub-transform has its own twiddles
+    if (!INV) {
+        ntt_pass<A, Tile, L, R1, 0, false, true, Tile::kRows ? kFoldSettled : kFwdIn>(sh, src, dst, tile, W, tw, g0, blk0,
+                                                                                       step, P, nthr, wide);
+        __syncthreads();
+        ntt_pass<A, Tile, L, R2, R1, false, false, kFoldSettled>(sh, src, dst, tile, W, tw, g0, blk0, step, P, nthr, wide);
+    } else {
+        ntt_pass<A, Tile, L, R2, R1, true, true, Tile::kRows ? kInvIn : kFoldSettled>(sh, src, dst, tile, W, tw, g0, blk0,
+                                                                                      step, P, nthr, wide);
+        __syncthreads();
+        ntt_pass<A, Tile, L, R1, 0, true, false, kFoldSettled>(sh, src, dst, tile, W, tw, g0, blk0, step, P, nthr, wide);
+    }
+}
 
 // tile t of a phase -> (group, row, position along the row)
 struct TileId {
@@ -267,131 +352,44 @@ __device__ __forceinline__ TileId tile_of(int t, int nb, int n_rows)
     return r;
 }
 
-// column phase: the first LOGM stages on M rows of stride N2 (COLS adjacent columns
-// per tile); each block loops over tiles with the next tile (and its twiddles,
-// indices below M) prefetched into the other half of shared memory
+// column phase: the first LOGM stages on M rows of stride N2, COLS adjacent columns per block
 template <class A, int LOGM, int COLS, bool INV, bool ALT>
-__global__ void __launch_bounds__((1 << (LOGM - Split<LOGM, ALT>::R1)) * COLS)
+__global__ void __launch_bounds__((1 << (LOGM - Split<LOGM, ALT>::R1)) * COLS,
+                                  A::kThreadsPerSm / ((1 << (LOGM - Split<LOGM, ALT>::R1)) * COLS))
 k_ntt_cols(const __grid_constant__ NttRows R, const typename A::Prime *__restrict__ primes,
-           const typename A::Tw *__restrict__ tw_all, int log_n, int n_tiles)
+           const typename A::Tw *__restrict__ tw_all, int log_n)
 {
-    constexpr int M = 1 << LOGM, E = M * COLS, R1 = Split<LOGM, ALT>::R1, R2 = Split<LOGM, ALT>::R2;
-    constexpr int T = (M >> R1) * COLS;
     extern __shared__ uint64_t sh[];
-    typename A::Tw *const stw = reinterpret_cast<typename A::Tw *>(sh + 2 * E);
-    const int N = 1 << log_n, N2 = N >> LOGM, nb = N2 / COLS;
-    auto prefetch = [&](int t, int slot) {
-        const TileId id = tile_of(t, nb, R.n_rows);
-        const int pr = R.prime[id.row];
-        const uint64_t *src = INV ? R.dst + (size_t)id.g * R.dst_gs + (size_t)R.dst_off[id.row] * N
-                                  : R.src + (size_t)id.g * R.src_gs + (size_t)R.src_off[id.row] * N;
-        const int c0 = id.bx * COLS;
-        for (int i = threadIdx.x; i < E / 2; i += T) {  // 16-byte pieces of COLS-word row segments
-            const int r = (2 * i) / COLS, c = (2 * i) % COLS;
-            cp_async16(sh + slot * E + 2 * i, src + (size_t)r * N2 + c0 + c);
-        }
-        const typename A::Tw *tw = tw_all + (size_t)pr * N;
-        for (int i = threadIdx.x; i < M; i += T) cp_async16(stw + slot * M + i, tw + i);
-        cp_async_commit();
-    };
-    int t = blockIdx.x, slot = 0;
-    if (t < n_tiles) prefetch(t, 0);
-    for (; t < n_tiles; t += gridDim.x, slot ^= 1) {
-        const int tn = t + gridDim.x;
-        if (tn < n_tiles) {
-            prefetch(tn, slot ^ 1);
-            cp_async_wait_all_but_one();
-        } else {
-            cp_async_wait_all();
-        }
-        __syncthreads();
-        const TileId id = tile_of(t, nb, R.n_rows);
-        const typename A::Prime P = primes[R.prime[id.row]];
-        uint64_t *dst = R.dst + (size_t)id.g * R.dst_gs + (size_t)R.dst_off[id.row] * N;
-        const int c0 = id.bx * COLS;
-        uint64_t *b = sh + slot * E;
-        const typename A::Tw *tws = stw + slot * M;
-        if (!INV) {
-            ntt_pass<A, LOGM, R1, 0, false, true, false, kFwdIn>(b, COLS, 1, COLS, tws, 0, 0, 0, P, T);
-            __syncthreads();
-            ntt_pass_out<A, LOGM, R2, R1, COLS, false>(b, tws, P, dst + c0, N2, T);
-        } else {
-            ntt_pass<A, LOGM, R2, R1, true, true, false, kFoldSettled>(b, COLS, 1, COLS, tws, 0, 0, 0, P, T);
-            __syncthreads();
-            ntt_pass_out<A, LOGM, R1, 0, COLS, true>(b, tws, P, dst + c0, N2, T);
-        }
-        __syncthreads();  // this half is refilled by the prefetch two tiles later
-    }
+    constexpr int T = (1 << (LOGM - Split<LOGM, ALT>::R1)) * COLS;
+    const int N = 1 << log_n, N2 = N >> LOGM;
+    const TileId id = tile_of(blockIdx.x, N2 / COLS, R.n_rows);
+    const int pr = R.prime[id.row];
+    const typename A::Prime P = primes[pr];
+    uint64_t *dst = R.dst + (size_t)id.g * R.dst_gs + (size_t)R.dst_off[id.row] * N + id.bx * COLS;
+    const uint64_t *src =
+        INV ? dst : R.src + (size_t)id.g * R.src_gs + (size_t)R.src_off[id.row] * N + id.bx * COLS;
+    ntt_tile<A, ColTile<LOGM, COLS, ALT>, LOGM, COLS, INV, ALT>(sh, src, dst, ColTile<LOGM, COLS, ALT>{N2},
+                                                                tw_all + (size_t)pr * N, 0, 0, P, T, false);
 }
 
-// row phase: the remaining LOGM stages on ROWS contiguous blocks of M words per tile
-// (padded layout, one spare word per 16), next tile prefetched in 8-byte pieces
+// row phase: the remaining LOGM stages on ROWS contiguous blocks of M words
 template <class A, int LOGM, int ROWS, bool INV, bool ALT>
-__global__ void __launch_bounds__((1 << (LOGM - Split<LOGM, ALT>::R1)) * ROWS)
+__global__ void __launch_bounds__((1 << (LOGM - Split<LOGM, ALT>::R1)) * ROWS,
+                                  A::kThreadsPerSm / ((1 << (LOGM - Split<LOGM, ALT>::R1)) * ROWS))
 k_ntt_rows(const __grid_constant__ NttRows R, const typename A::Prime *__restrict__ primes,
-           const typename A::Tw *__restrict__ tw_all, int log_n, int n_tiles)
+           const typename A::Tw *__restrict__ tw_all, int log_n, bool wide)
 {
-    constexpr int M = 1 << LOGM, E = M * ROWS, R1 = Split<LOGM, ALT>::R1, R2 = Split<LOGM, ALT>::R2;
-    constexpr int T = (M >> R1) * ROWS;
-    constexpr int SK = M + M / 8;  // padded block stride (two spare words per 16)
     extern __shared__ uint64_t sh[];
+    constexpr int T = (1 << (LOGM - Split<LOGM, ALT>::R1)) * ROWS;
     const int N = 1 << log_n;
-    const int g0 = log_n - LOGM;
-    const int nb = (N >> LOGM) / ROWS;
-    auto prefetch = [&](int t, int slot) {
-        const TileId id = tile_of(t, nb, R.n_rows);
-        const uint64_t *src = INV ? R.src + (size_t)id.g * R.src_gs + (size_t)R.src_off[id.row] * N
-                                  : R.dst + (size_t)id.g * R.dst_gs + (size_t)R.dst_off[id.row] * N;
-        const size_t base = (size_t)id.bx * ROWS * M;
-        for (int i = threadIdx.x; i < E / 2; i += T) {  // 16-byte pieces: pairs stay in one padding group
-            const int k = (2 * i) / M, e = (2 * i) % M;
-            cp_async16(sh + slot * ROWS * SK + k * SK + e + 2 * (e >> 4), src + base + 2 * i);
-        }
-        cp_async_commit();
-    };
-    int t = blockIdx.x, slot = 0;
-    if (t < n_tiles) prefetch(t, 0);
-    for (; t < n_tiles; t += gridDim.x, slot ^= 1) {
-        const int tn = t + gridDim.x;
-        if (tn < n_tiles) {
-            prefetch(tn, slot ^ 1);
-            cp_async_wait_all_but_one();
-        } else {
-            cp_async_wait_all();
-        }
-        __syncthreads();
-        const TileId id = tile_of(t, nb, R.n_rows);
-        const int pr = R.prime[id.row];
-        const typename A::Prime P = primes[pr];
-        const typename A::Tw *tw = tw_all + (size_t)pr * N;
-        uint64_t *dst = R.dst + (size_t)id.g * R.dst_gs + (size_t)R.dst_off[id.row] * N;
-        const int r_base = id.bx * ROWS;
-        const size_t base = (size_t)r_base * M;
-        uint64_t *b = sh + slot * ROWS * SK;
-        if (!INV) {
-            ntt_pass<A, LOGM, R1, 0, false, false, true, kFoldSettled>(b, ROWS, SK, 1, tw, g0, r_base, 1, P, T);
-            __syncthreads();
-            ntt_pass<A, LOGM, R2, R1, false, false, true, kFoldSettled, false>(b, ROWS, SK, 1, tw, g0, r_base, 1, P, T);
-            __syncthreads();
-            for (int i = threadIdx.x; i < E / 2; i += T) {  // pairs (e even, e+1) share a padding group
-                const int k = (2 * i) / M, e = (2 * i) % M;
-                const int sidx = k * SK + e + 2 * (e >> 4);
-                *reinterpret_cast<ulonglong2 *>(dst + base + 2 * i) =
-                    make_ulonglong2(A::finish(b[sidx], P), A::finish(b[sidx + 1], P));
-            }
-        } else {
-            ntt_pass<A, LOGM, R2, R1, true, false, true, kInvIn>(b, ROWS, SK, 1, tw, g0, r_base, 1, P, T);
-            __syncthreads();
-            ntt_pass<A, LOGM, R1, 0, true, false, true, kFoldSettled>(b, ROWS, SK, 1, tw, g0, r_base, 1, P, T);
-            __syncthreads();
-            for (int i = threadIdx.x; i < E / 2; i += T) {
-                const int k = (2 * i) / M, e = (2 * i) % M;
-                const int sidx = k * SK + e + 2 * (e >> 4);
-                *reinterpret_cast<ulonglong2 *>(dst + base + 2 * i) = make_ulonglong2(b[sidx], b[sidx + 1]);
-            }
-        }
-        __syncthreads();
-    }
+    const TileId id = tile_of(blockIdx.x, (N >> LOGM) / ROWS, R.n_rows);
+    const int pr = R.prime[id.row], r_base = id.bx * ROWS;
+    const typename A::Prime P = primes[pr];
+    uint64_t *dst = R.dst + (size_t)id.g * R.dst_gs + (size_t)R.dst_off[id.row] * N + ((size_t)r_base << LOGM);
+    const uint64_t *src =
+        INV ? R.src + (size_t)id.g * R.src_gs + (size_t)R.src_off[id.row] * N + ((size_t)r_base << LOGM) : dst;
+    ntt_tile<A, RowTile<LOGM, ROWS, ALT>, LOGM, ROWS, INV, ALT>(sh, src, dst, RowTile<LOGM, ROWS, ALT>{},
+                                                                tw_all + (size_t)pr * N, log_n - LOGM, r_base, P, T, wide);
 }
 
 // tile widths the autotuner chooses from (sub-transforms per block); a variant is a width index
@@ -401,50 +399,38 @@ constexpr const int *kNttTiles = kNttTileWidths;
 template <class A, int LOGM, int COLS, bool INV, bool ALT>
 void ntt_cols_w(const LaunchCtx &c, const NttRows &rows)
 {
-    constexpr int M = 1 << LOGM;
-    constexpr int E = M * COLS;
-    constexpr int T = (M >> Split<LOGM, ALT>::R1) * COLS;
+    constexpr int T = (1 << (LOGM - Split<LOGM, ALT>::R1)) * COLS;
     const int N2 = c.N >> LOGM;
     HX_CHECK(N2 % COLS == 0, HX_EINVAL, "NTT tile wider than the ring");
     const long long n_tiles = (long long)(N2 / COLS) * rows.n_rows * rows.n_groups;
     HX_CHECK(n_tiles < (1ll << 31), HX_EINVAL, "NTT batch too large");
-    const size_t smem = (size_t)E * 16 + (size_t)M * 32;  // two tiles + two twiddle sets
+    const size_t smem = sizeof(uint64_t) * ColTile<LOGM, COLS, ALT>::WORDS;
     static const bool attr =  // thread-safe one-time setup
         cudaFuncSetAttribute(k_ntt_cols<A, LOGM, COLS, INV, ALT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem) == cudaSuccess;
     (void)attr;
-    static const int per_sm = [&] {
-        int v = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_ntt_cols<A, LOGM, COLS, INV, ALT>, T, smem);
-        return v;
-    }();
-    const int grid = (int)std::min<long long>(n_tiles, (long long)std::max(1, per_sm) * c.t->n_sm);
-    k_ntt_cols<A, LOGM, COLS, INV, ALT><<<grid, T, smem, c.stream>>>(rows, A::primes(*c.t), A::twiddles(*c.t, INV), c.log_n,
-                                                                 (int)n_tiles);
+    k_ntt_cols<A, LOGM, COLS, INV, ALT><<<(unsigned)n_tiles, T, smem, c.stream>>>(rows, A::primes(*c.t),
+                                                                                 A::twiddles(*c.t, INV), c.log_n);
 }
 
 template <class A, int LOGM, int ROWS, bool INV, bool ALT>
 void ntt_rows_w(const LaunchCtx &c, const NttRows &rows)
 {
-    constexpr int M = 1 << LOGM;
-    constexpr int T = (M >> Split<LOGM, ALT>::R1) * ROWS;
+    constexpr int T = (1 << (LOGM - Split<LOGM, ALT>::R1)) * ROWS;
     const int N1 = c.N >> LOGM;
     HX_CHECK(N1 % ROWS == 0, HX_EINVAL, "NTT tile wider than the ring");
     const long long n_tiles = (long long)(N1 / ROWS) * rows.n_rows * rows.n_groups;
     HX_CHECK(n_tiles < (1ll << 31), HX_EINVAL, "NTT batch too large");
-    const size_t smem = (size_t)ROWS * (M + M / 8) * 16;  // two tiles
+    const size_t smem = sizeof(uint64_t) * RowTile<LOGM, ROWS, ALT>::WORDS;
     static const bool attr =  // thread-safe one-time setup
         cudaFuncSetAttribute(k_ntt_rows<A, LOGM, ROWS, INV, ALT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem) == cudaSuccess;
     (void)attr;
-    static const int per_sm = [&] {
-        int v = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_ntt_rows<A, LOGM, ROWS, INV, ALT>, T, smem);
-        return v;
-    }();
-    const int grid = (int)std::min<long long>(n_tiles, (long long)std::max(1, per_sm) * c.t->n_sm);
-    k_ntt_rows<A, LOGM, ROWS, INV, ALT><<<grid, T, smem, c.stream>>>(rows, A::primes(*c.t), A::twiddles(*c.t, INV), c.log_n,
-                                                                 (int)n_tiles);
+    // rows and blocks are multiples of 32 bytes: 32-byte pieces need only the bases and group strides aligned
+    const bool wide = ((reinterpret_cast<uintptr_t>(rows.src) | reinterpret_cast<uintptr_t>(rows.dst) |
+                        (rows.src_gs | rows.dst_gs) * sizeof(uint64_t)) & 31) == 0;
+    k_ntt_rows<A, LOGM, ROWS, INV, ALT><<<(unsigned)n_tiles, T, smem, c.stream>>>(
+        rows, A::primes(*c.t), A::twiddles(*c.t, INV), c.log_n, wide);
 }
 
 template <class A, bool INV, int LOGM, bool ALT>
@@ -488,9 +474,7 @@ namespace {
 
 // ---- several rings in one launch ------------------------------------------------
 // A job is n_rows rows of one ring (its own N, primes and twiddles), transformed
-// in place.  One persistent kernel per phase walks the tiles of every job, the
-// next tile (and for the column phase its twiddles) streaming into the other
-// half of shared memory while the current one is transformed; a tile's phase
+// in place.  One kernel per phase takes the tiles of every job; a tile's phase
 // size picks the template instance, with the tile width chosen so every
 // instance runs 128 threads.
 
@@ -498,8 +482,12 @@ constexpr int kMultiT = 128;
 template <int LOGM> struct MultiW {  // tile width per phase size: (M >> R1) * W = 128 threads
     static constexpr int W = kMultiT / ((1 << LOGM) >> Split<LOGM>::R1);
 };
-constexpr int kMultiColsBuf = 2048 + 2 * 256;  // words: the largest column tile and its twiddles
-constexpr int kMultiRowsBuf = 8 * (256 + 32);  // words: the largest padded row tile
+constexpr int max4(int a, int b, int c, int d) { return std::max(std::max(a, b), std::max(c, d)); }
+// words of the largest tile
+constexpr int kMultiColsBuf = max4(ColTile<5, MultiW<5>::W, false>::WORDS, ColTile<6, MultiW<6>::W, false>::WORDS,
+                                   ColTile<7, MultiW<7>::W, false>::WORDS, ColTile<8, MultiW<8>::W, false>::WORDS);
+constexpr int kMultiRowsBuf = max4(RowTile<5, MultiW<5>::W, false>::WORDS, RowTile<6, MultiW<6>::W, false>::WORDS,
+                                   RowTile<7, MultiW<7>::W, false>::WORDS, RowTile<8, MultiW<8>::W, false>::WORDS);
 
 template <class A> struct MultiTile {
     uint64_t *row;
@@ -534,137 +522,51 @@ __device__ __forceinline__ MultiTile<A> multi_tile(const NttJob *jobs, int n_job
     return m;
 }
 
-template <class A, int LOGM>
-__device__ void multi_cols_load(uint64_t *b, const MultiTile<A> &m)
+template <class A, int LOGM, bool INV, bool COLS_PHASE>
+__device__ __forceinline__ void multi_run(uint64_t *sh, const MultiTile<A> &m, const typename A::Prime &P)
 {
-    constexpr int M = 1 << LOGM, COLS = MultiW<LOGM>::W, E = M * COLS;
-    const int N2 = (1 << m.log_n) >> LOGM, c0 = m.bx * COLS;
-    typename A::Tw *stw = reinterpret_cast<typename A::Tw *>(b + 2048);
-    for (int i = threadIdx.x; i < E / 2; i += kMultiT) {
-        const int r = (2 * i) / COLS, c = (2 * i) % COLS;
-        cp_async16(b + 2 * i, m.row + (size_t)r * N2 + c0 + c);
-    }
-    for (int i = threadIdx.x; i < M; i += kMultiT) cp_async16(stw + i, m.tw + i);
-}
-
-template <class A, int LOGM, bool INV>
-__device__ void multi_cols_run(uint64_t *b, const MultiTile<A> &m, const typename A::Prime &P)
-{
-    constexpr int M = 1 << LOGM, COLS = MultiW<LOGM>::W, E = M * COLS;
-    constexpr int R1 = Split<LOGM>::R1, R2 = Split<LOGM>::R2;
-    const int N2 = (1 << m.log_n) >> LOGM, c0 = m.bx * COLS;
-    const typename A::Tw *stw = reinterpret_cast<const typename A::Tw *>(b + 2048);
-    // the column phase's output pass of the one-ring kernels: results from registers to global memory
-    if (!INV) {
-        ntt_pass<A, LOGM, R1, 0, false, true, false, kFwdIn>(b, COLS, 1, COLS, stw, 0, 0, 0, P, kMultiT);
-        __syncthreads();
-        ntt_pass_out<A, LOGM, R2, R1, COLS, false>(b, stw, P, m.row + c0, N2, kMultiT);
+    constexpr int W = MultiW<LOGM>::W;
+    if (COLS_PHASE) {
+        typedef ColTile<LOGM, W, false> Tile;
+        uint64_t *d = m.row + m.bx * W;
+        ntt_tile<A, Tile, LOGM, W, INV, false>(sh, d, d, Tile{(1 << m.log_n) >> LOGM}, m.tw, 0, 0, P, kMultiT, false);
     } else {
-        ntt_pass<A, LOGM, R2, R1, true, true, false, kFoldSettled>(b, COLS, 1, COLS, stw, 0, 0, 0, P, kMultiT);
-        __syncthreads();
-        ntt_pass_out<A, LOGM, R1, 0, COLS, true>(b, stw, P, m.row + c0, N2, kMultiT);
-    }
-}
-
-template <class A, int LOGM>
-__device__ void multi_rows_load(uint64_t *b, const MultiTile<A> &m)
-{
-    constexpr int M = 1 << LOGM, ROWS = MultiW<LOGM>::W, E = M * ROWS, SK = M + M / 8;
-    const size_t base = (size_t)m.bx * ROWS * M;
-    for (int i = threadIdx.x; i < E; i += kMultiT) {
-        const int k = i / M, e = i % M;
-        cp_async8(b + k * SK + e + 2 * (e >> 4), m.row + base + i);
-    }
-}
-
-template <class A, int LOGM, bool INV>
-__device__ void multi_rows_run(uint64_t *b, const MultiTile<A> &m, const typename A::Prime &P)
-{
-    constexpr int M = 1 << LOGM, ROWS = MultiW<LOGM>::W, E = M * ROWS, SK = M + M / 8;
-    constexpr int R1 = Split<LOGM>::R1, R2 = Split<LOGM>::R2;
-    const int g0 = m.log_n - LOGM, r_base = m.bx * ROWS;
-    const size_t base = (size_t)r_base * M;
-    if (!INV) {
-        ntt_pass<A, LOGM, R1, 0, false, false, true, kFoldSettled>(b, ROWS, SK, 1, m.tw, g0, r_base, 1, P, kMultiT);
-        __syncthreads();
-        ntt_pass<A, LOGM, R2, R1, false, false, true, kFoldSettled, false>(b, ROWS, SK, 1, m.tw, g0, r_base, 1, P, kMultiT);
-        __syncthreads();
-        for (int i = threadIdx.x; i < E; i += kMultiT) {
-            const int k = i / M, e = i % M;
-            m.row[base + i] = A::finish(b[k * SK + e + 2 * (e >> 4)], P);
-        }
-    } else {
-        ntt_pass<A, LOGM, R2, R1, true, false, true, kInvIn>(b, ROWS, SK, 1, m.tw, g0, r_base, 1, P, kMultiT);
-        __syncthreads();
-        ntt_pass<A, LOGM, R1, 0, true, false, true, kFoldSettled>(b, ROWS, SK, 1, m.tw, g0, r_base, 1, P, kMultiT);
-        __syncthreads();
-        for (int i = threadIdx.x; i < E; i += kMultiT) {
-            const int k = i / M, e = i % M;
-            m.row[base + i] = b[k * SK + e + 2 * (e >> 4)];
-        }
+        typedef RowTile<LOGM, W, false> Tile;
+        const int r_base = m.bx * W;
+        uint64_t *d = m.row + ((size_t)r_base << LOGM);
+        const bool wide = (reinterpret_cast<uintptr_t>(d) & 31) == 0;
+        ntt_tile<A, Tile, LOGM, W, INV, false>(sh, d, d, Tile{}, m.tw, m.log_n - LOGM, r_base, P, kMultiT, wide);
     }
 }
 
 template <class A, bool INV, bool COLS_PHASE>
-__global__ void __launch_bounds__(kMultiT) k_ntt_multi(const NttJob *__restrict__ jobs, int n_jobs, int n_tiles)
+__global__ void __launch_bounds__(kMultiT, A::kThreadsPerSm / kMultiT)
+    k_ntt_multi(const NttJob *__restrict__ jobs, int n_jobs)
 {
     extern __shared__ uint64_t sh[];
-    constexpr int BUF = COLS_PHASE ? kMultiColsBuf : kMultiRowsBuf;
-    auto load = [&](const MultiTile<A> &m, int slot) {
-        uint64_t *b = sh + slot * BUF;
-        switch (m.logm) {
-        case 5: COLS_PHASE ? multi_cols_load<A, 5>(b, m) : multi_rows_load<A, 5>(b, m); break;
-        case 6: COLS_PHASE ? multi_cols_load<A, 6>(b, m) : multi_rows_load<A, 6>(b, m); break;
-        case 7: COLS_PHASE ? multi_cols_load<A, 7>(b, m) : multi_rows_load<A, 7>(b, m); break;
-        default: COLS_PHASE ? multi_cols_load<A, 8>(b, m) : multi_rows_load<A, 8>(b, m); break;
-        }
-        cp_async_commit();
-    };
-    int t = blockIdx.x, slot = 0;
-    MultiTile<A> cur{};
-    if (t < n_tiles) {
-        cur = multi_tile<A>(jobs, n_jobs, t, COLS_PHASE, INV);
-        load(cur, 0);
-    }
-    for (; t < n_tiles; t += gridDim.x, slot ^= 1) {
-        const int tn = t + gridDim.x;
-        MultiTile<A> nxt{};
-        if (tn < n_tiles) {
-            nxt = multi_tile<A>(jobs, n_jobs, tn, COLS_PHASE, INV);
-            load(nxt, slot ^ 1);
-            cp_async_wait_all_but_one();
-        } else {
-            cp_async_wait_all();
-        }
-        __syncthreads();
-        const typename A::Prime P = cur.primes[cur.pr];
-        uint64_t *b = sh + slot * BUF;
-        switch (cur.logm) {
-        case 5: COLS_PHASE ? multi_cols_run<A, 5, INV>(b, cur, P) : multi_rows_run<A, 5, INV>(b, cur, P); break;
-        case 6: COLS_PHASE ? multi_cols_run<A, 6, INV>(b, cur, P) : multi_rows_run<A, 6, INV>(b, cur, P); break;
-        case 7: COLS_PHASE ? multi_cols_run<A, 7, INV>(b, cur, P) : multi_rows_run<A, 7, INV>(b, cur, P); break;
-        default: COLS_PHASE ? multi_cols_run<A, 8, INV>(b, cur, P) : multi_rows_run<A, 8, INV>(b, cur, P); break;
-        }
-        __syncthreads();  // this half is refilled by the prefetch two tiles later
-        cur = nxt;
+    const MultiTile<A> m = multi_tile<A>(jobs, n_jobs, blockIdx.x, COLS_PHASE, INV);
+    const typename A::Prime P = m.primes[m.pr];
+    switch (m.logm) {
+    case 5: multi_run<A, 5, INV, COLS_PHASE>(sh, m, P); break;
+    case 6: multi_run<A, 6, INV, COLS_PHASE>(sh, m, P); break;
+    case 7: multi_run<A, 7, INV, COLS_PHASE>(sh, m, P); break;
+    default: multi_run<A, 8, INV, COLS_PHASE>(sh, m, P); break;
     }
 }
-
 
 } // namespace
 
 // both phases of the several-ring transform over a job table on the device
-template <class A> void ntt_multi_phases(cudaStream_t s, const NttJob *jp, int n_jobs, int tc, int tr, bool inverse, int n_sm)
+template <class A> void ntt_multi_phases(cudaStream_t s, const NttJob *jp, int n_jobs, int tc, int tr, bool inverse)
 {
-    // two halves of shared memory per block (current tile, next tile)
-    const size_t smem_c = 2 * sizeof(uint64_t) * kMultiColsBuf, smem_r = 2 * sizeof(uint64_t) * kMultiRowsBuf;
-    const int grid_c = std::min(tc, n_sm * 8), grid_r = std::min(tr, n_sm * 8);
+    constexpr size_t smem_c = sizeof(uint64_t) * kMultiColsBuf, smem_r = sizeof(uint64_t) * kMultiRowsBuf;
+    static_assert(smem_c <= 48 * 1024 && smem_r <= 48 * 1024, "a tile fits without an attribute");
     if (!inverse) {
-        k_ntt_multi<A, false, true><<<grid_c, kMultiT, smem_c, s>>>(jp, n_jobs, tc);
-        k_ntt_multi<A, false, false><<<grid_r, kMultiT, smem_r, s>>>(jp, n_jobs, tr);
+        k_ntt_multi<A, false, true><<<tc, kMultiT, smem_c, s>>>(jp, n_jobs);
+        k_ntt_multi<A, false, false><<<tr, kMultiT, smem_r, s>>>(jp, n_jobs);
     } else {
-        k_ntt_multi<A, true, false><<<grid_r, kMultiT, smem_r, s>>>(jp, n_jobs, tr);
-        k_ntt_multi<A, true, true><<<grid_c, kMultiT, smem_c, s>>>(jp, n_jobs, tc);
+        k_ntt_multi<A, true, false><<<tr, kMultiT, smem_r, s>>>(jp, n_jobs);
+        k_ntt_multi<A, true, true><<<tc, kMultiT, smem_c, s>>>(jp, n_jobs);
     }
 }
 
