@@ -282,11 +282,16 @@ int64_t hx_keyset_export_switch_key(const hx_keyset *ks, uint64_t galois, uint64
     need(cap >= words, "buffer too small");
     HX_CUDA(cudaDeviceSynchronize());
     HX_CUDA(cudaMemcpy(host, k->buf->p, words * 8, cudaMemcpyDeviceToHost));
-    // Montgomery form -> standard residues: x * 2^-64 mod q
+    // the inner product's form -> standard residues: split at bit 30 and times 2^60 with fold
+    // arithmetic, else times 2^64
+    const bool split = c.t.fold != nullptr;
     for (size_t r = 0; r < (size_t)c.dnum * 2 * c.n_all; r++) {
         const uint64_t q = c.primes[r % c.n_all];
-        const uint64_t rinv = hinv((uint64_t)(((u128)1 << 64) % q), q);
-        for (int j = 0; j < c.N; j++) host[r * c.N + j] = hmul(host[r * c.N + j], rinv, q);
+        const uint64_t rinv = hinv((uint64_t)(((u128)1 << (split ? 60 : 64)) % q), q);
+        for (int j = 0; j < c.N; j++) {
+            const uint64_t w = host[r * c.N + j];
+            host[r * c.N + j] = hmul(split ? (w & 0x3fffffffu) | ((w >> 32) << 30) : w, rinv, q);
+        }
     }
     return (int64_t)words;
     HX_END

@@ -200,6 +200,10 @@ void build_context(hx_context &c, const hx_params &p)
             fold[i].mask = (1 << (b - 32)) - 1;
             fold[i].n_inv = fold_constant(c.h_primes[i].n_inv, q, b);
             fold[i].n_inv_w1 = fold_constant(c.h_primes[i].n_inv_w1, q, b);
+            fold[i].r60 = fold_constant(((uint64_t)1 << 60) % q, q, b);
+            fold[i].q0 = (uint32_t)(q & (((uint64_t)1 << 30) - 1));
+            fold[i].q1 = (uint32_t)(q >> 30);
+            fold[i].minv = (uint32_t)(mont_neg_inv(q) & (((uint64_t)1 << 30) - 1));
             for (int k = 0; k < N; k++) {
                 ftwf[(size_t)i * N + k] = fold_constant(twf[(size_t)i * N + k].x, q, b);
                 ftwi[(size_t)i * N + k] = fold_constant(twi[(size_t)i * N + k].x, q, b);

@@ -225,6 +225,7 @@ struct KeyIpJob {
     const uint64_t *D, *dnt, *key;
     size_t dnt_bstride;
     const PrimeConst *primes;
+    const FoldPrime *fold;  // not null: split keys
     int n_all, n_q, K, alpha, limbs, ndig, log_n, few;
     uint64_t g;
     int gx, gy, gz;

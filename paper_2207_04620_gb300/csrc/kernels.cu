@@ -4,6 +4,7 @@
 // encryption pieces, aggregation and the ALU calibration.
 #include <algorithm>
 #include <cstdio>
+#include <type_traits>
 
 #include "launch_util.cuh"
 
@@ -14,12 +15,12 @@ namespace {
 __device__ __forceinline__ int brv_bits(unsigned x, int bits) { return (int)(__brev(x) >> (32 - bits)); }
 
 // index of the NTT slot that the automorphism X -> X^g brings to slot j:
-// 2brv(j')+1 = (2brv(j)+1)*g mod 2N
+// 2brv(j')+1 = (2brv(j)+1)*g mod 2N, in 32 bits (2N <= 2^17 divides 2^32).  Slots j and j ^ 1 have
+// exponents N apart, and g is odd, so the slot brought to j ^ 1 is j' ^ 1.
 __device__ __forceinline__ int galois_src(int j, uint64_t g, int log_n)
 {
-    const uint64_t two_n_mask = (2ull << log_n) - 1;
-    uint64_t e = ((2ull * (uint64_t)brv_bits(j, log_n) + 1) * g) & two_n_mask;
-    return brv_bits((unsigned)((e - 1) >> 1), log_n);
+    const uint32_t e = (2u * (uint32_t)brv_bits(j, log_n) + 1) * (uint32_t)g;
+    return brv_bits((e >> 1) & ((1u << log_n) - 1), log_n);
 }
 
 // A block's coordinates and its grid's extent: the hardware's, or those of one job inside a launch
@@ -418,6 +419,203 @@ __device__ __forceinline__ void key_ip_body(const Blk &b, View acc, const uint64
     }
 }
 
+// The key inner products of chains with fold arithmetic: keys lie split at bit 30 and times 2^60
+// (modfold.cuh), so a product is four multiply-adds without carries and an output one reduction.
+// Two adjacent outputs per thread (their gathered sources are a pair as well) and blockDim.y batch
+// entries per block: their threads read the same key words within a short time, so L2 delivers a
+// key once per block and not once per entry.  What is left is the latency of the source rows, so a
+// thread has every digit's words in flight at once: the kernels are instantiated by digit count.
+// 163 inner products of the 64x64 product batch (16 entries, 4 digits, 9-10 rows of N = 2^14) took
+// 8.9 ms with Montgomery products of whole words and take 6.9 ms (30 us against 42 for one key,
+// 46 against 60 for two).
+struct SplitIp {
+    const uint64_t *D, *dnt;  // ModUp digits [entry][digit][row][n]; the input's own NTT rows
+    size_t dnt_bstride;
+    int n_q, K, alpha, limbs, ndig, log_n;
+    __device__ __forceinline__ int prime(int t) const { return t < limbs ? t : n_q + (t - limbs); }
+};
+
+// row t of every digit of entry bi: the ModUp output, and the input itself for the digit that holds t
+struct SplitRows {
+    const uint64_t *p, *own;
+    size_t stride;
+    int own_digit;
+    __device__ __forceinline__ SplitRows(const SplitIp &A, int bi, int t)
+    {
+        const size_t n = (size_t)1 << A.log_n;
+        stride = (size_t)(A.limbs + A.K) * n;
+        p = A.D + (size_t)bi * A.ndig * stride + t * n;
+        own = A.dnt + bi * A.dnt_bstride + t * n;
+        own_digit = t < A.limbs ? t / A.alpha : -1;
+    }
+    __device__ __forceinline__ const uint64_t *row(int d) const { return d == own_digit ? own : p + d * stride; }
+};
+
+// sums (output half h, coefficient of the pair): += pair x of a row (.) the key halves at kd and kd + half
+__device__ __forceinline__ void split_mac(Sum30 (&a)[2], Sum30 (&b)[2], ulonglong2 x, const uint64_t *kd, size_t half)
+{
+    const ulonglong2 k0 = *reinterpret_cast<const ulonglong2 *>(kd);
+    const ulonglong2 k1 = *reinterpret_cast<const ulonglong2 *>(kd + half);
+    const uint32_t a0 = (uint32_t)x.x & kMask30, a1 = (uint32_t)(x.x >> 30);
+    const uint32_t b0 = (uint32_t)x.y & kMask30, b1 = (uint32_t)(x.y >> 30);
+    a[0].mac(a0, a1, k0.x);
+    b[0].mac(b0, b1, k0.y);
+    a[1].mac(a0, a1, k1.x);
+    b[1].mac(b0, b1, k1.y);
+}
+
+// before product `count` of every sum: room for it
+__device__ __forceinline__ void split_room(Sum30 (&a)[2], Sum30 (&b)[2], int count, const FoldPrime &P)
+{
+    if (count > 0 && count % kSumTerms == 0 && (count % (2 * kSumTerms) == 0 || P.c == 28))
+        a[0].spill(P), a[1].spill(P), b[0].spill(P), b[1].spill(P);
+}
+
+// sums over the digits of a row's gathered pair times a key; ND: the number of digits, 0 for any
+template <int ND>
+__device__ __forceinline__ void split_ip(Sum30 (&a)[2], Sum30 (&b)[2], const SplitRows &R, int ndig, int s,
+                                         const uint64_t *kd, size_t half, const FoldPrime &P)
+{
+    if (ND == 0) {
+        for (int d = 0; d < ndig; d++) {
+            const uint64_t *row = R.row(d);
+            split_room(a, b, d, P);
+            split_mac(a, b, make_ulonglong2(row[s], row[s ^ 1]), kd + 2 * d * half, half);
+        }
+        return;
+    }
+    ulonglong2 x[ND ? ND : 1];
+#pragma unroll
+    for (int d = 0; d < ND; d++) {
+        const uint64_t *row = R.row(d);
+        x[d] = make_ulonglong2(row[s], row[s ^ 1]);
+    }
+#pragma unroll
+    for (int d = 0; d < ND; d++) {
+        split_room(a, b, d, P);
+        split_mac(a, b, x[d], kd + 2 * d * half, half);
+    }
+}
+
+// entry bi, row t, outputs j and j + 1 (j even): both halves of sum_d src_d[galois] key_d
+template <int ND>
+__device__ __forceinline__ void key_ip_split_body(const SplitIp &A, View acc, const uint64_t *__restrict__ key,
+                                                  const FoldPrime &P, int n_all, uint64_t g, bool accumulate, int bi, int t,
+                                                  int j)
+{
+    const size_t n = (size_t)1 << A.log_n, half = (size_t)n_all * n;
+    const int s = g == 1 ? j : galois_src(j, g, A.log_n);
+    Sum30 a[2], b[2];
+    split_ip<ND>(a, b, SplitRows(A, bi, t), A.ndig, s, key + (size_t)A.prime(t) * n + j, half, P);
+    ulonglong2 *o0 = reinterpret_cast<ulonglong2 *>(acc.p + bi * acc.bstride + (size_t)t * n + j);
+    ulonglong2 *o1 = reinterpret_cast<ulonglong2 *>(acc.p + bi * acc.bstride + acc.cstride + (size_t)t * n + j);
+    ulonglong2 r0 = make_ulonglong2(a[0].reduce(P), b[0].reduce(P)), r1 = make_ulonglong2(a[1].reduce(P), b[1].reduce(P));
+    if (accumulate) {
+        const ulonglong2 p0 = *o0, p1 = *o1;
+        r0.x = addmod(r0.x, p0.x, P.q), r0.y = addmod(r0.y, p0.y, P.q);
+        r1.x = addmod(r1.x, p1.x, P.q), r1.y = addmod(r1.y, p1.y, P.q);
+    }
+    *o0 = r0;
+    *o1 = r1;
+}
+
+constexpr int kSplitThreads = 128;
+
+template <int ND>
+__global__ void __launch_bounds__(kSplitThreads, 6)
+    k_key_ip_split(const SplitIp A, View acc, const uint64_t *__restrict__ key, const FoldPrime *__restrict__ primes,
+                   int n_all, uint64_t g, bool accumulate, int B)
+{
+    const int bi = blockIdx.z * blockDim.y + threadIdx.y, t = blockIdx.y;
+    if (bi >= B) return;
+    const FoldPrime P = primes[A.prime(t)];
+    key_ip_split_body<ND>(A, acc, key, P, n_all, g, accumulate, bi, t, 2 * (blockIdx.x * blockDim.x + threadIdx.x));
+}
+
+// the selection between two hoisted rotations (k_key_ip_mux below) over split keys
+template <int ND>
+__global__ void __launch_bounds__(kSplitThreads, 5)
+    k_key_ip_mux_split(const SplitIp A, View out, const uint64_t *__restrict__ key1, const uint64_t *__restrict__ key2,
+                       const uint64_t *__restrict__ v, const __grid_constant__ Scalars cs,
+                       const PrimeConst *__restrict__ primes, const FoldPrime *__restrict__ fold, int n_all, uint64_t g1,
+                       uint64_t g2, int B)
+{
+    const int bi = blockIdx.z * blockDim.y + threadIdx.y, t = blockIdx.y;
+    if (bi >= B) return;
+    const int pr = A.prime(t), j = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+    const FoldPrime F = fold[pr];
+    const size_t n = (size_t)1 << A.log_n, half = (size_t)n_all * n, ko = (size_t)pr * n + j;
+    const SplitRows R(A, bi, t);
+    uint64_t xr[4], yr[4];  // (half, coefficient)
+    {
+        Sum30 a[2], b[2];
+        split_ip<ND>(a, b, R, A.ndig, galois_src(j, g1, A.log_n), key1 + ko, half, F);
+        xr[0] = a[0].reduce(F), xr[1] = b[0].reduce(F), xr[2] = a[1].reduce(F), xr[3] = b[1].reduce(F);
+    }
+    {
+        Sum30 a[2], b[2];
+        split_ip<ND>(a, b, R, A.ndig, galois_src(j, g2, A.log_n), key2 + ko, half, F);
+        yr[0] = a[0].reduce(F), yr[1] = b[0].reduce(F), yr[2] = a[1].reduce(F), yr[3] = b[1].reduce(F);
+    }
+    const PrimeConst P = primes[pr];
+    // v holds the special primes' rows first, then the chain's (a mask of any level is a prefix)
+    const ulonglong2 vv = *reinterpret_cast<const ulonglong2 *>(v + (size_t)(t < A.limbs ? A.K + t : t - A.limbs) * n + j);
+    const uint64_t c = cs.v[t], csh = cs.sh[t];
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const uint64_t w = i % 2 ? vv.y : vv.x, d = submod(xr[i], yr[i], P.q);
+        xr[i] = addmod(shoup(yr[i], c, csh, P.q), redc_few(__umul64hi(w, d), w * d, P), P.q);
+    }
+    uint64_t *o = out.p + bi * out.bstride + (size_t)t * n + j;
+    *reinterpret_cast<ulonglong2 *>(o) = make_ulonglong2(xr[0], xr[1]);
+    *reinterpret_cast<ulonglong2 *>(o + out.cstride) = make_ulonglong2(xr[2], xr[3]);
+}
+
+// the same with premasked keys [2][ndig][2][ext][n]: one sum over both rotations
+template <int ND>
+__global__ void __launch_bounds__(kSplitThreads, 5)
+    k_key_ip_mux_pm_split(const SplitIp A, View out, const uint64_t *__restrict__ pk,
+                          const FoldPrime *__restrict__ primes, uint64_t g1, uint64_t g2, int B)
+{
+    const int bi = blockIdx.z * blockDim.y + threadIdx.y, t = blockIdx.y;
+    if (bi >= B) return;
+    const FoldPrime P = primes[A.prime(t)];
+    const int j = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+    const size_t n = (size_t)1 << A.log_n, half = (size_t)(A.limbs + A.K) * n, second = 2 * A.ndig * half;
+    const int s1 = galois_src(j, g1, A.log_n), s2 = galois_src(j, g2, A.log_n);
+    const SplitRows R(A, bi, t);
+    const uint64_t *kd = pk + (size_t)t * n + j;
+    Sum30 a[2], b[2];
+    if (ND == 0) {
+        for (int d = 0; d < A.ndig; d++) {
+            const uint64_t *row = R.row(d);
+            split_room(a, b, 2 * d, P);
+            split_mac(a, b, make_ulonglong2(row[s1], row[s1 ^ 1]), kd + 2 * d * half, half);
+            split_room(a, b, 2 * d + 1, P);
+            split_mac(a, b, make_ulonglong2(row[s2], row[s2 ^ 1]), kd + second + 2 * d * half, half);
+        }
+    } else {
+        ulonglong2 x[ND ? ND : 1], y[ND ? ND : 1];
+#pragma unroll
+        for (int d = 0; d < ND; d++) {
+            const uint64_t *row = R.row(d);
+            x[d] = make_ulonglong2(row[s1], row[s1 ^ 1]);
+            y[d] = make_ulonglong2(row[s2], row[s2 ^ 1]);
+        }
+#pragma unroll
+        for (int d = 0; d < ND; d++) {
+            split_room(a, b, 2 * d, P);
+            split_mac(a, b, x[d], kd + 2 * d * half, half);
+            split_room(a, b, 2 * d + 1, P);
+            split_mac(a, b, y[d], kd + second + 2 * d * half, half);
+        }
+    }
+    *reinterpret_cast<ulonglong2 *>(out.p + bi * out.bstride + (size_t)t * n + j) =
+        make_ulonglong2(a[0].reduce(P), b[0].reduce(P));
+    *reinterpret_cast<ulonglong2 *>(out.p + bi * out.bstride + out.cstride + (size_t)t * n + j) =
+        make_ulonglong2(a[1].reduce(P), b[1].reduce(P));
+}
+
 __global__ void k_key_ip(View acc, const uint64_t *__restrict__ D, const uint64_t *__restrict__ dnt, size_t dnt_bstride,
                          const uint64_t *__restrict__ key, const PrimeConst *__restrict__ primes, int n_all, int n_q,
                          int K, int alpha, int limbs, int ndig, uint64_t g, int log_n, bool accumulate, bool few)
@@ -476,7 +674,7 @@ __global__ void k_key_ip_mux(View out, const uint64_t *__restrict__ D, const uin
 __global__ void k_premask_keys(uint64_t *out, const uint64_t *__restrict__ key1, const uint64_t *__restrict__ key2,
                                const uint64_t *__restrict__ v, const __grid_constant__ Scalars cR,
                                const PrimeConst *__restrict__ primes, int n_all, int n_q, int K, int limbs, int ndig,
-                               int n)
+                               int n, bool split)
 {
     const int t = blockIdx.y, dh = blockIdx.z, d = dh / 2, h = dh % 2;
     const int ext = limbs + K;
@@ -488,10 +686,12 @@ __global__ void k_premask_keys(uint64_t *out, const uint64_t *__restrict__ key1,
     const uint64_t cr = cR.v[t];
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
         // v: the special primes' rows first, then the chain's
-        const uint64_t vv = v[(size_t)(t < limbs ? K + t : t - limbs) * n + j], k1 = key1[ko + j], k2 = key2[ko + j];
+        const uint64_t vv = v[(size_t)(t < limbs ? K + t : t - limbs) * n + j];
+        const uint64_t k1 = split ? join30(key1[ko + j]) : key1[ko + j], k2 = split ? join30(key2[ko + j]) : key2[ko + j];
         const uint64_t w = submod(cr, vv, P.q);  // (c - v) in Montgomery form
-        o1[j] = redc_few(__umul64hi(vv, k1), vv * k1, P);
-        o2[j] = redc_few(__umul64hi(w, k2), w * k2, P);
+        const uint64_t p1 = redc_few(__umul64hi(vv, k1), vv * k1, P), p2 = redc_few(__umul64hi(w, k2), w * k2, P);
+        o1[j] = split ? split30(p1) : p1;
+        o2[j] = split ? split30(p2) : p2;
     }
 }
 
@@ -751,9 +951,11 @@ __global__ void k_expand_masks(double *slots, const uint8_t *__restrict__ bits, 
 }
 
 // b = e - a*s + gad_r * s'  (all NTT form, row r modulo prime r); optionally
-// b and a are left in Montgomery form for the key inner product.
+// b and a are left in the form of the key inner product: split at bit 30 and times 2^60 where the
+// chain has fold arithmetic (fold not null), else in Montgomery form.
 __global__ void k_keygen_b(uint64_t *b, uint64_t *a, const uint64_t *e, const uint64_t *s, const uint64_t *sp,
-                           const uint64_t *gad, const PrimeConst *__restrict__ primes, int n, bool to_mont)
+                           const uint64_t *gad, const PrimeConst *__restrict__ primes,
+                           const FoldPrime *__restrict__ fold, int n, bool to_mont)
 {
     const int r = blockIdx.y;
     const PrimeConst P = primes[r];
@@ -762,7 +964,11 @@ __global__ void k_keygen_b(uint64_t *b, uint64_t *a, const uint64_t *e, const ui
         const size_t k = (size_t)r * n + j;
         uint64_t v = submod(e[k], mulmod(a[k], s[k], P), P.q);
         if (gr) v = addmod(v, mulmod(gr, sp[k], P), P.q);
-        if (to_mont) {
+        if (to_mont && fold) {
+            const FoldPrime &F = fold[r];
+            v = split30(fold_finish(fold_mul((int64_t)v, F.r60, F), F));
+            a[k] = split30(fold_finish(fold_mul((int64_t)a[k], F.r60, F), F));
+        } else if (to_mont) {
             v = shoup(v, P.r_mod, P.r_mod_sh, P.q);
             a[k] = shoup(a[k], P.r_mod, P.r_mod_sh, P.q);
         }
@@ -869,6 +1075,13 @@ __global__ void k_key_ip_jobs(const KeyIpJob *__restrict__ jobs, int n_jobs)
 {
     Blk b;
     const KeyIpJob &J = job_of_block(jobs, n_jobs, blockIdx.x, b);
+    if (J.fold) {
+        const SplitIp A{J.D, J.dnt, J.dnt_bstride, J.n_q, J.K, J.alpha, J.limbs, J.ndig, J.log_n};
+        const FoldPrime P = J.fold[A.prime(b.y)];
+        for (int j = 2 * (b.x * blockDim.x + threadIdx.x); j < 1 << J.log_n; j += 2 * b.gx * blockDim.x)
+            key_ip_split_body<0>(A, J.acc, J.key, P, J.n_all, J.g, false, b.z, b.y, j);
+        return;
+    }
     key_ip_body(b, J.acc, J.D, J.dnt, J.dnt_bstride, J.key, J.primes, J.n_all, J.n_q, J.K, J.alpha, J.limbs, J.ndig,
                 J.g, J.log_n, false, J.few != 0);
 }
@@ -990,11 +1203,41 @@ void launch_basis_convert(const LaunchCtx &c, const ConvTable *tab_dev, int max_
     post(c);
 }
 
+// f with the digit count as a constant where the kernels hold every digit's words, else with 0
+template <class F> static void by_digits(int ndig, F f)
+{
+    switch (ndig) {
+    case 1: f(std::integral_constant<int, 1>()); break;
+    case 2: f(std::integral_constant<int, 2>()); break;
+    case 3: f(std::integral_constant<int, 3>()); break;
+    case 4: f(std::integral_constant<int, 4>()); break;
+    case 5: f(std::integral_constant<int, 5>()); break;
+    case 6: f(std::integral_constant<int, 6>()); break;
+    default: f(std::integral_constant<int, 0>()); break;
+    }
+}
+
+// threads of a split inner product's block: up to four batch entries share its key words
+static dim3 split_block(int B)
+{
+    const int y = B >= 4 ? 4 : B >= 2 ? 2 : 1;
+    return dim3(kSplitThreads / y, y);
+}
+
 void launch_key_ip(const LaunchCtx &c, View acc, const uint64_t *D, const uint64_t *dnt, size_t dnt_bstride,
                    const uint64_t *key, int n_all, int n_q, int K, int alpha, int limbs, int ndig, uint64_t g, int B,
                    bool accumulate)
 {
     Timed tm_(c, K_KEYIP, 8.0 * c.N * ((double)B * ndig * (limbs + K) + 2.0 * ndig * (limbs + K) + 2.0 * B * (limbs + K)));
+    if (c.t->fold) {
+        const dim3 block = split_block(B), grid(c.N / 2 / block.x, limbs + K, (B + block.y - 1) / block.y);
+        const SplitIp A{D, dnt, dnt_bstride, n_q, K, alpha, limbs, ndig, c.log_n};
+        by_digits(ndig, [&](auto nd) {
+            k_key_ip_split<nd()><<<grid, block, 0, c.stream>>>(A, acc, key, c.t->fold, n_all, g, accumulate, B);
+        });
+        post(c);
+        return;
+    }
     dim3 grid(ew_blocks(c.N, 2), limbs + K, B);
     k_key_ip<<<grid, 256, 0, c.stream>>>(acc, D, dnt, dnt_bstride, key, c.t->primes, n_all, n_q, K, alpha, limbs, ndig, g,
                                          c.log_n, accumulate, ndig <= kRedcFewTerms);
@@ -1018,6 +1261,16 @@ void launch_key_ip_mux(const LaunchCtx &c, View out, const uint64_t *D, const ui
 {
     Timed tm_(c, K_KEYIP, 8.0 * c.N * ((double)B * ndig * (limbs + K) + 4.0 * ndig * (limbs + K) + (limbs + K) +
                                         2.0 * B * (limbs + K)));
+    if (c.t->fold) {
+        const dim3 block = split_block(B), grid(c.N / 2 / block.x, limbs + K, (B + block.y - 1) / block.y);
+        const SplitIp A{D, dnt, dnt_bstride, n_q, K, alpha, limbs, ndig, c.log_n};
+        by_digits(ndig, [&](auto nd) {
+            k_key_ip_mux_split<nd()><<<grid, block, 0, c.stream>>>(A, out, key1, key2, v, cs, c.t->primes, c.t->fold, n_all,
+                                                                  g1, g2, B);
+        });
+        post(c);
+        return;
+    }
     dim3 grid(ew_blocks(c.N, 1), limbs + K, B);
     k_key_ip_mux<<<grid, 256, 0, c.stream>>>(out, D, dnt, dnt_bstride, key1, key2, v, cs, c.t->primes, n_all, n_q, K,
                                              alpha, limbs, ndig, g1, g2, c.log_n, ndig <= kRedcFewTerms);
@@ -1028,7 +1281,8 @@ void launch_premask_keys(const LaunchCtx &c, uint64_t *out, const uint64_t *key1
                          const uint64_t *v, const Scalars &cR, int n_all, int n_q, int K, int limbs, int ndig)
 {
     dim3 grid(ew_blocks(c.N, 1), limbs + K, ndig * 2);
-    k_premask_keys<<<grid, 256, 0, c.stream>>>(out, key1, key2, v, cR, c.t->primes, n_all, n_q, K, limbs, ndig, c.N);
+    k_premask_keys<<<grid, 256, 0, c.stream>>>(out, key1, key2, v, cR, c.t->primes, n_all, n_q, K, limbs, ndig, c.N,
+                                           c.t->fold != nullptr);
     post(c);
 }
 
@@ -1038,6 +1292,15 @@ void launch_key_ip_mux_pm(const LaunchCtx &c, View out, const uint64_t *D, const
 {
     Timed tm_(c, K_KEYIP, 8.0 * c.N * ((double)B * ndig * (limbs + K) + 4.0 * ndig * (limbs + K) +
                                         2.0 * B * (limbs + K)));
+    if (c.t->fold) {
+        const dim3 block = split_block(B), grid(c.N / 2 / block.x, limbs + K, (B + block.y - 1) / block.y);
+        const SplitIp A{D, dnt, dnt_bstride, n_q, K, alpha, limbs, ndig, c.log_n};
+        by_digits(ndig, [&](auto nd) {
+            k_key_ip_mux_pm_split<nd()><<<grid, block, 0, c.stream>>>(A, out, pk, c.t->fold, g1, g2, B);
+        });
+        post(c);
+        return;
+    }
     dim3 grid(ew_blocks(c.N, 2), limbs + K, B);
     k_key_ip_mux_pm<<<grid, 256, 0, c.stream>>>(out, D, dnt, dnt_bstride, pk, c.t->primes, n_q, K, alpha, limbs, ndig, g1, g2,
                                                 c.log_n, 2 * ndig <= kRedcFewTerms);
@@ -1137,7 +1400,7 @@ void launch_keygen_b(const LaunchCtx &c, uint64_t *b, const uint64_t *a, const u
                      const uint64_t *sp, const uint64_t *gad, int rows, const int *, bool to_mont)
 {
     dim3 grid(ew_blocks(c.N, 1), rows, 1);
-    k_keygen_b<<<grid, 256, 0, c.stream>>>(b, const_cast<uint64_t *>(a), e, s, sp, gad, c.t->primes, c.N, to_mont);
+    k_keygen_b<<<grid, 256, 0, c.stream>>>(b, const_cast<uint64_t *>(a), e, s, sp, gad, c.t->primes, c.t->fold, c.N, to_mont);
     post(c);
 }
 

@@ -30,6 +30,9 @@ struct FoldPrime {
     int refold;    // != 0: the final reduction folds twice
     int4 n_inv;    // N^-1 mod q as a constant
     int4 n_inv_w1; // N^-1 * psi^-brv(1) mod q: the last inverse stage's twiddle with N^-1 folded in
+    int4 r60;      // 2^60 mod q as a constant
+    uint32_t q0, q1;  // q's low 30 bits and the rest
+    uint32_t minv;    // -q^-1 mod 2^30
 };
 
 // bounds in sixteenths of the unit u of a prime (u >= 2^b): a folded value, a product, the limit
@@ -77,6 +80,62 @@ __device__ __forceinline__ uint64_t fold_finish(int64_t v, const FoldPrime &P)
     else if (v >= q) v -= q;
     return (uint64_t)v;
 }
+
+// ---- sums of products in 30-bit parts
+//
+// Residues below 2^60 split at bit 30 into parts of at most 30 bits, so four multiply-adds per
+// product go into three 64-bit sums (weights 1, 2^30, 2^60) without carries.  A product adds
+// at most 2 (2^30 - 1)^2 to the middle sum: seven products and the reduction's two terms fit, and
+// fourteen below 2^59, where the outer sums' fourteen terms of (2^30 - 1)^2 are the limit.
+// The reduction takes two Montgomery steps of 30 bits, so one factor is kept times 2^60.
+constexpr uint32_t kMask30 = (1u << 30) - 1;
+constexpr int kSumTerms = 7;  // products between two spill()s, twice that below 2^59
+
+__device__ __forceinline__ uint64_t madu(uint32_t a, uint32_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
+}
+// a factor split for the sums: the low 30 bits in the low word, the rest in the high word
+__device__ __forceinline__ uint64_t split30(uint64_t x) { return (x & kMask30) | ((x >> 30) << 32); }
+__device__ __forceinline__ uint64_t join30(uint64_t x) { return (x & kMask30) | ((x >> 32) << 30); }
+
+// v - (v >> b) 2^b + (v >> b) d: congruent to v, below 2^b + 2^(64-b) d
+__device__ __forceinline__ uint64_t fold_u(uint64_t v, const FoldPrime &P)
+{
+    const uint32_t vh = (uint32_t)(v >> 32);
+    return madu(vh >> P.c, (uint32_t)P.d, ((uint64_t)(vh & (uint32_t)P.mask) << 32) | (uint32_t)v);
+}
+
+struct Sum30 {
+    uint64_t a = 0, b = 0, c = 0;
+    // += x k for split x (x0, x1) and k
+    __device__ __forceinline__ void mac(uint32_t x0, uint32_t x1, uint32_t k0, uint32_t k1)
+    {
+        a = madu(x0, k0, a);
+        b = madu(x0, k1, b);
+        c = madu(x1, k1, c);
+        b = madu(x1, k0, b);
+    }
+    __device__ __forceinline__ void mac(uint32_t x0, uint32_t x1, uint64_t k) { mac(x0, x1, (uint32_t)k, (uint32_t)(k >> 32)); }
+    // room for kSumTerms more products: the middle sum's high part moves up, the high sum is folded
+    __device__ __forceinline__ void spill(const FoldPrime &P)
+    {
+        c = fold_u(c + (b >> 30) + (a >> 60), P);
+        b &= kMask30;
+        a &= (1ull << 60) - 1;
+    }
+    // the sum times 2^-60 mod q, in [0, q)
+    __device__ __forceinline__ uint64_t reduce(const FoldPrime &P) const
+    {
+        const uint32_t m0 = ((uint32_t)a * P.minv) & kMask30;
+        uint64_t t = madu(m0, P.q1, b) + (madu(m0, P.q0, a) >> 30);
+        const uint32_t m1 = ((uint32_t)t * P.minv) & kMask30;
+        t = fold_u(madu(m1, P.q1, c) + (madu(m1, P.q0, t) >> 30), P);
+        return t >= P.q ? t - P.q : t;
+    }
+};
 #endif
 
 } // namespace hx

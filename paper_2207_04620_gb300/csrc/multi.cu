@@ -124,7 +124,7 @@ std::vector<Cts> rotate_jobs(const std::vector<RotateJob> &in, cudaStream_t s)
                                 ew_blocks((int)N, 2), 1, B * nd, 0});
         // a digit's own rows of D are never read (the inner product takes them from sigma_g(c1))
         n2.push_back(ntt_job(ctx, x.D->p, B * nd * ext, ext_primes));
-        kj.push_back(KeyIpJob{accv, x.D->p, x.t->p, x.key->buf->p, (size_t)L * N, ctx.t.primes, ctx.n_all, ctx.n_q,
+        kj.push_back(KeyIpJob{accv, x.D->p, x.t->p, x.key->buf->p, (size_t)L * N, ctx.t.primes, ctx.t.fold, ctx.n_all, ctx.n_q,
                               K, x.A, L, nd, ctx.log_n, nd <= kRedcFewTerms ? 1 : 0, 1, ew_blocks((int)N, 2), ext, B,
                               0});
         // ModDown: inverse NTT of the special rows, conversion to Q, forward NTT, epilogue

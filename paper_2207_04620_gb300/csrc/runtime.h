@@ -43,7 +43,7 @@ struct Cts {
 };
 
 struct SwitchKey {
-    BufPtr buf;  // [dnum][2][n_all][N] Montgomery form
+    BufPtr buf;  // [dnum][2][n_all][N]: split at bit 30 and times 2^60 with fold arithmetic, else Montgomery form
 };
 
 } // namespace hx
