@@ -362,6 +362,30 @@ void build_context(hx_context &c, const hx_params &p)
             }
         }
     }
+    if (all_fold) {
+        auto times60 = [&](uint64_t x, uint64_t q) {
+            const uint64_t y = (uint64_t)(((u128)x << 60) % q);
+            return (y & 0x3fffffffu) | ((y >> 30) << 32);
+        };
+        auto complete = [&](ConvTable &T) {
+            for (int i = 0; i < T.n_src; i++) {
+                const uint64_t q = c.primes[T.src_prime[i]];
+                const int b = fold_bits[T.src_prime[i]];
+                T.inv_f[i] = fold_constant(T.inv[i], q, b);
+                T.bits[i] = b;
+                T.recip[i] = (uint32_t)(((u128)1 << (b + 31)) / q);
+                for (int d = 0; d < T.n_dst; d++) T.w30[i][d] = times60(T.w[i][d], c.primes[T.dst_prime[d]]);
+            }
+            for (int d = 0; d < T.n_dst && T.shift; d++) {
+                const uint64_t q = c.primes[T.dst_prime[d]];
+                T.neg_prod30[d] = times60(q - T.prod_mod[d], q);
+                T.neg_sub30[d] = times60(q - T.sub_dst[d], q);
+            }
+        };
+        for (auto &T : c.h_modup) complete(T);
+        for (auto &M : c.h_moddown) complete(M.conv);
+        for (auto &M : c.h_relin_rs) complete(M.conv);
+    }
     c.t.primes = upload(c.h_primes);
     c.t.tw_fwd = upload(twf);
     c.t.tw_inv = upload(twi);

@@ -50,6 +50,12 @@ struct ConvTable {
     double inv_d[MAXK];                 // 1 / q_i in FP64
     uint64_t sub_dst[MAXP];             // h mod t
     uint64_t prod_mod[MAXP];            // (product of the sources) mod t
+    // the same constants for chains with fold arithmetic: inv as fold constants; w, -prod_mod and
+    // -sub_dst times 2^60 and split at bit 30; 2^(31 + bits) / q_i for the overshoot's estimate
+    int4 inv_f[MAXK];
+    uint64_t w30[MAXK][MAXP], neg_prod30[MAXP], neg_sub30[MAXP];
+    uint32_t recip[MAXK];
+    int bits[MAXK];
 };
 
 struct ModDownTable {
@@ -215,6 +221,7 @@ struct ConvertJob {
     const ConvTable *tabs;
     View out, in;
     const PrimeConst *primes;
+    const FoldPrime *fold;  // not null: by split sums
     int groups, n, max_src;
     size_t gstride_out, gstride_in;
     int gx, gy, gz;

@@ -365,6 +365,133 @@ __global__ void __launch_bounds__(256, MK <= 4 ? 4 : 2)
     basis_convert_body<MK>(Blk::hw(), tabs, out, in, primes, groups, gstride_out, gstride_in, n);
 }
 
+// The same for chains with fold arithmetic (modfold.cuh): a term is four multiply-adds into split
+// sums and an output one reduction, against a Shoup product and a correction per term.  A
+// two-source conversion to 32 x 7 rows of N = 2^14 took 21 us and takes 19 (a third of the time is
+// the reductions), the sign batch's (four sources, 16 limbs of N = 2^15) 2.27 ms and 1.6 per product.
+//
+// The shifted form's overshoot u = floor(sum of y_i / q_i rounded in FP64) comes from 32-bit
+// products (within 2^-29 of the sum) unless the sum lies within 2^-26 of an integer, where the
+// FP64 sum decides as in the form above: its pipe issues a sixteenth of a warp per cycle and
+// would take longer than the conversion.
+struct ConvShared {
+    uint64_t w[MAXK * MAXP], prod[MAXP], sub[MAXP];  // w: a destination's sources together
+    SumPrime dst[MAXP];
+    int row[MAXP];
+};
+
+// NS sources exactly; coefficients j, j + 1 of one (entry, digit)
+template <int NS>
+__device__ __forceinline__ void convert_split_pair(const ConvShared &S, const ConvTable &T, const uint64_t *src,
+                                                   uint64_t *dst, const FoldPrime *__restrict__ primes, int d0, int dstep,
+                                                   int n, int j)
+{
+    const int nd = T.n_dst;
+    const bool shift = T.shift != 0;
+    uint32_t l0[NS], h0[NS], l1[NS], h1[NS];
+    uint64_t v0 = 0, v1 = 0;  // the overshoot's estimate in units of 2^-60, each term short by less than 2^31
+#pragma unroll
+    for (int i = 0; i < NS; i++) {
+        const FoldPrime &P = primes[T.src_prime[i]];
+        ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(src + (size_t)T.src_row[i] * n + j);
+        if (shift) {
+            x.x = addmod(x.x, T.add_src[i], P.q);
+            x.y = addmod(x.y, T.add_src[i], P.q);
+        }
+        const uint64_t y0 = fold_finish(fold_mul((int64_t)x.x, T.inv_f[i], P), P);
+        const uint64_t y1 = fold_finish(fold_mul((int64_t)x.y, T.inv_f[i], P), P);
+        l0[i] = (uint32_t)y0 & kMask30, h0[i] = (uint32_t)(y0 >> 30);
+        l1[i] = (uint32_t)y1 & kMask30, h1[i] = (uint32_t)(y1 >> 30);
+        if (shift) {
+            const int drop = T.bits[i] - 32;
+            v0 += madu((uint32_t)(y0 >> drop), T.recip[i], 0) >> 3;
+            v1 += madu((uint32_t)(y1 >> drop), T.recip[i], 0) >> 3;
+        }
+    }
+    uint32_t u0 = (uint32_t)(v0 >> 60), u1 = (uint32_t)(v1 >> 60);  // the overshoot (shifted tables only)
+    if (shift) {
+        const uint64_t frac = (1ull << 60) - 1, low = 1ull << 14, high = (1ull << 60) - (1ull << 34);
+        if ((v0 & frac) < low || (v0 & frac) >= high || (v1 & frac) < low || (v1 & frac) >= high) {
+            double s0 = 0.0, s1 = 0.0;  // products and sums rounded to nearest, in source order
+#pragma unroll
+            for (int i = 0; i < NS; i++) {
+                const uint64_t y0 = l0[i] | (uint64_t)h0[i] << 30, y1 = l1[i] | (uint64_t)h1[i] << 30;
+                s0 = __dadd_rn(s0, __dmul_rn(__ull2double_rn(y0), T.inv_d[i]));
+                s1 = __dadd_rn(s1, __dmul_rn(__ull2double_rn(y1), T.inv_d[i]));
+            }
+            u0 = (uint32_t)__double2ull_rd(s0);
+            u1 = (uint32_t)__double2ull_rd(s1);
+        }
+    }
+    for (int d = d0; d < nd; d += dstep) {
+        Sum30 s0, s1;
+        if (shift) {  // - u (product of the sources) - h
+            const uint64_t np = S.prod[d], nh = S.sub[d];
+            s0.a = s1.a = (uint32_t)nh;
+            s0.b = s1.b = nh >> 32;
+            s0.a = madu(u0, (uint32_t)np, s0.a), s0.b = madu(u0, (uint32_t)(np >> 32), s0.b);
+            s1.a = madu(u1, (uint32_t)np, s1.a), s1.b = madu(u1, (uint32_t)(np >> 32), s1.b);
+        }
+#pragma unroll
+        for (int i = 0; i < NS; i++) {
+            const uint64_t w = S.w[d * NS + i];
+            s0.mac(l0[i], h0[i], w);
+            s1.mac(l1[i], h1[i], w);
+        }
+        const SumPrime P = S.dst[d];
+        *reinterpret_cast<ulonglong2 *>(dst + (size_t)S.row[d] * n + j) = make_ulonglong2(s0.reduce(P), s1.reduce(P));
+    }
+}
+
+// the instance for T's source count, at most NS
+template <int NS>
+__device__ __forceinline__ void convert_split_up_to(const ConvShared &S, const ConvTable &T, const uint64_t *src,
+                                                    uint64_t *dst, const FoldPrime *__restrict__ primes, int d0, int dstep,
+                                                    int n, int j)
+{
+    if constexpr (NS > 1) {
+        if (T.n_src != NS) {
+            convert_split_up_to<NS - 1>(S, T, src, dst, primes, d0, dstep, n, j);
+            return;
+        }
+    }
+    convert_split_pair<NS>(S, T, src, dst, primes, d0, dstep, n, j);
+}
+
+// blocks split at j over x, at the destinations over y; MK: the launch's largest source count (a
+// chain's last digit may have fewer)
+template <int MK>
+__device__ __forceinline__ void basis_convert_split_body(const Blk &b, const ConvTable *__restrict__ tabs, View out,
+                                                         View in, const FoldPrime *__restrict__ primes, int groups,
+                                                         size_t gstride_out, size_t gstride_in, int n)
+{
+    const int bi = b.z / groups, gi = b.z % groups;
+    const ConvTable &T = tabs[gi];
+    __shared__ ConvShared S;
+    const int ns = T.n_src, nd = T.n_dst;
+    for (int i = threadIdx.x; i < ns * nd; i += blockDim.x) S.w[i] = T.w30[i % ns][i / ns];
+    for (int d = threadIdx.x; d < nd; d += blockDim.x) {
+        S.dst[d] = SumPrime(primes[T.dst_prime[d]]);
+        S.row[d] = T.dst_row[d];
+        S.prod[d] = T.neg_prod30[d];
+        S.sub[d] = T.neg_sub30[d];
+    }
+    __syncthreads();
+    const uint64_t *src = in.p + bi * in.bstride + gi * gstride_in;
+    uint64_t *dst = out.p + bi * out.bstride + gi * gstride_out;
+    for (int j = (b.x * blockDim.x + threadIdx.x) * 2; j < n; j += b.gx * blockDim.x * 2) {
+        convert_split_up_to<MK>(S, T, src, dst, primes, b.y, b.gy, n, j);
+    }
+}
+
+template <int MK>
+__global__ void __launch_bounds__(256, MK <= 3 ? 4 : 3)
+    k_basis_convert_split(const ConvTable *__restrict__ tabs, View out, View in, const FoldPrime *__restrict__ primes,
+                          int groups, size_t gstride_out, size_t gstride_in, int n)
+{
+    basis_convert_split_body<MK>(Blk::hw(), tabs, out, in, primes, groups, gstride_out, gstride_in, n);
+}
+
 // Key inner product of hybrid key switching: for ext row t (Q_l then P),
 // acc_h[t] = sum_j src_j[t][galois(n)] * key[j][h][row(t)][n], where src_j is
 // the NTT-form input itself on digit j's own rows and the ModUp output D_j
@@ -1068,6 +1195,10 @@ __global__ void __launch_bounds__(256, MK <= 4 ? 4 : 2) k_convert_jobs(const Con
 {
     Blk b;
     const ConvertJob &J = job_of_block(jobs, n_jobs, blockIdx.x, b);
+    if (J.fold) {
+        basis_convert_split_body<MK>(b, J.tabs, J.out, J.in, J.fold, J.groups, J.gstride_out, J.gstride_in, J.n);
+        return;
+    }
     basis_convert_body<MK>(b, J.tabs, J.out, J.in, J.primes, J.groups, J.gstride_out, J.gstride_in, J.n);
 }
 
@@ -1194,6 +1325,27 @@ void launch_basis_convert(const LaunchCtx &c, const ConvTable *tab_dev, int max_
     HX_CHECK(B * groups < 65536, HX_EINVAL, "conversion batch too large");
     HX_CHECK(max_src >= 1 && max_src <= MAXK, HX_EINVAL, "too many conversion sources");
     dim3 grid(ew_blocks(c.N, 2), 1, B * groups);
+    if (c.t->fold) {
+        // a grid that leaves SMs idle is split over the destination rows (each block repeats the sources);
+        // one of more than two rounds of blocks takes several pairs per thread, so that fewer blocks
+        // stage the table
+        const long long blocks = (long long)grid.x * grid.z, round = 4ll * c.t->n_sm;
+        if (blocks < round / 2) grid.y = (unsigned)std::min<long long>(4, std::max<long long>(1, round / 2 / blocks));
+        while (grid.x > 1 && (long long)grid.x * grid.z > 2 * round) grid.x /= 2;
+        auto run = [&](auto mk) {
+            k_basis_convert_split<mk()><<<grid, 256, 0, c.stream>>>(tab_dev, out, in, c.t->fold, groups, gstride_out,
+                                                                    gstride_in, c.N);
+        };
+        switch (max_src) {
+        case 1: run(std::integral_constant<int, 1>()); break;
+        case 2: run(std::integral_constant<int, 2>()); break;
+        case 3: run(std::integral_constant<int, 3>()); break;
+        case 4: run(std::integral_constant<int, 4>()); break;
+        default: run(std::integral_constant<int, MAXK>()); break;
+        }
+        post(c);
+        return;
+    }
     if (max_src <= 4)
         k_basis_convert<4><<<grid, 256, 0, c.stream>>>(tab_dev, out, in, c.t->primes, groups, gstride_out, gstride_in,
                                                        c.N);

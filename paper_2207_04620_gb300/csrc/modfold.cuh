@@ -101,8 +101,20 @@ __device__ __forceinline__ uint64_t madu(uint32_t a, uint32_t b, uint64_t c)
 __device__ __forceinline__ uint64_t split30(uint64_t x) { return (x & kMask30) | ((x >> 30) << 32); }
 __device__ __forceinline__ uint64_t join30(uint64_t x) { return (x & kMask30) | ((x >> 32) << 30); }
 
+// what a sum's reduction needs of a prime
+struct SumPrime {
+    uint64_t q;
+    uint32_t q0, q1, minv;
+    int c, d, mask;
+    __device__ __forceinline__ SumPrime() {}
+    __device__ __forceinline__ SumPrime(const FoldPrime &P)
+        : q(P.q), q0(P.q0), q1(P.q1), minv(P.minv), c(P.c), d(P.d), mask(P.mask)
+    {
+    }
+};
+
 // v - (v >> b) 2^b + (v >> b) d: congruent to v, below 2^b + 2^(64-b) d
-__device__ __forceinline__ uint64_t fold_u(uint64_t v, const FoldPrime &P)
+template <class P_> __device__ __forceinline__ uint64_t fold_u(uint64_t v, const P_ &P)
 {
     const uint32_t vh = (uint32_t)(v >> 32);
     return madu(vh >> P.c, (uint32_t)P.d, ((uint64_t)(vh & (uint32_t)P.mask) << 32) | (uint32_t)v);
@@ -120,14 +132,14 @@ struct Sum30 {
     }
     __device__ __forceinline__ void mac(uint32_t x0, uint32_t x1, uint64_t k) { mac(x0, x1, (uint32_t)k, (uint32_t)(k >> 32)); }
     // room for kSumTerms more products: the middle sum's high part moves up, the high sum is folded
-    __device__ __forceinline__ void spill(const FoldPrime &P)
+    template <class P_> __device__ __forceinline__ void spill(const P_ &P)
     {
         c = fold_u(c + (b >> 30) + (a >> 60), P);
         b &= kMask30;
         a &= (1ull << 60) - 1;
     }
     // the sum times 2^-60 mod q, in [0, q)
-    __device__ __forceinline__ uint64_t reduce(const FoldPrime &P) const
+    template <class P_> __device__ __forceinline__ uint64_t reduce(const P_ &P) const
     {
         const uint32_t m0 = ((uint32_t)a * P.minv) & kMask30;
         uint64_t t = madu(m0, P.q1, b) + (madu(m0, P.q0, a) >> 30);

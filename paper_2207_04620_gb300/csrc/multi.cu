@@ -120,7 +120,7 @@ std::vector<Cts> rotate_jobs(const std::vector<RotateJob> &in, cudaStream_t s)
         for (int r = 0; r < K; r++) p_rows[r] = ctx.n_q + r;
         n1.push_back(ntt_job(ctx, x.coef->p, B * L, q_rows));
         c1.push_back(ConvertJob{ctx.t.modup + (size_t)L * ctx.dnum, View{x.D->p, (size_t)nd * ext * N, 0},
-                                View{x.coef->p, (size_t)L * N, 0}, ctx.t.primes, nd, (int)N, x.A, (size_t)ext * N, 0,
+                                View{x.coef->p, (size_t)L * N, 0}, ctx.t.primes, ctx.t.fold, nd, (int)N, x.A, (size_t)ext * N, 0,
                                 ew_blocks((int)N, 2), 1, B * nd, 0});
         // a digit's own rows of D are never read (the inner product takes them from sigma_g(c1))
         n2.push_back(ntt_job(ctx, x.D->p, B * nd * ext, ext_primes));
@@ -133,7 +133,7 @@ std::vector<Cts> rotate_jobs(const std::vector<RotateJob> &in, cudaStream_t s)
                 n3.push_back(ntt_job(ctx, x.acc->p + ((size_t)(b * 2 + c) * ext + L) * N, K, p_rows));
         const ModDownTable *md = ctx.t.moddown + L;
         c2.push_back(ConvertJob{reinterpret_cast<const ConvTable *>(md), View{x.conv->p, (size_t)L * N, 0},
-                                View{x.acc->p, (size_t)ext * N, 0}, ctx.t.primes, 1, (int)N, K, 0, 0,
+                                View{x.acc->p, (size_t)ext * N, 0}, ctx.t.primes, ctx.t.fold, 1, (int)N, K, 0, 0,
                                 ew_blocks((int)N, 2), 1, 2 * B, 0});
         n4.push_back(ntt_job(ctx, x.conv->p, 2 * B * L, q_rows));
         mj.push_back(ModDownJob{x.out.view((int)N), accv, View{x.conv->p, (size_t)2 * L * N, (size_t)L * N},
