@@ -693,8 +693,8 @@ hx_status hx_rotate_hoisted(hx_context *ctx, const hx_keyset *ks, const hx_ct *a
     mine(ctx, a);
     Eval ev(*ctx, S(stream));
     std::vector<int64_t> st(steps, steps + n);
-    std::vector<Cts> r = ev.rotate_hoisted(a->c, st, *ks);
-    for (int i = 0; i < n; i++) outs[i] = wrap(ctx, r[i]);
+    const Cts r = ev.rotate_hoisted(a->c, st, *ks);
+    scatter(*ctx, r, outs, S(stream));  // each handle owns its buffer
     return HX_OK;
     HX_END
 }

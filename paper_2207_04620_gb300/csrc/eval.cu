@@ -3,6 +3,7 @@
 // ModUp (iNTT, fast basis conversion per digit, NTT) -> key inner product ->
 // ModDown (iNTT of the special limbs, conversion P -> Q_l, NTT, subtract and
 // multiply by P^-1).
+#include <algorithm>
 #include <cmath>
 
 #include "runtime.h"
@@ -106,16 +107,6 @@ void Eval::from_mont(Cts &a)
     launch_mul_scalar(lc(), a.view(ctx.N), a.view(ctx.N), sc, a.B, a.comps, a.limbs);
 }
 
-void Eval::tensor_acc(Cts &acc, const Cts &a, const Cts &b, bool mont)
-{
-    HX_CHECK(a.B == b.B && a.limbs == b.limbs && acc.limbs == a.limbs && acc.comps == 3, HX_ESCALE,
-             "tensor operands differ");
-    HX_CHECK(std::fabs(acc.scale / (a.scale * b.scale) - 1.0) <= std::ldexp(1.0, -20), HX_ESCALE, "scale mismatch");
-    launch_tensor(lc(), acc.view(ctx.N), a.view(ctx.N), b.view(ctx.N), a.B, a.limbs, true, mont);
-    ctx.counters[C_MULCT] += a.B;
-    ctx.counters[C_ADD] += a.B;
-}
-
 Cts Eval::drop(const Cts &a, int limbs)
 {
     HX_CHECK(limbs >= 1 && limbs <= a.limbs, HX_EINVAL, "bad level drop");
@@ -190,67 +181,109 @@ BufPtr Eval::modup(const View &d, int B, int limbs)
     return D;
 }
 
+KeyTab one_key(const SwitchKey &key, uint64_t g)
+{
+    KeyTab t;
+    t.key[0] = key.buf->p;
+    t.g[0] = (uint32_t)g;
+    return t;
+}
+
 Cts Eval::ks_finish(const BufPtr &D, const View &dnt, int B, int limbs, const SwitchKey &key, uint64_t g,
                     const View &add, int add_mask, uint64_t add_g)
 {
     const int N = ctx.N, K = ctx.K, ext = limbs + K, nd = (limbs + ctx.alpha - 1) / ctx.alpha;
     DevBuf acc((size_t)B * 2 * ext * N, s);
     View accv{acc.p, (size_t)2 * ext * N, (size_t)ext * N};
-    launch_key_ip(lc(), accv, D->p, dnt.p, dnt.bstride, key.buf->p, ctx.n_all, ctx.n_q, K, ctx.alpha, limbs, nd, g, B);
+    launch_key_ip(lc(), accv, D->p, dnt.p, dnt.bstride, one_key(key, g), 1, true, false, ctx.n_all, ctx.n_q, K, ctx.alpha,
+                  limbs, nd, B);
     ctx.counters[C_KS] += B;
-    return moddown_add(accv, B, limbs, add, add_mask, add_g);
-}
-
-Cts Eval::moddown_add(const View &accv, int B, int limbs, const View &add, int add_mask, uint64_t add_g)
-{
-    const int N = ctx.N, K = ctx.K, ext = limbs + K;
-    ntt_inplace(accv.p, (size_t)ext * N, 2 * B, iota_vec(limbs, K), iota_vec(ctx.n_q, K), true);
-    DevBuf conv((size_t)B * 2 * limbs * N, s);
-    launch_basis_convert(lc(), reinterpret_cast<const ConvTable *>(ctx.t.moddown + limbs), ctx.K,
-                         View{conv.p, (size_t)limbs * N, 0}, View{accv.p, (size_t)ext * N, 0}, 2 * B, 1, 0, 0,
-                         8.0 * N * 2 * B * (K + limbs));
-    ntt_inplace(conv.p, (size_t)limbs * N, 2 * B, iota_vec(0, limbs), iota_vec(0, limbs), false);
     Cts o = alloc(B, 2, limbs);
-    launch_moddown_final(lc(), o.view(N), accv, View{conv.p, (size_t)2 * limbs * N, (size_t)limbs * N},
-                         ctx.t.moddown + limbs, B, limbs, add, add_mask, add_g);
+    moddown_add(o.view(N), accv, B, limbs, add, add_mask, one_galois(add_g, B));
     return o;
 }
 
-Cts Eval::rotate_sum(const std::vector<std::pair<Cts, int64_t>> &items, const hx_keyset &keys)
+void Eval::moddown_ntt(const View &accv, uint64_t *conv, int B, int limbs)
 {
-    HX_CHECK(!items.empty(), HX_EINVAL, "empty rotation sum");
-    const Cts &f = items[0].first;
-    const int N = ctx.N, K = ctx.K, limbs = f.limbs, B = f.B, ext = limbs + K, nd = (limbs + ctx.alpha - 1) / ctx.alpha;
+    const int N = ctx.N, K = ctx.K, ext = limbs + K;
+    ntt_inplace(accv.p, (size_t)ext * N, 2 * B, iota_vec(limbs, K), iota_vec(ctx.n_q, K), true);
+    launch_basis_convert(lc(), reinterpret_cast<const ConvTable *>(ctx.t.moddown + limbs), ctx.K,
+                         View{conv, (size_t)limbs * N, 0}, View{accv.p, (size_t)ext * N, 0}, 2 * B, 1, 0, 0,
+                         8.0 * N * 2 * B * (K + limbs));
+    ntt_inplace(conv, (size_t)limbs * N, 2 * B, iota_vec(0, limbs), iota_vec(0, limbs), false);
+}
+
+void Eval::moddown_add(const View &out, const View &accv, int B, int limbs, const View &add, int add_mask,
+                       const GaloisTab &gal, bool shared)
+{
+    const int N = ctx.N;
+    DevBuf conv((size_t)B * 2 * limbs * N, s);
+    moddown_ntt(accv, conv.p, B, limbs);
+    launch_moddown_final(lc(), out, accv, View{conv.p, (size_t)2 * limbs * N, (size_t)limbs * N}, ctx.t.moddown + limbs, B,
+                         limbs, add, add_mask, gal, shared);
+}
+
+// Rotations (or selections) of a batch of B per launch: as many as keep the launch's buffer small, so
+// that the stages that follow find it in L2.  One rotation of 16 entries of N = 2^14 (38 MB) already
+// fills the GPU; one of a single entry of N = 2^12 takes a few SMs, and with a launch per stage and
+// rotation the product of 16x16 matrices there waited on about 900 launches: 5.2 ms, 0.74 in groups
+// (five 32x32 products of N = 2^13: 4.0 ms, 2.6; a small dense layer of N = 2^14: 23.2 ms, 11.0).
+int Eval::rot_chunk(int B, int limbs, int most, size_t words)
+{
+    const size_t per = words ? words : (size_t)B * 2 * (limbs + ctx.K) * ctx.N;
+    const int grid = std::max(1, 16384 / (B * std::max(2, (limbs + ctx.alpha - 1) / ctx.alpha)));
+    return std::max(1, std::min({most, grid, (int)std::min<size_t>(MAX_ROT, ((size_t)32 << 20) / 8 / per)}));
+}
+
+Cts Eval::rotate_sum(const Cts &items, const std::vector<int64_t> &steps, const hx_keyset &keys)
+{
+    HX_CHECK(!steps.empty() && items.B % steps.size() == 0, HX_EINVAL, "empty rotation sum");
+    const int R = (int)steps.size(), B = items.B / R, N = ctx.N, K = ctx.K, limbs = items.limbs, ext = limbs + K,
+              nd = (limbs + ctx.alpha - 1) / ctx.alpha;
     Cts base = alloc(B, 2, limbs);
-    base.scale = f.scale;
+    base.scale = items.scale;
     HX_CUDA(cudaMemsetAsync(base.d, 0, sizeof(uint64_t) * base.bstride(N) * B, s));
     DevBuf acc((size_t)B * 2 * ext * N, s);
     View accv{acc.p, (size_t)2 * ext * N, (size_t)ext * N};
+    const int most = rot_chunk(B, limbs, MAX_ROT, (size_t)B * nd * ext * N / 2);  // the ModUp digits: up to 64 MB
     bool any = false;
-    for (auto &it : items) {
-        const Cts &ct = it.first;
-        check_same(ct, f);
-        const uint64_t g = galois_for_step(it.second, ctx.log_n);
-        if (g == 1) {
-            add_inplace(base, ct);
+    for (int r = 0; r < R;) {
+        Cts first = items;
+        first.d += (size_t)r * B * items.bstride(N);
+        first.B = B;
+        if (galois_for_step(steps[r], ctx.log_n) == 1) {
+            add_inplace(base, first);
+            r++;
             continue;
         }
-        const SwitchKey &key = rot_key(keys, g);
-        Cts t = alloc(B, 1, limbs);
-        View c1{ct.d + ct.cstride(N), ct.bstride(N), ct.cstride(N)};
-        launch_automorphism(lc(), t.view(N), c1, g, B, 1, limbs);
-        BufPtr D = modup(t.view(N), B, limbs);
-        launch_key_ip(lc(), accv, D->p, t.d, t.bstride(N), key.buf->p, ctx.n_all, ctx.n_q, K, ctx.alpha, limbs, nd, 1, B,
+        KeyTab kt;
+        GaloisTab gt;
+        gt.per = B;
+        int C = 0;
+        for (; C < most && r + C < R; C++) {
+            const uint64_t g = galois_for_step(steps[r + C], ctx.log_n);
+            if (g == 1) break;
+            kt.key[C] = rot_key(keys, g).buf->p;
+            kt.g[C] = 1;  // the items are rotated before their ModUp
+            gt.g[C] = (uint32_t)g;
+        }
+        Cts t = alloc(C * B, 1, limbs);
+        launch_automorphism(lc(), t.view(N), View{first.d + first.cstride(N), first.bstride(N), first.cstride(N)}, gt, C * B,
+                            1, limbs);
+        BufPtr D = modup(t.view(N), C * B, limbs);
+        launch_key_ip(lc(), accv, D->p, t.d, t.bstride(N), kt, C, false, true, ctx.n_all, ctx.n_q, K, ctx.alpha, limbs, nd, B,
                       any);
-        launch_automorphism(lc(), base.view(N), ct.view(N), g, B, 1, limbs, true);  // base.c0 += sigma_g(c0)
+        launch_automorphism_sum(lc(), base.view(N), first.view(N), gt, C, B, limbs);  // base.c0 += sigma_g(c0)
         any = true;
-        ctx.counters[C_ROT] += B;
-        ctx.counters[C_KS] += B;
-        ctx.counters[C_ADD] += B;
+        r += C;
+        ctx.counters[C_ROT] += (uint64_t)C * B;
+        ctx.counters[C_KS] += (uint64_t)C * B;
+        ctx.counters[C_ADD] += (uint64_t)C * B;
     }
     if (!any) return base;
-    Cts o = moddown_add(accv, B, limbs, base.view(N), 3, 1);
-    o.scale = f.scale;
+    Cts o = alloc(B, 2, limbs);
+    moddown_add(o.view(N), accv, B, limbs, base.view(N), 3, one_galois(1, B));
+    o.scale = items.scale;
     return o;
 }
 
@@ -280,7 +313,8 @@ Cts Eval::relin_rescale(const Cts &d, const SwitchKey &rk)
     BufPtr D = modup(d2, B, L);
     DevBuf acc((size_t)B * 2 * ext * N, s);
     View accv{acc.p, (size_t)2 * ext * N, (size_t)ext * N};
-    launch_key_ip(lc(), accv, D->p, d2.p, d2.bstride, rk.buf->p, ctx.n_all, ctx.n_q, K, ctx.alpha, L, nd, 1, B);
+    launch_key_ip(lc(), accv, D->p, d2.p, d2.bstride, one_key(rk, 1), 1, true, false, ctx.n_all, ctx.n_q, K, ctx.alpha, L,
+                  nd, B);
     ctx.counters[C_KS] += B;
     D.reset();
     const RelinRescaleTable *tab = ctx.t.relin_rs + L;
@@ -316,11 +350,40 @@ Cts Eval::rotate(const Cts &a, int64_t k, const hx_keyset &ks)
     const size_t N = ctx.N;
     Cts t = alloc(a.B, 1, a.limbs);
     View c1{a.d + a.cstride(N), a.bstride(N), a.cstride(N)};
-    launch_automorphism(lc(), t.view(N), c1, g, a.B, 1, a.limbs);
+    launch_automorphism(lc(), t.view(N), c1, one_galois(g, a.B), a.B, 1, a.limbs);
     BufPtr D = modup(t.view(N), a.B, a.limbs);
     Cts o = ks_finish(D, t.view(N), a.B, a.limbs, key, 1, a.view(N), 1, g);
     o.scale = a.scale;
     ctx.counters[C_ROT] += a.B;
+    return o;
+}
+
+Cts Eval::rotate_each(const Cts &a, const std::vector<int64_t> &steps, const hx_keyset &keys)
+{
+    const int R = (int)steps.size(), B = a.B / R, N = ctx.N, K = ctx.K, limbs = a.limbs, ext = limbs + K,
+              nd = (limbs + ctx.alpha - 1) / ctx.alpha;
+    HX_CHECK(R >= 1 && R <= MAX_ROT && a.B % R == 0 && a.comps == 2, HX_EINVAL, "bad batch of rotations");
+    KeyTab kt;
+    GaloisTab gt;
+    gt.per = B;
+    for (int r = 0; r < R; r++) {
+        const uint64_t g = galois_for_step(steps[r], ctx.log_n);
+        HX_CHECK(g != 1, HX_EINVAL, "a batch of rotations takes proper ones");
+        kt.key[r] = rot_key(keys, g).buf->p;
+        kt.g[r] = 1;
+        gt.g[r] = (uint32_t)g;
+    }
+    Cts t = alloc(a.B, 1, limbs);
+    launch_automorphism(lc(), t.view(N), View{a.d + a.cstride(N), a.bstride(N), a.cstride(N)}, gt, a.B, 1, limbs);
+    BufPtr D = modup(t.view(N), a.B, limbs);
+    DevBuf acc((size_t)a.B * 2 * ext * N, s);
+    View accv{acc.p, (size_t)2 * ext * N, (size_t)ext * N};
+    launch_key_ip(lc(), accv, D->p, t.d, t.bstride(N), kt, R, false, false, ctx.n_all, ctx.n_q, K, ctx.alpha, limbs, nd, B);
+    Cts o = alloc(a.B, 2, limbs);
+    moddown_add(o.view(N), accv, a.B, limbs, a.view(N), 1, gt);
+    o.scale = a.scale;
+    ctx.counters[C_ROT] += a.B;
+    ctx.counters[C_KS] += a.B;
     return o;
 }
 
@@ -331,27 +394,59 @@ BufPtr Eval::hoist(const Cts &a)
     return modup(c1, a.B, a.limbs);
 }
 
-Cts Eval::rotate_hoisted_one(const Cts &a, const BufPtr &D, int64_t k, const hx_keyset &keys)
+void Eval::rotate_hoisted_into(const Cts &out, const Cts &a, const BufPtr &D, const int64_t *steps, int R,
+                               const hx_keyset &keys)
 {
-    const size_t N = ctx.N;
-    const uint64_t g = galois_for_step(k, ctx.log_n);
-    if (g == 1) return copy(a);
-    const SwitchKey &key = rot_key(keys, g);
-    View c1{a.d + a.cstride(N), a.bstride(N), a.cstride(N)};
-    Cts o = ks_finish(D, c1, a.B, a.limbs, key, g, a.view(N), 1, g);
-    o.scale = a.scale;
-    ctx.counters[C_ROT] += a.B;
-    ctx.counters[C_ROT_HOIST] += a.B;
-    return o;
+    const int N = ctx.N, K = ctx.K, B = a.B, limbs = a.limbs, ext = limbs + K, nd = (limbs + ctx.alpha - 1) / ctx.alpha;
+    const View c1{a.d + a.cstride(N), a.bstride(N), a.cstride(N)};
+    const int most = rot_chunk(B, limbs, MAX_ROT);
+    for (int r = 0; r < R;) {
+        View o = out.view(N);
+        o.p += (size_t)r * B * o.bstride;
+        if (galois_for_step(steps[r], ctx.log_n) == 1) {
+            launch_copy(lc(), o, a.view(N), B, 2, limbs);
+            r++;
+            continue;
+        }
+        KeyTab kt;
+        GaloisTab gt;
+        gt.per = B;
+        int C = 0;
+        for (; C < most && r + C < R; C++) {
+            const uint64_t g = galois_for_step(steps[r + C], ctx.log_n);
+            if (g == 1) break;
+            kt.key[C] = rot_key(keys, g).buf->p;
+            kt.g[C] = gt.g[C] = (uint32_t)g;
+        }
+        DevBuf acc((size_t)C * B * 2 * ext * N, s);
+        View accv{acc.p, (size_t)2 * ext * N, (size_t)ext * N};
+        launch_key_ip(lc(), accv, D->p, c1.p, c1.bstride, kt, C, true, false, ctx.n_all, ctx.n_q, K, ctx.alpha, limbs, nd, B);
+        moddown_add(o, accv, C * B, limbs, a.view(N), 1, gt, true);
+        r += C;
+        ctx.counters[C_ROT] += (uint64_t)C * B;
+        ctx.counters[C_ROT_HOIST] += (uint64_t)C * B;
+        ctx.counters[C_KS] += (uint64_t)C * B;
+    }
 }
 
-Cts Eval::hoisted_mux(const Cts &a, const BufPtr &D, int64_t k1, int64_t k2, const uint64_t *v_ext, double v_scale,
-                      uint64_t c, const hx_keyset &keys, const uint64_t *premasked)
+Cts Eval::hoisted_mux(const Cts &a, const BufPtr &D, const std::vector<MuxItem> &items, double v_scale, uint64_t c,
+                      const hx_keyset &keys)
 {
     const int N = ctx.N, K = ctx.K, limbs = a.limbs, ext = limbs + K, nd = (limbs + ctx.alpha - 1) / ctx.alpha, B = a.B;
-    const uint64_t g1 = galois_for_step(k1, ctx.log_n), g2 = galois_for_step(k2, ctx.log_n);
-    HX_CHECK(g1 != 1 && g2 != 1, HX_EINVAL, "selection needs two proper rotations");
-    const SwitchKey &key1 = rot_key(keys, g1), &key2 = rot_key(keys, g2);
+    const int C = (int)items.size();
+    HX_CHECK(C >= 1 && C <= MAX_MUX, HX_EINVAL, "too many selections in one batch");
+    MuxTab tab;
+    const bool premasked = items[0].premasked != nullptr;
+    for (int i = 0; i < C; i++) {
+        const uint64_t g1 = galois_for_step(items[i].k1, ctx.log_n), g2 = galois_for_step(items[i].k2, ctx.log_n);
+        HX_CHECK(g1 != 1 && g2 != 1, HX_EINVAL, "selection needs two proper rotations");
+        tab.k1[i] = rot_key(keys, g1).buf->p;
+        tab.k2[i] = rot_key(keys, g2).buf->p;
+        if (premasked) tab.k1[i] = items[i].premasked;
+        tab.v[i] = items[i].v_ext;
+        tab.g1[i] = (uint32_t)g1;
+        tab.g2[i] = (uint32_t)g2;
+    }
     Scalars cs;
     for (int t = 0; t < ext; t++) {
         const uint64_t q = ctx.primes[t < limbs ? t : ctx.n_q + (t - limbs)];
@@ -359,40 +454,45 @@ Cts Eval::hoisted_mux(const Cts &a, const BufPtr &D, int64_t k1, int64_t k2, con
         cs.sh[t] = shoup_companion(cs.v[t], q);
     }
     const View c1{a.d + a.cstride(N), a.bstride(N), a.cstride(N)};
-    DevBuf z((size_t)B * 2 * ext * N, s);
+    DevBuf z((size_t)C * B * 2 * ext * N, s);
     View zv{z.p, (size_t)2 * ext * N, (size_t)ext * N};
     if (premasked)
-        launch_key_ip_mux_pm(lc(), zv, D->p, c1.p, c1.bstride, premasked, ctx.n_q, K, ctx.alpha, limbs, nd, g1, g2, B);
+        launch_key_ip_mux_pm(lc(), zv, D->p, c1.p, c1.bstride, tab, C, ctx.n_q, K, ctx.alpha, limbs, nd, B);
     else
-        launch_key_ip_mux(lc(), zv, D->p, c1.p, c1.bstride, key1.buf->p, key2.buf->p, v_ext, cs, ctx.n_all, ctx.n_q, K,
-                          ctx.alpha, limbs, nd, g1, g2, B);
-    ntt_inplace(z.p, (size_t)ext * N, 2 * B, iota_vec(limbs, K), iota_vec(ctx.n_q, K), true);
-    DevBuf conv((size_t)B * 2 * limbs * N, s);
-    launch_basis_convert(lc(), reinterpret_cast<const ConvTable *>(ctx.t.moddown + limbs), ctx.K,
-                         View{conv.p, (size_t)limbs * N, 0}, View{z.p, (size_t)ext * N, 0}, 2 * B, 1, 0, 0,
-                         8.0 * N * 2 * B * (ctx.K + limbs));
-    ntt_inplace(conv.p, (size_t)limbs * N, 2 * B, iota_vec(0, limbs), iota_vec(0, limbs), false);
-    Cts o = alloc(B, 2, limbs);
+        launch_key_ip_mux(lc(), zv, D->p, c1.p, c1.bstride, tab, C, cs, ctx.n_all, ctx.n_q, K, ctx.alpha, limbs, nd, B);
+    DevBuf conv((size_t)C * B * 2 * limbs * N, s);
+    moddown_ntt(zv, conv.p, C * B, limbs);
+    Cts o = alloc(C * B, 2, limbs);
     launch_moddown_final_mux(lc(), o.view(N), zv, View{conv.p, (size_t)2 * limbs * N, (size_t)limbs * N},
-                             ctx.t.moddown + limbs, B, limbs, a.view(N), v_ext + (size_t)K * N, cs, g1, g2);
+                             ctx.t.moddown + limbs, C, B, K, limbs, a.view(N), tab, cs);
     o.scale = a.scale * v_scale;
-    ctx.counters[C_ROT] += 2 * B;
-    ctx.counters[C_ROT_HOIST] += 2 * B;
-    ctx.counters[C_MULPT] += B;
-    ctx.counters[C_ADD] += B;
-    ctx.counters[C_KS] += B;
+    ctx.counters[C_ROT] += 2ull * C * B;
+    ctx.counters[C_ROT_HOIST] += 2ull * C * B;
+    ctx.counters[C_MULPT] += (uint64_t)C * B;
+    ctx.counters[C_ADD] += (uint64_t)C * B;
+    ctx.counters[C_KS] += (uint64_t)C * B;
     return o;
 }
 
-std::vector<Cts> Eval::rotate_hoisted(const Cts &a, const std::vector<int64_t> &ks, const hx_keyset &keys)
+Cts Eval::rotate_hoisted(const Cts &a, const std::vector<int64_t> &steps, const hx_keyset &keys)
 {
     BufPtr D;
-    std::vector<Cts> out;
-    for (int64_t k : ks) {
+    for (int64_t k : steps)
         if (!D && galois_for_step(k, ctx.log_n) != 1) D = hoist(a);
-        out.push_back(rotate_hoisted_one(a, D, k, keys));
-    }
+    Cts out = alloc(a.B * (int)steps.size(), 2, a.limbs);
+    out.scale = a.scale;
+    rotate_hoisted_into(out, a, D, steps.data(), (int)steps.size(), keys);
     return out;
+}
+
+void Eval::tensor_sum(Cts &acc, const Cts &a, const Cts &b)
+{
+    HX_CHECK(a.B == b.B && a.B % acc.B == 0 && a.limbs == b.limbs && acc.limbs == a.limbs && acc.comps == 3, HX_ESCALE,
+             "tensor operands differ");
+    HX_CHECK(std::fabs(acc.scale / (a.scale * b.scale) - 1.0) <= std::ldexp(1.0, -20), HX_ESCALE, "scale mismatch");
+    launch_tensor_sum(lc(), acc.view(ctx.N), a.view(ctx.N), b.view(ctx.N), a.B / acc.B, acc.B, a.limbs);
+    ctx.counters[C_MULCT] += a.B;
+    ctx.counters[C_ADD] += a.B;
 }
 
 Cts Eval::rescale(const Cts &a, int64_t c)

@@ -193,17 +193,46 @@ void launch_add_scalar_c0(const LaunchCtx &c, View out, View a, const Scalars &s
 // mont: the products left times 2^-64 (Montgomery reductions), to be scaled back once after summing
 void launch_tensor(const LaunchCtx &c, View out3, View a, View b, int B, int limbs, bool accumulate,
                    bool mont = false);
-void launch_automorphism(const LaunchCtx &c, View out, View in, uint64_t g, int B, int comps, int limbs,
-                         bool accumulate = false);
+// Rotations of one launch, by their place in the batch: entry e of R * per entries belongs to
+// rotation e / per, so a schedule's rotations by different amounts share a launch per stage
+constexpr int MAX_ROT = 32;
+struct GaloisTab {
+    int per;
+    uint32_t g[MAX_ROT];
+};
+struct KeyTab {
+    const uint64_t *key[MAX_ROT];
+    uint32_t g[MAX_ROT];
+};
+// selections between two rotations (Step 2): their keys (k1 alone: premasked ones), masks and elements
+constexpr int MAX_MUX = 16;
+struct MuxTab {
+    const uint64_t *k1[MAX_MUX], *k2[MAX_MUX], *v[MAX_MUX];
+    uint32_t g1[MAX_MUX], g2[MAX_MUX];
+};
+inline GaloisTab one_galois(uint64_t g, int B)
+{
+    GaloisTab t;
+    t.per = B;
+    t.g[0] = (uint32_t)g;
+    return t;
+}
+// entry e of `out` = sigma_g(entry e of `in`), g = tab.g[e / tab.per]
+void launch_automorphism(const LaunchCtx &c, View out, View in, const GaloisTab &tab, int B, int comps, int limbs);
+// out[b] += sum over r < R of sigma_g[r](in[r * B + b]), component 0
+void launch_automorphism_sum(const LaunchCtx &c, View out, View in, const GaloisTab &tab, int R, int B, int limbs);
 // alg_bytes: one read of every source row and one write of every destination row (profiling)
 void launch_basis_convert(const LaunchCtx &c, const ConvTable *tab_dev, int max_src, View out, View in, int B,
                           int groups, size_t gstride_out, size_t gstride_in, double alg_bytes = 0.0);
+// Inner products of R rotations of B entries: entry r * B + b of acc from D and dnt of that entry, or
+// of entry b for every r (shared: hoisted rotations of one batch); sum: entry b the sum over r
 void launch_key_ip(const LaunchCtx &c, View acc, const uint64_t *D, const uint64_t *dnt, size_t dnt_bstride,
-                   const uint64_t *key, int n_all, int n_q, int K, int alpha, int limbs, int ndig, uint64_t g, int B,
-                   bool accumulate = false);
-// out_c = (acc_c - conv_c) * P^-1, plus add_c[galois(j)] for the components set in add_mask
+                   const KeyTab &keys, int R, bool shared, bool sum, int n_all, int n_q, int K, int alpha, int limbs,
+                   int ndig, int B, bool accumulate = false);
+// out_c = (acc_c - conv_c) * P^-1, plus add_c[galois(j)] for the components set in add_mask; entry e
+// adds entry e of add, or (shared) entry e % tab.per
 void launch_moddown_final(const LaunchCtx &c, View out, View acc, View conv, const ModDownTable *tab, int B,
-                          int limbs, View add, int add_mask, uint64_t add_galois);
+                          int limbs, View add, int add_mask, const GaloisTab &gal, bool shared = false);
 
 // ---- several rings in one launch per key-switching stage (one job = one ring's batch) ----------
 // Each kernel runs the body of its one-ring counterpart over every job: a flat grid whose block
@@ -283,24 +312,34 @@ inline void set_ntt_tables(NttJob &j, const DeviceTables &t)
     j.ftw_inv = t.ftw_inv;
 }
 void launch_lintrans_mac(const LaunchCtx &c, const MacArgs &a, int B, int limbs, int n_terms);
-// two hoisted rotations selected by a mask in the extended basis (see kernels.cu)
+// C selections, each between two hoisted rotations by a mask in the extended basis (see kernels.cu):
+// entry i * B + b of out from entry b of D
 void launch_key_ip_mux(const LaunchCtx &c, View out, const uint64_t *D, const uint64_t *dnt, size_t dnt_bstride,
-                       const uint64_t *key1, const uint64_t *key2, const uint64_t *v, const Scalars &cs, int n_all,
-                       int n_q, int K, int alpha, int limbs, int ndig, uint64_t g1, uint64_t g2, int B);
+                       const MuxTab &tab, int C, const Scalars &cs, int n_all, int n_q, int K, int alpha, int limbs,
+                       int ndig, int B);
 // premasked keys of one selection: out = [2][ndig][2][ext][N] with
 // out[0] = v (.) key1, out[1] = (c - v) (.) key2 on the rows of the extended basis (Montgomery form);
 // cR[t] = c * 2^64 mod (prime of row t)
 void launch_premask_keys(const LaunchCtx &c, uint64_t *out, const uint64_t *key1, const uint64_t *key2,
                          const uint64_t *v, const Scalars &cR, int n_all, int n_q, int K, int limbs, int ndig);
-// the inner products of a selection with premasked keys: z_h = sum_d sigma_g1(D_d) pk[0][d][h]
-// + sigma_g2(D_d) pk[1][d][h], one Montgomery reduction
+// the inner products of C selections with premasked keys: z_h = sum_d sigma_g1(D_d) pk[0][d][h]
+// + sigma_g2(D_d) pk[1][d][h], one reduction
 void launch_key_ip_mux_pm(const LaunchCtx &c, View out, const uint64_t *D, const uint64_t *dnt, size_t dnt_bstride,
-                          const uint64_t *pk, int n_q, int K, int alpha, int limbs, int ndig, uint64_t g1, uint64_t g2,
-                          int B);
+                          const MuxTab &tab, int C, int n_q, int K, int alpha, int limbs, int ndig, int B);
 // measured rates of Shoup products and 128-bit multiply-accumulates on every SM (per second)
 void alu_calibrate(const LaunchCtx &c, uint64_t q, double *shoup_per_s, double *mac_per_s);
-void launch_moddown_final_mux(const LaunchCtx &c, View out, View acc, View conv, const ModDownTable *tab, int B,
-                              int limbs, View src, const uint64_t *v, const Scalars &cs, uint64_t g1, uint64_t g2);
+// their ModDown epilogue (v's chain rows start K rows in)
+void launch_moddown_final_mux(const LaunchCtx &c, View out, View acc, View conv, const ModDownTable *tab, int C, int B,
+                              int K, int limbs, View src, const MuxTab &mux, const Scalars &cs);
+// out (+)= sum over i < C of a[i * B + b] x b[i * B + b] (3 components), each product times 2^-64
+void launch_tensor_sum(const LaunchCtx &c, View out3, View a, View b, int C, int B, int limbs);
+// prefix sums P_m = sum_{l < m} T_l (T_0 = mask_0 b, T_l = mask_l rb[(l-1) B + b]): out[(h - m) B + b] = P_m
+struct PrefixTab {
+    const uint64_t *mask[256];
+};
+void launch_mask_prefix(const LaunchCtx &c, View out, View b, View rb, const PrefixTab &tab, int h, int B, int limbs);
+// out[(2 i) B + b] = P_(h-k), out[(2 i + 1) B + b] = P_h - P_(h-k) for k = k0 + i, i < C, of the sums above
+void launch_prefix_pairs(const LaunchCtx &c, View out, View prefix, int k0, int C, int B, int limbs);
 // slots[r*S + t*beta + j] = bits[r*hh + t] for j < beta (masks expanded over the packed matrices)
 void launch_expand_masks(const LaunchCtx &c, double *slots, const uint8_t *bits, int m, int hh, int beta, size_t S);
 void launch_relin_rs_top(const LaunchCtx &c, View acc, View d, const RelinRescaleTable *tab, int B, int limbs);

@@ -244,25 +244,110 @@ __global__ void k_tensor(View out, View a, View b, const PrimeConst *__restrict_
     }
 }
 
-// out = sigma_g(in) (accumulate: out += sigma_g(in), rows modulo prime index = row)
-__device__ __forceinline__ void automorphism_body(const Blk &b, View out, View in, uint64_t g, int comps, int log_n,
-                                                  bool accumulate, const PrimeConst *__restrict__ primes)
+// out (+)= sum_i a_i x b_i over C pairs of entries B apart, the products left times 2^-64
+__global__ void k_tensor_sum(View out, View a, View b, const PrimeConst *__restrict__ primes, int C, int B, int n)
 {
-    const int n = 1 << log_n;
-    const int l = b.y, bc = b.z, bi = bc / comps, ci = bc % comps;
-    const size_t oo = bi * out.bstride + ci * out.cstride + (size_t)l * n;
-    const size_t oi = bi * in.bstride + ci * in.cstride + (size_t)l * n;
-    const uint64_t q = accumulate ? primes[l].q : 0;
-    for (int j = b.x * blockDim.x + threadIdx.x; j < n; j += b.gx * blockDim.x) {
-        const uint64_t v = in.p[oi + galois_src(j, g, log_n)];
-        out.p[oo + j] = accumulate ? addmod(out.p[oo + j], v, q) : v;
+    const int l = blockIdx.y, bi = blockIdx.z;
+    const PrimeConst P = primes[l];
+    for (int j = (blockIdx.x * blockDim.x + threadIdx.x) * 2; j < n; j += gridDim.x * blockDim.x * 2) {
+        uint64_t *o = out.p + bi * out.bstride + (size_t)l * n + j;
+        ulonglong2 r[3];
+#pragma unroll
+        for (int h = 0; h < 3; h++) r[h] = *reinterpret_cast<const ulonglong2 *>(o + h * out.cstride);
+        for (int i = 0; i < C; i++) {
+            const uint64_t *pa = a.p + (size_t)(i * B + bi) * a.bstride + (size_t)l * n + j;
+            const uint64_t *pb = b.p + (size_t)(i * B + bi) * b.bstride + (size_t)l * n + j;
+            const ulonglong2 a0 = *reinterpret_cast<const ulonglong2 *>(pa);
+            const ulonglong2 a1 = *reinterpret_cast<const ulonglong2 *>(pa + a.cstride);
+            const ulonglong2 b0 = *reinterpret_cast<const ulonglong2 *>(pb);
+            const ulonglong2 b1 = *reinterpret_cast<const ulonglong2 *>(pb + b.cstride);
+            uint64_t x[3], y[3];
+            tensor_one(a0.x, a1.x, b0.x, b1.x, P, true, x[0], x[1], x[2]);
+            tensor_one(a0.y, a1.y, b0.y, b1.y, P, true, y[0], y[1], y[2]);
+#pragma unroll
+            for (int h = 0; h < 3; h++) r[h] = make_ulonglong2(addmod(r[h].x, x[h], P.q), addmod(r[h].y, y[h], P.q));
+        }
+#pragma unroll
+        for (int h = 0; h < 3; h++) *reinterpret_cast<ulonglong2 *>(o + h * out.cstride) = r[h];
     }
 }
 
-__global__ void k_automorphism(View out, View in, uint64_t g, int comps, int log_n, bool accumulate,
-                               const PrimeConst *__restrict__ primes)
+// the running sums of the masked rotations of b, the last first (see launch_mask_prefix)
+__global__ void k_mask_prefix(View out, View b, View rb, const __grid_constant__ PrefixTab tab,
+                              const PrimeConst *__restrict__ primes, int h, int B, int n)
 {
-    automorphism_body(Blk::hw(), out, in, g, comps, log_n, accumulate, primes);
+    const int l = blockIdx.y, bi = blockIdx.z / 2, ci = blockIdx.z % 2;
+    const PrimeConst P = primes[l];
+    const size_t row = (size_t)l * n;
+    for (int j = (blockIdx.x * blockDim.x + threadIdx.x) * 2; j < n; j += gridDim.x * blockDim.x * 2) {
+        ulonglong2 s = make_ulonglong2(0, 0);
+        for (int m = 0; m < h; m++) {
+            const View &v = m ? rb : b;
+            const uint64_t *x = v.p + (size_t)(m ? (m - 1) * B + bi : bi) * v.bstride + ci * v.cstride + row + j;
+            const ulonglong2 xv = *reinterpret_cast<const ulonglong2 *>(x);
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(tab.mask[m] + row + j);
+            s.x = addmod(s.x, redc_few(__umul64hi(xv.x, w.x), xv.x * w.x, P), P.q);
+            s.y = addmod(s.y, redc_few(__umul64hi(xv.y, w.y), xv.y * w.y, P), P.q);
+            *reinterpret_cast<ulonglong2 *>(out.p + (size_t)((h - 1 - m) * B + bi) * out.bstride + ci * out.cstride + row +
+                                            j) = s;
+        }
+    }
+}
+
+// grid z: (i, entry, component) of C pairs (see launch_prefix_pairs)
+__global__ void k_prefix_pairs(View out, View prefix, const PrimeConst *__restrict__ primes, int k0, int B, int n)
+{
+    const int l = blockIdx.y, ci = blockIdx.z % 2, bi = blockIdx.z / 2 % B, i = blockIdx.z / 2 / B;
+    const uint64_t q = primes[l].q;
+    const size_t row = ci * prefix.cstride + (size_t)l * n;
+    const uint64_t *x = prefix.p + (size_t)((k0 + i) * B + bi) * prefix.bstride + row;
+    const uint64_t *full = prefix.p + bi * prefix.bstride + row;
+    uint64_t *ox = out.p + (size_t)(2 * i * B + bi) * out.bstride + ci * out.cstride + (size_t)l * n;
+    uint64_t *oy = ox + B * out.bstride;
+    for (int j = (blockIdx.x * blockDim.x + threadIdx.x) * 2; j < n; j += gridDim.x * blockDim.x * 2) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(x + j);
+        const ulonglong2 f = *reinterpret_cast<const ulonglong2 *>(full + j);
+        *reinterpret_cast<ulonglong2 *>(ox + j) = v;
+        *reinterpret_cast<ulonglong2 *>(oy + j) = make_ulonglong2(submod(f.x, v.x, q), submod(f.y, v.y, q));
+    }
+}
+
+// out = sigma_g(in)
+__device__ __forceinline__ void automorphism_body(const Blk &b, View out, View in, uint64_t g, int comps, int log_n)
+{
+    const int n = 1 << log_n;
+    const int l = b.y, bc = b.z, bi = bc / comps, ci = bc % comps;
+    uint64_t *o = out.p + bi * out.bstride + ci * out.cstride + (size_t)l * n;
+    const uint64_t *x = in.p + bi * in.bstride + ci * in.cstride + (size_t)l * n;
+    for (int j = (b.x * blockDim.x + threadIdx.x) * 2; j < n; j += b.gx * blockDim.x * 2) {
+        const int src = galois_src(j, g, log_n);
+        *reinterpret_cast<ulonglong2 *>(o + j) = make_ulonglong2(x[src], x[src ^ 1]);
+    }
+}
+
+__global__ void k_automorphism(View out, View in, const __grid_constant__ GaloisTab tab, int comps, int log_n)
+{
+    automorphism_body(Blk::hw(), out, in, tab.g[gridDim.z == comps * tab.per ? 0 : blockIdx.z / comps / tab.per], comps,
+                      log_n);
+}
+
+// component 0 of entry b: += the sum of R rotated entries b, B + b, ...
+__global__ void k_automorphism_sum(View out, View in, const __grid_constant__ GaloisTab tab, int R, int B, int log_n,
+                                   const PrimeConst *__restrict__ primes)
+{
+    const int n = 1 << log_n, l = blockIdx.y, bi = blockIdx.z;
+    const uint64_t q = primes[l].q;
+    uint64_t *o = out.p + bi * out.bstride + (size_t)l * n;
+    for (int j = (blockIdx.x * blockDim.x + threadIdx.x) * 2; j < n; j += gridDim.x * blockDim.x * 2) {
+        ulonglong2 s = *reinterpret_cast<const ulonglong2 *>(o + j);
+        for (int r = 0; r < R; r++) {
+            const uint64_t *x = in.p + (size_t)(r * B + bi) * in.bstride + (size_t)l * n;
+            const int src = galois_src(j, tab.g[r], log_n);
+            s.x = addmod(s.x, x[src], q);
+            s.y = addmod(s.y, x[src ^ 1], q);
+        }
+        *reinterpret_cast<ulonglong2 *>(o + j) = s;
+    }
 }
 
 // Fast basis conversion; grid: x over coefficients, z = b * groups + grp (at most MK sources: register
@@ -624,50 +709,65 @@ __device__ __forceinline__ void split_ip(Sum30 (&a)[2], Sum30 (&b)[2], const Spl
     }
 }
 
-// entry bi, row t, outputs j and j + 1 (j even): both halves of sum_d src_d[galois] key_d
+// row t, outputs j and j + 1 (j even) of one rotation: both halves of sum_d src_d[galois] key_d, the
+// sources those of entry di
 template <int ND>
-__device__ __forceinline__ void key_ip_split_body(const SplitIp &A, View acc, const uint64_t *__restrict__ key,
-                                                  const FoldPrime &P, int n_all, uint64_t g, bool accumulate, int bi, int t,
-                                                  int j)
+__device__ __forceinline__ void key_ip_split_body(const SplitIp &A, const uint64_t *__restrict__ key, const FoldPrime &P,
+                                                  int n_all, uint64_t g, int di, int t, int j, ulonglong2 &r0,
+                                                  ulonglong2 &r1)
 {
     const size_t n = (size_t)1 << A.log_n, half = (size_t)n_all * n;
     const int s = g == 1 ? j : galois_src(j, g, A.log_n);
     Sum30 a[2], b[2];
-    split_ip<ND>(a, b, SplitRows(A, bi, t), A.ndig, s, key + (size_t)A.prime(t) * n + j, half, P);
-    ulonglong2 *o0 = reinterpret_cast<ulonglong2 *>(acc.p + bi * acc.bstride + (size_t)t * n + j);
-    ulonglong2 *o1 = reinterpret_cast<ulonglong2 *>(acc.p + bi * acc.bstride + acc.cstride + (size_t)t * n + j);
-    ulonglong2 r0 = make_ulonglong2(a[0].reduce(P), b[0].reduce(P)), r1 = make_ulonglong2(a[1].reduce(P), b[1].reduce(P));
-    if (accumulate) {
-        const ulonglong2 p0 = *o0, p1 = *o1;
-        r0.x = addmod(r0.x, p0.x, P.q), r0.y = addmod(r0.y, p0.y, P.q);
-        r1.x = addmod(r1.x, p1.x, P.q), r1.y = addmod(r1.y, p1.y, P.q);
-    }
-    *o0 = r0;
-    *o1 = r1;
+    split_ip<ND>(a, b, SplitRows(A, di, t), A.ndig, s, key + (size_t)A.prime(t) * n + j, half, P);
+    r0 = make_ulonglong2(a[0].reduce(P), b[0].reduce(P));
+    r1 = make_ulonglong2(a[1].reduce(P), b[1].reduce(P));
+}
+
+__device__ __forceinline__ ulonglong2 addmod2(ulonglong2 x, ulonglong2 y, uint64_t q)
+{
+    return make_ulonglong2(addmod(x.x, y.x, q), addmod(x.y, y.y, q));
 }
 
 constexpr int kSplitThreads = 128;
 
-template <int ND>
+// grid z: rotations times groups of blockDim.y entries; SUM: the groups alone, each thread over the
+// rotations
+template <int ND, bool SUM>
 __global__ void __launch_bounds__(kSplitThreads, 6)
-    k_key_ip_split(const SplitIp A, View acc, const uint64_t *__restrict__ key, const FoldPrime *__restrict__ primes,
-                   int n_all, uint64_t g, bool accumulate, int B)
+    k_key_ip_split(const SplitIp A, View acc, const __grid_constant__ KeyTab keys, int R, bool shared,
+                   const FoldPrime *__restrict__ primes, int n_all, bool accumulate, int B)
 {
-    const int bi = blockIdx.z * blockDim.y + threadIdx.y, t = blockIdx.y;
+    const int groups = (B + blockDim.y - 1) / blockDim.y, t = blockIdx.y;
+    const int r0 = SUM || R == 1 ? 0 : blockIdx.z / groups;
+    const int bi = (blockIdx.z - r0 * groups) * blockDim.y + threadIdx.y;
     if (bi >= B) return;
     const FoldPrime P = primes[A.prime(t)];
-    key_ip_split_body<ND>(A, acc, key, P, n_all, g, accumulate, bi, t, 2 * (blockIdx.x * blockDim.x + threadIdx.x));
+    const int j = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+    ulonglong2 s0, s1;
+    key_ip_split_body<ND>(A, keys.key[r0], P, n_all, keys.g[r0], shared ? bi : r0 * B + bi, t, j, s0, s1);
+    if (SUM) {
+        for (int r = 1; r < R; r++) {
+            ulonglong2 x0, x1;
+            key_ip_split_body<ND>(A, keys.key[r], P, n_all, keys.g[r], shared ? bi : r * B + bi, t, j, x0, x1);
+            s0 = addmod2(s0, x0, P.q), s1 = addmod2(s1, x1, P.q);
+        }
+    }
+    uint64_t *o = acc.p + (size_t)(r0 * B + bi) * acc.bstride + ((size_t)t << A.log_n) + j;
+    ulonglong2 *o0 = reinterpret_cast<ulonglong2 *>(o), *o1 = reinterpret_cast<ulonglong2 *>(o + acc.cstride);
+    if (accumulate) s0 = addmod2(s0, *o0, P.q), s1 = addmod2(s1, *o1, P.q);
+    *o0 = s0;
+    *o1 = s1;
 }
 
 // the selection between two hoisted rotations (k_key_ip_mux below) over split keys
 template <int ND>
 __global__ void __launch_bounds__(kSplitThreads, 5)
-    k_key_ip_mux_split(const SplitIp A, View out, const uint64_t *__restrict__ key1, const uint64_t *__restrict__ key2,
-                       const uint64_t *__restrict__ v, const __grid_constant__ Scalars cs,
-                       const PrimeConst *__restrict__ primes, const FoldPrime *__restrict__ fold, int n_all, uint64_t g1,
-                       uint64_t g2, int B)
+    k_key_ip_mux_split(const SplitIp A, View out, const __grid_constant__ MuxTab tab, const __grid_constant__ Scalars cs,
+                       const PrimeConst *__restrict__ primes, const FoldPrime *__restrict__ fold, int n_all, int B)
 {
-    const int bi = blockIdx.z * blockDim.y + threadIdx.y, t = blockIdx.y;
+    const int groups = (B + blockDim.y - 1) / blockDim.y, t = blockIdx.y;
+    const int i = gridDim.z == groups ? 0 : blockIdx.z / groups, bi = (blockIdx.z - i * groups) * blockDim.y + threadIdx.y;
     if (bi >= B) return;
     const int pr = A.prime(t), j = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     const FoldPrime F = fold[pr];
@@ -676,24 +776,25 @@ __global__ void __launch_bounds__(kSplitThreads, 5)
     uint64_t xr[4], yr[4];  // (half, coefficient)
     {
         Sum30 a[2], b[2];
-        split_ip<ND>(a, b, R, A.ndig, galois_src(j, g1, A.log_n), key1 + ko, half, F);
+        split_ip<ND>(a, b, R, A.ndig, galois_src(j, tab.g1[i], A.log_n), tab.k1[i] + ko, half, F);
         xr[0] = a[0].reduce(F), xr[1] = b[0].reduce(F), xr[2] = a[1].reduce(F), xr[3] = b[1].reduce(F);
     }
     {
         Sum30 a[2], b[2];
-        split_ip<ND>(a, b, R, A.ndig, galois_src(j, g2, A.log_n), key2 + ko, half, F);
+        split_ip<ND>(a, b, R, A.ndig, galois_src(j, tab.g2[i], A.log_n), tab.k2[i] + ko, half, F);
         yr[0] = a[0].reduce(F), yr[1] = b[0].reduce(F), yr[2] = a[1].reduce(F), yr[3] = b[1].reduce(F);
     }
     const PrimeConst P = primes[pr];
     // v holds the special primes' rows first, then the chain's (a mask of any level is a prefix)
-    const ulonglong2 vv = *reinterpret_cast<const ulonglong2 *>(v + (size_t)(t < A.limbs ? A.K + t : t - A.limbs) * n + j);
+    const ulonglong2 vv =
+        *reinterpret_cast<const ulonglong2 *>(tab.v[i] + (size_t)(t < A.limbs ? A.K + t : t - A.limbs) * n + j);
     const uint64_t c = cs.v[t], csh = cs.sh[t];
 #pragma unroll
-    for (int i = 0; i < 4; i++) {
-        const uint64_t w = i % 2 ? vv.y : vv.x, d = submod(xr[i], yr[i], P.q);
-        xr[i] = addmod(shoup(yr[i], c, csh, P.q), redc_few(__umul64hi(w, d), w * d, P), P.q);
+    for (int u = 0; u < 4; u++) {
+        const uint64_t w = u % 2 ? vv.y : vv.x, d = submod(xr[u], yr[u], P.q);
+        xr[u] = addmod(shoup(yr[u], c, csh, P.q), redc_few(__umul64hi(w, d), w * d, P), P.q);
     }
-    uint64_t *o = out.p + bi * out.bstride + (size_t)t * n + j;
+    uint64_t *o = out.p + (size_t)(i * B + bi) * out.bstride + (size_t)t * n + j;
     *reinterpret_cast<ulonglong2 *>(o) = make_ulonglong2(xr[0], xr[1]);
     *reinterpret_cast<ulonglong2 *>(o + out.cstride) = make_ulonglong2(xr[2], xr[3]);
 }
@@ -701,17 +802,18 @@ __global__ void __launch_bounds__(kSplitThreads, 5)
 // the same with premasked keys [2][ndig][2][ext][n]: one sum over both rotations
 template <int ND>
 __global__ void __launch_bounds__(kSplitThreads, 5)
-    k_key_ip_mux_pm_split(const SplitIp A, View out, const uint64_t *__restrict__ pk,
-                          const FoldPrime *__restrict__ primes, uint64_t g1, uint64_t g2, int B)
+    k_key_ip_mux_pm_split(const SplitIp A, View out, const __grid_constant__ MuxTab tab,
+                          const FoldPrime *__restrict__ primes, int B)
 {
-    const int bi = blockIdx.z * blockDim.y + threadIdx.y, t = blockIdx.y;
+    const int groups = (B + blockDim.y - 1) / blockDim.y, t = blockIdx.y;
+    const int i = gridDim.z == groups ? 0 : blockIdx.z / groups, bi = (blockIdx.z - i * groups) * blockDim.y + threadIdx.y;
     if (bi >= B) return;
     const FoldPrime P = primes[A.prime(t)];
     const int j = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     const size_t n = (size_t)1 << A.log_n, half = (size_t)(A.limbs + A.K) * n, second = 2 * A.ndig * half;
-    const int s1 = galois_src(j, g1, A.log_n), s2 = galois_src(j, g2, A.log_n);
+    const int s1 = galois_src(j, tab.g1[i], A.log_n), s2 = galois_src(j, tab.g2[i], A.log_n);
     const SplitRows R(A, bi, t);
-    const uint64_t *kd = pk + (size_t)t * n + j;
+    const uint64_t *kd = tab.k1[i] + (size_t)t * n + j;
     Sum30 a[2], b[2];
     if (ND == 0) {
         for (int d = 0; d < A.ndig; d++) {
@@ -737,10 +839,9 @@ __global__ void __launch_bounds__(kSplitThreads, 5)
             split_mac(a, b, y[d], kd + second + 2 * d * half, half);
         }
     }
-    *reinterpret_cast<ulonglong2 *>(out.p + bi * out.bstride + (size_t)t * n + j) =
-        make_ulonglong2(a[0].reduce(P), b[0].reduce(P));
-    *reinterpret_cast<ulonglong2 *>(out.p + bi * out.bstride + out.cstride + (size_t)t * n + j) =
-        make_ulonglong2(a[1].reduce(P), b[1].reduce(P));
+    uint64_t *o = out.p + (size_t)(i * B + bi) * out.bstride + (size_t)t * n + j;
+    *reinterpret_cast<ulonglong2 *>(o) = make_ulonglong2(a[0].reduce(P), b[0].reduce(P));
+    *reinterpret_cast<ulonglong2 *>(o + out.cstride) = make_ulonglong2(a[1].reduce(P), b[1].reduce(P));
 }
 
 __global__ void k_key_ip(View acc, const uint64_t *__restrict__ D, const uint64_t *__restrict__ dnt, size_t dnt_bstride,
@@ -912,30 +1013,32 @@ __global__ void k_calib_mac(uint64_t *out, int iters, uint64_t k0, uint64_t k1)
     out[t] = r;
 }
 
-// ModDown epilogue of k_key_ip_mux: out_h = (z_h - conv_h) * P^-1, plus for h = 0
+// ModDown epilogue of the selections: out_h = (z_h - conv_h) * P^-1, plus for h = 0
 // c*sigma_g2(c0) + v*(sigma_g1(c0) - sigma_g2(c0))
 __global__ void k_moddown_final_mux(View out, View acc, View conv, const ModDownTable *__restrict__ tab,
-                                    const PrimeConst *__restrict__ primes, View src, const uint64_t *__restrict__ v,
-                                    const __grid_constant__ Scalars cs, uint64_t g1, uint64_t g2, int log_n)
+                                    const PrimeConst *__restrict__ primes, View src, const __grid_constant__ MuxTab mux,
+                                    const __grid_constant__ Scalars cs, int B, int K, int log_n)
 {
     const int n = 1 << log_n;
-    const int t = blockIdx.y, bc = blockIdx.z, bi = bc / 2, ci = bc % 2;
+    const int t = blockIdx.y, e = blockIdx.z / 2, ci = blockIdx.z % 2;
+    const int i = gridDim.z == 2 * B ? 0 : e / B, bi = e - i * B;
     const PrimeConst P = primes[t];
     const uint64_t q = P.q, w = tab->pinv[t], wsh = tab->pinv_sh[t];
-    const uint64_t *a = acc.p + bi * acc.bstride + ci * acc.cstride + (size_t)t * n;
-    const uint64_t *cv = conv.p + bi * conv.bstride + ci * conv.cstride + (size_t)t * n;
-    uint64_t *o = out.p + bi * out.bstride + ci * out.cstride + (size_t)t * n;
-    const uint64_t *c0 = src.p + bi * src.bstride + (size_t)t * n;
+    const uint64_t *a = acc.p + e * acc.bstride + ci * acc.cstride + (size_t)t * n;
+    const uint64_t *cv = conv.p + e * conv.bstride + ci * conv.cstride + (size_t)t * n;
+    uint64_t *o = out.p + e * out.bstride + ci * out.cstride + (size_t)t * n;
+    const uint64_t *c0 = src.p + bi * src.bstride + (size_t)t * n, *v = mux.v[i] + (size_t)(K + t) * n;
     for (int j = (blockIdx.x * blockDim.x + threadIdx.x) * 2; j < n; j += gridDim.x * blockDim.x * 2) {
         const ulonglong2 av = *reinterpret_cast<const ulonglong2 *>(a + j);
         const ulonglong2 cw = *reinterpret_cast<const ulonglong2 *>(cv + j);
         uint64_t r[2] = {shoup(submod(av.x, cw.x, q), w, wsh, q), shoup(submod(av.y, cw.y, q), w, wsh, q)};
         if (ci == 0) {
-            const ulonglong2 vv2 = *reinterpret_cast<const ulonglong2 *>(v + (size_t)t * n + j);
+            const ulonglong2 vv2 = *reinterpret_cast<const ulonglong2 *>(v + j);
             const uint64_t vs[2] = {vv2.x, vv2.y};
+            const int j1 = galois_src(j, mux.g1[i], log_n), j2 = galois_src(j, mux.g2[i], log_n);
 #pragma unroll
             for (int u = 0; u < 2; u++) {
-                const uint64_t s1 = c0[galois_src(j + u, g1, log_n)], s2 = c0[galois_src(j + u, g2, log_n)];
+                const uint64_t s1 = c0[j1 ^ u], s2 = c0[j2 ^ u];
                 const uint64_t d = submod(s1, s2, q);
                 const uint64_t sel =
                     addmod(shoup(s2, cs.v[t], cs.sh[t], q), redc_few(__umul64hi(vs[u], d), vs[u] * d, P), q);
@@ -950,7 +1053,7 @@ __global__ void k_moddown_final_mux(View out, View acc, View conv, const ModDown
 __device__ __forceinline__ void moddown_final_body(const Blk &b, View out, View acc, View conv,
                                                    const ModDownTable *__restrict__ tab,
                                                    const PrimeConst *__restrict__ primes, View add, int add_mask,
-                                                   uint64_t g, int log_n)
+                                                   int add_entry, uint64_t g, int log_n)
 {
     const int n = 1 << log_n;
     const int t = b.y, bc = b.z, bi = bc / 2, ci = bc % 2;
@@ -959,7 +1062,7 @@ __device__ __forceinline__ void moddown_final_body(const Blk &b, View out, View 
     const uint64_t *cv = conv.p + bi * conv.bstride + ci * conv.cstride + (size_t)t * n;
     uint64_t *o = out.p + bi * out.bstride + ci * out.cstride + (size_t)t * n;
     const bool has = (add_mask >> ci) & 1;
-    const uint64_t *ap = has ? add.p + bi * add.bstride + ci * add.cstride + (size_t)t * n : nullptr;
+    const uint64_t *ap = has ? add.p + add_entry * add.bstride + ci * add.cstride + (size_t)t * n : nullptr;
     for (int j = (b.x * blockDim.x + threadIdx.x) * 2; j < n; j += b.gx * blockDim.x * 2) {
         const ulonglong2 av = *reinterpret_cast<const ulonglong2 *>(a + j);
         const ulonglong2 cw = *reinterpret_cast<const ulonglong2 *>(cv + j);
@@ -972,8 +1075,9 @@ __device__ __forceinline__ void moddown_final_body(const Blk &b, View out, View 
                 r.x = addmod(r.x, x.x, q);
                 r.y = addmod(r.y, x.y, q);
             } else {
-                r.x = addmod(r.x, ap[galois_src(j, g, log_n)], q);
-                r.y = addmod(r.y, ap[galois_src(j + 1, g, log_n)], q);
+                const int s = galois_src(j, g, log_n);
+                r.x = addmod(r.x, ap[s], q);
+                r.y = addmod(r.y, ap[s ^ 1], q);
             }
         }
         *reinterpret_cast<ulonglong2 *>(o + j) = r;
@@ -981,9 +1085,11 @@ __device__ __forceinline__ void moddown_final_body(const Blk &b, View out, View 
 }
 
 __global__ void k_moddown_final(View out, View acc, View conv, const ModDownTable *__restrict__ tab,
-                                const PrimeConst *__restrict__ primes, View add, int add_mask, uint64_t g, int log_n)
+                                const PrimeConst *__restrict__ primes, View add, int add_mask,
+                                const __grid_constant__ GaloisTab gal, bool shared, int log_n)
 {
-    moddown_final_body(Blk::hw(), out, acc, conv, tab, primes, add, add_mask, g, log_n);
+    const int e = blockIdx.z / 2, r = gridDim.z == 2 * gal.per ? 0 : e / gal.per;
+    moddown_final_body(Blk::hw(), out, acc, conv, tab, primes, add, add_mask, shared ? e - r * gal.per : e, gal.g[r], log_n);
 }
 
 // r_i = ([x + floor(q_t/2)]_{q_t} mod q_i - floor(q_t/2) mod q_i) for the lower limbs
@@ -1187,7 +1293,7 @@ __global__ void k_automorphism_jobs(const AutomorphismJob *__restrict__ jobs, in
 {
     Blk b;
     const AutomorphismJob &J = job_of_block(jobs, n_jobs, blockIdx.x, b);
-    automorphism_body(b, J.out, J.in, J.g, J.comps, J.log_n, false, J.primes);
+    automorphism_body(b, J.out, J.in, J.g, J.comps, J.log_n);
 }
 
 template <int MK>
@@ -1209,8 +1315,13 @@ __global__ void k_key_ip_jobs(const KeyIpJob *__restrict__ jobs, int n_jobs)
     if (J.fold) {
         const SplitIp A{J.D, J.dnt, J.dnt_bstride, J.n_q, J.K, J.alpha, J.limbs, J.ndig, J.log_n};
         const FoldPrime P = J.fold[A.prime(b.y)];
-        for (int j = 2 * (b.x * blockDim.x + threadIdx.x); j < 1 << J.log_n; j += 2 * b.gx * blockDim.x)
-            key_ip_split_body<0>(A, J.acc, J.key, P, J.n_all, J.g, false, b.z, b.y, j);
+        for (int j = 2 * (b.x * blockDim.x + threadIdx.x); j < 1 << J.log_n; j += 2 * b.gx * blockDim.x) {
+            ulonglong2 r0, r1;
+            key_ip_split_body<0>(A, J.key, P, J.n_all, J.g, b.z, b.y, j, r0, r1);
+            uint64_t *o = J.acc.p + b.z * J.acc.bstride + ((size_t)b.y << J.log_n) + j;
+            *reinterpret_cast<ulonglong2 *>(o) = r0;
+            *reinterpret_cast<ulonglong2 *>(o + J.acc.cstride) = r1;
+        }
         return;
     }
     key_ip_body(b, J.acc, J.D, J.dnt, J.dnt_bstride, J.key, J.primes, J.n_all, J.n_q, J.K, J.alpha, J.limbs, J.ndig,
@@ -1221,7 +1332,7 @@ __global__ void k_moddown_jobs(const ModDownJob *__restrict__ jobs, int n_jobs)
 {
     Blk b;
     const ModDownJob &J = job_of_block(jobs, n_jobs, blockIdx.x, b);
-    moddown_final_body(b, J.out, J.acc, J.conv, J.tab, J.primes, J.add, J.add_mask, J.g, J.log_n);
+    moddown_final_body(b, J.out, J.acc, J.conv, J.tab, J.primes, J.add, J.add_mask, b.z / 2, J.g, J.log_n);
 }
 
 } // namespace
@@ -1309,12 +1420,43 @@ void launch_tensor(const LaunchCtx &c, View out3, View a, View b, int B, int lim
     post(c);
 }
 
-void launch_automorphism(const LaunchCtx &c, View out, View in, uint64_t g, int B, int comps, int limbs,
-                         bool accumulate)
+void launch_automorphism(const LaunchCtx &c, View out, View in, const GaloisTab &tab, int B, int comps, int limbs)
 {
-    Timed tm_(c, K_AUTO, (accumulate ? 24.0 : 16.0) * B * comps * limbs * c.N);
-    dim3 grid(ew_blocks(c.N, 1), limbs, B * comps);
-    k_automorphism<<<grid, 256, 0, c.stream>>>(out, in, g, comps, c.log_n, accumulate, c.t->primes);
+    Timed tm_(c, K_AUTO, 16.0 * B * comps * limbs * c.N);
+    dim3 grid(ew_blocks(c.N, 2), limbs, B * comps);
+    k_automorphism<<<grid, 256, 0, c.stream>>>(out, in, tab, comps, c.log_n);
+    post(c);
+}
+
+void launch_automorphism_sum(const LaunchCtx &c, View out, View in, const GaloisTab &tab, int R, int B, int limbs)
+{
+    Timed tm_(c, K_AUTO, 8.0 * (R + 2) * B * limbs * c.N);
+    dim3 grid(ew_blocks(c.N, 2), limbs, B);
+    k_automorphism_sum<<<grid, 256, 0, c.stream>>>(out, in, tab, R, B, c.log_n, c.t->primes);
+    post(c);
+}
+
+void launch_tensor_sum(const LaunchCtx &c, View out3, View a, View b, int C, int B, int limbs)
+{
+    Timed tm_(c, K_TENSOR, 8.0 * B * limbs * c.N * (4 * C + 6));
+    dim3 grid(ew_blocks(c.N, 2), limbs, B);
+    k_tensor_sum<<<grid, 256, 0, c.stream>>>(out3, a, b, c.t->primes, C, B, c.N);
+    post(c);
+}
+
+void launch_mask_prefix(const LaunchCtx &c, View out, View b, View rb, const PrefixTab &tab, int h, int B, int limbs)
+{
+    Timed tm_(c, K_MULPT, 8.0 * (4 * B + 1) * h * limbs * c.N);
+    dim3 grid(ew_blocks(c.N, 2), limbs, B * 2);
+    k_mask_prefix<<<grid, 256, 0, c.stream>>>(out, b, rb, tab, c.t->primes, h, B, c.N);
+    post(c);
+}
+
+void launch_prefix_pairs(const LaunchCtx &c, View out, View prefix, int k0, int C, int B, int limbs)
+{
+    Timed tm_(c, K_ELEM, 8.0 * 6 * C * B * limbs * c.N);
+    dim3 grid(ew_blocks(c.N, 2), limbs, C * B * 2);
+    k_prefix_pairs<<<grid, 256, 0, c.stream>>>(out, prefix, c.t->primes, k0, B, c.N);
     post(c);
 }
 
@@ -1377,23 +1519,37 @@ static dim3 split_block(int B)
 }
 
 void launch_key_ip(const LaunchCtx &c, View acc, const uint64_t *D, const uint64_t *dnt, size_t dnt_bstride,
-                   const uint64_t *key, int n_all, int n_q, int K, int alpha, int limbs, int ndig, uint64_t g, int B,
-                   bool accumulate)
+                   const KeyTab &keys, int R, bool shared, bool sum, int n_all, int n_q, int K, int alpha, int limbs,
+                   int ndig, int B, bool accumulate)
 {
-    Timed tm_(c, K_KEYIP, 8.0 * c.N * ((double)B * ndig * (limbs + K) + 2.0 * ndig * (limbs + K) + 2.0 * B * (limbs + K)));
+    const double ext = limbs + K;
+    Timed tm_(c, K_KEYIP, 8.0 * c.N * ext * (ndig * ((shared ? 1.0 : R) * B + 2.0 * R) + 2.0 * B * (sum ? 1 : R)));
+    HX_CHECK(R >= 1 && R <= MAX_ROT, HX_EINVAL, "too many rotations in one launch");
     if (c.t->fold) {
-        const dim3 block = split_block(B), grid(c.N / 2 / block.x, limbs + K, (B + block.y - 1) / block.y);
+        const dim3 block = split_block(B);
+        const dim3 grid(c.N / 2 / block.x, limbs + K, (sum ? 1 : R) * ((B + block.y - 1) / block.y));
         const SplitIp A{D, dnt, dnt_bstride, n_q, K, alpha, limbs, ndig, c.log_n};
         by_digits(ndig, [&](auto nd) {
-            k_key_ip_split<nd()><<<grid, block, 0, c.stream>>>(A, acc, key, c.t->fold, n_all, g, accumulate, B);
+            if (sum)
+                k_key_ip_split<nd(), true><<<grid, block, 0, c.stream>>>(A, acc, keys, R, shared, c.t->fold, n_all, accumulate,
+                                                                        B);
+            else
+                k_key_ip_split<nd(), false><<<grid, block, 0, c.stream>>>(A, acc, keys, R, shared, c.t->fold, n_all,
+                                                                         accumulate, B);
         });
         post(c);
         return;
     }
     dim3 grid(ew_blocks(c.N, 2), limbs + K, B);
-    k_key_ip<<<grid, 256, 0, c.stream>>>(acc, D, dnt, dnt_bstride, key, c.t->primes, n_all, n_q, K, alpha, limbs, ndig, g,
-                                         c.log_n, accumulate, ndig <= kRedcFewTerms);
-    post(c);
+    for (int r = 0; r < R; r++) {
+        const size_t at = shared ? 0 : (size_t)r * B;
+        View o = acc;
+        if (!sum) o.p += (size_t)r * B * acc.bstride;
+        k_key_ip<<<grid, 256, 0, c.stream>>>(o, D + at * ndig * (limbs + K) * c.N, dnt + at * dnt_bstride, dnt_bstride,
+                                             keys.key[r], c.t->primes, n_all, n_q, K, alpha, limbs, ndig, keys.g[r], c.log_n,
+                                             accumulate || (sum && r > 0), ndig <= kRedcFewTerms);
+        post(c);
+    }
 }
 
 void launch_lintrans_mac(const LaunchCtx &c, const MacArgs &a, int B, int limbs, int n_terms)
@@ -1408,25 +1564,30 @@ void launch_lintrans_mac(const LaunchCtx &c, const MacArgs &a, int B, int limbs,
 }
 
 void launch_key_ip_mux(const LaunchCtx &c, View out, const uint64_t *D, const uint64_t *dnt, size_t dnt_bstride,
-                       const uint64_t *key1, const uint64_t *key2, const uint64_t *v, const Scalars &cs, int n_all,
-                       int n_q, int K, int alpha, int limbs, int ndig, uint64_t g1, uint64_t g2, int B)
+                       const MuxTab &tab, int C, const Scalars &cs, int n_all, int n_q, int K, int alpha, int limbs,
+                       int ndig, int B)
 {
-    Timed tm_(c, K_KEYIP, 8.0 * c.N * ((double)B * ndig * (limbs + K) + 4.0 * ndig * (limbs + K) + (limbs + K) +
-                                        2.0 * B * (limbs + K)));
+    const double ext = limbs + K;
+    Timed tm_(c, K_KEYIP, 8.0 * c.N * ext * ((double)B * ndig + C * (4.0 * ndig + 1.0 + 2.0 * B)));
+    HX_CHECK(C >= 1 && C <= MAX_MUX, HX_EINVAL, "too many selections in one launch");
     if (c.t->fold) {
-        const dim3 block = split_block(B), grid(c.N / 2 / block.x, limbs + K, (B + block.y - 1) / block.y);
+        const dim3 block = split_block(B), grid(c.N / 2 / block.x, limbs + K, C * ((B + block.y - 1) / block.y));
         const SplitIp A{D, dnt, dnt_bstride, n_q, K, alpha, limbs, ndig, c.log_n};
         by_digits(ndig, [&](auto nd) {
-            k_key_ip_mux_split<nd()><<<grid, block, 0, c.stream>>>(A, out, key1, key2, v, cs, c.t->primes, c.t->fold, n_all,
-                                                                  g1, g2, B);
+            k_key_ip_mux_split<nd()><<<grid, block, 0, c.stream>>>(A, out, tab, cs, c.t->primes, c.t->fold, n_all, B);
         });
         post(c);
         return;
     }
     dim3 grid(ew_blocks(c.N, 1), limbs + K, B);
-    k_key_ip_mux<<<grid, 256, 0, c.stream>>>(out, D, dnt, dnt_bstride, key1, key2, v, cs, c.t->primes, n_all, n_q, K,
-                                             alpha, limbs, ndig, g1, g2, c.log_n, ndig <= kRedcFewTerms);
-    post(c);
+    for (int i = 0; i < C; i++) {
+        View o = out;
+        o.p += (size_t)i * B * out.bstride;
+        k_key_ip_mux<<<grid, 256, 0, c.stream>>>(o, D, dnt, dnt_bstride, tab.k1[i], tab.k2[i], tab.v[i], cs, c.t->primes,
+                                                 n_all, n_q, K, alpha, limbs, ndig, tab.g1[i], tab.g2[i], c.log_n,
+                                                 ndig <= kRedcFewTerms);
+        post(c);
+    }
 }
 
 void launch_premask_keys(const LaunchCtx &c, uint64_t *out, const uint64_t *key1, const uint64_t *key2,
@@ -1439,24 +1600,28 @@ void launch_premask_keys(const LaunchCtx &c, uint64_t *out, const uint64_t *key1
 }
 
 void launch_key_ip_mux_pm(const LaunchCtx &c, View out, const uint64_t *D, const uint64_t *dnt, size_t dnt_bstride,
-                          const uint64_t *pk, int n_q, int K, int alpha, int limbs, int ndig, uint64_t g1, uint64_t g2,
-                          int B)
+                          const MuxTab &tab, int C, int n_q, int K, int alpha, int limbs, int ndig, int B)
 {
-    Timed tm_(c, K_KEYIP, 8.0 * c.N * ((double)B * ndig * (limbs + K) + 4.0 * ndig * (limbs + K) +
-                                        2.0 * B * (limbs + K)));
+    const double ext = limbs + K;
+    Timed tm_(c, K_KEYIP, 8.0 * c.N * ext * ((double)B * ndig + C * (4.0 * ndig + 2.0 * B)));
+    HX_CHECK(C >= 1 && C <= MAX_MUX, HX_EINVAL, "too many selections in one launch");
     if (c.t->fold) {
-        const dim3 block = split_block(B), grid(c.N / 2 / block.x, limbs + K, (B + block.y - 1) / block.y);
+        const dim3 block = split_block(B), grid(c.N / 2 / block.x, limbs + K, C * ((B + block.y - 1) / block.y));
         const SplitIp A{D, dnt, dnt_bstride, n_q, K, alpha, limbs, ndig, c.log_n};
         by_digits(ndig, [&](auto nd) {
-            k_key_ip_mux_pm_split<nd()><<<grid, block, 0, c.stream>>>(A, out, pk, c.t->fold, g1, g2, B);
+            k_key_ip_mux_pm_split<nd()><<<grid, block, 0, c.stream>>>(A, out, tab, c.t->fold, B);
         });
         post(c);
         return;
     }
     dim3 grid(ew_blocks(c.N, 2), limbs + K, B);
-    k_key_ip_mux_pm<<<grid, 256, 0, c.stream>>>(out, D, dnt, dnt_bstride, pk, c.t->primes, n_q, K, alpha, limbs, ndig, g1, g2,
-                                                c.log_n, 2 * ndig <= kRedcFewTerms);
-    post(c);
+    for (int i = 0; i < C; i++) {
+        View o = out;
+        o.p += (size_t)i * B * out.bstride;
+        k_key_ip_mux_pm<<<grid, 256, 0, c.stream>>>(o, D, dnt, dnt_bstride, tab.k1[i], c.t->primes, n_q, K, alpha, limbs,
+                                                    ndig, tab.g1[i], tab.g2[i], c.log_n, 2 * ndig <= kRedcFewTerms);
+        post(c);
+    }
 }
 
 void alu_calibrate(const LaunchCtx &c, uint64_t q, double *shoup_per_s, double *mac_per_s)
@@ -1485,21 +1650,21 @@ void alu_calibrate(const LaunchCtx &c, uint64_t q, double *shoup_per_s, double *
     *mac_per_s = ops / (ms2 * 1e-3);
 }
 
-void launch_moddown_final_mux(const LaunchCtx &c, View out, View acc, View conv, const ModDownTable *tab, int B,
-                              int limbs, View src, const uint64_t *v, const Scalars &cs, uint64_t g1, uint64_t g2)
+void launch_moddown_final_mux(const LaunchCtx &c, View out, View acc, View conv, const ModDownTable *tab, int C, int B,
+                              int K, int limbs, View src, const MuxTab &mux, const Scalars &cs)
 {
-    Timed tm_(c, K_MODDOWN, 8.0 * B * limbs * c.N * 9.0);
-    dim3 grid(ew_blocks(c.N, 2), limbs, B * 2);
-    k_moddown_final_mux<<<grid, 256, 0, c.stream>>>(out, acc, conv, tab, c.t->primes, src, v, cs, g1, g2, c.log_n);
+    Timed tm_(c, K_MODDOWN, 8.0 * C * B * limbs * c.N * 9.0);
+    dim3 grid(ew_blocks(c.N, 2), limbs, C * B * 2);
+    k_moddown_final_mux<<<grid, 256, 0, c.stream>>>(out, acc, conv, tab, c.t->primes, src, mux, cs, B, K, c.log_n);
     post(c);
 }
 
 void launch_moddown_final(const LaunchCtx &c, View out, View acc, View conv, const ModDownTable *tab, int B,
-                          int limbs, View add, int add_mask, uint64_t g)
+                          int limbs, View add, int add_mask, const GaloisTab &gal, bool shared)
 {
     Timed tm_(c, K_MODDOWN, 8.0 * B * 2 * limbs * c.N * ((add_mask ? 4.0 : 3.0)));
     dim3 grid(ew_blocks(c.N, 2), limbs, B * 2);
-    k_moddown_final<<<grid, 256, 0, c.stream>>>(out, acc, conv, tab, c.t->primes, add, add_mask, g, c.log_n);
+    k_moddown_final<<<grid, 256, 0, c.stream>>>(out, acc, conv, tab, c.t->primes, add, add_mask, gal, shared, c.log_n);
     post(c);
 }
 

@@ -264,7 +264,7 @@ void add_rotation_keys(hx_context &ctx, hx_keyset &ks, const std::vector<int64_t
     for (int64_t k : steps) {
         const uint64_t g = galois_for_step(k, ctx.log_n);
         if (g == 1 || ks.rot.count(g)) continue;
-        launch_automorphism(ev.lc(), View{sg.p, 0, 0}, View{ks.s_ntt->p, 0, 0}, g, 1, 1, ctx.n_all);
+        launch_automorphism(ev.lc(), View{sg.p, 0, 0}, View{ks.s_ntt->p, 0, 0}, one_galois(g, 1), 1, 1, ctx.n_all);
         SwitchKey key;
         gen_switch_key(ctx, ks, g, sg.p, key, s);
         ks.rot[g] = key;

@@ -76,8 +76,8 @@ extern "C" hx_status hx_rotate_noalloc(hx_context *ctx, const hx_keyset *ks, con
         LaunchCtx lc{ctx->log_n, N, &ctx->t, s, &ctx->counters[C_LAUNCH], nullptr};
         const View vin{const_cast<uint64_t *>(in), 2 * limbs * n, limbs * n};
         // sigma_g(c1), then ModUp of it
-        launch_automorphism(lc, View{tmp, limbs * n, n}, View{vin.p + vin.cstride, vin.bstride, vin.cstride}, g, 1, 1,
-                            limbs);
+        launch_automorphism(lc, View{tmp, limbs * n, n}, View{vin.p + vin.cstride, vin.bstride, vin.cstride},
+                            one_galois(g, 1), 1, 1, limbs);
         NttRows r;
         r.src = tmp;
         r.dst = coef;
@@ -103,7 +103,10 @@ extern "C" hx_status hx_rotate_noalloc(hx_context *ctx, const hx_keyset *ks, con
         launch_ntt(lc, r, false);
         // key inner product and ModDown, sigma_g(c0) added to the first component
         View accv{acc, 2 * (size_t)ext * n, (size_t)ext * n};
-        launch_key_ip(lc, accv, D, tmp, limbs * n, it->second.buf->p, ctx->n_all, ctx->n_q, K, A, limbs, nd, 1, 1);
+        KeyTab key;
+        key.key[0] = it->second.buf->p;
+        key.g[0] = 1;
+        launch_key_ip(lc, accv, D, tmp, limbs * n, key, 1, true, false, ctx->n_all, ctx->n_q, K, A, limbs, nd, 1);
         r.src = r.dst = acc;
         r.src_gs = r.dst_gs = (size_t)ext * n;
         r.n_groups = 2;
@@ -121,7 +124,7 @@ extern "C" hx_status hx_rotate_noalloc(hx_context *ctx, const hx_keyset *ks, con
         for (int l = 0; l < limbs; l++) r.src_off[l] = r.dst_off[l] = r.prime[l] = (int16_t)l;
         launch_ntt(lc, r, false);
         launch_moddown_final(lc, View{out, 2 * limbs * n, limbs * n}, accv, View{conv, 2 * limbs * n, limbs * n},
-                             ctx->t.moddown + limbs, 1, limbs, vin, 1, g);
+                             ctx->t.moddown + limbs, 1, limbs, vin, 1, one_galois(g, 1));
         ctx->counters[C_ROT] += 1;
         ctx->counters[C_KS] += 1;
         ctx->counters[C_MODUP] += 1;

@@ -182,7 +182,8 @@ struct Eval {
     Cts add_const(const Cts &a, double value);
     // mont: the products times 2^-64 (Montgomery form), for a sum scaled back once by from_mont
     Cts tensor(const Cts &a, const Cts &b, bool mont = false);
-    void tensor_acc(Cts &acc, const Cts &a, const Cts &b, bool mont = false);
+    // acc[b] += sum_i a[i acc.B + b] x b[i acc.B + b], the products in Montgomery form
+    void tensor_sum(Cts &acc, const Cts &a, const Cts &b);
     void from_mont(Cts &a);  // a *= 2^64, in place
     Cts relinearize(const Cts &d, const SwitchKey &rk);
     Cts rescale(const Cts &a, int64_t c = 1);  // rescale(c * a), c an integer scalar
@@ -190,26 +191,42 @@ struct Eval {
     Cts drop(const Cts &a, int limbs);  // shares storage
     Cts copy(const Cts &a);
     Cts rotate(const Cts &a, int64_t k, const hx_keyset &ks);
-    std::vector<Cts> rotate_hoisted(const Cts &a, const std::vector<int64_t> &ks, const hx_keyset &keys);
+    // a's entries in steps.size() equal groups, group i rotated by steps[i] (none 0 mod N/2)
+    Cts rotate_each(const Cts &a, const std::vector<int64_t> &steps, const hx_keyset &keys);
+    // every rotation of a's batch, from one ModUp: entry i a.B + b is entry b rotated by steps[i]
+    Cts rotate_hoisted(const Cts &a, const std::vector<int64_t> &steps, const hx_keyset &keys);
     // hoisting in two steps: the ModUp of c1 once, then any number of rotations
     BufPtr hoist(const Cts &a);
-    Cts rotate_hoisted_one(const Cts &a, const BufPtr &D, int64_t k, const hx_keyset &keys);
-    // v . Rot(a, k1) + (1 - v) . Rot(a, k2) from the ModUp D of a; the selection is applied in
-    // the extended basis before one ModDown; v_ext: mask over P then Q_l (Montgomery), encoded
-    // at scale v_scale whose integer value is c.  premasked (optional): the two rotation keys
-    // already multiplied by v and c - v (premask_keys), so the inner product gives the selection
-    Cts hoisted_mux(const Cts &a, const BufPtr &D, int64_t k1, int64_t k2, const uint64_t *v_ext, double v_scale,
-                    uint64_t c, const hx_keyset &keys, const uint64_t *premasked = nullptr);
+    void rotate_hoisted_into(const Cts &out, const Cts &a, const BufPtr &D, const int64_t *steps, int R,
+                             const hx_keyset &keys);
+    // rotations of a batch of B at `limbs` limbs (or buffers of `words` each) to run in one launch per
+    // stage, at most `most`
+    int rot_chunk(int B, int limbs, int most, size_t words = 0);
+    // v . Rot(a, k1) + (1 - v) . Rot(a, k2) from the ModUp D of a, for several (k1, k2, v) at once
+    // (entry i a.B + b: item i of entry b); the selection is applied in the extended basis before one
+    // ModDown; v_ext: mask over P then Q_l (Montgomery), encoded at scale v_scale whose integer value
+    // is c.  premasked (optional, for all items): the two rotation keys already multiplied by v and
+    // c - v (premask_keys), so the inner product gives the selection
+    struct MuxItem {
+        int64_t k1, k2;
+        const uint64_t *v_ext, *premasked;
+    };
+    Cts hoisted_mux(const Cts &a, const BufPtr &D, const std::vector<MuxItem> &items, double v_scale, uint64_t c,
+                    const hx_keyset &keys);
     void check_same(const Cts &a, const Cts &b);
 
     // hybrid key switching pieces
     BufPtr modup(const View &d, int B, int limbs);
     Cts ks_finish(const BufPtr &D, const View &dnt, int B, int limbs, const SwitchKey &key, uint64_t g,
                   const View &add, int add_mask, uint64_t add_g);
-    // ModDown of an extended-basis pair accv ([B][2][limbs+K][N]) plus `add`
-    Cts moddown_add(const View &accv, int B, int limbs, const View &add, int add_mask, uint64_t add_g);
-    // sum_i Rot(ct_i, k_i) with a single ModDown (terms with k = 0 are added unrotated)
-    Cts rotate_sum(const std::vector<std::pair<Cts, int64_t>> &items, const hx_keyset &keys);
+    // ModDown of extended-basis pairs accv ([B][2][limbs+K][N]): the converted special rows in NTT form
+    // ([B][2][limbs][N]); and the epilogue with it, plus `add`
+    void moddown_ntt(const View &accv, uint64_t *conv, int B, int limbs);
+    void moddown_add(const View &out, const View &accv, int B, int limbs, const View &add, int add_mask,
+                     const GaloisTab &gal, bool shared = false);
+    // sum_i Rot(ct_i, k_i) with a single ModDown (terms with k = 0 are added unrotated), ct_i the i-th
+    // of steps.size() equal groups of items' entries
+    Cts rotate_sum(const Cts &items, const std::vector<int64_t> &steps, const hx_keyset &keys);
     void ntt_inplace(uint64_t *p, size_t gstride, int groups, const std::vector<int> &rows_off,
                      const std::vector<int> &rows_prime, bool inverse);
     void ntt_oop(const uint64_t *src, size_t sgs, uint64_t *dst, size_t dgs, int groups,

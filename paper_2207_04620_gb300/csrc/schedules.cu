@@ -446,7 +446,7 @@ Cts lintrans(Eval &ev, const hx_keyset &ks, const Cts &ct, int lmin, int lmax, i
     std::sort(js.begin(), js.end());
     std::vector<int64_t> steps;
     for (int j : js) steps.push_back((int64_t)beta * stride * j);
-    std::vector<Cts> babies = ev.rotate_hoisted(ct, steps, ks);
+    const Cts babies = ev.rotate_hoisted(ct, steps, ks);
     std::map<int, int> jpos;
     for (size_t k = 0; k < js.size(); k++) jpos[js[k]] = (int)k;
     // every inner sum sum_j Mul_pt(baby_j, mask_(i,j)) in one fused launch
@@ -456,9 +456,9 @@ Cts lintrans(Eval &ev, const hx_keyset &ks, const Cts &ct, int lmin, int lmax, i
     std::unique_ptr<MacArgs> ma(new MacArgs());
     ma->n_baby = (int)js.size();
     ma->n_group = (int)groups.size();
-    for (size_t m = 0; m < js.size(); m++) ma->baby[m] = babies[m].d;
-    ma->baby_bstride = babies[0].bstride(N);
-    ma->baby_cstride = babies[0].cstride(N);
+    for (size_t m = 0; m < js.size(); m++) ma->baby[m] = babies.d + m * B * babies.bstride(N);
+    ma->baby_bstride = babies.bstride(N);
+    ma->baby_cstride = babies.cstride(N);
     double sc = 0;
     int g = 0, n_terms = 0;
     for (auto &kv : groups) {
@@ -473,21 +473,17 @@ Cts lintrans(Eval &ev, const hx_keyset &ks, const Cts &ct, int lmin, int lmax, i
     launch_lintrans_mac(ev.lc(), *ma, B, limbs, n_terms);
     ev.ctx.counters[C_MULPT] += (uint64_t)B * n_terms;
     ev.ctx.counters[C_ADD] += (uint64_t)B * (n_terms - ma->n_group);
-    std::vector<std::pair<Cts, int64_t>> items;
-    g = 0;
-    for (auto &kv : groups) {
-        Cts inner;
-        inner.buf = inner_buf;
-        inner.d = inner_buf->p + (size_t)g * B * 2 * limbs * N;
-        inner.B = B;
-        inner.comps = 2;
-        inner.limbs = inner.cap = limbs;
-        inner.scale = ct.scale * sc;
-        items.push_back({inner, (int64_t)beta * stride * b * kv.first});
-        g++;
-    }
+    Cts inner;
+    inner.buf = inner_buf;
+    inner.d = inner_buf->p;
+    inner.B = ma->n_group * B;
+    inner.comps = 2;
+    inner.limbs = inner.cap = limbs;
+    inner.scale = ct.scale * sc;
+    std::vector<int64_t> giant;
+    for (auto &kv : groups) giant.push_back((int64_t)beta * stride * b * kv.first);
     // giant steps: one ModDown for the whole sum
-    return ev.rotate_sum(items, ks);
+    return ev.rotate_sum(inner, giant, ks);
 }
 
 // t < h: only the terms k < t of Steps 2-3 (the rectangular product, App. D)
@@ -525,22 +521,33 @@ Cts matmul_alg3(Eval &ev, const hx_keyset &ks, const hx_matmul_plan &p, const Ct
     acc_odd.scale = acc.scale;
     HX_CUDA(cudaEventRecord(e[5], ev.s));
     HX_CUDA(cudaStreamWaitEvent(ss.s, e[5], 0));  // B0's read by the main stream comes before its release
+    // the k are taken in groups of C: a group's rotations, selections and products share a launch per
+    // stage; groups alternate between the two streams and accumulators
     Cts held[2];  // B^(k) stays alive until its consumer's use is ordered before the release
-    for (int k = 1; k < t; k++) {
-        const int par = k & 1;
-        if (held[par].buf) {  // B^(k-2): released on sb after its consumer (same parity) used it
+    const int C = ev.rot_chunk(A0.B, A0.limbs, MAX_MUX);
+    for (int k0 = 1, grp = 1; k0 < t; k0 += C, grp++) {
+        const int par = grp & 1, n = std::min(C, t - k0);
+        if (held[par].buf) {  // the last but one group's B^(k): released on sb after its consumer used it
             HX_CUDA(cudaStreamWaitEvent(ss.s, e[5 + par], 0));
             held[par] = Cts();
         }
-        held[par] = evb.rotate_hoisted_one(B0, DB, (int64_t)beta * h * k, ks);
+        std::vector<int64_t> bsteps(n);
+        std::vector<Eval::MuxItem> sel(n);
+        double sc = 0;
+        for (int i = 0; i < n; i++) {
+            const int k = k0 + i;
+            bsteps[i] = (int64_t)beta * h * k;
+            sel[i] = {(int64_t)beta * k, (int64_t)beta * (k - h), mask_pt(p, 2, k, &sc),
+                      (p.bound_uid && p.bound_uid == ks.uid) ? p.premasked[k]->p : nullptr};
+        }
+        held[par] = evb.alloc(n * B0.B, 2, B0.limbs);
+        held[par].scale = B0.scale;
+        evb.rotate_hoisted_into(held[par], B0, DB, bsteps.data(), n, ks);
         HX_CUDA(cudaEventRecord(e[3 + par], ss.s));
         Eval &ec = par ? eva : ev;
-        double sc;
-        const uint64_t *v = mask_pt(p, 2, k, &sc);
-        const uint64_t *pm = (p.bound_uid && p.bound_uid == ks.uid) ? p.premasked[k]->p : nullptr;
-        Cts Ak = ec.hoisted_mux(A0, DA, (int64_t)beta * k, (int64_t)beta * (k - h), v, sc, cm, ks, pm);
+        Cts Ak = ec.hoisted_mux(A0, DA, sel, sc, cm, ks);
         HX_CUDA(cudaStreamWaitEvent(ec.s, e[3 + par], 0));
-        ec.tensor_acc(par ? acc_odd : acc, Ak, held[par], true);
+        ec.tensor_sum(par ? acc_odd : acc, Ak, held[par]);
         HX_CUDA(cudaEventRecord(e[5 + par], ec.s));
     }
     for (int par = 0; par < 2; par++)
@@ -562,31 +569,47 @@ Cts matmul_alg3(Eval &ev, const hx_keyset &ks, const hx_matmul_plan &p, const Ct
 
 Cts matmul_depth2(Eval &ev, const hx_keyset &ks, const hx_matmul_plan &p, const Cts &A, const Cts &B, int t)
 {
-    const int h = p.h, beta = p.beta;
+    hx_context &ctx = ev.ctx;
+    const int h = p.h, beta = p.beta, N = ctx.N, n = B.B;
     Cts A0 = ev.rescale(lintrans(ev, ks, A, -h + 1, h - 1, 1, p, 0));
     std::vector<int64_t> st;
     for (int l = 1; l < h; l++) st.push_back((int64_t)beta * h * l);
-    std::vector<Cts> Rb = ev.rotate_hoisted(B, st, ks);
-    std::vector<Cts> prefix(h + 1);  // prefix[m] = S_m = sum_{l<m} T_l
-    for (int l = 0; l < h; l++) {
-        double sc;
-        const uint64_t *pt = mask_pt(p, 1, l, &sc);
-        Cts T = ev.mul_plain(l == 0 ? B : Rb[l - 1], pt, sc);
-        prefix[l + 1] = l == 0 ? T : ev.add(prefix[l], T);
+    // prefix sums S_m = sum_{l<m} T_l of T_l = mask_l . Rot(b, hl), the last (S_h) first
+    Cts S = ev.alloc(h * n, 2, B.limbs);
+    {
+        const Cts Rb = ev.rotate_hoisted(B, st, ks);
+        PrefixTab tab;
+        HX_CHECK(h <= 256, HX_EINVAL, "too many masks for the prefix sums");
+        double sc = 0;
+        for (int l = 0; l < h; l++) tab.mask[l] = mask_pt(p, 1, l, &sc);
+        S.scale = B.scale * sc;
+        launch_mask_prefix(ev.lc(), S.view(N), B.view(N), Rb.view(N), tab, h, n, B.limbs);
+        ctx.counters[C_MULPT] += (uint64_t)h * n;
+        ctx.counters[C_ADD] += (uint64_t)(h - 1) * n;
     }
-    Rb.clear();
-    const Cts &Bfull = prefix[h];
-    Cts B0 = ev.rescale(Bfull);
-    std::vector<int64_t> ast;
-    for (int k = 1; k < t; k++) ast.push_back((int64_t)beta * k);
-    for (int k = 1; k < t; k++) ast.push_back((int64_t)beta * (k - h));
-    std::vector<Cts> RA = ev.rotate_hoisted(A0, ast, ks);
+    Cts full = S;  // S_h: the first n entries
+    full.B = n;
+    const Cts B0 = ev.rescale(full);
+    BufPtr DA = t > 1 ? ev.hoist(A0) : BufPtr();
     Cts acc = ev.tensor(A0, B0, true);  // summed in Montgomery form, scaled back once
-    for (int k = 1; k < t; k++) {
-        Cts X = ev.rescale(prefix[h - k]);
-        Cts Y = ev.rescale(ev.add(Bfull, prefix[h - k], true));
-        ev.tensor_acc(acc, RA[k - 1], ev.rotate(X, (int64_t)beta * h * k, ks), true);
-        ev.tensor_acc(acc, RA[t - 1 + k - 1], ev.rotate(Y, (int64_t)beta * h * k, ks), true);
+    const int C = ev.rot_chunk(2 * n, A0.limbs, MAX_ROT / 2);
+    for (int k0 = 1; k0 < t; k0 += C) {  // groups of k share a launch per stage
+        const int c = std::min(C, t - k0);
+        std::vector<int64_t> ra, rb;
+        for (int k = k0; k < k0 + c; k++) {
+            ra.push_back((int64_t)beta * k);
+            ra.push_back((int64_t)beta * (k - h));
+            rb.push_back((int64_t)beta * h * k);
+        }
+        Cts XY = ev.alloc(2 * c * n, 2, S.limbs);  // per k: X_k = S_{h-k}, then Y_k = S_h - S_{h-k}
+        XY.scale = S.scale;
+        launch_prefix_pairs(ev.lc(), XY.view(N), S.view(N), k0, c, n, S.limbs);
+        ctx.counters[C_ADD] += (uint64_t)c * n;
+        XY = ev.rotate_each(ev.rescale(XY), rb, ks);
+        Cts RA = ev.alloc(2 * c * n, 2, A0.limbs);
+        RA.scale = A0.scale;
+        ev.rotate_hoisted_into(RA, A0, DA, ra.data(), 2 * c, ks);
+        ev.tensor_sum(acc, RA, XY);
     }
     ev.from_mont(acc);
     return ev.rescale(ev.relinearize(acc, ks.relin));
