@@ -466,13 +466,12 @@ struct ConvShared {
 };
 
 // NS sources exactly; coefficients j, j + 1 of one (entry, digit)
-template <int NS>
+template <int NS, bool shift>
 __device__ __forceinline__ void convert_split_pair(const ConvShared &S, const ConvTable &T, const uint64_t *src,
                                                    uint64_t *dst, const FoldPrime *__restrict__ primes, int d0, int dstep,
                                                    int n, int j)
 {
     const int nd = T.n_dst;
-    const bool shift = T.shift != 0;
     uint32_t l0[NS], h0[NS], l1[NS], h1[NS];
     uint64_t v0 = 0, v1 = 0;  // the overshoot's estimate in units of 2^-60, each term short by less than 2^31
 #pragma unroll
@@ -483,8 +482,10 @@ __device__ __forceinline__ void convert_split_pair(const ConvShared &S, const Co
             x.x = addmod(x.x, T.add_src[i], P.q);
             x.y = addmod(x.y, T.add_src[i], P.q);
         }
-        const uint64_t y0 = fold_finish(fold_mul((int64_t)x.x, T.inv_f[i], P), P);
-        const uint64_t y1 = fold_finish(fold_mul((int64_t)x.y, T.inv_f[i], P), P);
+        const int4 inv = T.inv_f[i];
+        uint64_t y[2] = {(uint64_t)fold_mul((int64_t)x.x, inv, P), (uint64_t)fold_mul((int64_t)x.y, inv, P)};
+        fold_finish(y, P);
+        const uint64_t y0 = y[0], y1 = y[1];
         l0[i] = (uint32_t)y0 & kMask30, h0[i] = (uint32_t)(y0 >> 30);
         l1[i] = (uint32_t)y1 & kMask30, h1[i] = (uint32_t)(y1 >> 30);
         if (shift) {
@@ -508,6 +509,7 @@ __device__ __forceinline__ void convert_split_pair(const ConvShared &S, const Co
             u1 = (uint32_t)__double2ull_rd(s1);
         }
     }
+#pragma unroll 2
     for (int d = d0; d < nd; d += dstep) {
         Sum30 s0, s1;
         if (shift) {  // - u (product of the sources) - h
@@ -524,7 +526,9 @@ __device__ __forceinline__ void convert_split_pair(const ConvShared &S, const Co
             s1.mac(l1[i], h1[i], w);
         }
         const SumPrime P = S.dst[d];
-        *reinterpret_cast<ulonglong2 *>(dst + (size_t)S.row[d] * n + j) = make_ulonglong2(s0.reduce(P), s1.reduce(P));
+        uint64_t r[2] = {s0.reduce(P), s1.reduce(P)};
+        settle_rare(r, P.q);
+        *reinterpret_cast<ulonglong2 *>(dst + (size_t)S.row[d] * n + j) = make_ulonglong2(r[0], r[1]);
     }
 }
 
@@ -540,7 +544,8 @@ __device__ __forceinline__ void convert_split_up_to(const ConvShared &S, const C
             return;
         }
     }
-    convert_split_pair<NS>(S, T, src, dst, primes, d0, dstep, n, j);
+    if (T.shift) convert_split_pair<NS, true>(S, T, src, dst, primes, d0, dstep, n, j);
+    else convert_split_pair<NS, false>(S, T, src, dst, primes, d0, dstep, n, j);
 }
 
 // blocks split at j over x, at the destinations over y; MK: the launch's largest source count (a
@@ -720,8 +725,10 @@ __device__ __forceinline__ void key_ip_split_body(const SplitIp &A, const uint64
     const int s = g == 1 ? j : galois_src(j, g, A.log_n);
     Sum30 a[2], b[2];
     split_ip<ND>(a, b, SplitRows(A, di, t), A.ndig, s, key + (size_t)A.prime(t) * n + j, half, P);
-    r0 = make_ulonglong2(a[0].reduce(P), b[0].reduce(P));
-    r1 = make_ulonglong2(a[1].reduce(P), b[1].reduce(P));
+    uint64_t r[4] = {a[0].reduce(P), b[0].reduce(P), a[1].reduce(P), b[1].reduce(P)};
+    settle_rare(r, P.q);
+    r0 = make_ulonglong2(r[0], r[1]);
+    r1 = make_ulonglong2(r[2], r[3]);
 }
 
 __device__ __forceinline__ ulonglong2 addmod2(ulonglong2 x, ulonglong2 y, uint64_t q)
@@ -778,11 +785,13 @@ __global__ void __launch_bounds__(kSplitThreads, 5)
         Sum30 a[2], b[2];
         split_ip<ND>(a, b, R, A.ndig, galois_src(j, tab.g1[i], A.log_n), tab.k1[i] + ko, half, F);
         xr[0] = a[0].reduce(F), xr[1] = b[0].reduce(F), xr[2] = a[1].reduce(F), xr[3] = b[1].reduce(F);
+        settle_rare(xr, F.q);
     }
     {
         Sum30 a[2], b[2];
         split_ip<ND>(a, b, R, A.ndig, galois_src(j, tab.g2[i], A.log_n), tab.k2[i] + ko, half, F);
         yr[0] = a[0].reduce(F), yr[1] = b[0].reduce(F), yr[2] = a[1].reduce(F), yr[3] = b[1].reduce(F);
+        settle_rare(yr, F.q);
     }
     const PrimeConst P = primes[pr];
     // v holds the special primes' rows first, then the chain's (a mask of any level is a prefix)
@@ -839,9 +848,11 @@ __global__ void __launch_bounds__(kSplitThreads, 5)
             split_mac(a, b, y[d], kd + second + 2 * d * half, half);
         }
     }
+    uint64_t r[4] = {a[0].reduce(P), b[0].reduce(P), a[1].reduce(P), b[1].reduce(P)};
+    settle_rare(r, P.q);
     uint64_t *o = out.p + (size_t)(i * B + bi) * out.bstride + (size_t)t * n + j;
-    *reinterpret_cast<ulonglong2 *>(o) = make_ulonglong2(a[0].reduce(P), b[0].reduce(P));
-    *reinterpret_cast<ulonglong2 *>(o + out.cstride) = make_ulonglong2(a[1].reduce(P), b[1].reduce(P));
+    *reinterpret_cast<ulonglong2 *>(o) = make_ulonglong2(r[0], r[1]);
+    *reinterpret_cast<ulonglong2 *>(o + out.cstride) = make_ulonglong2(r[2], r[3]);
 }
 
 __global__ void k_key_ip(View acc, const uint64_t *__restrict__ D, const uint64_t *__restrict__ dnt, size_t dnt_bstride,

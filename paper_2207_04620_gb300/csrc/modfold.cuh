@@ -70,15 +70,36 @@ __device__ __forceinline__ int64_t fold(int64_t v, const FoldPrime &P)
     return mad_wide(vh >> P.c, P.d, l);
 }
 
-// v mod q in [0, q)
+// Values just folded lie in [0, q) except for about d in 2^b of them: q is added or subtracted in a
+// branch that is hardly ever taken, of one test for all N values
+template <int N> __device__ __forceinline__ void settle_rare(uint64_t (&v)[N], uint64_t q)
+{
+    bool out = false;
+#pragma unroll
+    for (int i = 0; i < N; i++) out |= v[i] >= q;  // negative ones too
+    if (out) {
+        asm volatile("");  // a branch, not selects
+#pragma unroll
+        for (int i = 0; i < N; i++) v[i] += (int64_t)v[i] < 0 ? q : v[i] >= q ? 0 - q : 0;
+    }
+}
+
+// v mod q in [0, q), for every v
+template <int N> __device__ __forceinline__ void fold_finish(uint64_t (&v)[N], const FoldPrime &P)
+{
+#pragma unroll
+    for (int i = 0; i < N; i++) v[i] = (uint64_t)fold((int64_t)v[i], P);
+    if (P.refold) {
+#pragma unroll
+        for (int i = 0; i < N; i++) v[i] = (uint64_t)fold((int64_t)v[i], P);
+    }
+    settle_rare(v, P.q);
+}
 __device__ __forceinline__ uint64_t fold_finish(int64_t v, const FoldPrime &P)
 {
-    v = fold(v, P);
-    if (P.refold) v = fold(v, P);
-    const int64_t q = (int64_t)P.q;
-    if (v < 0) v += q;
-    else if (v >= q) v -= q;
-    return (uint64_t)v;
+    uint64_t x[1] = {(uint64_t)v};
+    fold_finish(x, P);
+    return x[0];
 }
 
 // ---- sums of products in 30-bit parts
@@ -138,14 +159,13 @@ struct Sum30 {
         b &= kMask30;
         a &= (1ull << 60) - 1;
     }
-    // the sum times 2^-60 mod q, in [0, q)
+    // the sum times 2^-60 mod q, below 2^b + 2^(64-b) d (settle_rare() brings it below q)
     template <class P_> __device__ __forceinline__ uint64_t reduce(const P_ &P) const
     {
         const uint32_t m0 = ((uint32_t)a * P.minv) & kMask30;
         uint64_t t = madu(m0, P.q1, b) + (madu(m0, P.q0, a) >> 30);
         const uint32_t m1 = ((uint32_t)t * P.minv) & kMask30;
-        t = fold_u(madu(m1, P.q1, c) + (madu(m1, P.q0, t) >> 30), P);
-        return t >= P.q ? t - P.q : t;
+        return fold_u(madu(m1, P.q1, c) + (madu(m1, P.q0, t) >> 30), P);
     }
 };
 #endif

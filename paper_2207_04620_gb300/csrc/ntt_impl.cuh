@@ -42,20 +42,21 @@ struct ArithShoup {
         x = u;
         y = shoup_lazy(d, w.x, w.y, P.q);
     }
-    // the last inverse stage with N^-1 folded in, outputs in [0, q)
+    // the last inverse stage with N^-1 folded in, outputs in [0, 2q)
     static __device__ __forceinline__ void gs_last(uint64_t &x, uint64_t &y, const Prime &P)
     {
         const uint64_t two_q = 2 * P.q;
         uint64_t u = x + y;
         if (u >= two_q) u -= two_q;
         const uint64_t d = x - y + two_q;
-        x = shoup(u, P.n_inv, P.n_inv_sh, P.q);
-        y = shoup(d, P.n_inv_w1, P.n_inv_w1_sh, P.q);
+        x = shoup_lazy(u, P.n_inv, P.n_inv_sh, P.q);
+        y = shoup_lazy(d, P.n_inv_w1, P.n_inv_w1_sh, P.q);
     }
     static __device__ __forceinline__ uint64_t settle(uint64_t v, const Prime &) { return v; }
-    static __device__ __forceinline__ uint64_t finish(uint64_t v, const Prime &P)
+    template <int N> static __device__ __forceinline__ void finish(uint64_t (&v)[N], const Prime &P)
     {
-        return csub(csub(v, 2 * P.q), P.q);
+#pragma unroll
+        for (int i = 0; i < N; i++) v[i] = csub(csub(v[i], 2 * P.q), P.q);
     }
     static const Prime *primes(const DeviceTables &t) { return t.primes; }
     static const Tw *twiddles(const DeviceTables &t, bool inv) { return inv ? t.tw_inv : t.tw_fwd; }
@@ -93,11 +94,11 @@ struct ArithFold {
     static __device__ __forceinline__ void gs_last(uint64_t &x, uint64_t &y, const Prime &P)
     {
         const uint64_t d = x - y, u = x + y;
-        x = fold_finish(fold_mul((int64_t)u, P.n_inv, P), P);
-        y = fold_finish(fold_mul((int64_t)d, P.n_inv_w1, P), P);
+        x = (uint64_t)fold_mul((int64_t)u, P.n_inv, P);
+        y = (uint64_t)fold_mul((int64_t)d, P.n_inv_w1, P);
     }
     static __device__ __forceinline__ uint64_t settle(uint64_t v, const Prime &P) { return (uint64_t)fold((int64_t)v, P); }
-    static __device__ __forceinline__ uint64_t finish(uint64_t v, const Prime &P) { return fold_finish((int64_t)v, P); }
+    template <int N> static __device__ __forceinline__ void finish(uint64_t (&v)[N], const Prime &P) { fold_finish(v, P); }
     static const Prime *primes(const DeviceTables &t) { return t.fold; }
     static const Tw *twiddles(const DeviceTables &t, bool inv) { return inv ? t.ftw_inv : t.ftw_fwd; }
     static __device__ __forceinline__ const Prime *job_primes(const NttJob &J) { return J.fold; }
@@ -136,7 +137,7 @@ template <class Tw> __device__ __forceinline__ void load_pair(const Tw *p, Tw &a
 
 // R stages in registers.  IN: the inputs' bound in sixteenths (tracked arithmetic).  A forward sum
 // x +- w y only bounds x: y may reach the limit.  An inverse sum folds the larger operand first
-// where it would pass the limit.  SCALE: the inverse's stage 0 applies N^-1 and finishes.
+// where it would pass the limit.  SCALE: the inverse's stage 0 applies N^-1.
 template <class A, int R, int S0, bool INV, int IN, bool SCALE = false>
 __device__ __forceinline__ void ntt_stages(uint64_t (&v)[1 << R], const typename A::Tw *__restrict__ tw, int g0, int blk,
                                            int hi, const typename A::Prime &P)
@@ -303,10 +304,11 @@ __device__ __forceinline__ void ntt_pass(uint64_t *sh, const uint64_t *src, uint
             for (int m = 0; m < RR; m++) v[m] = sh[Tile::shared(base + m * TL, k)];
         }
         ntt_stages<A, R, S0, INV, IN, kScale>(v, tw, g0, blk0 + k * blk_step, hi, P);
-        if (!kScale) {
+        if (!FIRST && INV != Tile::kRows) {  // the transform's results
+            A::finish(v, P);
+        } else {
 #pragma unroll
-            for (int m = 0; m < RR; m++)
-                v[m] = (!INV && !FIRST && Tile::kRows) ? A::finish(v[m], P) : A::settle(v[m], P);
+            for (int m = 0; m < RR; m++) v[m] = A::settle(v[m], P);
         }
         if (FIRST) {
 #pragma unroll
