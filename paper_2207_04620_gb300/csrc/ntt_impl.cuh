@@ -72,8 +72,9 @@ struct ArithShoup {
 // so a radix-16 pass of the forward transform folds none of its 64 sums and the inverse one a few.
 //
 // The butterflies set the transform's time, so this is where it was won: 1600 limbs of N = 2^14
-// take 215 us forward and 223 us inverse against 274 and 283 with Shoup butterflies in the same
-// tiles (8.5e11 butterflies/s; the five multiply-adds alone allow 2.0e12).
+// take 199 us forward and 205 us inverse against 274 and 283 with Shoup butterflies in the same
+// tiles (9.2e11 butterflies/s; a network of them alone in registers runs at 1.5e12, and the L1 pipe
+// that returns 16 bytes of twiddle per thread and multiplication is 50-75 % busy).
 struct ArithFold {
     typedef FoldPrime Prime;
     typedef int4 Tw;
@@ -135,17 +136,16 @@ template <class Tw> __device__ __forceinline__ void load_pair(const Tw *p, Tw &a
     b = u.t[1];
 }
 
-// R stages in registers.  IN: the inputs' bound in sixteenths (tracked arithmetic).  A forward sum
-// x +- w y only bounds x: y may reach the limit.  An inverse sum folds the larger operand first
-// where it would pass the limit.  SCALE: the inverse's stage 0 applies N^-1.
-template <class A, int R, int S0, bool INV, int IN, bool SCALE = false>
-__device__ __forceinline__ void ntt_stages(uint64_t (&v)[1 << R], const typename A::Tw *__restrict__ tw, int g0, int blk,
-                                           int hi, const typename A::Prime &P)
+// R stages in registers.  bound: the values' bounds in sixteenths before and after (tracked
+// arithmetic; compile-time constants once unrolled).  A forward sum x +- w y only bounds x: y may
+// reach the limit.  An inverse sum folds its larger operand, and the other if need be, where it
+// would pass the limit.  SCALE: the inverse's stage 0 applies N^-1.
+template <class A, int R, int S0, bool INV, bool SCALE = false>
+__device__ __forceinline__ void ntt_stages(uint64_t (&v)[1 << R], int (&bound)[1 << R],
+                                           const typename A::Tw *__restrict__ tw, int g0, int blk, int hi,
+                                           const typename A::Prime &P)
 {
     constexpr int RR = 1 << R;
-    int bound[RR];
-#pragma unroll
-    for (int m = 0; m < RR; m++) bound[m] = IN;
 #pragma unroll
     for (int step = 0; step < R; step++) {
         const int vv = INV ? R - 1 - step : step;
@@ -170,11 +170,13 @@ __device__ __forceinline__ void ntt_stages(uint64_t (&v)[1 << R], const typename
                         }
                         bound[ix] = bound[iy] = bound[ix] + kFoldProduct;
                     } else {
-                        if (bound[ix] + bound[iy] > kFoldLimit) {
-                            const int k = bound[ix] >= bound[iy] ? ix : iy;
-                            v[k] = A::settle(v[k], P);
-                            bound[k] = kFoldSettled;
-                        }
+#pragma unroll
+                        for (int again = 0; again < 2; again++)
+                            if (bound[ix] + bound[iy] > kFoldLimit) {
+                                const int k = bound[ix] >= bound[iy] ? ix : iy;
+                                v[k] = A::settle(v[k], P);
+                                bound[k] = kFoldSettled;
+                            }
                         bound[ix] = bound[ix] + bound[iy];
                         bound[iy] = kFoldProduct;
                     }
@@ -186,6 +188,17 @@ __device__ __forceinline__ void ntt_stages(uint64_t (&v)[1 << R], const typename
         }
     }
 }
+
+// the bound after R forward stages (every value has the same)
+constexpr int fwd_bound(int in, int R)
+{
+    for (int i = 0; i < R; i++) in = (in + kFoldProduct > kFoldLimit ? kFoldSettled : in) + kFoldProduct;
+    return in;
+}
+// bounds between the passes of a transform: a value above its pass's bound is folded before it is
+// stored.  Forward, the column phase hands over what most of its sizes end with, unfolded; inverse,
+// every pass hands over the products as they are and folds the sums.
+constexpr int kFwdMid = 67, kInvMid = kFoldProduct;
 
 // bounds of a transform's inputs in sixteenths (tracked arithmetic): below 4q forward, 2q inverse,
 // as the Shoup butterflies take them
@@ -208,7 +221,8 @@ template <int L, int W, bool ALT> struct ColTile {
     int n2;
     __device__ __forceinline__ static int sub(int w, int) { return w % W; }
     __device__ __forceinline__ static int group(int w, int) { return w / W; }
-    __device__ __forceinline__ size_t global(int e, int k) const { return (size_t)e * n2 + k; }
+    // byte offset: 32 bits on the block's uniform base
+    __device__ __forceinline__ uint32_t global(int e, int k) const { return 8u * ((uint32_t)e * n2 + k); }
     __device__ __forceinline__ static int shared(int e, int k) { return e * W + k; }
 };
 // Rows: W contiguous blocks of M words.  The first pass of the stages takes elements 2^R2 apart
@@ -220,7 +234,7 @@ template <int L, int W, bool ALT> struct RowTile {
     static constexpr int DATA = M + (M >> R2), SK = DATA + ((RUN - DATA) % 16 + 16) % 16, WORDS = SK * W;
     __device__ __forceinline__ static int sub(int w, int items) { return w / items; }
     __device__ __forceinline__ static int group(int w, int items) { return w % items; }
-    __device__ __forceinline__ size_t global(int e, int k) const { return (size_t)k * M + e; }
+    __device__ __forceinline__ uint32_t global(int e, int k) const { return 8u * (k * M + e); }
     __device__ __forceinline__ static int shared(int e, int k) { return k * SK + e + (e >> R2); }
 };
 
@@ -234,13 +248,22 @@ __device__ __forceinline__ void st_global_32(uint64_t *p, uint64_t a, uint64_t b
     asm volatile("st.global.v4.u64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
 }
 
+__device__ __forceinline__ const uint64_t *at_bytes(const uint64_t *p, uint32_t off)
+{
+    return reinterpret_cast<const uint64_t *>(reinterpret_cast<const char *>(p) + off);
+}
+__device__ __forceinline__ uint64_t *at_bytes(uint64_t *p, uint32_t off)
+{
+    return reinterpret_cast<uint64_t *>(reinterpret_cast<char *>(p) + off);
+}
+
 // RR elements of a butterfly group, TL apart, from or to global memory; consecutive ones (TL = 1)
 // of a row in 16-byte pieces, or in 32-byte ones where the caller found the rows aligned (wide)
 template <class Tile, int RR, int TL>
 __device__ __forceinline__ void load_group(uint64_t (&v)[RR], const uint64_t *src, const Tile &t, int base, int k, bool wide)
 {
     if (Tile::kRows && TL == 1) {
-        const uint64_t *p = src + t.global(base, k);
+        const uint64_t *p = at_bytes(src, t.global(base, k));
         if (wide) {
 #pragma unroll
             for (int m = 0; m < RR; m += 4) ld_global_32(p + m, v[m], v[m + 1], v[m + 2], v[m + 3]);
@@ -254,14 +277,14 @@ __device__ __forceinline__ void load_group(uint64_t (&v)[RR], const uint64_t *sr
         }
     } else {
 #pragma unroll
-        for (int m = 0; m < RR; m++) v[m] = src[t.global(base + m * TL, k)];
+        for (int m = 0; m < RR; m++) v[m] = *at_bytes(src, t.global(base + m * TL, k));
     }
 }
 template <class Tile, int RR, int TL>
 __device__ __forceinline__ void store_group(const uint64_t (&v)[RR], uint64_t *dst, const Tile &t, int base, int k, bool wide)
 {
     if (Tile::kRows && TL == 1) {
-        uint64_t *p = dst + t.global(base, k);
+        uint64_t *p = at_bytes(dst, t.global(base, k));
         if (wide) {
 #pragma unroll
             for (int m = 0; m < RR; m += 4) st_global_32(p + m, v[m], v[m + 1], v[m + 2], v[m + 3]);
@@ -272,7 +295,7 @@ __device__ __forceinline__ void store_group(const uint64_t (&v)[RR], uint64_t *d
         }
     } else {
 #pragma unroll
-        for (int m = 0; m < RR; m++) dst[t.global(base + m * TL, k)] = v[m];
+        for (int m = 0; m < RR; m++) *at_bytes(dst, t.global(base + m * TL, k)) = v[m];
     }
 }
 
@@ -285,30 +308,36 @@ __device__ __forceinline__ void store_group(const uint64_t (&v)[RR], uint64_t *d
 // lazy values; the column phase ends with stage 0, whose butterfly also applies N^-1 --
 // x' = (x+y) N^-1 and y' = (x-y) psi^-brv(1) N^-1, one product each instead of a butterfly product
 // and two scalings -- and finishes.
-template <class A, class Tile, int L, int R, int S0, bool INV, bool FIRST, int IN>
+//
+// IN, OUT: the bounds of the values taken and handed on.
+template <class A, class Tile, int L, int R, int S0, bool INV, bool FIRST, int IN, int OUT>
 __device__ __forceinline__ void ntt_pass(uint64_t *sh, const uint64_t *src, uint64_t *dst, const Tile &tile, int n_sub,
                                          const typename A::Tw *__restrict__ tw, int g0, int blk0, int blk_step,
                                          const typename A::Prime &P, int nthr, bool wide)
 {
     constexpr int M = 1 << L, RR = 1 << R, TL = M >> (S0 + R), ITEMS = M >> R;
-    constexpr bool kScale = INV && !FIRST && !Tile::kRows;  // the pass that applies N^-1
+    constexpr bool kLast = !FIRST && INV != Tile::kRows;  // the pass that ends the transform
     for (int w = threadIdx.x; w < ITEMS * n_sub; w += nthr) {
         const int k = Tile::sub(w, ITEMS), u = Tile::group(w, ITEMS);
         const int hi = u / TL, lo = u % TL;
         const int base = hi * TL * RR + lo;
         uint64_t v[RR];
+        int bound[RR];
+#pragma unroll
+        for (int m = 0; m < RR; m++) bound[m] = IN;
         if (FIRST) {
             load_group<Tile, RR, TL>(v, src, tile, base, k, wide);
         } else {
 #pragma unroll
             for (int m = 0; m < RR; m++) v[m] = sh[Tile::shared(base + m * TL, k)];
         }
-        ntt_stages<A, R, S0, INV, IN, kScale>(v, tw, g0, blk0 + k * blk_step, hi, P);
-        if (!FIRST && INV != Tile::kRows) {  // the transform's results
+        ntt_stages<A, R, S0, INV, INV && kLast>(v, bound, tw, g0, blk0 + k * blk_step, hi, P);
+        if (kLast) {
             A::finish(v, P);
         } else {
 #pragma unroll
-            for (int m = 0; m < RR; m++) v[m] = A::settle(v[m], P);
+            for (int m = 0; m < RR; m++)
+                if (bound[m] > OUT) v[m] = A::settle(v[m], P);
         }
         if (FIRST) {
 #pragma unroll
@@ -328,32 +357,20 @@ __device__ __forceinline__ void ntt_tile(uint64_t *sh, const uint64_t *src, uint
     constexpr int R1 = Split<L, ALT>::R1, R2 = Split<L, ALT>::R2;
     constexpr int step = Tile::kRows ? 1 : 0;  // rows: every sub-transform has its own twiddles
     if (!INV) {
-        ntt_pass<A, Tile, L, R1, 0, false, true, Tile::kRows ? kFoldSettled : kFwdIn>(sh, src, dst, tile, W, tw, g0, blk0,
-                                                                                       step, P, nthr, wide);
+        constexpr int in = Tile::kRows ? kFwdMid : kFwdIn, mid = fwd_bound(in, R1);
+        ntt_pass<A, Tile, L, R1, 0, false, true, in, mid>(sh, src, dst, tile, W, tw, g0, blk0, step, P, nthr, wide);
         __syncthreads();
-        ntt_pass<A, Tile, L, R2, R1, false, false, kFoldSettled>(sh, src, dst, tile, W, tw, g0, blk0, step, P, nthr, wide);
+        ntt_pass<A, Tile, L, R2, R1, false, false, mid, kFwdMid>(sh, src, dst, tile, W, tw, g0, blk0, step, P, nthr, wide);
     } else {
-        ntt_pass<A, Tile, L, R2, R1, true, true, Tile::kRows ? kInvIn : kFoldSettled>(sh, src, dst, tile, W, tw, g0, blk0,
-                                                                                      step, P, nthr, wide);
+        constexpr int in = Tile::kRows ? kInvIn : kInvMid;
+        ntt_pass<A, Tile, L, R2, R1, true, true, in, kInvMid>(sh, src, dst, tile, W, tw, g0, blk0, step, P, nthr, wide);
         __syncthreads();
-        ntt_pass<A, Tile, L, R1, 0, true, false, kFoldSettled>(sh, src, dst, tile, W, tw, g0, blk0, step, P, nthr, wide);
+        ntt_pass<A, Tile, L, R1, 0, true, false, kInvMid, kInvMid>(sh, src, dst, tile, W, tw, g0, blk0, step, P, nthr, wide);
     }
 }
 
-// tile t of a phase -> (group, row, position along the row)
-struct TileId {
-    int g, row, bx;
-};
-__device__ __forceinline__ TileId tile_of(int t, int nb, int n_rows)
-{
-    TileId r;
-    r.bx = t % nb;
-    const int rest = t / nb;
-    r.row = rest % n_rows;
-    r.g = rest / n_rows;
-    return r;
-}
-
+// grid: tiles of a row, rows, groups
+//
 // column phase: the first LOGM stages on M rows of stride N2, COLS adjacent columns per block
 template <class A, int LOGM, int COLS, bool INV, bool ALT>
 __global__ void __launch_bounds__((1 << (LOGM - Split<LOGM, ALT>::R1)) * COLS,
@@ -363,13 +380,11 @@ k_ntt_cols(const __grid_constant__ NttRows R, const typename A::Prime *__restric
 {
     extern __shared__ uint64_t sh[];
     constexpr int T = (1 << (LOGM - Split<LOGM, ALT>::R1)) * COLS;
-    const int N = 1 << log_n, N2 = N >> LOGM;
-    const TileId id = tile_of(blockIdx.x, N2 / COLS, R.n_rows);
-    const int pr = R.prime[id.row];
+    const int N = 1 << log_n, N2 = N >> LOGM, row = blockIdx.y, c0 = blockIdx.x * COLS;
+    const int pr = R.prime[row];
     const typename A::Prime P = primes[pr];
-    uint64_t *dst = R.dst + (size_t)id.g * R.dst_gs + (size_t)R.dst_off[id.row] * N + id.bx * COLS;
-    const uint64_t *src =
-        INV ? dst : R.src + (size_t)id.g * R.src_gs + (size_t)R.src_off[id.row] * N + id.bx * COLS;
+    uint64_t *dst = R.dst + blockIdx.z * R.dst_gs + (size_t)R.dst_off[row] * N + c0;
+    const uint64_t *src = INV ? dst : R.src + blockIdx.z * R.src_gs + (size_t)R.src_off[row] * N + c0;
     ntt_tile<A, ColTile<LOGM, COLS, ALT>, LOGM, COLS, INV, ALT>(sh, src, dst, ColTile<LOGM, COLS, ALT>{N2},
                                                                 tw_all + (size_t)pr * N, 0, 0, P, T, false);
 }
@@ -384,12 +399,11 @@ k_ntt_rows(const __grid_constant__ NttRows R, const typename A::Prime *__restric
     extern __shared__ uint64_t sh[];
     constexpr int T = (1 << (LOGM - Split<LOGM, ALT>::R1)) * ROWS;
     const int N = 1 << log_n;
-    const TileId id = tile_of(blockIdx.x, (N >> LOGM) / ROWS, R.n_rows);
-    const int pr = R.prime[id.row], r_base = id.bx * ROWS;
+    const int row = blockIdx.y, pr = R.prime[row], r_base = blockIdx.x * ROWS;
     const typename A::Prime P = primes[pr];
-    uint64_t *dst = R.dst + (size_t)id.g * R.dst_gs + (size_t)R.dst_off[id.row] * N + ((size_t)r_base << LOGM);
+    uint64_t *dst = R.dst + blockIdx.z * R.dst_gs + (size_t)R.dst_off[row] * N + (r_base << LOGM);
     const uint64_t *src =
-        INV ? R.src + (size_t)id.g * R.src_gs + (size_t)R.src_off[id.row] * N + ((size_t)r_base << LOGM) : dst;
+        INV ? R.src + blockIdx.z * R.src_gs + (size_t)R.src_off[row] * N + (r_base << LOGM) : dst;
     ntt_tile<A, RowTile<LOGM, ROWS, ALT>, LOGM, ROWS, INV, ALT>(sh, src, dst, RowTile<LOGM, ROWS, ALT>{},
                                                                 tw_all + (size_t)pr * N, log_n - LOGM, r_base, P, T, wide);
 }
@@ -404,14 +418,12 @@ void ntt_cols_w(const LaunchCtx &c, const NttRows &rows)
     constexpr int T = (1 << (LOGM - Split<LOGM, ALT>::R1)) * COLS;
     const int N2 = c.N >> LOGM;
     HX_CHECK(N2 % COLS == 0, HX_EINVAL, "NTT tile wider than the ring");
-    const long long n_tiles = (long long)(N2 / COLS) * rows.n_rows * rows.n_groups;
-    HX_CHECK(n_tiles < (1ll << 31), HX_EINVAL, "NTT batch too large");
     const size_t smem = sizeof(uint64_t) * ColTile<LOGM, COLS, ALT>::WORDS;
     static const bool attr =  // thread-safe one-time setup
         cudaFuncSetAttribute(k_ntt_cols<A, LOGM, COLS, INV, ALT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem) == cudaSuccess;
     (void)attr;
-    k_ntt_cols<A, LOGM, COLS, INV, ALT><<<(unsigned)n_tiles, T, smem, c.stream>>>(rows, A::primes(*c.t),
+    k_ntt_cols<A, LOGM, COLS, INV, ALT><<<dim3(N2 / COLS, rows.n_rows, rows.n_groups), T, smem, c.stream>>>(rows, A::primes(*c.t),
                                                                                  A::twiddles(*c.t, INV), c.log_n);
 }
 
@@ -421,8 +433,6 @@ void ntt_rows_w(const LaunchCtx &c, const NttRows &rows)
     constexpr int T = (1 << (LOGM - Split<LOGM, ALT>::R1)) * ROWS;
     const int N1 = c.N >> LOGM;
     HX_CHECK(N1 % ROWS == 0, HX_EINVAL, "NTT tile wider than the ring");
-    const long long n_tiles = (long long)(N1 / ROWS) * rows.n_rows * rows.n_groups;
-    HX_CHECK(n_tiles < (1ll << 31), HX_EINVAL, "NTT batch too large");
     const size_t smem = sizeof(uint64_t) * RowTile<LOGM, ROWS, ALT>::WORDS;
     static const bool attr =  // thread-safe one-time setup
         cudaFuncSetAttribute(k_ntt_rows<A, LOGM, ROWS, INV, ALT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -431,7 +441,7 @@ void ntt_rows_w(const LaunchCtx &c, const NttRows &rows)
     // rows and blocks are multiples of 32 bytes: 32-byte pieces need only the bases and group strides aligned
     const bool wide = ((reinterpret_cast<uintptr_t>(rows.src) | reinterpret_cast<uintptr_t>(rows.dst) |
                         (rows.src_gs | rows.dst_gs) * sizeof(uint64_t)) & 31) == 0;
-    k_ntt_rows<A, LOGM, ROWS, INV, ALT><<<(unsigned)n_tiles, T, smem, c.stream>>>(
+    k_ntt_rows<A, LOGM, ROWS, INV, ALT><<<dim3(N1 / ROWS, rows.n_rows, rows.n_groups), T, smem, c.stream>>>(
         rows, A::primes(*c.t), A::twiddles(*c.t, INV), c.log_n, wide);
 }
 
