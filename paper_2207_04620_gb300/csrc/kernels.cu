@@ -38,6 +38,7 @@ struct Blk {
 
 __global__ void k_add(View out, View a, View b, const PrimeConst *__restrict__ primes, int comps, int n, bool sub)
 {
+    after_previous_kernel();
     const int l = blockIdx.y, bc = blockIdx.z, bi = bc / comps, ci = bc % comps;
     const uint64_t q = primes[l].q;
     const size_t oo = bi * out.bstride + ci * out.cstride + (size_t)l * n;
@@ -55,6 +56,7 @@ __global__ void k_add(View out, View a, View b, const PrimeConst *__restrict__ p
 
 __global__ void k_copy(View out, View a, int comps, int n)
 {
+    after_previous_kernel();
     const int l = blockIdx.y, bc = blockIdx.z, bi = bc / comps, ci = bc % comps;
     const size_t oo = bi * out.bstride + ci * out.cstride + (size_t)l * n;
     const size_t oa = bi * a.bstride + ci * a.cstride + (size_t)l * n;
@@ -68,6 +70,7 @@ __global__ void k_copy(View out, View a, int comps, int n)
 __global__ void k_aggregate(View out, const AggSrc *__restrict__ src, int n_parties, int count,
                             const __grid_constant__ Scalars C, const PrimeConst *__restrict__ primes, int comps, int n)
 {
+    after_previous_kernel();
     const int l = blockIdx.y, bc = blockIdx.z, m = bc / comps, ci = bc % comps;
     const PrimeConst P = primes[l];
     const size_t off = (size_t)l * n;
@@ -109,6 +112,7 @@ template <int NB>
 __global__ void __launch_bounds__(128) k_lintrans_mac(const __grid_constant__ MacArgs A,
                                                       const PrimeConst *__restrict__ primes, int B, int limbs, int n)
 {
+    after_previous_kernel();
     // batch entries vary fastest over the grid: the blocks reading one mask tile run together and
     // share it through L2 (a plan's masks are larger than L2)
     const int bi = blockIdx.x, l = blockIdx.z;
@@ -150,6 +154,7 @@ __global__ void __launch_bounds__(128) k_lintrans_mac(const __grid_constant__ Ma
 __global__ void k_mul_plain(View out, View a, const uint64_t *__restrict__ pt, const PrimeConst *__restrict__ primes,
                             int n)
 {
+    after_previous_kernel();
     const int l = blockIdx.y, bc = blockIdx.z, bi = bc / 2, ci = bc % 2;
     const PrimeConst P = primes[l];
     const size_t oo = bi * out.bstride + ci * out.cstride + (size_t)l * n;
@@ -168,6 +173,7 @@ __global__ void k_mul_plain(View out, View a, const uint64_t *__restrict__ pt, c
 __global__ void k_mul_scalar(View out, View a, const __grid_constant__ Scalars sc, const PrimeConst *__restrict__ primes,
                              int comps, int n)
 {
+    after_previous_kernel();
     const int l = blockIdx.y, bc = blockIdx.z, bi = bc / comps, ci = bc % comps;
     const uint64_t q = primes[l].q, w = sc.v[l], wsh = sc.sh[l];
     const size_t oo = bi * out.bstride + ci * out.cstride + (size_t)l * n;
@@ -185,6 +191,7 @@ __global__ void k_mul_scalar(View out, View a, const __grid_constant__ Scalars s
 __global__ void k_add_scalar_c0(View out, View a, const __grid_constant__ Scalars sc,
                                 const PrimeConst *__restrict__ primes, int n)
 {
+    after_previous_kernel();
     const int l = blockIdx.y, bc = blockIdx.z, bi = bc / 2, ci = bc % 2;
     const uint64_t q = primes[l].q, s = ci == 0 ? sc.v[l] : 0;
     const size_t oo = bi * out.bstride + ci * out.cstride + (size_t)l * n;
@@ -216,6 +223,7 @@ __device__ __forceinline__ void tensor_one(uint64_t a0, uint64_t a1, uint64_t b0
 
 __global__ void k_tensor(View out, View a, View b, const PrimeConst *__restrict__ primes, int n, bool acc, bool mont)
 {
+    after_previous_kernel();
     const int l = blockIdx.y, bi = blockIdx.z;
     const PrimeConst P = primes[l];
     const size_t la = bi * a.bstride + (size_t)l * n, lb = bi * b.bstride + (size_t)l * n;
@@ -247,6 +255,7 @@ __global__ void k_tensor(View out, View a, View b, const PrimeConst *__restrict_
 // out (+)= sum_i a_i x b_i over C pairs of entries B apart, the products left times 2^-64
 __global__ void k_tensor_sum(View out, View a, View b, const PrimeConst *__restrict__ primes, int C, int B, int n)
 {
+    after_previous_kernel();
     const int l = blockIdx.y, bi = blockIdx.z;
     const PrimeConst P = primes[l];
     for (int j = (blockIdx.x * blockDim.x + threadIdx.x) * 2; j < n; j += gridDim.x * blockDim.x * 2) {
@@ -276,6 +285,7 @@ __global__ void k_tensor_sum(View out, View a, View b, const PrimeConst *__restr
 __global__ void k_mask_prefix(View out, View b, View rb, const __grid_constant__ PrefixTab tab,
                               const PrimeConst *__restrict__ primes, int h, int B, int n)
 {
+    after_previous_kernel();
     const int l = blockIdx.y, bi = blockIdx.z / 2, ci = blockIdx.z % 2;
     const PrimeConst P = primes[l];
     const size_t row = (size_t)l * n;
@@ -297,6 +307,7 @@ __global__ void k_mask_prefix(View out, View b, View rb, const __grid_constant__
 // grid z: (i, entry, component) of C pairs (see launch_prefix_pairs)
 __global__ void k_prefix_pairs(View out, View prefix, const PrimeConst *__restrict__ primes, int k0, int B, int n)
 {
+    after_previous_kernel();
     const int l = blockIdx.y, ci = blockIdx.z % 2, bi = blockIdx.z / 2 % B, i = blockIdx.z / 2 / B;
     const uint64_t q = primes[l].q;
     const size_t row = ci * prefix.cstride + (size_t)l * n;
@@ -327,6 +338,7 @@ __device__ __forceinline__ void automorphism_body(const Blk &b, View out, View i
 
 __global__ void k_automorphism(View out, View in, const __grid_constant__ GaloisTab tab, int comps, int log_n)
 {
+    after_previous_kernel();
     automorphism_body(Blk::hw(), out, in, tab.g[gridDim.z == comps * tab.per ? 0 : blockIdx.z / comps / tab.per], comps,
                       log_n);
 }
@@ -335,6 +347,7 @@ __global__ void k_automorphism(View out, View in, const __grid_constant__ Galois
 __global__ void k_automorphism_sum(View out, View in, const __grid_constant__ GaloisTab tab, int R, int B, int log_n,
                                    const PrimeConst *__restrict__ primes)
 {
+    after_previous_kernel();
     const int n = 1 << log_n, l = blockIdx.y, bi = blockIdx.z;
     const uint64_t q = primes[l].q;
     uint64_t *o = out.p + bi * out.bstride + (size_t)l * n;
@@ -579,6 +592,7 @@ __global__ void __launch_bounds__(256, MK <= 3 ? 4 : 3)
     k_basis_convert_split(const ConvTable *__restrict__ tabs, View out, View in, const FoldPrime *__restrict__ primes,
                           int groups, size_t gstride_out, size_t gstride_in, int n)
 {
+    after_previous_kernel();
     basis_convert_split_body<MK>(Blk::hw(), tabs, out, in, primes, groups, gstride_out, gstride_in, n);
 }
 
@@ -745,6 +759,7 @@ __global__ void __launch_bounds__(kSplitThreads, 6)
     k_key_ip_split(const SplitIp A, View acc, const __grid_constant__ KeyTab keys, int R, bool shared,
                    const FoldPrime *__restrict__ primes, int n_all, bool accumulate, int B)
 {
+    after_previous_kernel();
     const int groups = (B + blockDim.y - 1) / blockDim.y, t = blockIdx.y;
     const int r0 = SUM || R == 1 ? 0 : blockIdx.z / groups;
     const int bi = (blockIdx.z - r0 * groups) * blockDim.y + threadIdx.y;
@@ -773,6 +788,7 @@ __global__ void __launch_bounds__(kSplitThreads, 5)
     k_key_ip_mux_split(const SplitIp A, View out, const __grid_constant__ MuxTab tab, const __grid_constant__ Scalars cs,
                        const PrimeConst *__restrict__ primes, const FoldPrime *__restrict__ fold, int n_all, int B)
 {
+    after_previous_kernel();
     const int groups = (B + blockDim.y - 1) / blockDim.y, t = blockIdx.y;
     const int i = gridDim.z == groups ? 0 : blockIdx.z / groups, bi = (blockIdx.z - i * groups) * blockDim.y + threadIdx.y;
     if (bi >= B) return;
@@ -814,6 +830,7 @@ __global__ void __launch_bounds__(kSplitThreads, 5)
     k_key_ip_mux_pm_split(const SplitIp A, View out, const __grid_constant__ MuxTab tab,
                           const FoldPrime *__restrict__ primes, int B)
 {
+    after_previous_kernel();
     const int groups = (B + blockDim.y - 1) / blockDim.y, t = blockIdx.y;
     const int i = gridDim.z == groups ? 0 : blockIdx.z / groups, bi = (blockIdx.z - i * groups) * blockDim.y + threadIdx.y;
     if (bi >= B) return;
@@ -1030,6 +1047,7 @@ __global__ void k_moddown_final_mux(View out, View acc, View conv, const ModDown
                                     const PrimeConst *__restrict__ primes, View src, const __grid_constant__ MuxTab mux,
                                     const __grid_constant__ Scalars cs, int B, int K, int log_n)
 {
+    after_previous_kernel();
     const int n = 1 << log_n;
     const int t = blockIdx.y, e = blockIdx.z / 2, ci = blockIdx.z % 2;
     const int i = gridDim.z == 2 * B ? 0 : e / B, bi = e - i * B;
@@ -1099,6 +1117,7 @@ __global__ void k_moddown_final(View out, View acc, View conv, const ModDownTabl
                                 const PrimeConst *__restrict__ primes, View add, int add_mask,
                                 const __grid_constant__ GaloisTab gal, bool shared, int log_n)
 {
+    after_previous_kernel();
     const int e = blockIdx.z / 2, r = gridDim.z == 2 * gal.per ? 0 : e / gal.per;
     moddown_final_body(Blk::hw(), out, acc, conv, tab, primes, add, add_mask, shared ? e - r * gal.per : e, gal.g[r], log_n);
 }
@@ -1108,6 +1127,7 @@ __global__ void k_rescale_prep(View r, View xtop, const RescaleTable *__restrict
                                const PrimeConst *__restrict__ primes, int comps, int top, int n,
                                const __grid_constant__ Scalars sc, bool scaled)
 {
+    after_previous_kernel();
     const int i = blockIdx.y, bc = blockIdx.z, bi = bc / comps, ci = bc % comps;
     const uint64_t qt = primes[top].q, half = tab->half;
     const PrimeConst Pi = primes[i];
@@ -1131,6 +1151,7 @@ __global__ void k_rescale_final(View out, View in, View r, const RescaleTable *_
                                 const PrimeConst *__restrict__ primes, int comps, int n,
                                 const __grid_constant__ Scalars sc, bool scaled)
 {
+    after_previous_kernel();
     const int i = blockIdx.y, bc = blockIdx.z, bi = bc / comps, ci = bc % comps;
     const uint64_t q = primes[i].q, w = tab->qinv[i], wsh = tab->qinv_sh[i];
     const uint64_t *a = in.p + bi * in.bstride + ci * in.cstride + (size_t)i * n;
@@ -1153,6 +1174,7 @@ __global__ void k_rescale_final(View out, View in, View r, const RescaleTable *_
 __global__ void k_relin_rs_top(View acc, View d, const RelinRescaleTable *__restrict__ tab,
                                const PrimeConst *__restrict__ primes, int top, int n)
 {
+    after_previous_kernel();
     const int bc = blockIdx.z, bi = bc / 2, ci = bc % 2;
     const uint64_t q = primes[top].q, w = tab->pmod[top], wsh = tab->pmod_sh[top];
     uint64_t *a = acc.p + bi * acc.bstride + ci * acc.cstride + (size_t)top * n;
@@ -1169,6 +1191,7 @@ __global__ void k_relin_rs_top(View acc, View d, const RelinRescaleTable *__rest
 __global__ void k_relin_rs_final(View out, View acc, View d, View conv, const RelinRescaleTable *__restrict__ tab,
                                  const PrimeConst *__restrict__ primes, int n)
 {
+    after_previous_kernel();
     const int i = blockIdx.y, bc = blockIdx.z, bi = bc / 2, ci = bc % 2;
     const uint64_t q = primes[i].q, pm = tab->pmod[i], pmsh = tab->pmod_sh[i];
     const uint64_t w = tab->pqinv[i], wsh = tab->pqinv_sh[i];
@@ -1225,6 +1248,7 @@ __global__ void k_encrypt_combine(uint64_t *ct, const uint64_t *v, const uint64_
                                   const uint64_t *m, const uint64_t *pk, const PrimeConst *__restrict__ primes,
                                   int n_q, int limbs, int n)
 {
+    after_previous_kernel();
     const int l = blockIdx.y;
     const PrimeConst P = primes[l];
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
@@ -1240,6 +1264,7 @@ __global__ void k_encrypt_combine(uint64_t *ct, const uint64_t *v, const uint64_
 __global__ void k_signed_to_rows(uint64_t *out, const int64_t *in, int rows, size_t in_stride, const int *prime,
                                  const PrimeConst *__restrict__ primes, int n)
 {
+    after_previous_kernel();
     const int r = blockIdx.y, p = blockIdx.z;
     const uint64_t q = primes[prime[r]].q;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
@@ -1251,6 +1276,7 @@ __global__ void k_signed_to_rows(uint64_t *out, const int64_t *in, int rows, siz
 
 __global__ void k_to_mont(uint64_t *p, const int *prime, const PrimeConst *__restrict__ primes, int n)
 {
+    after_previous_kernel();
     const int r = blockIdx.y;
     const PrimeConst P = primes[prime[r]];
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
@@ -1273,6 +1299,7 @@ __global__ void k_mul_rows(uint64_t *out, const uint64_t *a, const uint64_t *b, 
 __global__ void k_ddec_shares(uint64_t *out, View ct, const uint64_t *shares, const PrimeConst *__restrict__ primes,
                               int np, int n)
 {
+    after_previous_kernel();
     const int p = blockIdx.y, bi = blockIdx.z;
     const PrimeConst P = primes[0];
     const uint64_t *c0 = ct.p + bi * ct.bstride;
@@ -1302,6 +1329,7 @@ __device__ __forceinline__ const J &job_of_block(const J *__restrict__ jobs, int
 
 __global__ void k_automorphism_jobs(const AutomorphismJob *__restrict__ jobs, int n_jobs)
 {
+    after_previous_kernel();
     Blk b;
     const AutomorphismJob &J = job_of_block(jobs, n_jobs, blockIdx.x, b);
     automorphism_body(b, J.out, J.in, J.g, J.comps, J.log_n);
@@ -1310,6 +1338,7 @@ __global__ void k_automorphism_jobs(const AutomorphismJob *__restrict__ jobs, in
 template <int MK>
 __global__ void __launch_bounds__(256, MK <= 4 ? 4 : 2) k_convert_jobs(const ConvertJob *__restrict__ jobs, int n_jobs)
 {
+    after_previous_kernel();
     Blk b;
     const ConvertJob &J = job_of_block(jobs, n_jobs, blockIdx.x, b);
     if (J.fold) {
@@ -1321,6 +1350,7 @@ __global__ void __launch_bounds__(256, MK <= 4 ? 4 : 2) k_convert_jobs(const Con
 
 __global__ void k_key_ip_jobs(const KeyIpJob *__restrict__ jobs, int n_jobs)
 {
+    after_previous_kernel();
     Blk b;
     const KeyIpJob &J = job_of_block(jobs, n_jobs, blockIdx.x, b);
     if (J.fold) {
@@ -1341,6 +1371,7 @@ __global__ void k_key_ip_jobs(const KeyIpJob *__restrict__ jobs, int n_jobs)
 
 __global__ void k_moddown_jobs(const ModDownJob *__restrict__ jobs, int n_jobs)
 {
+    after_previous_kernel();
     Blk b;
     const ModDownJob &J = job_of_block(jobs, n_jobs, blockIdx.x, b);
     moddown_final_body(b, J.out, J.acc, J.conv, J.tab, J.primes, J.add, J.add_mask, b.z / 2, J.g, J.log_n);
@@ -1377,7 +1408,7 @@ void launch_add(const LaunchCtx &c, View out, View a, View b, int B, int comps, 
 {
     Timed tm_(c, K_ELEM, 24.0 * B * comps * limbs * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs, B * comps);
-    k_add<<<grid, 256, 0, c.stream>>>(out, a, b, c.t->primes, comps, c.N, sub);
+    launch(c, k_add, grid, 256, 0, out, a, b, c.t->primes, comps, c.N, sub);
     post(c);
 }
 
@@ -1385,7 +1416,7 @@ void launch_copy(const LaunchCtx &c, View out, View a, int B, int comps, int lim
 {
     Timed tm_(c, K_ELEM, 16.0 * B * comps * limbs * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs, B * comps);
-    k_copy<<<grid, 256, 0, c.stream>>>(out, a, comps, c.N);
+    launch(c, k_copy, grid, 256, 0, out, a, comps, c.N);
     post(c);
 }
 
@@ -1395,7 +1426,7 @@ void launch_aggregate(const LaunchCtx &c, View out, const AggSrc *src_dev, int n
     Timed tm_(c, K_AGG, 8.0 * (n_parties + 1.0) * count * comps * limbs * c.N);
     HX_CHECK(count * comps < 65536 && limbs < 65536, HX_EINVAL, "aggregation batch too large");
     dim3 grid(ew_blocks(c.N, 2), limbs, count * comps);
-    k_aggregate<<<grid, 256, 0, c.stream>>>(out, src_dev, n_parties, count, C, c.t->primes, comps, c.N);
+    launch(c, k_aggregate, grid, 256, 0, out, src_dev, n_parties, count, C, c.t->primes, comps, c.N);
     post(c);
 }
 
@@ -1403,7 +1434,7 @@ void launch_mul_plain(const LaunchCtx &c, View out, View a, const uint64_t *pt, 
 {
     Timed tm_(c, K_MULPT, 8.0 * (4 * B + 1) * limbs * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs, B * 2);
-    k_mul_plain<<<grid, 256, 0, c.stream>>>(out, a, pt, c.t->primes, c.N);
+    launch(c, k_mul_plain, grid, 256, 0, out, a, pt, c.t->primes, c.N);
     post(c);
 }
 
@@ -1411,7 +1442,7 @@ void launch_mul_scalar(const LaunchCtx &c, View out, View a, const Scalars &sc, 
 {
     Timed tm_(c, K_ELEM, 16.0 * B * comps * limbs * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs, B * comps);
-    k_mul_scalar<<<grid, 256, 0, c.stream>>>(out, a, sc, c.t->primes, comps, c.N);
+    launch(c, k_mul_scalar, grid, 256, 0, out, a, sc, c.t->primes, comps, c.N);
     post(c);
 }
 
@@ -1419,7 +1450,7 @@ void launch_add_scalar_c0(const LaunchCtx &c, View out, View a, const Scalars &s
 {
     Timed tm_(c, K_ELEM, 32.0 * B * limbs * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs, B * 2);
-    k_add_scalar_c0<<<grid, 256, 0, c.stream>>>(out, a, sc, c.t->primes, c.N);
+    launch(c, k_add_scalar_c0, grid, 256, 0, out, a, sc, c.t->primes, c.N);
     post(c);
 }
 
@@ -1427,7 +1458,7 @@ void launch_tensor(const LaunchCtx &c, View out3, View a, View b, int B, int lim
 {
     Timed tm_(c, K_TENSOR, 8.0 * B * limbs * c.N * (accumulate ? 10 : 7));
     dim3 grid(ew_blocks(c.N, 2), limbs, B);
-    k_tensor<<<grid, 256, 0, c.stream>>>(out3, a, b, c.t->primes, c.N, accumulate, mont);
+    launch(c, k_tensor, grid, 256, 0, out3, a, b, c.t->primes, c.N, accumulate, mont);
     post(c);
 }
 
@@ -1435,7 +1466,7 @@ void launch_automorphism(const LaunchCtx &c, View out, View in, const GaloisTab 
 {
     Timed tm_(c, K_AUTO, 16.0 * B * comps * limbs * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs, B * comps);
-    k_automorphism<<<grid, 256, 0, c.stream>>>(out, in, tab, comps, c.log_n);
+    launch(c, k_automorphism, grid, 256, 0, out, in, tab, comps, c.log_n);
     post(c);
 }
 
@@ -1443,7 +1474,7 @@ void launch_automorphism_sum(const LaunchCtx &c, View out, View in, const Galois
 {
     Timed tm_(c, K_AUTO, 8.0 * (R + 2) * B * limbs * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs, B);
-    k_automorphism_sum<<<grid, 256, 0, c.stream>>>(out, in, tab, R, B, c.log_n, c.t->primes);
+    launch(c, k_automorphism_sum, grid, 256, 0, out, in, tab, R, B, c.log_n, c.t->primes);
     post(c);
 }
 
@@ -1451,7 +1482,7 @@ void launch_tensor_sum(const LaunchCtx &c, View out3, View a, View b, int C, int
 {
     Timed tm_(c, K_TENSOR, 8.0 * B * limbs * c.N * (4 * C + 6));
     dim3 grid(ew_blocks(c.N, 2), limbs, B);
-    k_tensor_sum<<<grid, 256, 0, c.stream>>>(out3, a, b, c.t->primes, C, B, c.N);
+    launch(c, k_tensor_sum, grid, 256, 0, out3, a, b, c.t->primes, C, B, c.N);
     post(c);
 }
 
@@ -1459,7 +1490,7 @@ void launch_mask_prefix(const LaunchCtx &c, View out, View b, View rb, const Pre
 {
     Timed tm_(c, K_MULPT, 8.0 * (4 * B + 1) * h * limbs * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs, B * 2);
-    k_mask_prefix<<<grid, 256, 0, c.stream>>>(out, b, rb, tab, c.t->primes, h, B, c.N);
+    launch(c, k_mask_prefix, grid, 256, 0, out, b, rb, tab, c.t->primes, h, B, c.N);
     post(c);
 }
 
@@ -1467,7 +1498,7 @@ void launch_prefix_pairs(const LaunchCtx &c, View out, View prefix, int k0, int 
 {
     Timed tm_(c, K_ELEM, 8.0 * 6 * C * B * limbs * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs, C * B * 2);
-    k_prefix_pairs<<<grid, 256, 0, c.stream>>>(out, prefix, c.t->primes, k0, B, c.N);
+    launch(c, k_prefix_pairs, grid, 256, 0, out, prefix, c.t->primes, k0, B, c.N);
     post(c);
 }
 
@@ -1486,7 +1517,7 @@ void launch_basis_convert(const LaunchCtx &c, const ConvTable *tab_dev, int max_
         if (blocks < round / 2) grid.y = (unsigned)std::min<long long>(4, std::max<long long>(1, round / 2 / blocks));
         while (grid.x > 1 && (long long)grid.x * grid.z > 2 * round) grid.x /= 2;
         auto run = [&](auto mk) {
-            k_basis_convert_split<mk()><<<grid, 256, 0, c.stream>>>(tab_dev, out, in, c.t->fold, groups, gstride_out,
+            launch(c, k_basis_convert_split<mk()>, grid, 256, 0, tab_dev, out, in, c.t->fold, groups, gstride_out,
                                                                     gstride_in, c.N);
         };
         switch (max_src) {
@@ -1542,10 +1573,10 @@ void launch_key_ip(const LaunchCtx &c, View acc, const uint64_t *D, const uint64
         const SplitIp A{D, dnt, dnt_bstride, n_q, K, alpha, limbs, ndig, c.log_n};
         by_digits(ndig, [&](auto nd) {
             if (sum)
-                k_key_ip_split<nd(), true><<<grid, block, 0, c.stream>>>(A, acc, keys, R, shared, c.t->fold, n_all, accumulate,
+                launch(c, k_key_ip_split<nd(), true>, grid, block, 0, A, acc, keys, R, shared, c.t->fold, n_all, accumulate,
                                                                         B);
             else
-                k_key_ip_split<nd(), false><<<grid, block, 0, c.stream>>>(A, acc, keys, R, shared, c.t->fold, n_all,
+                launch(c, k_key_ip_split<nd(), false>, grid, block, 0, A, acc, keys, R, shared, c.t->fold, n_all,
                                                                          accumulate, B);
         });
         post(c);
@@ -1568,9 +1599,9 @@ void launch_lintrans_mac(const LaunchCtx &c, const MacArgs &a, int B, int limbs,
     Timed tm_(c, K_MULPT, 8.0 * limbs * c.N * ((double)B * 2 * (a.n_baby + a.n_group) + n_terms));
     HX_CHECK(B >= 1 && limbs < 65536, HX_EINVAL, "bad BSGS batch");
     dim3 grid(B, (c.N / 2 + 127) / 128, limbs);
-    if (a.n_baby <= 4) k_lintrans_mac<4><<<grid, 128, 0, c.stream>>>(a, c.t->primes, B, limbs, c.N);
-    else if (a.n_baby <= 8) k_lintrans_mac<8><<<grid, 128, 0, c.stream>>>(a, c.t->primes, B, limbs, c.N);
-    else k_lintrans_mac<16><<<grid, 128, 0, c.stream>>>(a, c.t->primes, B, limbs, c.N);
+    if (a.n_baby <= 4) launch(c, k_lintrans_mac<4>, grid, 128, 0, a, c.t->primes, B, limbs, c.N);
+    else if (a.n_baby <= 8) launch(c, k_lintrans_mac<8>, grid, 128, 0, a, c.t->primes, B, limbs, c.N);
+    else launch(c, k_lintrans_mac<16>, grid, 128, 0, a, c.t->primes, B, limbs, c.N);
     post(c);
 }
 
@@ -1585,7 +1616,7 @@ void launch_key_ip_mux(const LaunchCtx &c, View out, const uint64_t *D, const ui
         const dim3 block = split_block(B), grid(c.N / 2 / block.x, limbs + K, C * ((B + block.y - 1) / block.y));
         const SplitIp A{D, dnt, dnt_bstride, n_q, K, alpha, limbs, ndig, c.log_n};
         by_digits(ndig, [&](auto nd) {
-            k_key_ip_mux_split<nd()><<<grid, block, 0, c.stream>>>(A, out, tab, cs, c.t->primes, c.t->fold, n_all, B);
+            launch(c, k_key_ip_mux_split<nd()>, grid, block, 0, A, out, tab, cs, c.t->primes, c.t->fold, n_all, B);
         });
         post(c);
         return;
@@ -1620,7 +1651,7 @@ void launch_key_ip_mux_pm(const LaunchCtx &c, View out, const uint64_t *D, const
         const dim3 block = split_block(B), grid(c.N / 2 / block.x, limbs + K, C * ((B + block.y - 1) / block.y));
         const SplitIp A{D, dnt, dnt_bstride, n_q, K, alpha, limbs, ndig, c.log_n};
         by_digits(ndig, [&](auto nd) {
-            k_key_ip_mux_pm_split<nd()><<<grid, block, 0, c.stream>>>(A, out, tab, c.t->fold, B);
+            launch(c, k_key_ip_mux_pm_split<nd()>, grid, block, 0, A, out, tab, c.t->fold, B);
         });
         post(c);
         return;
@@ -1666,7 +1697,7 @@ void launch_moddown_final_mux(const LaunchCtx &c, View out, View acc, View conv,
 {
     Timed tm_(c, K_MODDOWN, 8.0 * C * B * limbs * c.N * 9.0);
     dim3 grid(ew_blocks(c.N, 2), limbs, C * B * 2);
-    k_moddown_final_mux<<<grid, 256, 0, c.stream>>>(out, acc, conv, tab, c.t->primes, src, mux, cs, B, K, c.log_n);
+    launch(c, k_moddown_final_mux, grid, 256, 0, out, acc, conv, tab, c.t->primes, src, mux, cs, B, K, c.log_n);
     post(c);
 }
 
@@ -1675,7 +1706,7 @@ void launch_moddown_final(const LaunchCtx &c, View out, View acc, View conv, con
 {
     Timed tm_(c, K_MODDOWN, 8.0 * B * 2 * limbs * c.N * ((add_mask ? 4.0 : 3.0)));
     dim3 grid(ew_blocks(c.N, 2), limbs, B * 2);
-    k_moddown_final<<<grid, 256, 0, c.stream>>>(out, acc, conv, tab, c.t->primes, add, add_mask, gal, shared, c.log_n);
+    launch(c, k_moddown_final, grid, 256, 0, out, acc, conv, tab, c.t->primes, add, add_mask, gal, shared, c.log_n);
     post(c);
 }
 
@@ -1691,7 +1722,7 @@ void launch_relin_rs_top(const LaunchCtx &c, View acc, View d, const RelinRescal
 {
     Timed tm_(c, K_RESCALE, 24.0 * B * 2 * c.N);
     dim3 grid(ew_blocks(c.N, 2), 1, B * 2);
-    k_relin_rs_top<<<grid, 256, 0, c.stream>>>(acc, d, tab, c.t->primes, limbs - 1, c.N);
+    launch(c, k_relin_rs_top, grid, 256, 0, acc, d, tab, c.t->primes, limbs - 1, c.N);
     post(c);
 }
 
@@ -1700,7 +1731,7 @@ void launch_relin_rs_final(const LaunchCtx &c, View out, View acc, View d, View 
 {
     Timed tm_(c, K_MODDOWN, 32.0 * B * 2 * (limbs - 1) * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs - 1, B * 2);
-    k_relin_rs_final<<<grid, 256, 0, c.stream>>>(out, acc, d, conv, tab, c.t->primes, c.N);
+    launch(c, k_relin_rs_final, grid, 256, 0, out, acc, d, conv, tab, c.t->primes, c.N);
     post(c);
 }
 
@@ -1709,7 +1740,7 @@ void launch_rescale_prep(const LaunchCtx &c, View r, View xtop, const RescaleTab
 {
     Timed tm_(c, K_RESCALE, 8.0 * B * comps * (top + 1) * c.N);
     dim3 grid(ew_blocks(c.N, 2), top, B * comps);
-    k_rescale_prep<<<grid, 256, 0, c.stream>>>(r, xtop, tab, c.t->primes, comps, top, c.N, sc ? *sc : Scalars{},
+    launch(c, k_rescale_prep, grid, 256, 0, r, xtop, tab, c.t->primes, comps, top, c.N, sc ? *sc : Scalars{},
                                                sc != nullptr);
     post(c);
 }
@@ -1719,7 +1750,7 @@ void launch_rescale_final(const LaunchCtx &c, View out, View in, View r, const R
 {
     Timed tm_(c, K_RESCALE, 24.0 * B * comps * top * c.N);
     dim3 grid(ew_blocks(c.N, 2), top, B * comps);
-    k_rescale_final<<<grid, 256, 0, c.stream>>>(out, in, r, tab, c.t->primes, comps, c.N, sc ? *sc : Scalars{},
+    launch(c, k_rescale_final, grid, 256, 0, out, in, r, tab, c.t->primes, comps, c.N, sc ? *sc : Scalars{},
                                                 sc != nullptr);
     post(c);
 }
@@ -1736,7 +1767,7 @@ void launch_encrypt_combine(const LaunchCtx &c, uint64_t *ct, const uint64_t *v,
                             const uint64_t *e1, const uint64_t *m, const uint64_t *pk, int n_q, int limbs)
 {
     dim3 grid(ew_blocks(c.N, 1), limbs, 1);
-    k_encrypt_combine<<<grid, 256, 0, c.stream>>>(ct, v, e0, e1, m, pk, c.t->primes, n_q, limbs, c.N);
+    launch(c, k_encrypt_combine, grid, 256, 0, ct, v, e0, e1, m, pk, c.t->primes, n_q, limbs, c.N);
     post(c);
 }
 
@@ -1744,14 +1775,14 @@ void launch_signed_to_rows(const LaunchCtx &c, uint64_t *out, const int64_t *in,
                            size_t in_stride, const int *prime_dev)
 {
     dim3 grid(ew_blocks(c.N, 1), rows, n_in_polys);
-    k_signed_to_rows<<<grid, 256, 0, c.stream>>>(out, in, rows, in_stride, prime_dev, c.t->primes, c.N);
+    launch(c, k_signed_to_rows, grid, 256, 0, out, in, rows, in_stride, prime_dev, c.t->primes, c.N);
     post(c);
 }
 
 void launch_to_mont(const LaunchCtx &c, uint64_t *p, int rows, const int *prime_dev)
 {
     dim3 grid(ew_blocks(c.N, 1), rows, 1);
-    k_to_mont<<<grid, 256, 0, c.stream>>>(p, prime_dev, c.t->primes, c.N);
+    launch(c, k_to_mont, grid, 256, 0, p, prime_dev, c.t->primes, c.N);
     post(c);
 }
 
@@ -1765,7 +1796,7 @@ void launch_mul_rows(const LaunchCtx &c, uint64_t *out, const uint64_t *a, const
 void launch_ddec_shares(const LaunchCtx &c, uint64_t *out, View ct, const uint64_t *shares, int n_parties, int B)
 {
     dim3 grid(ew_blocks(c.N, 1), n_parties + 1, B);
-    k_ddec_shares<<<grid, 256, 0, c.stream>>>(out, ct, shares, c.t->primes, n_parties, c.N);
+    launch(c, k_ddec_shares, grid, 256, 0, out, ct, shares, c.t->primes, n_parties, c.N);
     post(c);
 }
 
@@ -1776,39 +1807,39 @@ static void check_job_grid(long long blocks, int n_jobs)
 }
 
 void launch_automorphism_jobs(cudaStream_t s, const AutomorphismJob *jobs, int n_jobs, long long blocks,
-                              std::atomic<uint64_t> *launches)
+                              std::atomic<uint64_t> *launches, int n_sm)
 {
     check_job_grid(blocks, n_jobs);
-    k_automorphism_jobs<<<(unsigned)blocks, 256, 0, s>>>(jobs, n_jobs);
+    launch_on(s, n_sm, k_automorphism_jobs, (unsigned)blocks, 256, 0, jobs, n_jobs);
     HX_CUDA(cudaGetLastError());
     if (launches) *launches += 1;
 }
 
 void launch_convert_jobs(cudaStream_t s, const ConvertJob *jobs, int n_jobs, long long blocks, int max_src,
-                         std::atomic<uint64_t> *launches)
+                         std::atomic<uint64_t> *launches, int n_sm)
 {
     check_job_grid(blocks, n_jobs);
     HX_CHECK(max_src >= 1 && max_src <= MAXK, HX_EINVAL, "too many conversion sources");
-    if (max_src <= 4) k_convert_jobs<4><<<(unsigned)blocks, 256, 0, s>>>(jobs, n_jobs);
-    else k_convert_jobs<MAXK><<<(unsigned)blocks, 256, 0, s>>>(jobs, n_jobs);
+    if (max_src <= 4) launch_on(s, n_sm, k_convert_jobs<4>, (unsigned)blocks, 256, 0, jobs, n_jobs);
+    else launch_on(s, n_sm, k_convert_jobs<MAXK>, (unsigned)blocks, 256, 0, jobs, n_jobs);
     HX_CUDA(cudaGetLastError());
     if (launches) *launches += 1;
 }
 
 void launch_key_ip_jobs(cudaStream_t s, const KeyIpJob *jobs, int n_jobs, long long blocks,
-                        std::atomic<uint64_t> *launches)
+                        std::atomic<uint64_t> *launches, int n_sm)
 {
     check_job_grid(blocks, n_jobs);
-    k_key_ip_jobs<<<(unsigned)blocks, 256, 0, s>>>(jobs, n_jobs);
+    launch_on(s, n_sm, k_key_ip_jobs, (unsigned)blocks, 256, 0, jobs, n_jobs);
     HX_CUDA(cudaGetLastError());
     if (launches) *launches += 1;
 }
 
 void launch_moddown_jobs(cudaStream_t s, const ModDownJob *jobs, int n_jobs, long long blocks,
-                         std::atomic<uint64_t> *launches)
+                         std::atomic<uint64_t> *launches, int n_sm)
 {
     check_job_grid(blocks, n_jobs);
-    k_moddown_jobs<<<(unsigned)blocks, 256, 0, s>>>(jobs, n_jobs);
+    launch_on(s, n_sm, k_moddown_jobs, (unsigned)blocks, 256, 0, jobs, n_jobs);
     HX_CUDA(cudaGetLastError());
     if (launches) *launches += 1;
 }

@@ -378,6 +378,7 @@ __global__ void __launch_bounds__((1 << (LOGM - Split<LOGM, ALT>::R1)) * COLS,
 k_ntt_cols(const __grid_constant__ NttRows R, const typename A::Prime *__restrict__ primes,
            const typename A::Tw *__restrict__ tw_all, int log_n)
 {
+    after_previous_kernel();
     extern __shared__ uint64_t sh[];
     constexpr int T = (1 << (LOGM - Split<LOGM, ALT>::R1)) * COLS;
     const int N = 1 << log_n, N2 = N >> LOGM, row = blockIdx.y, c0 = blockIdx.x * COLS;
@@ -396,6 +397,7 @@ __global__ void __launch_bounds__((1 << (LOGM - Split<LOGM, ALT>::R1)) * ROWS,
 k_ntt_rows(const __grid_constant__ NttRows R, const typename A::Prime *__restrict__ primes,
            const typename A::Tw *__restrict__ tw_all, int log_n, bool wide)
 {
+    after_previous_kernel();
     extern __shared__ uint64_t sh[];
     constexpr int T = (1 << (LOGM - Split<LOGM, ALT>::R1)) * ROWS;
     const int N = 1 << log_n;
@@ -423,8 +425,8 @@ void ntt_cols_w(const LaunchCtx &c, const NttRows &rows)
         cudaFuncSetAttribute(k_ntt_cols<A, LOGM, COLS, INV, ALT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem) == cudaSuccess;
     (void)attr;
-    k_ntt_cols<A, LOGM, COLS, INV, ALT><<<dim3(N2 / COLS, rows.n_rows, rows.n_groups), T, smem, c.stream>>>(rows, A::primes(*c.t),
-                                                                                 A::twiddles(*c.t, INV), c.log_n);
+    launch(c, k_ntt_cols<A, LOGM, COLS, INV, ALT>, dim3(N2 / COLS, rows.n_rows, rows.n_groups), T, smem, rows,
+           A::primes(*c.t), A::twiddles(*c.t, INV), c.log_n);
 }
 
 template <class A, int LOGM, int ROWS, bool INV, bool ALT>
@@ -441,8 +443,8 @@ void ntt_rows_w(const LaunchCtx &c, const NttRows &rows)
     // rows and blocks are multiples of 32 bytes: 32-byte pieces need only the bases and group strides aligned
     const bool wide = ((reinterpret_cast<uintptr_t>(rows.src) | reinterpret_cast<uintptr_t>(rows.dst) |
                         (rows.src_gs | rows.dst_gs) * sizeof(uint64_t)) & 31) == 0;
-    k_ntt_rows<A, LOGM, ROWS, INV, ALT><<<dim3(N1 / ROWS, rows.n_rows, rows.n_groups), T, smem, c.stream>>>(
-        rows, A::primes(*c.t), A::twiddles(*c.t, INV), c.log_n, wide);
+    launch(c, k_ntt_rows<A, LOGM, ROWS, INV, ALT>, dim3(N1 / ROWS, rows.n_rows, rows.n_groups), T, smem, rows,
+           A::primes(*c.t), A::twiddles(*c.t, INV), c.log_n, wide);
 }
 
 template <class A, bool INV, int LOGM, bool ALT>
@@ -555,6 +557,7 @@ template <class A, bool INV, bool COLS_PHASE>
 __global__ void __launch_bounds__(kMultiT, A::kThreadsPerSm / kMultiT)
     k_ntt_multi(const NttJob *__restrict__ jobs, int n_jobs)
 {
+    after_previous_kernel();
     extern __shared__ uint64_t sh[];
     const MultiTile<A> m = multi_tile<A>(jobs, n_jobs, blockIdx.x, COLS_PHASE, INV);
     const typename A::Prime P = m.primes[m.pr];
@@ -569,16 +572,16 @@ __global__ void __launch_bounds__(kMultiT, A::kThreadsPerSm / kMultiT)
 } // namespace
 
 // both phases of the several-ring transform over a job table on the device
-template <class A> void ntt_multi_phases(cudaStream_t s, const NttJob *jp, int n_jobs, int tc, int tr, bool inverse)
+template <class A> void ntt_multi_phases(cudaStream_t s, const NttJob *jp, int n_jobs, int tc, int tr, bool inverse, int n_sm)
 {
     constexpr size_t smem_c = sizeof(uint64_t) * kMultiColsBuf, smem_r = sizeof(uint64_t) * kMultiRowsBuf;
     static_assert(smem_c <= 48 * 1024 && smem_r <= 48 * 1024, "a tile fits without an attribute");
     if (!inverse) {
-        k_ntt_multi<A, false, true><<<tc, kMultiT, smem_c, s>>>(jp, n_jobs);
-        k_ntt_multi<A, false, false><<<tr, kMultiT, smem_r, s>>>(jp, n_jobs);
+        launch_on(s, n_sm, k_ntt_multi<A, false, true>, tc, kMultiT, smem_c, jp, n_jobs);
+        launch_on(s, n_sm, k_ntt_multi<A, false, false>, tr, kMultiT, smem_r, jp, n_jobs);
     } else {
-        k_ntt_multi<A, true, false><<<tr, kMultiT, smem_r, s>>>(jp, n_jobs);
-        k_ntt_multi<A, true, true><<<tc, kMultiT, smem_c, s>>>(jp, n_jobs);
+        launch_on(s, n_sm, k_ntt_multi<A, true, false>, tr, kMultiT, smem_r, jp, n_jobs);
+        launch_on(s, n_sm, k_ntt_multi<A, true, true>, tc, kMultiT, smem_c, jp, n_jobs);
     }
 }
 
