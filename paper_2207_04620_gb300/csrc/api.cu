@@ -742,7 +742,7 @@ hx_status hx_ntt_multi(const hx_ntt_job *jobs, int n_jobs, int inverse, void *st
         }
     }
     hx_context *c0 = const_cast<hx_context *>(jobs[0].ctx);
-    launch_ntt_multi(S(stream), v, inverse != 0, c0->t.n_sm, &c0->counters[C_LAUNCH]);
+    launch_ntt_multi(S(stream), v, inverse != 0, &c0->counters[C_LAUNCH]);
     return HX_OK;
     HX_END
 }

@@ -171,7 +171,7 @@ struct NttJob {
     int16_t prime[64];
 };
 // every job's transform in one launch per phase (several ring degrees together)
-void launch_ntt_multi(cudaStream_t s, const std::vector<NttJob> &jobs, bool inverse, int n_sm,
+void launch_ntt_multi(cudaStream_t s, const std::vector<NttJob> &jobs, bool inverse,
                       std::atomic<uint64_t> *launches);
 
 // times every NTT variant (tile width, radix split) of each phase on `rows` limbs of buf and
@@ -288,19 +288,19 @@ template <class J> long long plan_job_blocks(std::vector<J> &jobs)
 }
 // one grid over the jobs of a table already on the device (blocks from plan_job_blocks)
 void launch_automorphism_jobs(cudaStream_t s, const AutomorphismJob *jobs, int n_jobs, long long blocks,
-                              std::atomic<uint64_t> *launches, int n_sm);
+                              std::atomic<uint64_t> *launches);
 void launch_convert_jobs(cudaStream_t s, const ConvertJob *jobs, int n_jobs, long long blocks, int max_src,
-                         std::atomic<uint64_t> *launches, int n_sm);
+                         std::atomic<uint64_t> *launches);
 void launch_key_ip_jobs(cudaStream_t s, const KeyIpJob *jobs, int n_jobs, long long blocks,
-                        std::atomic<uint64_t> *launches, int n_sm);
+                        std::atomic<uint64_t> *launches);
 void launch_moddown_jobs(cudaStream_t s, const ModDownJob *jobs, int n_jobs, long long blocks,
-                         std::atomic<uint64_t> *launches, int n_sm);
+                         std::atomic<uint64_t> *launches);
 // the NTT over several rings in two steps: tile offsets of every job (host), then the two phase
 // launches over a job table already on the device
 void plan_ntt_jobs(std::vector<NttJob> &jobs, int *tiles_cols, int *tiles_rows);
 // fold: every job's ring has fold tables
 void launch_ntt_jobs(cudaStream_t s, const NttJob *jobs, int n_jobs, int tiles_cols, int tiles_rows, bool fold,
-                     bool inverse, int n_sm, std::atomic<uint64_t> *launches);
+                     bool inverse, std::atomic<uint64_t> *launches);
 // the tables of a context that its NTT jobs carry
 inline void set_ntt_tables(NttJob &j, const DeviceTables &t)
 {

@@ -1408,7 +1408,7 @@ void launch_add(const LaunchCtx &c, View out, View a, View b, int B, int comps, 
 {
     Timed tm_(c, K_ELEM, 24.0 * B * comps * limbs * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs, B * comps);
-    launch(c, k_add, grid, 256, 0, out, a, b, c.t->primes, comps, c.N, sub);
+    launch(c.stream, k_add, grid, 256, 0, out, a, b, c.t->primes, comps, c.N, sub);
     post(c);
 }
 
@@ -1416,7 +1416,7 @@ void launch_copy(const LaunchCtx &c, View out, View a, int B, int comps, int lim
 {
     Timed tm_(c, K_ELEM, 16.0 * B * comps * limbs * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs, B * comps);
-    launch(c, k_copy, grid, 256, 0, out, a, comps, c.N);
+    launch(c.stream, k_copy, grid, 256, 0, out, a, comps, c.N);
     post(c);
 }
 
@@ -1426,7 +1426,7 @@ void launch_aggregate(const LaunchCtx &c, View out, const AggSrc *src_dev, int n
     Timed tm_(c, K_AGG, 8.0 * (n_parties + 1.0) * count * comps * limbs * c.N);
     HX_CHECK(count * comps < 65536 && limbs < 65536, HX_EINVAL, "aggregation batch too large");
     dim3 grid(ew_blocks(c.N, 2), limbs, count * comps);
-    launch(c, k_aggregate, grid, 256, 0, out, src_dev, n_parties, count, C, c.t->primes, comps, c.N);
+    launch(c.stream, k_aggregate, grid, 256, 0, out, src_dev, n_parties, count, C, c.t->primes, comps, c.N);
     post(c);
 }
 
@@ -1434,7 +1434,7 @@ void launch_mul_plain(const LaunchCtx &c, View out, View a, const uint64_t *pt, 
 {
     Timed tm_(c, K_MULPT, 8.0 * (4 * B + 1) * limbs * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs, B * 2);
-    launch(c, k_mul_plain, grid, 256, 0, out, a, pt, c.t->primes, c.N);
+    launch(c.stream, k_mul_plain, grid, 256, 0, out, a, pt, c.t->primes, c.N);
     post(c);
 }
 
@@ -1442,7 +1442,7 @@ void launch_mul_scalar(const LaunchCtx &c, View out, View a, const Scalars &sc, 
 {
     Timed tm_(c, K_ELEM, 16.0 * B * comps * limbs * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs, B * comps);
-    launch(c, k_mul_scalar, grid, 256, 0, out, a, sc, c.t->primes, comps, c.N);
+    launch(c.stream, k_mul_scalar, grid, 256, 0, out, a, sc, c.t->primes, comps, c.N);
     post(c);
 }
 
@@ -1450,7 +1450,7 @@ void launch_add_scalar_c0(const LaunchCtx &c, View out, View a, const Scalars &s
 {
     Timed tm_(c, K_ELEM, 32.0 * B * limbs * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs, B * 2);
-    launch(c, k_add_scalar_c0, grid, 256, 0, out, a, sc, c.t->primes, c.N);
+    launch(c.stream, k_add_scalar_c0, grid, 256, 0, out, a, sc, c.t->primes, c.N);
     post(c);
 }
 
@@ -1458,7 +1458,7 @@ void launch_tensor(const LaunchCtx &c, View out3, View a, View b, int B, int lim
 {
     Timed tm_(c, K_TENSOR, 8.0 * B * limbs * c.N * (accumulate ? 10 : 7));
     dim3 grid(ew_blocks(c.N, 2), limbs, B);
-    launch(c, k_tensor, grid, 256, 0, out3, a, b, c.t->primes, c.N, accumulate, mont);
+    launch(c.stream, k_tensor, grid, 256, 0, out3, a, b, c.t->primes, c.N, accumulate, mont);
     post(c);
 }
 
@@ -1466,7 +1466,7 @@ void launch_automorphism(const LaunchCtx &c, View out, View in, const GaloisTab 
 {
     Timed tm_(c, K_AUTO, 16.0 * B * comps * limbs * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs, B * comps);
-    launch(c, k_automorphism, grid, 256, 0, out, in, tab, comps, c.log_n);
+    launch(c.stream, k_automorphism, grid, 256, 0, out, in, tab, comps, c.log_n);
     post(c);
 }
 
@@ -1474,7 +1474,7 @@ void launch_automorphism_sum(const LaunchCtx &c, View out, View in, const Galois
 {
     Timed tm_(c, K_AUTO, 8.0 * (R + 2) * B * limbs * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs, B);
-    launch(c, k_automorphism_sum, grid, 256, 0, out, in, tab, R, B, c.log_n, c.t->primes);
+    launch(c.stream, k_automorphism_sum, grid, 256, 0, out, in, tab, R, B, c.log_n, c.t->primes);
     post(c);
 }
 
@@ -1482,7 +1482,7 @@ void launch_tensor_sum(const LaunchCtx &c, View out3, View a, View b, int C, int
 {
     Timed tm_(c, K_TENSOR, 8.0 * B * limbs * c.N * (4 * C + 6));
     dim3 grid(ew_blocks(c.N, 2), limbs, B);
-    launch(c, k_tensor_sum, grid, 256, 0, out3, a, b, c.t->primes, C, B, c.N);
+    launch(c.stream, k_tensor_sum, grid, 256, 0, out3, a, b, c.t->primes, C, B, c.N);
     post(c);
 }
 
@@ -1490,7 +1490,7 @@ void launch_mask_prefix(const LaunchCtx &c, View out, View b, View rb, const Pre
 {
     Timed tm_(c, K_MULPT, 8.0 * (4 * B + 1) * h * limbs * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs, B * 2);
-    launch(c, k_mask_prefix, grid, 256, 0, out, b, rb, tab, c.t->primes, h, B, c.N);
+    launch(c.stream, k_mask_prefix, grid, 256, 0, out, b, rb, tab, c.t->primes, h, B, c.N);
     post(c);
 }
 
@@ -1498,7 +1498,7 @@ void launch_prefix_pairs(const LaunchCtx &c, View out, View prefix, int k0, int 
 {
     Timed tm_(c, K_ELEM, 8.0 * 6 * C * B * limbs * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs, C * B * 2);
-    launch(c, k_prefix_pairs, grid, 256, 0, out, prefix, c.t->primes, k0, B, c.N);
+    launch(c.stream, k_prefix_pairs, grid, 256, 0, out, prefix, c.t->primes, k0, B, c.N);
     post(c);
 }
 
@@ -1517,7 +1517,7 @@ void launch_basis_convert(const LaunchCtx &c, const ConvTable *tab_dev, int max_
         if (blocks < round / 2) grid.y = (unsigned)std::min<long long>(4, std::max<long long>(1, round / 2 / blocks));
         while (grid.x > 1 && (long long)grid.x * grid.z > 2 * round) grid.x /= 2;
         auto run = [&](auto mk) {
-            launch(c, k_basis_convert_split<mk()>, grid, 256, 0, tab_dev, out, in, c.t->fold, groups, gstride_out,
+            launch(c.stream, k_basis_convert_split<mk()>, grid, 256, 0, tab_dev, out, in, c.t->fold, groups, gstride_out,
                                                                     gstride_in, c.N);
         };
         switch (max_src) {
@@ -1573,10 +1573,10 @@ void launch_key_ip(const LaunchCtx &c, View acc, const uint64_t *D, const uint64
         const SplitIp A{D, dnt, dnt_bstride, n_q, K, alpha, limbs, ndig, c.log_n};
         by_digits(ndig, [&](auto nd) {
             if (sum)
-                launch(c, k_key_ip_split<nd(), true>, grid, block, 0, A, acc, keys, R, shared, c.t->fold, n_all, accumulate,
+                launch(c.stream, k_key_ip_split<nd(), true>, grid, block, 0, A, acc, keys, R, shared, c.t->fold, n_all, accumulate,
                                                                         B);
             else
-                launch(c, k_key_ip_split<nd(), false>, grid, block, 0, A, acc, keys, R, shared, c.t->fold, n_all,
+                launch(c.stream, k_key_ip_split<nd(), false>, grid, block, 0, A, acc, keys, R, shared, c.t->fold, n_all,
                                                                          accumulate, B);
         });
         post(c);
@@ -1599,9 +1599,9 @@ void launch_lintrans_mac(const LaunchCtx &c, const MacArgs &a, int B, int limbs,
     Timed tm_(c, K_MULPT, 8.0 * limbs * c.N * ((double)B * 2 * (a.n_baby + a.n_group) + n_terms));
     HX_CHECK(B >= 1 && limbs < 65536, HX_EINVAL, "bad BSGS batch");
     dim3 grid(B, (c.N / 2 + 127) / 128, limbs);
-    if (a.n_baby <= 4) launch(c, k_lintrans_mac<4>, grid, 128, 0, a, c.t->primes, B, limbs, c.N);
-    else if (a.n_baby <= 8) launch(c, k_lintrans_mac<8>, grid, 128, 0, a, c.t->primes, B, limbs, c.N);
-    else launch(c, k_lintrans_mac<16>, grid, 128, 0, a, c.t->primes, B, limbs, c.N);
+    if (a.n_baby <= 4) launch(c.stream, k_lintrans_mac<4>, grid, 128, 0, a, c.t->primes, B, limbs, c.N);
+    else if (a.n_baby <= 8) launch(c.stream, k_lintrans_mac<8>, grid, 128, 0, a, c.t->primes, B, limbs, c.N);
+    else launch(c.stream, k_lintrans_mac<16>, grid, 128, 0, a, c.t->primes, B, limbs, c.N);
     post(c);
 }
 
@@ -1616,7 +1616,7 @@ void launch_key_ip_mux(const LaunchCtx &c, View out, const uint64_t *D, const ui
         const dim3 block = split_block(B), grid(c.N / 2 / block.x, limbs + K, C * ((B + block.y - 1) / block.y));
         const SplitIp A{D, dnt, dnt_bstride, n_q, K, alpha, limbs, ndig, c.log_n};
         by_digits(ndig, [&](auto nd) {
-            launch(c, k_key_ip_mux_split<nd()>, grid, block, 0, A, out, tab, cs, c.t->primes, c.t->fold, n_all, B);
+            launch(c.stream, k_key_ip_mux_split<nd()>, grid, block, 0, A, out, tab, cs, c.t->primes, c.t->fold, n_all, B);
         });
         post(c);
         return;
@@ -1651,7 +1651,7 @@ void launch_key_ip_mux_pm(const LaunchCtx &c, View out, const uint64_t *D, const
         const dim3 block = split_block(B), grid(c.N / 2 / block.x, limbs + K, C * ((B + block.y - 1) / block.y));
         const SplitIp A{D, dnt, dnt_bstride, n_q, K, alpha, limbs, ndig, c.log_n};
         by_digits(ndig, [&](auto nd) {
-            launch(c, k_key_ip_mux_pm_split<nd()>, grid, block, 0, A, out, tab, c.t->fold, B);
+            launch(c.stream, k_key_ip_mux_pm_split<nd()>, grid, block, 0, A, out, tab, c.t->fold, B);
         });
         post(c);
         return;
@@ -1697,7 +1697,7 @@ void launch_moddown_final_mux(const LaunchCtx &c, View out, View acc, View conv,
 {
     Timed tm_(c, K_MODDOWN, 8.0 * C * B * limbs * c.N * 9.0);
     dim3 grid(ew_blocks(c.N, 2), limbs, C * B * 2);
-    launch(c, k_moddown_final_mux, grid, 256, 0, out, acc, conv, tab, c.t->primes, src, mux, cs, B, K, c.log_n);
+    launch(c.stream, k_moddown_final_mux, grid, 256, 0, out, acc, conv, tab, c.t->primes, src, mux, cs, B, K, c.log_n);
     post(c);
 }
 
@@ -1706,7 +1706,7 @@ void launch_moddown_final(const LaunchCtx &c, View out, View acc, View conv, con
 {
     Timed tm_(c, K_MODDOWN, 8.0 * B * 2 * limbs * c.N * ((add_mask ? 4.0 : 3.0)));
     dim3 grid(ew_blocks(c.N, 2), limbs, B * 2);
-    launch(c, k_moddown_final, grid, 256, 0, out, acc, conv, tab, c.t->primes, add, add_mask, gal, shared, c.log_n);
+    launch(c.stream, k_moddown_final, grid, 256, 0, out, acc, conv, tab, c.t->primes, add, add_mask, gal, shared, c.log_n);
     post(c);
 }
 
@@ -1722,7 +1722,7 @@ void launch_relin_rs_top(const LaunchCtx &c, View acc, View d, const RelinRescal
 {
     Timed tm_(c, K_RESCALE, 24.0 * B * 2 * c.N);
     dim3 grid(ew_blocks(c.N, 2), 1, B * 2);
-    launch(c, k_relin_rs_top, grid, 256, 0, acc, d, tab, c.t->primes, limbs - 1, c.N);
+    launch(c.stream, k_relin_rs_top, grid, 256, 0, acc, d, tab, c.t->primes, limbs - 1, c.N);
     post(c);
 }
 
@@ -1731,7 +1731,7 @@ void launch_relin_rs_final(const LaunchCtx &c, View out, View acc, View d, View 
 {
     Timed tm_(c, K_MODDOWN, 32.0 * B * 2 * (limbs - 1) * c.N);
     dim3 grid(ew_blocks(c.N, 2), limbs - 1, B * 2);
-    launch(c, k_relin_rs_final, grid, 256, 0, out, acc, d, conv, tab, c.t->primes, c.N);
+    launch(c.stream, k_relin_rs_final, grid, 256, 0, out, acc, d, conv, tab, c.t->primes, c.N);
     post(c);
 }
 
@@ -1740,7 +1740,7 @@ void launch_rescale_prep(const LaunchCtx &c, View r, View xtop, const RescaleTab
 {
     Timed tm_(c, K_RESCALE, 8.0 * B * comps * (top + 1) * c.N);
     dim3 grid(ew_blocks(c.N, 2), top, B * comps);
-    launch(c, k_rescale_prep, grid, 256, 0, r, xtop, tab, c.t->primes, comps, top, c.N, sc ? *sc : Scalars{},
+    launch(c.stream, k_rescale_prep, grid, 256, 0, r, xtop, tab, c.t->primes, comps, top, c.N, sc ? *sc : Scalars{},
                                                sc != nullptr);
     post(c);
 }
@@ -1750,7 +1750,7 @@ void launch_rescale_final(const LaunchCtx &c, View out, View in, View r, const R
 {
     Timed tm_(c, K_RESCALE, 24.0 * B * comps * top * c.N);
     dim3 grid(ew_blocks(c.N, 2), top, B * comps);
-    launch(c, k_rescale_final, grid, 256, 0, out, in, r, tab, c.t->primes, comps, c.N, sc ? *sc : Scalars{},
+    launch(c.stream, k_rescale_final, grid, 256, 0, out, in, r, tab, c.t->primes, comps, c.N, sc ? *sc : Scalars{},
                                                 sc != nullptr);
     post(c);
 }
@@ -1767,7 +1767,7 @@ void launch_encrypt_combine(const LaunchCtx &c, uint64_t *ct, const uint64_t *v,
                             const uint64_t *e1, const uint64_t *m, const uint64_t *pk, int n_q, int limbs)
 {
     dim3 grid(ew_blocks(c.N, 1), limbs, 1);
-    launch(c, k_encrypt_combine, grid, 256, 0, ct, v, e0, e1, m, pk, c.t->primes, n_q, limbs, c.N);
+    launch(c.stream, k_encrypt_combine, grid, 256, 0, ct, v, e0, e1, m, pk, c.t->primes, n_q, limbs, c.N);
     post(c);
 }
 
@@ -1775,14 +1775,14 @@ void launch_signed_to_rows(const LaunchCtx &c, uint64_t *out, const int64_t *in,
                            size_t in_stride, const int *prime_dev)
 {
     dim3 grid(ew_blocks(c.N, 1), rows, n_in_polys);
-    launch(c, k_signed_to_rows, grid, 256, 0, out, in, rows, in_stride, prime_dev, c.t->primes, c.N);
+    launch(c.stream, k_signed_to_rows, grid, 256, 0, out, in, rows, in_stride, prime_dev, c.t->primes, c.N);
     post(c);
 }
 
 void launch_to_mont(const LaunchCtx &c, uint64_t *p, int rows, const int *prime_dev)
 {
     dim3 grid(ew_blocks(c.N, 1), rows, 1);
-    launch(c, k_to_mont, grid, 256, 0, p, prime_dev, c.t->primes, c.N);
+    launch(c.stream, k_to_mont, grid, 256, 0, p, prime_dev, c.t->primes, c.N);
     post(c);
 }
 
@@ -1796,7 +1796,7 @@ void launch_mul_rows(const LaunchCtx &c, uint64_t *out, const uint64_t *a, const
 void launch_ddec_shares(const LaunchCtx &c, uint64_t *out, View ct, const uint64_t *shares, int n_parties, int B)
 {
     dim3 grid(ew_blocks(c.N, 1), n_parties + 1, B);
-    launch(c, k_ddec_shares, grid, 256, 0, out, ct, shares, c.t->primes, n_parties, c.N);
+    launch(c.stream, k_ddec_shares, grid, 256, 0, out, ct, shares, c.t->primes, n_parties, c.N);
     post(c);
 }
 
@@ -1807,39 +1807,39 @@ static void check_job_grid(long long blocks, int n_jobs)
 }
 
 void launch_automorphism_jobs(cudaStream_t s, const AutomorphismJob *jobs, int n_jobs, long long blocks,
-                              std::atomic<uint64_t> *launches, int n_sm)
+                              std::atomic<uint64_t> *launches)
 {
     check_job_grid(blocks, n_jobs);
-    launch_on(s, n_sm, k_automorphism_jobs, (unsigned)blocks, 256, 0, jobs, n_jobs);
+    launch(s, k_automorphism_jobs, (unsigned)blocks, 256, 0, jobs, n_jobs);
     HX_CUDA(cudaGetLastError());
     if (launches) *launches += 1;
 }
 
 void launch_convert_jobs(cudaStream_t s, const ConvertJob *jobs, int n_jobs, long long blocks, int max_src,
-                         std::atomic<uint64_t> *launches, int n_sm)
+                         std::atomic<uint64_t> *launches)
 {
     check_job_grid(blocks, n_jobs);
     HX_CHECK(max_src >= 1 && max_src <= MAXK, HX_EINVAL, "too many conversion sources");
-    if (max_src <= 4) launch_on(s, n_sm, k_convert_jobs<4>, (unsigned)blocks, 256, 0, jobs, n_jobs);
-    else launch_on(s, n_sm, k_convert_jobs<MAXK>, (unsigned)blocks, 256, 0, jobs, n_jobs);
+    if (max_src <= 4) launch(s, k_convert_jobs<4>, (unsigned)blocks, 256, 0, jobs, n_jobs);
+    else launch(s, k_convert_jobs<MAXK>, (unsigned)blocks, 256, 0, jobs, n_jobs);
     HX_CUDA(cudaGetLastError());
     if (launches) *launches += 1;
 }
 
 void launch_key_ip_jobs(cudaStream_t s, const KeyIpJob *jobs, int n_jobs, long long blocks,
-                        std::atomic<uint64_t> *launches, int n_sm)
+                        std::atomic<uint64_t> *launches)
 {
     check_job_grid(blocks, n_jobs);
-    launch_on(s, n_sm, k_key_ip_jobs, (unsigned)blocks, 256, 0, jobs, n_jobs);
+    launch(s, k_key_ip_jobs, (unsigned)blocks, 256, 0, jobs, n_jobs);
     HX_CUDA(cudaGetLastError());
     if (launches) *launches += 1;
 }
 
 void launch_moddown_jobs(cudaStream_t s, const ModDownJob *jobs, int n_jobs, long long blocks,
-                         std::atomic<uint64_t> *launches, int n_sm)
+                         std::atomic<uint64_t> *launches)
 {
     check_job_grid(blocks, n_jobs);
-    launch_on(s, n_sm, k_moddown_jobs, (unsigned)blocks, 256, 0, jobs, n_jobs);
+    launch(s, k_moddown_jobs, (unsigned)blocks, 256, 0, jobs, n_jobs);
     HX_CUDA(cudaGetLastError());
     if (launches) *launches += 1;
 }

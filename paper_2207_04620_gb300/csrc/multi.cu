@@ -155,21 +155,20 @@ std::vector<Cts> rotate_jobs(const std::vector<RotateJob> &in, cudaStream_t s)
     HX_CUDA(cudaMemcpyAsync(d, tb.host.data(), tb.host.size(), cudaMemcpyHostToDevice, s));
     hx_context &c0 = *w[0].ctx;
     std::atomic<uint64_t> *launches = &c0.counters[C_LAUNCH];
-    const int n_sm = c0.t.n_sm;
     bool fold = true;
     for (const Work &x : w) fold = fold && x.ctx->t.fold;
 
-    launch_automorphism_jobs(s, reinterpret_cast<const AutomorphismJob *>(d + oa), (int)aj.size(), ba, launches, n_sm);
+    launch_automorphism_jobs(s, reinterpret_cast<const AutomorphismJob *>(d + oa), (int)aj.size(), ba, launches);
     for (Work &x : w)
         HX_CUDA(cudaMemcpyAsync(x.coef->p, x.t->p, sizeof(uint64_t) * x.B * x.L * x.N, cudaMemcpyDeviceToDevice, s));
-    launch_ntt_jobs(s, reinterpret_cast<const NttJob *>(d + o1), (int)n1.size(), t1c, t1r, fold, true, n_sm, launches);
-    launch_convert_jobs(s, reinterpret_cast<const ConvertJob *>(d + oc1), (int)c1.size(), bc1, max_a, launches, n_sm);
-    launch_ntt_jobs(s, reinterpret_cast<const NttJob *>(d + o2), (int)n2.size(), t2c, t2r, fold, false, n_sm, launches);
-    launch_key_ip_jobs(s, reinterpret_cast<const KeyIpJob *>(d + ok), (int)kj.size(), bk, launches, n_sm);
-    launch_ntt_jobs(s, reinterpret_cast<const NttJob *>(d + o3), (int)n3.size(), t3c, t3r, fold, true, n_sm, launches);
-    launch_convert_jobs(s, reinterpret_cast<const ConvertJob *>(d + oc2), (int)c2.size(), bc2, max_k, launches, n_sm);
-    launch_ntt_jobs(s, reinterpret_cast<const NttJob *>(d + o4), (int)n4.size(), t4c, t4r, fold, false, n_sm, launches);
-    launch_moddown_jobs(s, reinterpret_cast<const ModDownJob *>(d + om), (int)mj.size(), bm, launches, n_sm);
+    launch_ntt_jobs(s, reinterpret_cast<const NttJob *>(d + o1), (int)n1.size(), t1c, t1r, fold, true, launches);
+    launch_convert_jobs(s, reinterpret_cast<const ConvertJob *>(d + oc1), (int)c1.size(), bc1, max_a, launches);
+    launch_ntt_jobs(s, reinterpret_cast<const NttJob *>(d + o2), (int)n2.size(), t2c, t2r, fold, false, launches);
+    launch_key_ip_jobs(s, reinterpret_cast<const KeyIpJob *>(d + ok), (int)kj.size(), bk, launches);
+    launch_ntt_jobs(s, reinterpret_cast<const NttJob *>(d + o3), (int)n3.size(), t3c, t3r, fold, true, launches);
+    launch_convert_jobs(s, reinterpret_cast<const ConvertJob *>(d + oc2), (int)c2.size(), bc2, max_k, launches);
+    launch_ntt_jobs(s, reinterpret_cast<const NttJob *>(d + o4), (int)n4.size(), t4c, t4r, fold, false, launches);
+    launch_moddown_jobs(s, reinterpret_cast<const ModDownJob *>(d + om), (int)mj.size(), bm, launches);
 
     for (size_t k = 0; k < w.size(); k++) {
         hx_context &ctx = *w[k].ctx;

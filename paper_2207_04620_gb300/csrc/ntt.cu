@@ -5,9 +5,9 @@
 namespace hx {
 
 template void ntt_phase<ArithShoup>(const LaunchCtx &, const NttRows &, bool, bool, int, int);
-template void ntt_multi_phases<ArithShoup>(cudaStream_t, const NttJob *, int, int, int, bool, int);
+template void ntt_multi_phases<ArithShoup>(cudaStream_t, const NttJob *, int, int, int, bool);
 extern template void ntt_phase<ArithFold>(const LaunchCtx &, const NttRows &, bool, bool, int, int);
-extern template void ntt_multi_phases<ArithFold>(cudaStream_t, const NttJob *, int, int, int, bool, int);
+extern template void ntt_multi_phases<ArithFold>(cudaStream_t, const NttJob *, int, int, int, bool);
 
 // ---- launcher (host code: it picks the tuned variants and the phase split of the kernels above)
 static void run_phase(const LaunchCtx &c, const NttRows &rows, bool inverse, bool cols, int logm, int var)
@@ -132,17 +132,17 @@ void plan_ntt_jobs(std::vector<NttJob> &jobs, int *tiles_cols, int *tiles_rows)
     *tiles_rows = tr;
 }
 
-void launch_ntt_jobs(cudaStream_t s, const NttJob *jp, int n_jobs, int tc, int tr, bool fold, bool inverse, int n_sm,
+void launch_ntt_jobs(cudaStream_t s, const NttJob *jp, int n_jobs, int tc, int tr, bool fold, bool inverse,
                      std::atomic<uint64_t> *launches)
 {
     if (tc == 0) return;
-    if (fold) ntt_multi_phases<ArithFold>(s, jp, n_jobs, tc, tr, inverse, n_sm);
-    else ntt_multi_phases<ArithShoup>(s, jp, n_jobs, tc, tr, inverse, n_sm);
+    if (fold) ntt_multi_phases<ArithFold>(s, jp, n_jobs, tc, tr, inverse);
+    else ntt_multi_phases<ArithShoup>(s, jp, n_jobs, tc, tr, inverse);
     HX_CUDA(cudaGetLastError());
     if (launches) *launches += 2;
 }
 
-void launch_ntt_multi(cudaStream_t s, const std::vector<NttJob> &jobs_in, bool inverse, int n_sm,
+void launch_ntt_multi(cudaStream_t s, const std::vector<NttJob> &jobs_in, bool inverse,
                       std::atomic<uint64_t> *launches)
 {
     std::vector<NttJob> jobs = jobs_in;
@@ -155,7 +155,7 @@ void launch_ntt_multi(cudaStream_t s, const std::vector<NttJob> &jobs_in, bool i
     HX_CUDA(cudaMallocAsync(&jd, jobs.size() * sizeof(NttJob), s));
     HX_CUDA(cudaMemcpyAsync(jd, jobs.data(), jobs.size() * sizeof(NttJob), cudaMemcpyHostToDevice, s));
     try {
-        launch_ntt_jobs(s, reinterpret_cast<const NttJob *>(jd), (int)jobs.size(), tc, tr, fold, inverse, n_sm, launches);
+        launch_ntt_jobs(s, reinterpret_cast<const NttJob *>(jd), (int)jobs.size(), tc, tr, fold, inverse, launches);
     } catch (...) {
         cudaFreeAsync(jd, s);
         throw;

@@ -4,6 +4,6 @@
 namespace hx {
 
 template void ntt_phase<ArithFold>(const LaunchCtx &, const NttRows &, bool, bool, int, int);
-template void ntt_multi_phases<ArithFold>(cudaStream_t, const NttJob *, int, int, int, bool, int);
+template void ntt_multi_phases<ArithFold>(cudaStream_t, const NttJob *, int, int, int, bool);
 
 } // namespace hx

@@ -425,7 +425,7 @@ void ntt_cols_w(const LaunchCtx &c, const NttRows &rows)
         cudaFuncSetAttribute(k_ntt_cols<A, LOGM, COLS, INV, ALT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem) == cudaSuccess;
     (void)attr;
-    launch(c, k_ntt_cols<A, LOGM, COLS, INV, ALT>, dim3(N2 / COLS, rows.n_rows, rows.n_groups), T, smem, rows,
+    launch(c.stream, k_ntt_cols<A, LOGM, COLS, INV, ALT>, dim3(N2 / COLS, rows.n_rows, rows.n_groups), T, smem, rows,
            A::primes(*c.t), A::twiddles(*c.t, INV), c.log_n);
 }
 
@@ -443,7 +443,7 @@ void ntt_rows_w(const LaunchCtx &c, const NttRows &rows)
     // rows and blocks are multiples of 32 bytes: 32-byte pieces need only the bases and group strides aligned
     const bool wide = ((reinterpret_cast<uintptr_t>(rows.src) | reinterpret_cast<uintptr_t>(rows.dst) |
                         (rows.src_gs | rows.dst_gs) * sizeof(uint64_t)) & 31) == 0;
-    launch(c, k_ntt_rows<A, LOGM, ROWS, INV, ALT>, dim3(N1 / ROWS, rows.n_rows, rows.n_groups), T, smem, rows,
+    launch(c.stream, k_ntt_rows<A, LOGM, ROWS, INV, ALT>, dim3(N1 / ROWS, rows.n_rows, rows.n_groups), T, smem, rows,
            A::primes(*c.t), A::twiddles(*c.t, INV), c.log_n, wide);
 }
 
@@ -572,16 +572,16 @@ __global__ void __launch_bounds__(kMultiT, A::kThreadsPerSm / kMultiT)
 } // namespace
 
 // both phases of the several-ring transform over a job table on the device
-template <class A> void ntt_multi_phases(cudaStream_t s, const NttJob *jp, int n_jobs, int tc, int tr, bool inverse, int n_sm)
+template <class A> void ntt_multi_phases(cudaStream_t s, const NttJob *jp, int n_jobs, int tc, int tr, bool inverse)
 {
     constexpr size_t smem_c = sizeof(uint64_t) * kMultiColsBuf, smem_r = sizeof(uint64_t) * kMultiRowsBuf;
     static_assert(smem_c <= 48 * 1024 && smem_r <= 48 * 1024, "a tile fits without an attribute");
     if (!inverse) {
-        launch_on(s, n_sm, k_ntt_multi<A, false, true>, tc, kMultiT, smem_c, jp, n_jobs);
-        launch_on(s, n_sm, k_ntt_multi<A, false, false>, tr, kMultiT, smem_r, jp, n_jobs);
+        launch(s, k_ntt_multi<A, false, true>, tc, kMultiT, smem_c, jp, n_jobs);
+        launch(s, k_ntt_multi<A, false, false>, tr, kMultiT, smem_r, jp, n_jobs);
     } else {
-        launch_on(s, n_sm, k_ntt_multi<A, true, false>, tr, kMultiT, smem_r, jp, n_jobs);
-        launch_on(s, n_sm, k_ntt_multi<A, true, true>, tc, kMultiT, smem_c, jp, n_jobs);
+        launch(s, k_ntt_multi<A, true, false>, tr, kMultiT, smem_r, jp, n_jobs);
+        launch(s, k_ntt_multi<A, true, true>, tc, kMultiT, smem_c, jp, n_jobs);
     }
 }
 
