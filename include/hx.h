@@ -136,7 +136,7 @@ hx_status hx_encrypt_batch(hx_context *ctx, const hx_keyset *ks, const double *s
 hx_status hx_encrypt_coeffs(hx_context *ctx, const hx_keyset *ks, const int64_t *coeffs, double scale, int limbs,
                             uint64_t seed, uint32_t tag, uint32_t index, hx_ct **out);
 /* DDec: every simulated party's share c1*s_i is computed on the device, the
- * shares are summed with c0 on the host modulo q_0 and decoded (Dcd).  Writes
+ * shares are summed with c0 modulo q_0 and decoded (Dcd) there.  Writes
  * min(n, N/2) real slots. */
 hx_status hx_decrypt(hx_context *ctx, const hx_keyset *ks, const hx_ct *ct, double *slots, size_t n);
 /* The same collective decryption stopped before decoding: N centered integer

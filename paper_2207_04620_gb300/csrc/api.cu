@@ -413,8 +413,7 @@ hx_status hx_decrypt(hx_context *ctx, const hx_keyset *ks, const hx_ct *ct, doub
     mine(ctx, ks);
     mine(ctx, ct);
     HX_CUDA(cudaDeviceSynchronize());
-    std::vector<int64_t> v = decrypt_coeffs(*ctx, *ks, ct->c, nullptr);
-    ctx->enc->decode(v.data(), ct->c.scale, slots, std::min(n, (size_t)ctx->N / 2));
+    decrypt_slots(*ctx, *ks, ct->c, slots, n, nullptr);
     return HX_OK;
     HX_END
 }
@@ -432,8 +431,7 @@ hx_status hx_decrypt_parties(hx_context *ctx, const hx_keyset *ks, const hx_ct *
                  "party " + std::to_string(i) + " sent no decryption share; DDec needs all " +
                      std::to_string(ks->n_parties) + " parties");
     HX_CUDA(cudaDeviceSynchronize());
-    std::vector<int64_t> v = decrypt_coeffs(*ctx, *ks, ct->c, nullptr);
-    ctx->enc->decode(v.data(), ct->c.scale, slots, std::min(n, (size_t)ctx->N / 2));
+    decrypt_slots(*ctx, *ks, ct->c, slots, n, nullptr);
     return HX_OK;
     HX_END
 }

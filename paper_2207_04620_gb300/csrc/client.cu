@@ -234,6 +234,86 @@ __global__ void k_enc_sample(int64_t *out, size_t entry_stride, const uint64_t *
     }
 }
 
+// ---- decoding (Dcd): z_j = sum_i c_i zeta^(i e_j) / scale (real part), zeta = e^(i pi / N), by an
+// iterative radix-2 transform of length 2N in doubles, every product and sum rounded once.  The same
+// operations on one host core took 0.46 ms for N = 2^14; a whole decryption 0.56 ms, now 0.10.
+
+__device__ __forceinline__ void dec_butterfly(double2 &u, double2 &v, const double4 w)
+{
+    // v times the conjugate of w = (w.x, w.z)
+    const double wi = -w.z;
+    const double tr = __dsub_rn(__dmul_rn(v.x, w.x), __dmul_rn(v.y, wi));
+    const double ti = __dadd_rn(__dmul_rn(v.x, wi), __dmul_rn(v.y, w.x));
+    v = make_double2(__dsub_rn(u.x, tr), __dsub_rn(u.y, ti));
+    u = make_double2(__dadd_rn(u.x, tr), __dadd_rn(u.y, ti));
+}
+
+// DDec's sum over the shares ([1 + n_parties][n], coefficient form mod q) at coefficient i, centred,
+// placed for the 2n-point transform.  The upper n inputs are zero, so the first stage copies each
+// value to its neighbour.
+__global__ void k_dec_place(double2 *A, const uint64_t *__restrict__ sh, int n_parties, uint64_t q, int log_m)
+{
+    const int n = 1 << (log_m - 1);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        uint64_t acc = 0;
+        for (int p = 0; p <= n_parties; p++) acc = addmod(acc, sh[(size_t)p * n + i], q);
+        const int64_t v = acc > q / 2 ? (int64_t)acc - (int64_t)q : (int64_t)acc;
+        const double2 z = make_double2((double)v, 0.0);
+        const unsigned at = __brev((unsigned)i) >> (32 - log_m);
+        A[at] = z;
+        A[at + 1] = z;
+    }
+}
+
+constexpr int kDecTile = 2048;  // points of the contiguous sub-transforms
+constexpr int kDecCols = 16;    // columns per block of the stages beyond them
+
+// stages len = 4 .. kDecTile
+__global__ void __launch_bounds__(512) k_dec_tile(double2 *A, const double4 *__restrict__ roots, int log_m)
+{
+    __shared__ double2 s[kDecTile];
+    const int m = 1 << log_m;
+    double2 *a = A + (size_t)blockIdx.x * kDecTile;
+    for (int i = threadIdx.x; i < kDecTile; i += blockDim.x) s[i] = a[i];
+    for (int len = 4; len <= kDecTile; len <<= 1) {
+        __syncthreads();
+        const int half = len >> 1, step = m / len;
+        for (int t = threadIdx.x; t < kDecTile / 2; t += blockDim.x) {
+            const int k = t & (half - 1), i = 2 * t - k;
+            dec_butterfly(s[i], s[i + half], roots[(size_t)k * step]);
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kDecTile; i += blockDim.x) a[i] = s[i];
+}
+
+// stages len > kDecTile on kDecCols columns (points kDecTile apart); real parts over the scale
+__global__ void __launch_bounds__(256) k_dec_cols(double *re, const double2 *A, const double4 *__restrict__ roots,
+                                                  int log_m, double scale)
+{
+    __shared__ double2 s[64 * kDecCols];  // N = 2^16: 64 rows
+    const int m = 1 << log_m, rows = m / kDecTile, c0 = blockIdx.x * kDecCols;
+    for (int i = threadIdx.x; i < rows * kDecCols; i += blockDim.x)
+        s[i] = A[(size_t)(i / kDecCols) * kDecTile + c0 + i % kDecCols];
+    for (int half = 1; half < rows; half <<= 1) {
+        __syncthreads();
+        const int step = m / (2 * half * kDecTile);
+        for (int t = threadIdx.x; t < rows / 2 * kDecCols; t += blockDim.x) {
+            const int c = t % kDecCols, b = t / kDecCols, k = b & (half - 1), i = 2 * b - k;
+            dec_butterfly(s[i * kDecCols + c], s[(i + half) * kDecCols + c],
+                          roots[(size_t)(k * kDecTile + c0 + c) * step]);
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < rows * kDecCols; i += blockDim.x)
+        re[(size_t)(i / kDecCols) * kDecTile + c0 + i % kDecCols] = __ddiv_rn(s[i].x, scale);
+}
+
+__global__ void k_dec_gather(double *slots, const double *__restrict__ re, const int *__restrict__ e, int count)
+{
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < count; j += gridDim.x * blockDim.x) slots[j] = re[e[j]];
+}
+
 int grid_for(size_t work) { return (int)std::min<size_t>((work + 255) / 256, 4096); }
 
 // device copies of the host encoder's tables (2N-th roots, 5^j mod 2N) and of
@@ -338,6 +418,23 @@ void encode_real_batch(hx_context &ctx, const double *slots_dev, size_t n_slots,
         ctx.counters[C_LAUNCH] += 1;
     }
     HX_CUDA(cudaStreamSynchronize(s));  // the work buffer is released at return
+}
+
+void decode_shares(hx_context &ctx, const uint64_t *sh, int n_parties, double scale, double *slots_dev, int count,
+                   cudaStream_t s)
+{
+    const int N = ctx.N, log_m = ctx.log_n + 1;
+    const EncTables &t = enc_tables(ctx);
+    const double4 *roots = reinterpret_cast<const double4 *>(t.roots->p);
+    DevBuf work((size_t)6 * N, s);  // 2N complex points, 2N real parts
+    double2 *A = reinterpret_cast<double2 *>(work.p);
+    double *re = reinterpret_cast<double *>(work.p + (size_t)4 * N);
+    k_dec_place<<<grid_for(N), 256, 0, s>>>(A, sh, n_parties, ctx.primes[0], log_m);
+    k_dec_tile<<<2 * N / kDecTile, 512, 0, s>>>(A, roots, log_m);
+    k_dec_cols<<<kDecTile / kDecCols, 256, 0, s>>>(re, A, roots, log_m, scale);
+    k_dec_gather<<<grid_for(count), 256, 0, s>>>(slots_dev, re, reinterpret_cast<const int *>(t.e->p), count);
+    HX_CUDA(cudaGetLastError());
+    ctx.counters[C_LAUNCH] += 4;
 }
 
 // rows[r] of the output = the encoding at `scale` of the slot vector whose real coefficients

@@ -252,7 +252,6 @@ Encoder::Encoder(int ln) : log_n(ln), n(1 << ln)
     auto neg = [](DD x) { return DD{-x.hi, -x.lo}; };
     roots_re.resize(n);
     roots_im.resize(n);
-    roots.resize(n);
     for (int k = 0; k < n; k++) {
         DD c, si;
         if (k <= m8) {
@@ -270,30 +269,6 @@ Encoder::Encoder(int ln) : log_n(ln), n(1 << ln)
         }
         roots_re[k] = c;
         roots_im[k] = neg(si);
-        roots[k] = std::complex<double>(c.hi, -si.hi);
-    }
-}
-
-// iterative radix-2 FFT of length 2N: A_k = sum_i a_i w^(ik), w = e^(-+2 pi i / 2N)
-void Encoder::fft(std::vector<std::complex<double>> &a, bool inverse) const
-{
-    const int m = 2 * n;
-    for (int i = 1, j = 0; i < m; i++) {
-        int bit = m >> 1;
-        for (; j & bit; bit >>= 1) j ^= bit;
-        j ^= bit;
-        if (i < j) std::swap(a[i], a[j]);
-    }
-    for (int len = 2; len <= m; len <<= 1) {
-        const int step = m / len;
-        for (int i = 0; i < m; i += len)
-            for (int k = 0; k < len / 2; k++) {
-                std::complex<double> w = roots[k * step];
-                if (inverse) w = std::conj(w);
-                std::complex<double> u = a[i + k], v = a[i + k + len / 2] * w;
-                a[i + k] = u + v;
-                a[i + k + len / 2] = u - v;
-            }
     }
 }
 
@@ -348,15 +323,6 @@ void Encoder::encode(const double *slots, size_t count, double scale, int64_t *c
     std::vector<DD> m;
     encode_real(slots, count, m);
     for (int i = 0; i < n; i++) coeffs[i] = dd_round_coeff(dd_mul_d(m[i], scale));
-}
-
-void Encoder::decode(const int64_t *coeffs, double scale, double *slots, size_t count) const
-{
-    const int m = 2 * n;
-    std::vector<std::complex<double>> big(m);
-    for (int i = 0; i < n; i++) big[i] = (double)coeffs[i];
-    fft(big, true);  // sum_i c_i e^(+2 pi i ik / 2N) = sum_i c_i zeta^(ik)
-    for (size_t j = 0; j < count && j < (size_t)(n / 2); j++) slots[j] = big[e[j]].real() / scale;
 }
 
 } // namespace hx

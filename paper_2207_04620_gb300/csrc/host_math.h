@@ -64,7 +64,7 @@ DD dd_mul_d(DD a, double b);
 // 2^-20 of a half-integer taken as that half-integer.  Throws past 2^62.
 int64_t dd_round_coeff(DD x);
 
-// Canonical-embedding encoder/decoder (slot j at zeta^(5^j), zeta = e^(i pi/N)).
+// Canonical-embedding encoder (slot j at zeta^(5^j), zeta = e^(i pi/N)).
 // Encoding is exact: coefficient i is scale * (2/N) * sum_j z_j cos(pi (i e_j mod 2N)/N)
 // under dd_round_coeff, the sum taken by a double-double FFT of length 2N whose error
 // (about 2^-90 relative) lies far inside the rounding rule's band.
@@ -72,17 +72,11 @@ struct Encoder {
     int log_n, n;
     std::vector<int64_t> e;  // 5^j mod 2N
     std::vector<DD> roots_re, roots_im;  // e^(-2 pi i k / 2N), k < N, double-double
-    std::vector<std::complex<double>> roots;  // the same rounded to double (decoding)
     explicit Encoder(int log_n);
     // m_i = (2/N) sum_j z_j cos(pi (i e_j mod 2N)/N) before the scale, double-double
     void encode_real(const double *slots, size_t count, std::vector<DD> &m) const;
     // coeffs = dd_round_coeff(scale * m)
     void encode(const double *slots, size_t count, double scale, int64_t *coeffs) const;
-    // z_j = sum_i c_i zeta^(i e_j) / scale (real part)
-    void decode(const int64_t *coeffs, double scale, double *slots, size_t count) const;
-
-  private:
-    void fft(std::vector<std::complex<double>> &a, bool inverse) const;
 };
 
 } // namespace hx

@@ -2,6 +2,7 @@
 // toy scale: the parties are simulated in this process; their randomness is
 // drawn on the host from SplitMix64 streams and the ring arithmetic runs on
 // the device with the evaluation kernels.
+#include <algorithm>
 #include <cstring>
 
 #include "runtime.h"
@@ -311,6 +312,21 @@ std::vector<int64_t> decrypt_coeffs(hx_context &ctx, const hx_keyset &ks, const 
             out[(size_t)b * N + i] = acc > q / 2 ? (int64_t)acc - (int64_t)q : (int64_t)acc;
         }
     return out;
+}
+
+void decrypt_slots(hx_context &ctx, const hx_keyset &ks, const Cts &c, double *slots, size_t count, cudaStream_t s)
+{
+    HX_CHECK(c.comps == 2 && c.B == 1, HX_EINVAL, "decryption needs a 2-component ciphertext");
+    const int N = ctx.N, np = ks.n_parties;
+    count = std::min(count, (size_t)N / 2);
+    if (count == 0) return;
+    Eval ev(ctx, s);
+    DevBuf sh((size_t)(np + 1) * N, s), out(count, s);
+    launch_ddec_shares(ev.lc(), sh.p, c.view(N), ks.s_parts0->p, np, 1);
+    ev.ntt_inplace(sh.p, (size_t)N, np + 1, {0}, {0}, true);
+    decode_shares(ctx, sh.p, np, c.scale, reinterpret_cast<double *>(out.p), (int)count, s);
+    HX_CUDA(cudaMemcpyAsync(slots, out.p, sizeof(double) * count, cudaMemcpyDeviceToHost, s));
+    HX_CUDA(cudaStreamSynchronize(s));
 }
 
 // Fig. 1 item 13: collective public-key switch of every entry of ct to the
