@@ -519,6 +519,10 @@ int64_t hx_ct_export(const hx_ct *ct, uint64_t *host, size_t cap)
     const size_t N = ct->ctx->N, words = (size_t)c.comps * c.limbs * N;
     need(cap >= words, "buffer too small");
     HX_CUDA(cudaDeviceSynchronize());
+    if (c.cap == c.limbs) {  // the components follow one another
+        HX_CUDA(cudaMemcpy(host, c.d, sizeof(uint64_t) * words, cudaMemcpyDeviceToHost));
+        return (int64_t)words;
+    }
     for (int k = 0; k < c.comps; k++)
         HX_CUDA(cudaMemcpy(host + (size_t)k * c.limbs * N, c.d + k * c.cstride(N), sizeof(uint64_t) * c.limbs * N,
                            cudaMemcpyDeviceToHost));
@@ -728,7 +732,7 @@ hx_status hx_ntt_multi(const hx_ntt_job *jobs, int n_jobs, int inverse, void *st
         need(dev < 0 || j.ctx->device == dev, "jobs on several devices");
         dev = j.ctx->device;
         NttJob &J = v[i];
-        J.data = j.data;
+        J.src = J.data = j.data;
         set_ntt_tables(J, j.ctx->t);
         J.log_n = j.ctx->log_n;
         J.n_rows = j.n_polys * j.n_limbs;

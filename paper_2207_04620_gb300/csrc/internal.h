@@ -158,9 +158,10 @@ struct LaunchCtx {
 };
 
 void launch_ntt(const LaunchCtx &c, const NttRows &rows, bool inverse);
-// one job of a multi-ring NTT: n_rows rows of 2^log_n words at data (in place), row r modulo
-// prime[r % n_limbs] of its own context's tables
+// one job of a multi-ring NTT: n_rows rows of 2^log_n words from src to data (they may be the same),
+// row r modulo prime[r % n_limbs] of its own context's tables
 struct NttJob {
+    const uint64_t *src;
     uint64_t *data;
     const PrimeConst *primes;
     const ulonglong2 *tw_fwd, *tw_inv;

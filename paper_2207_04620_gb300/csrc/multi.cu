@@ -27,9 +27,10 @@ struct Tables {
     }
 };
 
-NttJob ntt_job(const hx_context &ctx, uint64_t *data, int rows, const std::vector<int> &primes)
+NttJob ntt_job(const hx_context &ctx, const uint64_t *src, uint64_t *data, int rows, const std::vector<int> &primes)
 {
     NttJob j{};
+    j.src = src;
     j.data = data;
     set_ntt_tables(j, ctx.t);
     j.log_n = ctx.log_n;
@@ -49,7 +50,7 @@ std::vector<Cts> rotate_jobs(const std::vector<RotateJob> &in, cudaStream_t s)
         uint64_t g;
         const SwitchKey *key;
         int N, L, K, A, nd, ext, B;
-        BufPtr t, coef, D, acc, conv;
+        uint64_t *t, *coef, *D, *acc, *conv;  // in the call's one work buffer
         Cts out;
     };
     std::vector<Cts> out(in.size());
@@ -95,48 +96,60 @@ std::vector<Cts> rotate_jobs(const std::vector<RotateJob> &in, cudaStream_t s)
     std::vector<KeyIpJob> kj;
     std::vector<ModDownJob> mj;
     int max_a = 1, max_k = 1;
+    size_t words = 0;
+    for (const Work &x : w) words += (size_t)x.B * x.N * (4 * x.L + (x.nd + 2) * x.ext);
+    DevBuf work(words, s);
+    uint64_t *at = work.p;
+    auto take = [&](size_t n) {
+        uint64_t *p = at;
+        at += n;
+        return p;
+    };
     for (Work &x : w) {
         hx_context &ctx = *x.ctx;
         const size_t N = x.N;
         const int L = x.L, K = x.K, ext = x.ext, nd = x.nd, B = x.B;
-        x.t = std::make_shared<DevBuf>((size_t)B * L * N, s);
-        x.coef = std::make_shared<DevBuf>((size_t)B * L * N, s);
-        x.D = std::make_shared<DevBuf>((size_t)B * nd * ext * N, s);
-        x.acc = std::make_shared<DevBuf>((size_t)B * 2 * ext * N, s);
-        x.conv = std::make_shared<DevBuf>((size_t)B * 2 * L * N, s);
+        x.t = take((size_t)B * L * N);
+        x.coef = take((size_t)B * L * N);
+        x.D = take((size_t)B * nd * ext * N);
+        x.acc = take((size_t)B * 2 * ext * N);
+        x.conv = take((size_t)B * 2 * L * N);
         x.out = Eval(ctx, s).alloc(B, 2, L);
         x.out.scale = x.a->scale;
         max_a = std::max(max_a, x.A);
         max_k = std::max(max_k, K);
-        const View tv{x.t->p, (size_t)L * N, (size_t)L * N};
+        const View tv{x.t, (size_t)L * N, (size_t)L * N};
         const View c1v{x.a->d + x.a->cstride(N), x.a->bstride(N), x.a->cstride(N)};
-        const View accv{x.acc->p, (size_t)2 * ext * N, (size_t)ext * N};
+        const View accv{x.acc, (size_t)2 * ext * N, (size_t)ext * N};
         // sigma_g(c1)
         aj.push_back(AutomorphismJob{tv, c1v, x.g, 1, ctx.log_n, ctx.t.primes, ew_blocks((int)N, 1), L, B, 0});
-        // ModUp: inverse NTT of a copy, conversion of every digit, forward NTT of the extended rows
+        // ModUp: inverse NTT, conversion of every digit, forward NTT of the extended rows
         std::vector<int> q_rows(L), ext_primes(ext), p_rows(K);
         for (int r = 0; r < L; r++) q_rows[r] = r;
         for (int r = 0; r < ext; r++) ext_primes[r] = r < L ? r : ctx.n_q + (r - L);
         for (int r = 0; r < K; r++) p_rows[r] = ctx.n_q + r;
-        n1.push_back(ntt_job(ctx, x.coef->p, B * L, q_rows));
-        c1.push_back(ConvertJob{ctx.t.modup + (size_t)L * ctx.dnum, View{x.D->p, (size_t)nd * ext * N, 0},
-                                View{x.coef->p, (size_t)L * N, 0}, ctx.t.primes, ctx.t.fold, nd, (int)N, x.A, (size_t)ext * N, 0,
+        n1.push_back(ntt_job(ctx, x.t, x.coef, B * L, q_rows));
+        c1.push_back(ConvertJob{ctx.t.modup + (size_t)L * ctx.dnum, View{x.D, (size_t)nd * ext * N, 0},
+                                View{x.coef, (size_t)L * N, 0}, ctx.t.primes, ctx.t.fold, nd, (int)N, x.A, (size_t)ext * N, 0,
                                 ew_blocks((int)N, 2), 1, B * nd, 0});
         // a digit's own rows of D are never read (the inner product takes them from sigma_g(c1))
-        n2.push_back(ntt_job(ctx, x.D->p, B * nd * ext, ext_primes));
-        kj.push_back(KeyIpJob{accv, x.D->p, x.t->p, x.key->buf->p, (size_t)L * N, ctx.t.primes, ctx.t.fold, ctx.n_all, ctx.n_q,
+        n2.push_back(ntt_job(ctx, x.D, x.D, B * nd * ext, ext_primes));
+        kj.push_back(KeyIpJob{accv, x.D, x.t, x.key->buf->p, (size_t)L * N, ctx.t.primes, ctx.t.fold, ctx.n_all, ctx.n_q,
                               K, x.A, L, nd, ctx.log_n, nd <= kRedcFewTerms ? 1 : 0, 1, ew_blocks((int)N, 2), ext, B,
                               0});
         // ModDown: inverse NTT of the special rows, conversion to Q, forward NTT, epilogue
         for (int b = 0; b < B; b++)
             for (int c = 0; c < 2; c++)
-                n3.push_back(ntt_job(ctx, x.acc->p + ((size_t)(b * 2 + c) * ext + L) * N, K, p_rows));
+            {
+                uint64_t *rows = x.acc + ((size_t)(b * 2 + c) * ext + L) * N;
+                n3.push_back(ntt_job(ctx, rows, rows, K, p_rows));
+            }
         const ModDownTable *md = ctx.t.moddown + L;
-        c2.push_back(ConvertJob{reinterpret_cast<const ConvTable *>(md), View{x.conv->p, (size_t)L * N, 0},
-                                View{x.acc->p, (size_t)ext * N, 0}, ctx.t.primes, ctx.t.fold, 1, (int)N, K, 0, 0,
+        c2.push_back(ConvertJob{reinterpret_cast<const ConvTable *>(md), View{x.conv, (size_t)L * N, 0},
+                                View{x.acc, (size_t)ext * N, 0}, ctx.t.primes, ctx.t.fold, 1, (int)N, K, 0, 0,
                                 ew_blocks((int)N, 2), 1, 2 * B, 0});
-        n4.push_back(ntt_job(ctx, x.conv->p, 2 * B * L, q_rows));
-        mj.push_back(ModDownJob{x.out.view((int)N), accv, View{x.conv->p, (size_t)2 * L * N, (size_t)L * N},
+        n4.push_back(ntt_job(ctx, x.conv, x.conv, 2 * B * L, q_rows));
+        mj.push_back(ModDownJob{x.out.view((int)N), accv, View{x.conv, (size_t)2 * L * N, (size_t)L * N},
                                 x.a->view((int)N), md, ctx.t.primes, 1, ctx.log_n, x.g, ew_blocks((int)N, 2), L,
                                 2 * B, 0});
     }
@@ -159,8 +172,6 @@ std::vector<Cts> rotate_jobs(const std::vector<RotateJob> &in, cudaStream_t s)
     for (const Work &x : w) fold = fold && x.ctx->t.fold;
 
     launch_automorphism_jobs(s, reinterpret_cast<const AutomorphismJob *>(d + oa), (int)aj.size(), ba, launches);
-    for (Work &x : w)
-        HX_CUDA(cudaMemcpyAsync(x.coef->p, x.t->p, sizeof(uint64_t) * x.B * x.L * x.N, cudaMemcpyDeviceToDevice, s));
     launch_ntt_jobs(s, reinterpret_cast<const NttJob *>(d + o1), (int)n1.size(), t1c, t1r, fold, true, launches);
     launch_convert_jobs(s, reinterpret_cast<const ConvertJob *>(d + oc1), (int)c1.size(), bc1, max_a, launches);
     launch_ntt_jobs(s, reinterpret_cast<const NttJob *>(d + o2), (int)n2.size(), t2c, t2r, fold, false, launches);

@@ -487,8 +487,7 @@ template <class A> void ntt_phase(const LaunchCtx &c, const NttRows &r, bool inv
 namespace {
 
 // ---- several rings in one launch ------------------------------------------------
-// A job is n_rows rows of one ring (its own N, primes and twiddles), transformed
-// in place.  One kernel per phase takes the tiles of every job; a tile's phase
+// A job is n_rows rows of one ring (its own N, primes and twiddles).  One kernel per phase takes the tiles of every job; a tile's phase
 // size picks the template instance, with the tile width chosen so every
 // instance runs 128 threads.
 
@@ -504,6 +503,7 @@ constexpr int kMultiRowsBuf = max4(RowTile<5, MultiW<5>::W, false>::WORDS, RowTi
                                    RowTile<7, MultiW<7>::W, false>::WORDS, RowTile<8, MultiW<8>::W, false>::WORDS);
 
 template <class A> struct MultiTile {
+    const uint64_t *src;  // the first phase's source
     uint64_t *row;
     const typename A::Tw *tw;
     const typename A::Prime *primes;
@@ -531,6 +531,7 @@ __device__ __forceinline__ MultiTile<A> multi_tile(const NttJob *jobs, int n_job
     m.bx = local % nb;
     m.pr = J.prime[r % J.n_limbs];
     m.primes = A::job_primes(J);
+    m.src = J.src + (size_t)r * n;
     m.row = J.data + (size_t)r * n;
     m.tw = A::job_twiddles(J, inv) + (size_t)m.pr * n;
     return m;
@@ -543,13 +544,14 @@ __device__ __forceinline__ void multi_run(uint64_t *sh, const MultiTile<A> &m, c
     if (COLS_PHASE) {
         typedef ColTile<LOGM, W, false> Tile;
         uint64_t *d = m.row + m.bx * W;
-        ntt_tile<A, Tile, LOGM, W, INV, false>(sh, d, d, Tile{(1 << m.log_n) >> LOGM}, m.tw, 0, 0, P, kMultiT, false);
+        ntt_tile<A, Tile, LOGM, W, INV, false>(sh, INV ? d : m.src + m.bx * W, d, Tile{(1 << m.log_n) >> LOGM}, m.tw, 0, 0, P, kMultiT, false);
     } else {
         typedef RowTile<LOGM, W, false> Tile;
         const int r_base = m.bx * W;
         uint64_t *d = m.row + ((size_t)r_base << LOGM);
-        const bool wide = (reinterpret_cast<uintptr_t>(d) & 31) == 0;
-        ntt_tile<A, Tile, LOGM, W, INV, false>(sh, d, d, Tile{}, m.tw, m.log_n - LOGM, r_base, P, kMultiT, wide);
+        const uint64_t *from = INV ? m.src + ((size_t)r_base << LOGM) : d;
+        const bool wide = ((reinterpret_cast<uintptr_t>(d) | reinterpret_cast<uintptr_t>(from)) & 31) == 0;
+        ntt_tile<A, Tile, LOGM, W, INV, false>(sh, from, d, Tile{}, m.tw, m.log_n - LOGM, r_base, P, kMultiT, wide);
     }
 }
 
