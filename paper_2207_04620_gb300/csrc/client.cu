@@ -11,6 +11,9 @@
 // Knuth's two-sum), so its error is far inside that band and the integer is the
 // one the exact value gives -- the host encoder's, whatever the order of the
 // operations.
+#include <algorithm>
+
+#include "launch_util.cuh"
 #include "runtime.h"
 
 namespace hx {
@@ -18,7 +21,7 @@ namespace hx {
 namespace {
 
 constexpr uint64_t kGamma = 0x9E3779B97F4A7C15ull;
-constexpr int kFftTile = 1024;  // points of the sub-transforms done in shared memory
+constexpr int kFftTile = 256;  // points of the contiguous sub-transforms
 
 __device__ __forceinline__ uint64_t dmix64(uint64_t z)
 {
@@ -126,41 +129,67 @@ __global__ void k_enc_place(double4 *A, const double *slots, size_t n_slots, con
     }
 }
 
-// stages len = 2 .. kFftTile (radix-2 decimation in time) on contiguous tiles of the compact
-// second half in shared memory
+// v times -i, the twiddle of the second butterfly of four points
+__device__ __forceinline__ double4 times_minus_i(const double4 v) { return make_double4(v.z, v.w, -v.x, -v.y); }
+
+__device__ __forceinline__ void butterfly_plain(double4 &u, double4 &v)  // twiddle 1
+{
+    const ddv ur{u.x, u.y}, ui{u.z, u.w}, tr{v.x, v.y}, ti{v.z, v.w};
+    const ddv a = dd_plus(ur, tr), b = dd_plus(ui, ti), c = dd_minus(ur, tr), d = dd_minus(ui, ti);
+    u = make_double4(a.hi, a.lo, b.hi, b.lo);
+    v = make_double4(c.hi, c.lo, d.hi, d.lo);
+}
+
+// The transform's stages in two kernels, each through shared memory once: stages len = 2 .. kFftTile on
+// contiguous tiles of the compact second half, then the others on columns of points kFftTile apart.
+// The FP64 pipe sets the time (two lanes a cycle and SM, some 160 operations a butterfly), so the tiles
+// are small enough to load every SM alike, and the first two stages, whose twiddles are 1 and -i,
+// multiply nothing: twelve vectors of N = 2^14 took 600 us with tiles of 1024 points and a kernel per
+// later stage and take 432.
 __global__ void __launch_bounds__(kFftTile / 2) k_enc_fft_tile(double4 *A, const double4 *__restrict__ roots, int log_m)
 {
     __shared__ double4 s[kFftTile];
     const int m = 1 << log_m;
     double4 *a = A + (size_t)blockIdx.y * (m >> 1) + (size_t)blockIdx.x * kFftTile;
-    for (int i = threadIdx.x; i < kFftTile; i += blockDim.x) s[i] = a[i];
-    __syncthreads();
+    const int t = threadIdx.x;
+    for (int i = t; i < kFftTile; i += blockDim.x) s[i] = a[i];
     for (int len = 2; len <= kFftTile; len <<= 1) {
-        const int half = len >> 1, step = m / len;
-        for (int t = threadIdx.x; t < kFftTile / 2; t += blockDim.x) {
-            const int g = t / half, k = t % half, i = g * len + k;
-            double4 u = s[i], v = s[i + half];
-            butterfly(u, v, roots[(size_t)k * step]);
-            s[i] = u;
-            s[i + half] = v;
-        }
         __syncthreads();
+        const int half = len >> 1, step = m / len, k = t & (half - 1), i = 2 * t - k;
+        double4 u = s[i], v = s[i + half];
+        if (len <= 4) {
+            if (k) v = times_minus_i(v);
+            butterfly_plain(u, v);
+        } else {
+            butterfly(u, v, roots[(size_t)k * step]);
+        }
+        s[i] = u;
+        s[i + half] = v;
     }
-    for (int i = threadIdx.x; i < kFftTile; i += blockDim.x) a[i] = s[i];
+    __syncthreads();
+    for (int i = t; i < kFftTile; i += blockDim.x) a[i] = s[i];
 }
 
-// one later stage (kFftTile < len <= N) over the compact second half in global memory
-__global__ void k_enc_fft_stage(double4 *A, const double4 *__restrict__ roots, int log_m, int len)
+constexpr int kFftCols = 2;  // columns per block
+
+__global__ void k_enc_fft_cols(double4 *A, const double4 *__restrict__ roots, int log_m)
 {
-    const int m = 1 << log_m, half = len >> 1, step = m / len;
-    double4 *a = A + (size_t)blockIdx.y * (m >> 1);
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < m / 4; t += gridDim.x * blockDim.x) {
-        const int g = t / half, k = t % half, i = g * len + k;
-        double4 u = a[i], v = a[i + half];
-        butterfly(u, v, roots[(size_t)k * step]);
-        a[i] = u;
-        a[i + half] = v;
+    extern __shared__ double4 cols[];  // [rows][kFftCols]
+    const int m = 1 << log_m, rows = (m >> 1) / kFftTile, c0 = blockIdx.x * kFftCols;
+    double4 *a = A + (size_t)blockIdx.y * (m >> 1) + c0;
+    for (int i = threadIdx.x; i < rows * kFftCols; i += blockDim.x)
+        cols[i] = a[(size_t)(i / kFftCols) * kFftTile + i % kFftCols];
+    for (int half = 1; half < rows; half <<= 1) {
+        __syncthreads();
+        const int step = m / (2 * half * kFftTile);
+        for (int t = threadIdx.x; t < rows / 2 * kFftCols; t += blockDim.x) {
+            const int c = t % kFftCols, b = t / kFftCols, k = b & (half - 1), i = (2 * b - k) * kFftCols + c;
+            butterfly(cols[i], cols[i + half * kFftCols], roots[(size_t)(k * kFftTile + c0 + c) * step]);
+        }
     }
+    __syncthreads();
+    for (int i = threadIdx.x; i < rows * kFftCols; i += blockDim.x)
+        a[(size_t)(i / kFftCols) * kFftTile + i % kFftCols] = cols[i];
 }
 
 // Re A_i = Re(w_i B_i), the last stage's butterfly on a zero first-half entry
@@ -253,6 +282,7 @@ __device__ __forceinline__ void dec_butterfly(double2 &u, double2 &v, const doub
 // value to its neighbour.
 __global__ void k_dec_place(double2 *A, const uint64_t *__restrict__ sh, int n_parties, uint64_t q, int log_m)
 {
+    after_previous_kernel();
     const int n = 1 << (log_m - 1);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         uint64_t acc = 0;
@@ -265,12 +295,15 @@ __global__ void k_dec_place(double2 *A, const uint64_t *__restrict__ sh, int n_p
     }
 }
 
-constexpr int kDecTile = 2048;  // points of the contiguous sub-transforms
-constexpr int kDecCols = 16;    // columns per block of the stages beyond them
+// small tiles again, to spread one transform over the SMs' FP64 pipes: with tiles of 2048 points and 16
+// columns a block, 16 and 128 of them, one decryption at N = 2^14 took 101 us, and takes 67
+constexpr int kDecTile = 256;  // points of the contiguous sub-transforms
+constexpr int kDecCols = 2;    // columns per block of the stages beyond them
 
 // stages len = 4 .. kDecTile
-__global__ void __launch_bounds__(512) k_dec_tile(double2 *A, const double4 *__restrict__ roots, int log_m)
+__global__ void __launch_bounds__(kDecTile / 2) k_dec_tile(double2 *A, const double4 *__restrict__ roots, int log_m)
 {
+    after_previous_kernel();
     __shared__ double2 s[kDecTile];
     const int m = 1 << log_m;
     double2 *a = A + (size_t)blockIdx.x * kDecTile;
@@ -291,7 +324,8 @@ __global__ void __launch_bounds__(512) k_dec_tile(double2 *A, const double4 *__r
 __global__ void __launch_bounds__(256) k_dec_cols(double *re, const double2 *A, const double4 *__restrict__ roots,
                                                   int log_m, double scale)
 {
-    __shared__ double2 s[64 * kDecCols];  // N = 2^16: 64 rows
+    after_previous_kernel();
+    __shared__ double2 s[512 * kDecCols];  // N = 2^16: 512 rows
     const int m = 1 << log_m, rows = m / kDecTile, c0 = blockIdx.x * kDecCols;
     for (int i = threadIdx.x; i < rows * kDecCols; i += blockDim.x)
         s[i] = A[(size_t)(i / kDecCols) * kDecTile + c0 + i % kDecCols];
@@ -311,6 +345,7 @@ __global__ void __launch_bounds__(256) k_dec_cols(double *re, const double2 *A, 
 
 __global__ void k_dec_gather(double *slots, const double *__restrict__ re, const int *__restrict__ e, int count)
 {
+    after_previous_kernel();
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < count; j += gridDim.x * blockDim.x) slots[j] = re[e[j]];
 }
 
@@ -356,10 +391,11 @@ void enc_transform(hx_context &ctx, const EncTables &t, double4 *a, const double
     k_enc_place<<<dim3(grid_for(N / 2), count), 256, 0, s>>>(a, slots_dev, n_slots,
                                                              reinterpret_cast<const int *>(t.e->p), log_m, N / 2);
     k_enc_fft_tile<<<dim3(N / kFftTile, count), kFftTile / 2, 0, s>>>(a, roots, log_m);
-    for (int len = 2 * kFftTile; len <= N; len <<= 1)
-        k_enc_fft_stage<<<dim3(grid_for(N / 2), count), 256, 0, s>>>(a, roots, log_m, len);
+    const int rows = N / kFftTile;  // at most 256
+    k_enc_fft_cols<<<dim3(kFftTile / kFftCols, count), std::max(32, rows / 2 * kFftCols), sizeof(double4) * rows * kFftCols,
+                     s>>>(a, roots, log_m);
     HX_CUDA(cudaGetLastError());
-    ctx.counters[C_LAUNCH] += 2 + (log_m - 11);
+    ctx.counters[C_LAUNCH] += 3;
 }
 
 // vectors transformed per pass: bounds the complex double-double work buffer (32 B per point)
@@ -373,7 +409,7 @@ void encode_batch(hx_context &ctx, const double *slots_dev, size_t n_slots, int 
                   size_t out_stride, cudaStream_t s)
 {
     const int N = ctx.N;
-    HX_CHECK(N % kFftTile == 0, HX_EINVAL, "the device encoder needs N >= 1024");
+    HX_CHECK(N % kFftTile == 0, HX_EINVAL, "the device encoder needs N >= 256");
     HX_CHECK(n_slots <= (size_t)N / 2 && count >= 1 && count < 65536, HX_EINVAL, "bad slot batch");
     const EncTables &t = enc_tables(ctx);
     const double4 *roots = reinterpret_cast<const double4 *>(t.roots->p);
@@ -403,7 +439,7 @@ void encode_real_batch(hx_context &ctx, const double *slots_dev, size_t n_slots,
                        cudaStream_t s)
 {
     const int N = ctx.N;
-    HX_CHECK(N % kFftTile == 0, HX_EINVAL, "the device encoder needs N >= 1024");
+    HX_CHECK(N % kFftTile == 0, HX_EINVAL, "the device encoder needs N >= 256");
     HX_CHECK(n_slots <= (size_t)N / 2 && count >= 1 && count < 65536, HX_EINVAL, "bad slot batch");
     const EncTables &t = enc_tables(ctx);
     const double4 *roots = reinterpret_cast<const double4 *>(t.roots->p);
@@ -429,10 +465,10 @@ void decode_shares(hx_context &ctx, const uint64_t *sh, int n_parties, double sc
     DevBuf work((size_t)6 * N, s);  // 2N complex points, 2N real parts
     double2 *A = reinterpret_cast<double2 *>(work.p);
     double *re = reinterpret_cast<double *>(work.p + (size_t)4 * N);
-    k_dec_place<<<grid_for(N), 256, 0, s>>>(A, sh, n_parties, ctx.primes[0], log_m);
-    k_dec_tile<<<2 * N / kDecTile, 512, 0, s>>>(A, roots, log_m);
-    k_dec_cols<<<kDecTile / kDecCols, 256, 0, s>>>(re, A, roots, log_m, scale);
-    k_dec_gather<<<grid_for(count), 256, 0, s>>>(slots_dev, re, reinterpret_cast<const int *>(t.e->p), count);
+    launch(s, k_dec_place, grid_for(N), 256, 0, A, sh, n_parties, ctx.primes[0], log_m);
+    launch(s, k_dec_tile, 2 * N / kDecTile, kDecTile / 2, 0, A, roots, log_m);
+    launch(s, k_dec_cols, kDecTile / kDecCols, 256, 0, re, A, roots, log_m, scale);
+    launch(s, k_dec_gather, grid_for(count), 256, 0, slots_dev, re, reinterpret_cast<const int *>(t.e->p), count);
     HX_CUDA(cudaGetLastError());
     ctx.counters[C_LAUNCH] += 4;
 }
@@ -486,11 +522,8 @@ Cts encrypt_batch(hx_context &ctx, const hx_keyset &ks, const double *slots_dev,
     Cts c = ev.alloc(count, 2, limbs);
     c.scale = ctx.scale;
     const size_t st4 = (size_t)limbs * N;
-    for (int b = 0; b < count; b++) {
-        const uint64_t *pb = polys.p + (size_t)b * 4 * st4;
-        launch_encrypt_combine(ev.lc(), c.d + (size_t)b * c.bstride(N), pb, pb + st4, pb + 2 * st4, pb + 3 * st4,
-                               ks.pk->p, ctx.n_q, limbs);
-    }
+    launch_encrypt_combine(ev.lc(), c.d, polys.p, polys.p + st4, polys.p + 2 * st4, polys.p + 3 * st4, ks.pk->p, ctx.n_q, limbs,
+                           count, 4 * st4);
     HX_CUDA(cudaStreamSynchronize(s));  // the staging buffers above are released at return
     return c;
 }

@@ -354,7 +354,8 @@ void launch_keygen_b(const LaunchCtx &c, uint64_t *b, const uint64_t *a, const u
                      const uint64_t *sp, const uint64_t *gadget_mask, int rows, const int *prime_of_row_dev,
                      bool to_mont);
 void launch_encrypt_combine(const LaunchCtx &c, uint64_t *ct, const uint64_t *v, const uint64_t *e0,
-                            const uint64_t *e1, const uint64_t *m, const uint64_t *pk, int n_q, int limbs);
+                            const uint64_t *e1, const uint64_t *m, const uint64_t *pk, int n_q, int limbs,
+                            int count = 1, size_t stride = 0);  // count entries, their polynomials stride words apart
 void launch_signed_to_rows(const LaunchCtx &c, uint64_t *out, const int64_t *in, int rows, int n_in_polys,
                            size_t in_stride, const int *prime_dev);
 void launch_to_mont(const LaunchCtx &c, uint64_t *p, int rows, const int *prime_dev);

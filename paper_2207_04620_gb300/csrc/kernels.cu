@@ -1246,11 +1246,14 @@ __global__ void k_keygen_b(uint64_t *b, uint64_t *a, const uint64_t *e, const ui
 // c0 = v*pk_b + e0 + m, c1 = v*pk_a + e1 on the first `limbs` primes
 __global__ void k_encrypt_combine(uint64_t *ct, const uint64_t *v, const uint64_t *e0, const uint64_t *e1,
                                   const uint64_t *m, const uint64_t *pk, const PrimeConst *__restrict__ primes,
-                                  int n_q, int limbs, int n)
+                                  int n_q, int limbs, int n, size_t stride)
 {
     after_previous_kernel();
     const int l = blockIdx.y;
     const PrimeConst P = primes[l];
+    ct += (size_t)blockIdx.z * 2 * limbs * n;
+    const size_t at = blockIdx.z * stride;  // entry z's polynomials
+    v += at, e0 += at, e1 += at, m += at;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
         const size_t k = (size_t)l * n + j;
         const uint64_t vb = mulmod(v[k], pk[k], P);
@@ -1266,10 +1269,11 @@ __global__ void k_signed_to_rows(uint64_t *out, const int64_t *in, int rows, siz
 {
     after_previous_kernel();
     const int r = blockIdx.y, p = blockIdx.z;
-    const uint64_t q = primes[prime[r]].q;
+    const uint64_t q = primes[prime[r]].q, bar = primes[prime[r]].bar;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
         const int64_t v = in[p * in_stride + j];
-        const uint64_t m = v >= 0 ? (uint64_t)v % q : (q - ((uint64_t)(-v) % q)) % q;
+        const uint64_t a = reduce64(v >= 0 ? (uint64_t)v : 0 - (uint64_t)v, q, bar);
+        const uint64_t m = v >= 0 || a == 0 ? a : q - a;
         out[((size_t)p * rows + r) * n + j] = m;
     }
 }
@@ -1764,10 +1768,11 @@ void launch_keygen_b(const LaunchCtx &c, uint64_t *b, const uint64_t *a, const u
 }
 
 void launch_encrypt_combine(const LaunchCtx &c, uint64_t *ct, const uint64_t *v, const uint64_t *e0,
-                            const uint64_t *e1, const uint64_t *m, const uint64_t *pk, int n_q, int limbs)
+                            const uint64_t *e1, const uint64_t *m, const uint64_t *pk, int n_q, int limbs, int count,
+                            size_t stride)
 {
-    dim3 grid(ew_blocks(c.N, 1), limbs, 1);
-    launch(c.stream, k_encrypt_combine, grid, 256, 0, ct, v, e0, e1, m, pk, c.t->primes, n_q, limbs, c.N);
+    dim3 grid(ew_blocks(c.N, 1), limbs, count);
+    launch(c.stream, k_encrypt_combine, grid, 256, 0, ct, v, e0, e1, m, pk, c.t->primes, n_q, limbs, c.N, stride);
     post(c);
 }
 
