@@ -77,13 +77,19 @@ Cts Eval::mul_int(const Cts &a, int64_t c, double new_scale)
     return o;
 }
 
+int64_t const_int(double value, double scale)
+{
+    const double r = round_half_away(value * scale);
+    HX_CHECK(std::fabs(r) < 9.2e18, HX_EINVAL, "constant too large");
+    return (int64_t)r;
+}
+
 Cts Eval::add_const(const Cts &a, double value)
 {
-    const double r = round_half_away(value * a.scale);
-    HX_CHECK(std::fabs(r) < 9.2e18, HX_EINVAL, "constant too large");
+    const int64_t r = const_int(value, a.scale);
     Cts o = alloc(a.B, 2, a.limbs);
     o.scale = a.scale;
-    launch_add_scalar_c0(lc(), o.view(ctx.N), a.view(ctx.N), scalars_for(ctx, a.limbs, (int64_t)r), a.B, a.limbs);
+    launch_add_scalar_c0(lc(), o.view(ctx.N), a.view(ctx.N), scalars_for(ctx, a.limbs, r), a.B, a.limbs);
     return o;
 }
 
@@ -495,7 +501,7 @@ void Eval::tensor_sum(Cts &acc, const Cts &a, const Cts &b)
     ctx.counters[C_ADD] += a.B;
 }
 
-Cts Eval::rescale(const Cts &a, int64_t c)
+Cts Eval::rescale(const Cts &a, int64_t c, const Tail *tail)
 {
     HX_CHECK(a.limbs >= 2, HX_ELEVEL, "no level left to rescale");
     const int N = ctx.N, top = a.limbs - 1, comps = a.comps, B = a.B;
@@ -506,12 +512,24 @@ Cts Eval::rescale(const Cts &a, int64_t c)
     const RescaleTable *tab = ctx.t.rescale + a.limbs;
     // rescale(c * a) for an integer c: a's residues times c in the two elementwise passes
     // (the top limb after its inverse NTT), the same values as multiplying first
-    const Scalars sc = c != 1 ? scalars_for(ctx, a.limbs, c) : Scalars{};
-    const Scalars *scp = c != 1 ? &sc : nullptr;
+    const Scalars sc = c != 1 || tail ? scalars_for(ctx, a.limbs, c) : Scalars{};
+    const Scalars *scp = c != 1 || tail ? &sc : nullptr;
     launch_rescale_prep(lc(), rv, View{xtop.p, (size_t)comps * N, (size_t)N}, tab, B, comps, top, scp);
     ntt_inplace(r.p, (size_t)top * N, B * comps, iota_vec(0, top), iota_vec(0, top), false);
     Cts o = alloc(B, comps, top);
-    launch_rescale_final(lc(), o.view(N), a.view(N), rv, tab, B, comps, top, scp);
+    if (tail) {
+        RescaleTail t{scalars_for(ctx, top, tail->times), scalars_for(ctx, top, tail->add_times),
+                      scalars_for(ctx, top, tail->c0), View{nullptr, 0, 0}, tail->times != 1, 0};
+        if (tail->add) {
+            HX_CHECK(tail->add->B == B && tail->add->limbs == top && tail->add->comps == comps, HX_ESCALE, "addend's shape differs");
+            t.add = tail->add->view(N);
+            t.has_add = tail->add_times != 1 ? 2 : 1;
+            ctx.counters[C_ADD] += B;
+        }
+        launch_rescale_tail(lc(), o.view(N), a.view(N), rv, tab, sc, t, B, comps, top);
+    } else {
+        launch_rescale_final(lc(), o.view(N), a.view(N), rv, tab, B, comps, top, scp);
+    }
     o.scale = a.scale / (double)ctx.primes[top];
     ctx.counters[C_RESCALE] += B;
     return o;

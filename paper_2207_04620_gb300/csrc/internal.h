@@ -113,6 +113,13 @@ struct View {
     size_t bstride, cstride;
 };
 
+// what follows a rescale's division x in the same pass: w x + add_w add + c0 (c0 on component 0)
+struct RescaleTail {
+    Scalars w, add_w, c0;
+    View add;
+    int has_w, has_add;  // 0: none (a factor 1, no addend), 1: as it is, 2: times add_w
+};
+
 struct DeviceTables {
     PrimeConst *primes = nullptr;   // [n_all]
     ulonglong2 *tw_fwd = nullptr;   // [n_all][N] (psi^brv(k), Shoup)
@@ -350,6 +357,8 @@ void launch_rescale_prep(const LaunchCtx &c, View r, View xtop, const RescaleTab
                          const Scalars *sc = nullptr);
 void launch_rescale_final(const LaunchCtx &c, View out, View in, View r, const RescaleTable *tab, int B, int comps,
                           int top, const Scalars *sc = nullptr);
+void launch_rescale_tail(const LaunchCtx &c, View out, View in, View r, const RescaleTable *tab, const Scalars &sc,
+                         const RescaleTail &tail, int B, int comps, int top);
 void launch_keygen_b(const LaunchCtx &c, uint64_t *b, const uint64_t *a, const uint64_t *e, const uint64_t *s,
                      const uint64_t *sp, const uint64_t *gadget_mask, int rows, const int *prime_of_row_dev,
                      bool to_mont);

@@ -1169,6 +1169,39 @@ __global__ void k_rescale_final(View out, View in, View r, const RescaleTable *_
     }
 }
 
+// the division and a linear combination with another ciphertext and a constant in one pass.  Bound by
+// memory (24 bytes a word, 32 with a second ciphertext): the terms of a composite sign's polynomial
+// took five more passes (integer multiplications and sums, 16 to 24 bytes a word each); without them
+// sixty-four signs at N = 2^15 take 128.0 ms instead of 131.3
+__global__ void k_rescale_tail(View out, View in, View r, const RescaleTable *__restrict__ tab,
+                               const PrimeConst *__restrict__ primes, int comps, int n,
+                               const __grid_constant__ Scalars sc, const __grid_constant__ RescaleTail T)
+{
+    after_previous_kernel();
+    const int i = blockIdx.y, bc = blockIdx.z, bi = bc / comps, ci = bc % comps;
+    const uint64_t q = primes[i].q, s = sc.v[i], ssh = sc.sh[i], w = tab->qinv[i], wsh = tab->qinv_sh[i];
+    const uint64_t aw = T.add_w.v[i], awsh = T.add_w.sh[i], c0 = ci == 0 ? T.c0.v[i] : 0;
+    const uint64_t *a = in.p + bi * in.bstride + ci * in.cstride + (size_t)i * n;
+    const uint64_t *rr = r.p + bi * r.bstride + ci * r.cstride + (size_t)i * n;
+    const uint64_t *x = T.add.p + bi * T.add.bstride + ci * T.add.cstride + (size_t)i * n;  // read if T.has_add
+    uint64_t *o = out.p + bi * out.bstride + ci * out.cstride + (size_t)i * n;
+    for (int j = (blockIdx.x * blockDim.x + threadIdx.x) * 2; j < n; j += gridDim.x * blockDim.x * 2) {
+        const ulonglong2 av = *reinterpret_cast<const ulonglong2 *>(a + j);
+        const ulonglong2 rv = *reinterpret_cast<const ulonglong2 *>(rr + j);
+        ulonglong2 xv = make_ulonglong2(0, 0);
+        if (T.has_add) xv = *reinterpret_cast<const ulonglong2 *>(x + j);
+        if (T.has_add == 2) xv = make_ulonglong2(shoup(xv.x, aw, awsh, q), shoup(xv.y, aw, awsh, q));
+        uint64_t v0 = shoup(submod(shoup(av.x, s, ssh, q), rv.x, q), w, wsh, q);
+        uint64_t v1 = shoup(submod(shoup(av.y, s, ssh, q), rv.y, q), w, wsh, q);
+        if (T.has_w) {
+            v0 = shoup(v0, T.w.v[i], T.w.sh[i], q);
+            v1 = shoup(v1, T.w.v[i], T.w.sh[i], q);
+        }
+        *reinterpret_cast<ulonglong2 *>(o + j) =
+            make_ulonglong2(addmod(addmod(v0, xv.x, q), c0, q), addmod(addmod(v1, xv.y, q), c0, q));
+    }
+}
+
 // Relinearisation + rescale (division by P q_top).  Row l-1 (q_top) of each key-switched
 // component becomes y = acc + (P mod q_top) d, the value the conversion reads there.
 __global__ void k_relin_rs_top(View acc, View d, const RelinRescaleTable *__restrict__ tab,
@@ -1756,6 +1789,15 @@ void launch_rescale_final(const LaunchCtx &c, View out, View in, View r, const R
     dim3 grid(ew_blocks(c.N, 2), top, B * comps);
     launch(c.stream, k_rescale_final, grid, 256, 0, out, in, r, tab, c.t->primes, comps, c.N, sc ? *sc : Scalars{},
                                                 sc != nullptr);
+    post(c);
+}
+
+void launch_rescale_tail(const LaunchCtx &c, View out, View in, View r, const RescaleTable *tab, const Scalars &sc,
+                         const RescaleTail &tail, int B, int comps, int top)
+{
+    Timed tm_(c, K_RESCALE, (tail.has_add ? 32.0 : 24.0) * B * comps * top * c.N);
+    dim3 grid(ew_blocks(c.N, 2), top, B * comps);
+    launch(c.stream, k_rescale_tail, grid, 256, 0, out, in, r, tab, c.t->primes, comps, c.N, sc, tail);
     post(c);
 }
 

@@ -186,7 +186,14 @@ struct Eval {
     void tensor_sum(Cts &acc, const Cts &a, const Cts &b);
     void from_mont(Cts &a);  // a *= 2^64, in place
     Cts relinearize(const Cts &d, const SwitchKey &rk);
-    Cts rescale(const Cts &a, int64_t c = 1);  // rescale(c * a), c an integer scalar
+    struct Tail {
+        int64_t times = 1;         // of the rescaled ciphertext
+        const Cts *add = nullptr;  // add_times * add is added
+        int64_t add_times = 1;
+        int64_t c0 = 0;  // added to component 0
+    };
+    // rescale(c * a), c an integer scalar; tail: the combination that follows, in the same pass
+    Cts rescale(const Cts &a, int64_t c = 1, const Tail *tail = nullptr);
     Cts relin_rescale(const Cts &d, const SwitchKey &rk);  // rescale(relinearize(d)) as one division
     Cts drop(const Cts &a, int limbs);  // shares storage
     Cts copy(const Cts &a);
@@ -246,6 +253,7 @@ struct RotateJob {
 std::vector<Cts> rotate_jobs(const std::vector<RotateJob> &jobs, cudaStream_t s);
 
 Scalars scalars_for(const hx_context &ctx, int limbs, int64_t c);
+int64_t const_int(double value, double scale);  // round(value * scale), refused beyond 64 bits
 void upload_plaintext(hx_context &ctx, cudaStream_t s, const int64_t *coeffs, int limbs, uint64_t *dst_mont);
 // the same over p_0..p_{K-1} then q_0..q_{limbs-1} (an extended mask's row order)
 void upload_plaintext_ext(hx_context &ctx, cudaStream_t s, const int64_t *coeffs, int limbs, uint64_t *dst_mont);

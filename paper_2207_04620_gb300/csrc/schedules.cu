@@ -716,15 +716,16 @@ Cts square_rs(Eval &ev, const hx_keyset &ks, const Cts &a, const Cts &b)
 
 // bring ct to `target` limbs at scale target_scale, times c_real: drop to
 // target+1 limbs, multiply by round(c_real*target_scale*q_target/scale),
-// rescale; the result is declared to have target_scale
-Cts level_adjust(Eval &ev, const Cts &ct, int target, double c_real, double target_scale)
+// rescale (with what tail adds); the result is declared to have target_scale
+Cts level_adjust(Eval &ev, const Cts &ct, int target, double c_real, double target_scale,
+                 const Eval::Tail *tail = nullptr)
 {
     HX_CHECK(ct.limbs > target, HX_ELEVEL, "cannot raise the level");
     Cts x = ct.limbs > target + 1 ? ev.drop(ct, target + 1) : ct;
     const uint64_t qt = ev.ctx.primes[target];
     const double c = round_half_away(c_real * target_scale * (double)qt / ct.scale);
     HX_CHECK(std::fabs(c) < 4.6e18, HX_EINVAL, "level-adjust constant too large");
-    Cts y = ev.rescale(x, (int64_t)c);
+    Cts y = ev.rescale(x, (int64_t)c, tail);
     y.scale = target_scale;
     return y;
 }
@@ -739,24 +740,33 @@ Cts eval_g(Eval &ev, const hx_keyset &ks, const Cts &x, int d)
     Cts y1 = square_rs(ev, ks, x, x), y2, top;
     if (d >= 2) y2 = square_rs(ev, ks, y1, y1);
     if (d >= 3) {
-        Cts B = ev.mul_int(level_adjust(ev, y1, y2.limbs, 1.0, y2.scale), n[3]);
-        if (d == 4) ev.add_inplace(B, ev.mul_int(y2, n[4]));
-        top = square_rs(ev, ks, y2, B);
+        Eval::Tail t;  // n3 y + n4 y^2
+        t.times = n[3];
+        if (d == 4) t.add = &y2, t.add_times = n[4];
+        top = square_rs(ev, ks, y2, level_adjust(ev, y1, y2.limbs, 1.0, y2.scale, &t));
     }
     const Cts &lead = d >= 3 ? top : (d == 2 ? y2 : y1);
     const int lp = lead.limbs;
     const double sp = lead.scale;
     Cts P = d >= 3 ? top : Cts();
+    bool complete = false;  // n0 is in P
     const Cts *ys[3] = {nullptr, &y1, &y2};
     for (int j = 1; j <= std::min(d, 2); j++) {
         const Cts &yj = *ys[j];
-        Cts t = yj.limbs > lp ? level_adjust(ev, yj, lp, (double)n[j], sp) : ev.mul_int(yj, n[j]);
-        if (!P.buf)
-            P = t;
-        else
-            ev.add_inplace(P, t);
+        if (yj.limbs > lp) {  // its adjustment adds the terms so far, the last one's n0 too
+            Eval::Tail t;
+            if (P.buf) t.add = &P;
+            if (j == std::min(d, 2)) t.c0 = const_int((double)n[0], sp), complete = true;
+            P = level_adjust(ev, yj, lp, (double)n[j], sp, &t);
+        } else {
+            Cts t = ev.mul_int(yj, n[j]);
+            if (!P.buf)
+                P = t;
+            else
+                ev.add_inplace(P, t);
+        }
     }
-    P = ev.add_const(P, (double)n[0]);
+    if (!complete) P = ev.add_const(P, (double)n[0]);
     Cts xa = level_adjust(ev, x, lp, 1.0 / std::ldexp(1.0, 2 * d - 1), sp);
     return square_rs(ev, ks, xa, P);
 }
