@@ -1062,15 +1062,13 @@ hx_status hx_matmul_exec_run(hx_matmul_exec *ex, const hx_ct *const *A, const hx
                  "inputs must have the executor's scale");
     }
     cudaStream_t s = S(stream);
+    std::vector<CopyPair> copies;
     for (size_t i = 0; i < ex->count; i++)
         for (int c = 0; c < 2; c++) {
-            HX_CUDA(cudaMemcpyAsync(ex->A.d + i * ex->A.bstride(N) + c * ex->A.cstride(N),
-                                    A[i]->c.d + c * A[i]->c.cstride(N), sizeof(uint64_t) * ex->A.limbs * N,
-                                    cudaMemcpyDeviceToDevice, s));
-            HX_CUDA(cudaMemcpyAsync(ex->B.d + i * ex->B.bstride(N) + c * ex->B.cstride(N),
-                                    B[i]->c.d + c * B[i]->c.cstride(N), sizeof(uint64_t) * ex->B.limbs * N,
-                                    cudaMemcpyDeviceToDevice, s));
+            copies.push_back({ex->A.d + i * ex->A.bstride(N) + c * ex->A.cstride(N), A[i]->c.d + c * A[i]->c.cstride(N)});
+            copies.push_back({ex->B.d + i * ex->B.bstride(N) + c * ex->B.cstride(N), B[i]->c.d + c * B[i]->c.cstride(N)});
         }
+    launch_copies(Eval(ctx, s).lc(), copies, ex->A.limbs * N);
     HX_CUDA(cudaGraphLaunch(ex->exec, s));
     ctx.counters[C_LAUNCH] += ex->launches;
     scatter(ctx, ex->out, out, s);

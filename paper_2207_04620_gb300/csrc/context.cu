@@ -492,11 +492,11 @@ Cts gather(hx_context &ctx, const hx_ct *const *cts, size_t count, cudaStream_t 
     Cts out = ev.alloc((int)count, f.comps, f.limbs);
     out.scale = f.scale;
     const size_t N = ctx.N;
+    std::vector<CopyPair> copies;
     for (size_t i = 0; i < count; i++)
         for (int c = 0; c < f.comps; c++)
-            HX_CUDA(cudaMemcpyAsync(out.d + i * out.bstride(N) + c * out.cstride(N),
-                                    cts[i]->c.d + c * cts[i]->c.cstride(N), sizeof(uint64_t) * f.limbs * N,
-                                    cudaMemcpyDeviceToDevice, s));
+            copies.push_back({out.d + i * out.bstride(N) + c * out.cstride(N), cts[i]->c.d + c * cts[i]->c.cstride(N)});
+    launch_copies(ev.lc(), copies, f.limbs * N);
     return out;
 }
 
@@ -504,16 +504,17 @@ void scatter(hx_context &ctx, const Cts &b, hx_ct **out, cudaStream_t s)
 {
     const size_t N = ctx.N;
     Eval ev(ctx, s);
+    std::vector<CopyPair> copies;
     for (int i = 0; i < b.B; i++) {
         hx_ct *h = new hx_ct;
         h->ctx = &ctx;
         h->c = ev.alloc(1, b.comps, b.limbs);
         h->c.scale = b.scale;
         for (int c = 0; c < b.comps; c++)
-            HX_CUDA(cudaMemcpyAsync(h->c.d + c * h->c.cstride(N), b.d + i * b.bstride(N) + c * b.cstride(N),
-                                    sizeof(uint64_t) * b.limbs * N, cudaMemcpyDeviceToDevice, s));
+            copies.push_back({h->c.d + c * h->c.cstride(N), b.d + i * b.bstride(N) + c * b.cstride(N)});
         out[i] = h;
     }
+    launch_copies(ev.lc(), copies, b.limbs * N);
 }
 
 } // namespace hx

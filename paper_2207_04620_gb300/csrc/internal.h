@@ -113,6 +113,17 @@ struct View {
     size_t bstride, cstride;
 };
 
+// copies of one launch
+constexpr int MAX_COPIES = 128;
+struct CopyPair {
+    uint64_t *dst;
+    const uint64_t *src;
+};
+struct CopyTab {
+    const uint64_t *src[MAX_COPIES];
+    uint64_t *dst[MAX_COPIES];
+};
+
 // what follows a rescale's division x in the same pass: w x + add_w add + c0 (c0 on component 0)
 struct RescaleTail {
     Scalars w, add_w, c0;
@@ -187,6 +198,8 @@ void launch_ntt_multi(cudaStream_t s, const std::vector<NttJob> &jobs, bool inve
 void autotune_ntt(const LaunchCtx &c, uint64_t *buf, int rows, int *best, float *ms_out);
 void launch_add(const LaunchCtx &c, View out, View a, View b, int B, int comps, int limbs, bool sub);
 void launch_copy(const LaunchCtx &c, View out, View a, int B, int comps, int limbs);
+// words of each pair (a multiple of 2^11), the pairs' buffers disjoint
+void launch_copies(const LaunchCtx &c, const std::vector<CopyPair> &copies, size_t words);
 // one ciphertext read in place: component c, limb l at p + c*cstride + l*N
 struct AggSrc {
     const uint64_t *p;

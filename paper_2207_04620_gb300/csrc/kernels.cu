@@ -64,6 +64,25 @@ __global__ void k_copy(View out, View a, int comps, int n)
         *reinterpret_cast<ulonglong2 *>(out.p + oo + j) = *reinterpret_cast<const ulonglong2 *>(a.p + oa + j);
 }
 
+// Copies of equal length between ciphertexts' own buffers and a batch: a table of addresses in one
+// launch, where one device-to-device copy each took 2-4 us of the host and of the stream:
+// one aggregation of 8 models over 16 parties 494 -> 386 us with it and with the update's sum in the rescale.
+// A block moves kCopyWords, 64 bytes a thread in flight.
+constexpr int kCopyWords = 2048;
+
+__global__ void __launch_bounds__(256) k_copy_table(const __grid_constant__ CopyTab T)
+{
+    after_previous_kernel();
+    const size_t at = (size_t)blockIdx.x * (kCopyWords / 2) + threadIdx.x;
+    const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(T.src[blockIdx.y]) + at;
+    ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(T.dst[blockIdx.y]) + at;
+    ulonglong2 x[kCopyWords / 512];
+#pragma unroll
+    for (int i = 0; i < kCopyWords / 512; i++) x[i] = src[i * 256];
+#pragma unroll
+    for (int i = 0; i < kCopyWords / 512; i++) dst[i * 256] = x[i];
+}
+
 // Alg. 6 Aggregation: the sum over parties of one gradient ciphertext, times a
 // constant, streamed from the parties' buffers in place (16-byte loads, four
 // parties in flight per thread, a Barrett reduction every 4 terms).
@@ -1455,6 +1474,19 @@ void launch_copy(const LaunchCtx &c, View out, View a, int B, int comps, int lim
     dim3 grid(ew_blocks(c.N, 2), limbs, B * comps);
     launch(c.stream, k_copy, grid, 256, 0, out, a, comps, c.N);
     post(c);
+}
+
+void launch_copies(const LaunchCtx &c, const std::vector<CopyPair> &copies, size_t words)
+{
+    Timed tm_(c, K_ELEM, 16.0 * copies.size() * words);
+    HX_CHECK(words % kCopyWords == 0, HX_EINVAL, "whole rows of at least 2^11 words are copied");
+    for (size_t at = 0; at < copies.size(); at += MAX_COPIES) {
+        CopyTab t;
+        const int k = (int)std::min<size_t>(MAX_COPIES, copies.size() - at);
+        for (int i = 0; i < k; i++) t.src[i] = copies[at + i].src, t.dst[i] = copies[at + i].dst;
+        launch(c.stream, k_copy_table, dim3((unsigned)(words / kCopyWords), k), 256, 0, t);
+        post(c);
+    }
 }
 
 void launch_aggregate(const LaunchCtx &c, View out, const AggSrc *src_dev, int n_parties, int count, int comps,

@@ -935,9 +935,12 @@ Cts aggregate(hx_context &ctx, const std::vector<const Cts *> &grads, int n_part
     sum.scale = g0.scale;
     launch_aggregate(ev.lc(), sum.view(ctx.N), reinterpret_cast<const AggSrc *>(tab_dev.p), n_parties, count, 2, L,
                      scalars_for(ctx, L, (int64_t)cr));
-    Cts upd = ev.rescale(sum);
+    const Cts low = ev.drop(models, target);
+    Eval::Tail t;
+    t.add = &low;
+    Cts upd = ev.rescale(sum, 1, &t);
     upd.scale = models.scale;
-    return ev.add(ev.drop(models, target), upd);
+    return upd;
 }
 
 } // namespace hx

@@ -207,17 +207,19 @@ void hx_server::run_lane(Lane &L)
                 Cts A = ev.alloc(B, 2, r0.a.limbs);
                 A.scale = r0.a.scale;
                 const size_t N = ctx.N;
+                std::vector<CopyPair> copies;
                 auto pack = [&](Cts &dst, int i, const Cts &src) {
                     for (int c = 0; c < 2; c++)
-                        HX_CUDA(cudaMemcpyAsync(dst.d + i * dst.bstride(N) + c * dst.cstride(N),
-                                                src.d + c * src.cstride(N), sizeof(uint64_t) * dst.limbs * N,
-                                                cudaMemcpyDeviceToDevice, L.s));
+                        copies.push_back({dst.d + i * dst.bstride(N) + c * dst.cstride(N), src.d + c * src.cstride(N)});
                 };
                 for (int i = 0; i < B; i++) pack(A, i, batch[i].a);
+                launch_copies(ev.lc(), copies, A.limbs * N);
                 if (r0.kind == 0) {
                     Cts Bc = ev.alloc(B, 2, r0.b.limbs);
                     Bc.scale = r0.b.scale;
+                    copies.clear();
                     for (int i = 0; i < B; i++) pack(Bc, i, batch[i].b);
+                    launch_copies(ev.lc(), copies, Bc.limbs * N);
                     plan = cached_plan(ctx, r0.h, r0.a.limbs);  // held until the lane's stream is done
                     out = matmul_batch(ctx, *r0.ks, *plan, A, Bc, L.s);
                 } else {
