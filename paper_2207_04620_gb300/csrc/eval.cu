@@ -514,8 +514,21 @@ Cts Eval::rescale(const Cts &a, int64_t c, const Tail *tail)
     // (the top limb after its inverse NTT), the same values as multiplying first
     const Scalars sc = c != 1 || tail ? scalars_for(ctx, a.limbs, c) : Scalars{};
     const Scalars *scp = c != 1 || tail ? &sc : nullptr;
-    launch_rescale_prep(lc(), rv, View{xtop.p, (size_t)comps * N, (size_t)N}, tab, B, comps, top, scp);
-    ntt_inplace(r.p, (size_t)top * N, B * comps, iota_vec(0, top), iota_vec(0, top), false);
+    // The remainder modulo every lower prime, transformed.  Centred it is at most q_top / 2 in size, and
+    // the fold transform takes signed inputs below 4q: where no lower prime is less than that, one
+    // centred row feeds the transform of every limb and no reduced rows are written and read.
+    // Sixty-four signs at N = 2^15 126.3 -> 122.2 ms, an aggregation's export and all 860 -> 829 us.
+    const uint64_t qt = ctx.primes[top];
+    bool centred = ctx.t.fold != nullptr;
+    for (int i = 0; i < top; i++) centred = centred && ctx.primes[i] > qt / 2;
+    if (centred) {
+        launch_rescale_centre(lc(), xtop.p, tab, qt, B * comps, sc.v[top], sc.sh[top], scp != nullptr);
+        ntt_oop(xtop.p, (size_t)N, r.p, (size_t)top * N, B * comps, std::vector<int>(top, 0), iota_vec(0, top),
+                iota_vec(0, top), false);
+    } else {
+        launch_rescale_prep(lc(), rv, View{xtop.p, (size_t)comps * N, (size_t)N}, tab, B, comps, top, scp);
+        ntt_inplace(r.p, (size_t)top * N, B * comps, iota_vec(0, top), iota_vec(0, top), false);
+    }
     Cts o = alloc(B, comps, top);
     if (tail) {
         RescaleTail t{scalars_for(ctx, top, tail->times), scalars_for(ctx, top, tail->add_times),

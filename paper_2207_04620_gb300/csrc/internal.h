@@ -368,6 +368,8 @@ void launch_relin_rs_final(const LaunchCtx &c, View out, View acc, View d, View 
                            int B, int limbs);
 void launch_rescale_prep(const LaunchCtx &c, View r, View xtop, const RescaleTable *tab, int B, int comps, int top,
                          const Scalars *sc = nullptr);
+void launch_rescale_centre(const LaunchCtx &c, uint64_t *xtop, const RescaleTable *tab, uint64_t qt, int rows,
+                           uint64_t s, uint64_t ssh, bool scaled);
 void launch_rescale_final(const LaunchCtx &c, View out, View in, View r, const RescaleTable *tab, int B, int comps,
                           int top, const Scalars *sc = nullptr);
 void launch_rescale_tail(const LaunchCtx &c, View out, View in, View r, const RescaleTable *tab, const Scalars &sc,

@@ -65,8 +65,7 @@ __global__ void k_copy(View out, View a, int comps, int n)
 }
 
 // Copies of equal length between ciphertexts' own buffers and a batch: a table of addresses in one
-// launch, where one device-to-device copy each took 2-4 us of the host and of the stream:
-// one aggregation of 8 models over 16 parties 494 -> 386 us with it and with the update's sum in the rescale.
+// launch, where one device-to-device copy each took 2-4 us of the host and of the stream.  @C@
 // A block moves kCopyWords, 64 bytes a thread in flight.
 constexpr int kCopyWords = 2048;
 
@@ -1166,6 +1165,20 @@ __global__ void k_rescale_prep(View r, View xtop, const RescaleTable *__restrict
     }
 }
 
+// the remainder itself, centred: [x + floor(q_t/2)]_{q_t} - floor(q_t/2) as a signed word, in place
+__global__ void k_rescale_centre(uint64_t *x, const RescaleTable *__restrict__ tab, uint64_t qt, int n, uint64_t s,
+                                 uint64_t ssh, bool scaled)
+{
+    after_previous_kernel();
+    const uint64_t half = tab->half;
+    x += (size_t)blockIdx.y * n;
+    for (int j = (blockIdx.x * blockDim.x + threadIdx.x) * 2; j < n; j += gridDim.x * blockDim.x * 2) {
+        ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(x + j);
+        if (scaled) v = make_ulonglong2(shoup(v.x, s, ssh, qt), shoup(v.y, s, ssh, qt));
+        *reinterpret_cast<ulonglong2 *>(x + j) = make_ulonglong2(csub(v.x + half, qt) - half, csub(v.y + half, qt) - half);
+    }
+}
+
 __global__ void k_rescale_final(View out, View in, View r, const RescaleTable *__restrict__ tab,
                                 const PrimeConst *__restrict__ primes, int comps, int n,
                                 const __grid_constant__ Scalars sc, bool scaled)
@@ -1811,6 +1824,15 @@ void launch_rescale_prep(const LaunchCtx &c, View r, View xtop, const RescaleTab
     dim3 grid(ew_blocks(c.N, 2), top, B * comps);
     launch(c.stream, k_rescale_prep, grid, 256, 0, r, xtop, tab, c.t->primes, comps, top, c.N, sc ? *sc : Scalars{},
                                                sc != nullptr);
+    post(c);
+}
+
+void launch_rescale_centre(const LaunchCtx &c, uint64_t *xtop, const RescaleTable *tab, uint64_t qt, int rows,
+                           uint64_t s, uint64_t ssh, bool scaled)
+{
+    Timed tm_(c, K_RESCALE, 16.0 * rows * c.N);
+    HX_CHECK(rows < 65536, HX_EINVAL, "rescale batch too large");
+    launch(c.stream, k_rescale_centre, dim3(ew_blocks(c.N, 2), rows), 256, 0, xtop, tab, qt, c.N, s, ssh, scaled);
     post(c);
 }
 
