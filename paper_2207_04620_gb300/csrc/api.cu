@@ -1268,7 +1268,7 @@ hx_status hx_autotune(hx_context *ctx, int32_t *choice, void *stream)
     HX_CUDA(cudaMemsetAsync(buf.p, 0, sizeof(uint64_t) * rows_max * ctx->N, S(stream)));
     Eval ev(*ctx, S(stream));
     for (int b = 0; b < NTT_BUCKETS; b++) {
-        int best[5] = {2, 2, 2, 2, 0};
+        int best[5];
         float ms[4];
         autotune_ntt(ev.lc(), buf.p, std::min(kNttBucketTune[b], rows_max), best, ms);
         for (int i = 0; i < 5; i++) ctx->t.ntt_var[b][i] = best[i];
@@ -1295,7 +1295,7 @@ hx_status hx_ntt_tiles(hx_context *ctx, const int32_t *set, int32_t *get)
         }
         for (int b = 0; b < NTT_BUCKETS; b++) {
             for (int i = 0; i < 4; i++) ctx->t.ntt_var[b][i] = v[i];
-            ctx->t.ntt_var[b][4] = 0;  // the default split of an odd log N
+            ctx->t.ntt_var[b][4] = ntt_default_split(ctx->log_n);
         }
     }
     if (get)

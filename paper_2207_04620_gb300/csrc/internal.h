@@ -23,6 +23,22 @@ constexpr int kNttTileWidths[NTT_WIDTHS] = {4, 8, 16, 32};
 constexpr int NTT_VARIANTS = 2 * NTT_WIDTHS;  // a width, with the register passes' radices as is or swapped
 // NTT batch sizes tuned separately: a launch of n limbs uses the first bucket with n <= its bound
 constexpr int NTT_BUCKETS = 4;
+// Untuned, the column phase takes the larger half of an odd log N from 2^13 on: its threads of a warp
+// share their twiddles, a row phase's do not, and the L1 pipe that returns them is as busy as the
+// multiply pipe.  1200 rows of N = 2^15 take 294 us forward and 309 inverse instead of 326 and 359,
+// 3200 of N = 2^13 177 and 189 instead of 190 and 201; 960 of N = 2^11 15.9 instead of 15.3, so there
+// the smaller half stays.
+__host__ __device__ constexpr int ntt_default_split(int log_n) { return (log_n & 1) && log_n >= 13 ? 1 : 0; }
+// Untuned tile widths: 8 for a phase of 256 points, else 16, blocks of 128 threads either way (400 rows of
+// N = 2^16 228 us forward and 243 inverse, 236 and 258 with blocks of 256)
+constexpr int ntt_default_var(int logm) { return logm >= 8 ? 1 : 2; }
+inline void ntt_defaults(int log_n, int (&v)[5])
+{
+    const int cols = log_n / 2 + ntt_default_split(log_n), rows = log_n - cols;
+    v[0] = v[2] = ntt_default_var(cols);
+    v[1] = v[3] = ntt_default_var(rows);
+    v[4] = ntt_default_split(log_n);
+}
 constexpr int kNttBucketMax[NTT_BUCKETS] = {64, 256, 768, 1 << 30};
 constexpr int kNttBucketTune[NTT_BUCKETS] = {48, 176, 512, 1024};  // limbs timed for each bucket
 inline int ntt_bucket(long long limbs)
@@ -146,7 +162,7 @@ struct DeviceTables {
     // NTT variant per batch-size bucket and phase (fwd cols, fwd rows, inv cols, inv rows)
     // per bucket: the four phases' variants (forward column, forward row, inverse column, inverse
     // row), then the split of an odd log N (0: the column phase takes floor(log N / 2) stages, 1: ceil)
-    int ntt_var[NTT_BUCKETS][5] = {{2, 2, 2, 2, 0}, {2, 2, 2, 2, 0}, {2, 2, 2, 2, 0}, {2, 2, 2, 2, 0}};
+    int ntt_var[NTT_BUCKETS][5];
     int n_sm = 1;                   // multiprocessors of the device
 };
 

@@ -54,13 +54,13 @@ void autotune_ntt(const LaunchCtx &c, uint64_t *buf, int rows, int *best, float 
     HX_CUDA(cudaEventCreate(&e0));
     HX_CUDA(cudaEventCreate(&e1));
     // Each variant's time is the best of three rounds of five transforms, the rounds interleaved
-    // over the variants so drift hits them alike.  A variant replaces the default (width 16: four
-    // warps per block in the 128-point phases) only when it is clearly faster: the widths' isolated
+    // over the variants so drift hits them alike.  A variant replaces the default (four warps per
+    // block) only when it is clearly faster: the widths' isolated
     // times differ by about their noise (1-2 % at the batch sizes of a product's launches), and
     // blocks of the default size share the SMs best with the kernels of concurrent chains.  The
     // other split of an odd log N replaces the default one on the same rule, by the sum of its
     // four phases' times.
-    constexpr int kDefault = 2, kRounds = 3, kRuns = 5;
+    constexpr int kRounds = 3, kRuns = 5;
     constexpr float kClearWin = 0.98f;
     float split_ms[2] = {0.f, 0.f};
     int split_best[2][4];
@@ -70,7 +70,7 @@ void autotune_ntt(const LaunchCtx &c, uint64_t *buf, int rows, int *best, float 
         const int logm1 = c.log_n / 2 + sp, logm2 = c.log_n - logm1;
         for (int ph = 0; ph < 4; ph++) {
             const bool cols = ph == 0 || ph == 2, inv = ph >= 2;
-            const int logm = cols ? logm1 : logm2;
+            const int logm = cols ? logm1 : logm2, kDefault = ntt_default_var(logm);
             float t[NTT_VARIANTS];
             bool ok[NTT_VARIANTS];
             for (int v = 0; v < NTT_VARIANTS; v++) {
@@ -100,7 +100,8 @@ void autotune_ntt(const LaunchCtx &c, uint64_t *buf, int rows, int *best, float 
             split_ms[sp] += split_phase_ms[sp][ph];
         }
     }
-    const int sp = (n_splits == 2 && split_ms[1] < kClearWin * split_ms[0]) ? 1 : 0;
+    const int def = ntt_default_split(c.log_n);
+    const int sp = (n_splits == 2 && split_ms[1 - def] < kClearWin * split_ms[def]) ? 1 - def : def;
     for (int ph = 0; ph < 4; ph++) {
         best[ph] = split_best[sp][ph];
         if (ms_out) ms_out[ph] = split_phase_ms[sp][ph];
@@ -119,7 +120,7 @@ void plan_ntt_jobs(std::vector<NttJob> &jobs, int *tiles_cols, int *tiles_rows)
     for (auto &J : jobs) {
         HX_CHECK(J.log_n >= 11 && J.log_n <= 16, HX_EINVAL, "ring degree outside 2^11..2^16");
         HX_CHECK(J.n_limbs >= 1 && J.n_limbs <= 64 && J.n_rows >= 0, HX_EINVAL, "bad job rows");
-        const int n = 1 << J.log_n, l1 = J.log_n / 2, l2 = J.log_n - l1;
+        const int n = 1 << J.log_n, l1 = J.log_n / 2 + ntt_default_split(J.log_n), l2 = J.log_n - l1;
         const int w1 = 128 / ((1 << l1) >> ((l1 + 1) / 2)), w2 = 128 / ((1 << l2) >> ((l2 + 1) / 2));
         J.tile0_cols = tc;
         J.tile0_rows = tr;

@@ -523,7 +523,8 @@ __device__ __forceinline__ MultiTile<A> multi_tile(const NttJob *jobs, int n_job
     MultiTile<A> m;
     const int local = t - (cols ? J.tile0_cols : J.tile0_rows);
     m.log_n = J.log_n;
-    m.logm = cols ? J.log_n / 2 : J.log_n - J.log_n / 2;
+    const int logc = J.log_n / 2 + ntt_default_split(J.log_n);
+    m.logm = cols ? logc : J.log_n - logc;
     const int n = 1 << J.log_n;
     const int W = kMultiT / ((1 << m.logm) >> ((m.logm + 1) / 2));
     const int nb = (n >> m.logm) / W;
