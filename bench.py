@@ -1097,8 +1097,8 @@ def run_micro_ntt_multi(args):
     cases = {"large": [(13, 12, 8), (14, 8, 16), (15, 16, 4), (16, 20, 2)],
              "many_small": [(12 + (i % 3), 1 + (i % 4), 1) for i in range(48)]}
     out = {"micro": "ntt_multi", "peak_gbs": peak, "peak_kind": kind,
-           "note": "fused: one persistent launch per phase for all rings (128-thread tiles, next tile "
-                   "prefetched); per-ring: one hx_ntt call (two launches, autotuned persistent kernels) per ring"}
+           "note": "fused: one launch per phase for all rings (128-thread tiles); "
+                   "per-ring: one hx_ntt call (two launches, autotuned kernels) per ring"}
     for name, specs in cases.items():
         jobs, bufs, byt = make_jobs(specs)
 
