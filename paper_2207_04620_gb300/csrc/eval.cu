@@ -229,8 +229,10 @@ void Eval::moddown_add(const View &out, const View &accv, int B, int limbs, cons
                          limbs, add, add_mask, gal, shared);
 }
 
-// Rotations (or selections) of a batch of B per launch: as many as keep the launch's buffer small, so
-// that the stages that follow find it in L2.  One rotation of 16 entries of N = 2^14 (38 MB) already
+// Rotations (or selections) of a batch of B per launch: as many as keep the launch's buffer within
+// 128 MB, about L2's size, so that the stages that follow find most of it there (sixteen 64x64 pairs
+// 21.9 ms with 32 MB, 20.8 with 128; five 32x32 products 2.11 and 2.03, 2.33 with 16; a small dense layer
+// 8.66 and 7.85, 10.6 with 16).  One rotation of 16 entries of N = 2^14 (38 MB) already
 // fills the GPU; one of a single entry of N = 2^12 takes a few SMs, and with a launch per stage and
 // rotation the product of 16x16 matrices there waited on about 900 launches: 5.2 ms, 0.74 in groups
 // (five 32x32 products of N = 2^13: 4.0 ms, 2.6; a small dense layer of N = 2^14: 23.2 ms, 11.0).
@@ -238,7 +240,7 @@ int Eval::rot_chunk(int B, int limbs, int most, size_t words)
 {
     const size_t per = words ? words : (size_t)B * 2 * (limbs + ctx.K) * ctx.N;
     const int grid = std::max(1, 16384 / (B * std::max(2, (limbs + ctx.alpha - 1) / ctx.alpha)));
-    return std::max(1, std::min({most, grid, (int)std::min<size_t>(MAX_ROT, ((size_t)32 << 20) / 8 / per)}));
+    return std::max(1, std::min({most, grid, (int)std::min<size_t>(MAX_ROT, kGroupBytes / 8 / per)}));
 }
 
 Cts Eval::rotate_sum(const Cts &items, const std::vector<int64_t> &steps, const hx_keyset &keys)
@@ -251,7 +253,7 @@ Cts Eval::rotate_sum(const Cts &items, const std::vector<int64_t> &steps, const 
     HX_CUDA(cudaMemsetAsync(base.d, 0, sizeof(uint64_t) * base.bstride(N) * B, s));
     DevBuf acc((size_t)B * 2 * ext * N, s);
     View accv{acc.p, (size_t)2 * ext * N, (size_t)ext * N};
-    const int most = rot_chunk(B, limbs, MAX_ROT, (size_t)B * nd * ext * N / 2);  // the ModUp digits: up to 64 MB
+    const int most = rot_chunk(B, limbs, MAX_ROT, (size_t)B * nd * ext * N / 2);  // the ModUp digits: up to 256 MB
     bool any = false;
     for (int r = 0; r < R;) {
         Cts first = items;

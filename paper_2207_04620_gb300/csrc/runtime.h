@@ -253,6 +253,7 @@ struct RotateJob {
 std::vector<Cts> rotate_jobs(const std::vector<RotateJob> &jobs, cudaStream_t s);
 
 Scalars scalars_for(const hx_context &ctx, int limbs, int64_t c);
+constexpr size_t kGroupBytes = (size_t)128 << 20;  // see Eval::rot_chunk
 int64_t const_int(double value, double scale);  // round(value * scale), refused beyond 64 bits
 void upload_plaintext(hx_context &ctx, cudaStream_t s, const int64_t *coeffs, int limbs, uint64_t *dst_mont);
 // the same over p_0..p_{K-1} then q_0..q_{limbs-1} (an extended mask's row order)

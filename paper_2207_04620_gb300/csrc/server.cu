@@ -66,6 +66,14 @@ size_t estimate(const Request &r)
     return r.kind == 0 ? 48 * ct : 24 * ct + (size_t)2 * r.ctx->n_q * r.ctx->N * 8;
 }
 
+// a product's grouped rotations and selections on top of that: some eight buffers over its three
+// streams, each of a group's size
+size_t group_bytes(const Request &r, size_t entries)
+{
+    if (r.kind != 0) return 0;
+    return 8 * std::min(kGroupBytes, entries * MAX_MUX * 2 * (r.a.limbs + r.ctx->K) * r.ctx->N * 8);
+}
+
 size_t key_bytes(const hx_keyset &ks)
 {
     size_t b = ks.relin.buf ? ks.relin.buf->words * 8 : 0;
@@ -157,7 +165,8 @@ void hx_server::run_dispatch()
                 ++it;
                 continue;
             }
-            if (admitted + est + it->est > budget) break;
+            // beside running batches a group's buffers have to fit too; a batch alone runs as before
+            if (admitted + est + it->est + (admitted ? group_bytes(*it, batch.size() + 1) : 0) > budget) break;
             est += it->est;
             batch.push_back(std::move(*it));
             it = pending.erase(it);
@@ -166,8 +175,9 @@ void hx_server::run_dispatch()
             sleep();
             continue;
         }
+        peak = std::max(peak, admitted + est);
+        est += group_bytes(batch[0], batch.size());
         admitted += est;
-        peak = std::max(peak, admitted);
         n_batches++;
         max_seen_batch = std::max<uint64_t>(max_seen_batch, batch.size());
         idle->batch = std::move(batch);
