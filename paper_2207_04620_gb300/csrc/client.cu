@@ -280,7 +280,7 @@ __device__ __forceinline__ void dec_butterfly(double2 &u, double2 &v, const doub
 // DDec's sum over the shares ([1 + n_parties][n], coefficient form mod q) at coefficient i, centred,
 // placed for the 2n-point transform.  The upper n inputs are zero, so the first stage copies each
 // value to its neighbour.
-__global__ void k_dec_place(double2 *A, const uint64_t *__restrict__ sh, int n_parties, uint64_t q, int log_m)
+__global__ void k_dec_place(double2 *A, const uint64_t *sh, int n_parties, uint64_t q, int log_m)
 {
     after_previous_kernel();
     const int n = 1 << (log_m - 1);
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(256) k_dec_cols(double *re, const double2 *A, 
         re[(size_t)(i / kDecCols) * kDecTile + c0 + i % kDecCols] = __ddiv_rn(s[i].x, scale);
 }
 
-__global__ void k_dec_gather(double *slots, const double *__restrict__ re, const int *__restrict__ e, int count)
+__global__ void k_dec_gather(double *slots, const double *re, const int *__restrict__ e, int count)
 {
     after_previous_kernel();
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < count; j += gridDim.x * blockDim.x) slots[j] = re[e[j]];

@@ -169,8 +169,7 @@ __global__ void __launch_bounds__(128) k_lintrans_mac(const __grid_constant__ Ma
 }
 
 // out_c = a_c * pt  with pt in Montgomery form (pt * 2^64 mod q): one reduction
-__global__ void k_mul_plain(View out, View a, const uint64_t *__restrict__ pt, const PrimeConst *__restrict__ primes,
-                            int n)
+__global__ void k_mul_plain(View out, View a, const uint64_t *pt, const PrimeConst *__restrict__ primes, int n)
 {
     after_previous_kernel();
     const int l = blockIdx.y, bc = blockIdx.z, bi = bc / 2, ci = bc % 2;

@@ -34,7 +34,10 @@ struct Timed {
 
 // Kernels launched by launch(): first of all they wait until the stream's previous kernel has
 // finished and its writes are visible, and then let the next one be scheduled (in this order, so that
-// one kernel at most waits on the SMs)
+// one kernel at most waits on the SMs).  Such a kernel exists while its predecessor still writes, so what
+// a kernel may have written -- every residue and every double -- is read through plain pointers:
+// `const ... * __restrict__` allows the read-only path, which is defined only for data that nobody
+// writes as long as the kernel exists.  Context tables and job lists (written by copies) keep it.
 __device__ __forceinline__ void after_previous_kernel()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
