@@ -694,9 +694,17 @@ hx_status hx_rotate_hoisted(hx_context *ctx, const hx_keyset *ks, const hx_ct *a
     mine(ctx, ks);
     mine(ctx, a);
     Eval ev(*ctx, S(stream));
-    std::vector<int64_t> st(steps, steps + n);
-    const Cts r = ev.rotate_hoisted(a->c, st, *ks);
-    scatter(*ctx, r, outs, S(stream));  // each handle owns its buffer
+    const std::vector<int64_t> st(steps, steps + n);
+    // each handle owns its buffer, and the rotations write there
+    std::vector<Cts> r(n);
+    std::vector<uint64_t *> at(n);
+    for (int i = 0; i < n; i++) {
+        r[i] = ev.alloc(1, 2, a->c.limbs);
+        r[i].scale = a->c.scale;
+        at[i] = r[i].d;
+    }
+    ev.rotate_hoisted_into(at, a->c, ev.hoist_for(a->c, st), st, *ks);
+    for (int i = 0; i < n; i++) outs[i] = wrap(ctx, r[i]);
     return HX_OK;
     HX_END
 }

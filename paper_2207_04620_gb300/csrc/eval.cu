@@ -205,7 +205,7 @@ Cts Eval::ks_finish(const BufPtr &D, const View &dnt, int B, int limbs, const Sw
                   limbs, nd, B);
     ctx.counters[C_KS] += B;
     Cts o = alloc(B, 2, limbs);
-    moddown_add(o.view(N), accv, B, limbs, add, add_mask, one_galois(add_g, B));
+    moddown_add(batch_out(o.view(N), B), accv, B, limbs, add, add_mask, one_galois(add_g, B));
     return o;
 }
 
@@ -219,7 +219,7 @@ void Eval::moddown_ntt(const View &accv, uint64_t *conv, int B, int limbs)
     ntt_inplace(conv, (size_t)limbs * N, 2 * B, iota_vec(0, limbs), iota_vec(0, limbs), false);
 }
 
-void Eval::moddown_add(const View &out, const View &accv, int B, int limbs, const View &add, int add_mask,
+void Eval::moddown_add(const OutTab &out, const View &accv, int B, int limbs, const View &add, int add_mask,
                        const GaloisTab &gal, bool shared)
 {
     const int N = ctx.N;
@@ -290,7 +290,7 @@ Cts Eval::rotate_sum(const Cts &items, const std::vector<int64_t> &steps, const 
     }
     if (!any) return base;
     Cts o = alloc(B, 2, limbs);
-    moddown_add(o.view(N), accv, B, limbs, base.view(N), 3, one_galois(1, B));
+    moddown_add(batch_out(o.view(N), B), accv, B, limbs, base.view(N), 3, one_galois(1, B));
     o.scale = items.scale;
     return o;
 }
@@ -388,7 +388,7 @@ Cts Eval::rotate_each(const Cts &a, const std::vector<int64_t> &steps, const hx_
     View accv{acc.p, (size_t)2 * ext * N, (size_t)ext * N};
     launch_key_ip(lc(), accv, D->p, t.d, t.bstride(N), kt, R, false, false, ctx.n_all, ctx.n_q, K, ctx.alpha, limbs, nd, B);
     Cts o = alloc(a.B, 2, limbs);
-    moddown_add(o.view(N), accv, a.B, limbs, a.view(N), 1, gt);
+    moddown_add(batch_out(o.view(N), B, R), accv, a.B, limbs, a.view(N), 1, gt);
     o.scale = a.scale;
     ctx.counters[C_ROT] += a.B;
     ctx.counters[C_KS] += a.B;
@@ -402,17 +402,33 @@ BufPtr Eval::hoist(const Cts &a)
     return modup(c1, a.B, a.limbs);
 }
 
-void Eval::rotate_hoisted_into(const Cts &out, const Cts &a, const BufPtr &D, const int64_t *steps, int R,
-                               const hx_keyset &keys)
+BufPtr Eval::hoist_for(const Cts &a, const std::vector<int64_t> &steps)
 {
+    for (int64_t k : steps)
+        if (galois_for_step(k, ctx.log_n) != 1) return hoist(a);
+    return BufPtr();
+}
+
+std::vector<uint64_t *> Eval::groups_of(const Cts &c, int R) const
+{
+    std::vector<uint64_t *> p(R);
+    for (int r = 0; r < R; r++) p[r] = c.d + (size_t)r * (c.B / R) * c.bstride(ctx.N);
+    return p;
+}
+
+void Eval::rotate_hoisted_into(const std::vector<uint64_t *> &out, const Cts &a, const BufPtr &D,
+                               const std::vector<int64_t> &steps, const hx_keyset &keys)
+{
+    const int R = (int)steps.size();
     const int N = ctx.N, K = ctx.K, B = a.B, limbs = a.limbs, ext = limbs + K, nd = (limbs + ctx.alpha - 1) / ctx.alpha;
+    OutTab ot;
+    ot.cstride = (size_t)limbs * N;
+    ot.bstride = 2 * ot.cstride;
     const View c1{a.d + a.cstride(N), a.bstride(N), a.cstride(N)};
     const int most = rot_chunk(B, limbs, MAX_ROT);
     for (int r = 0; r < R;) {
-        View o = out.view(N);
-        o.p += (size_t)r * B * o.bstride;
         if (galois_for_step(steps[r], ctx.log_n) == 1) {
-            launch_copy(lc(), o, a.view(N), B, 2, limbs);
+            launch_copy(lc(), View{out[r], ot.bstride, ot.cstride}, a.view(N), B, 2, limbs);
             r++;
             continue;
         }
@@ -425,11 +441,12 @@ void Eval::rotate_hoisted_into(const Cts &out, const Cts &a, const BufPtr &D, co
             if (g == 1) break;
             kt.key[C] = rot_key(keys, g).buf->p;
             kt.g[C] = gt.g[C] = (uint32_t)g;
+            ot.p[C] = out[r + C];
         }
         DevBuf acc((size_t)C * B * 2 * ext * N, s);
         View accv{acc.p, (size_t)2 * ext * N, (size_t)ext * N};
         launch_key_ip(lc(), accv, D->p, c1.p, c1.bstride, kt, C, true, false, ctx.n_all, ctx.n_q, K, ctx.alpha, limbs, nd, B);
-        moddown_add(o, accv, C * B, limbs, a.view(N), 1, gt, true);
+        moddown_add(ot, accv, C * B, limbs, a.view(N), 1, gt, true);
         r += C;
         ctx.counters[C_ROT] += (uint64_t)C * B;
         ctx.counters[C_ROT_HOIST] += (uint64_t)C * B;
@@ -484,12 +501,10 @@ Cts Eval::hoisted_mux(const Cts &a, const BufPtr &D, const std::vector<MuxItem> 
 
 Cts Eval::rotate_hoisted(const Cts &a, const std::vector<int64_t> &steps, const hx_keyset &keys)
 {
-    BufPtr D;
-    for (int64_t k : steps)
-        if (!D && galois_for_step(k, ctx.log_n) != 1) D = hoist(a);
+    const BufPtr D = hoist_for(a, steps);
     Cts out = alloc(a.B * (int)steps.size(), 2, a.limbs);
     out.scale = a.scale;
-    rotate_hoisted_into(out, a, D, steps.data(), (int)steps.size(), keys);
+    rotate_hoisted_into(groups_of(out, (int)steps.size()), a, D, steps, keys);
     return out;
 }
 

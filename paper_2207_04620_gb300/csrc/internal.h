@@ -247,6 +247,20 @@ struct MuxTab {
     const uint64_t *k1[MAX_MUX], *k2[MAX_MUX], *v[MAX_MUX];
     uint32_t g1[MAX_MUX], g2[MAX_MUX];
 };
+// where the entries of one launch's rotations go: those of rotation r follow one another from p[r]
+struct OutTab {
+    uint64_t *p[MAX_ROT];
+    size_t bstride, cstride;
+};
+// all R rotations of `per` entries in one batch
+inline OutTab batch_out(const View &v, int per, int R = 1)
+{
+    OutTab t;
+    t.bstride = v.bstride;
+    t.cstride = v.cstride;
+    for (int r = 0; r < R; r++) t.p[r] = v.p + (size_t)r * per * v.bstride;
+    return t;
+}
 inline GaloisTab one_galois(uint64_t g, int B)
 {
     GaloisTab t;
@@ -267,8 +281,8 @@ void launch_key_ip(const LaunchCtx &c, View acc, const uint64_t *D, const uint64
                    const KeyTab &keys, int R, bool shared, bool sum, int n_all, int n_q, int K, int alpha, int limbs,
                    int ndig, int B, bool accumulate = false);
 // out_c = (acc_c - conv_c) * P^-1, plus add_c[galois(j)] for the components set in add_mask; entry e
-// adds entry e of add, or (shared) entry e % tab.per
-void launch_moddown_final(const LaunchCtx &c, View out, View acc, View conv, const ModDownTable *tab, int B,
+// adds entry e of add, or (shared) entry e % tab.per.  The results go where `out` says by rotation
+void launch_moddown_final(const LaunchCtx &c, const OutTab &out, View acc, View conv, const ModDownTable *tab, int B,
                           int limbs, View add, int add_mask, const GaloisTab &gal, bool shared = false);
 
 // ---- several rings in one launch per key-switching stage (one job = one ring's batch) ----------

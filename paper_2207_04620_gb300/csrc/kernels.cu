@@ -1096,7 +1096,8 @@ __global__ void k_moddown_final_mux(View out, View acc, View conv, const ModDown
 }
 
 // out_c[t] = (acc_c[t] - conv_c[t]) * P^-1 (+ add_c[t][galois(j)] for the components in add_mask)
-__device__ __forceinline__ void moddown_final_body(const Blk &b, View out, View acc, View conv,
+// the entry's two components at out and out + out_cstride
+__device__ __forceinline__ void moddown_final_body(const Blk &b, uint64_t *out, size_t out_cstride, View acc, View conv,
                                                    const ModDownTable *__restrict__ tab,
                                                    const PrimeConst *__restrict__ primes, View add, int add_mask,
                                                    int add_entry, uint64_t g, int log_n)
@@ -1106,7 +1107,7 @@ __device__ __forceinline__ void moddown_final_body(const Blk &b, View out, View 
     const uint64_t q = primes[t].q, w = tab->pinv[t], wsh = tab->pinv_sh[t];
     const uint64_t *a = acc.p + bi * acc.bstride + ci * acc.cstride + (size_t)t * n;
     const uint64_t *cv = conv.p + bi * conv.bstride + ci * conv.cstride + (size_t)t * n;
-    uint64_t *o = out.p + bi * out.bstride + ci * out.cstride + (size_t)t * n;
+    uint64_t *o = out + ci * out_cstride + (size_t)t * n;
     const bool has = (add_mask >> ci) & 1;
     const uint64_t *ap = has ? add.p + add_entry * add.bstride + ci * add.cstride + (size_t)t * n : nullptr;
     for (int j = (b.x * blockDim.x + threadIdx.x) * 2; j < n; j += b.gx * blockDim.x * 2) {
@@ -1130,13 +1131,14 @@ __device__ __forceinline__ void moddown_final_body(const Blk &b, View out, View 
     }
 }
 
-__global__ void k_moddown_final(View out, View acc, View conv, const ModDownTable *__restrict__ tab,
+__global__ void k_moddown_final(const __grid_constant__ OutTab out, View acc, View conv, const ModDownTable *__restrict__ tab,
                                 const PrimeConst *__restrict__ primes, View add, int add_mask,
                                 const __grid_constant__ GaloisTab gal, bool shared, int log_n)
 {
     after_previous_kernel();
-    const int e = blockIdx.z / 2, r = gridDim.z == 2 * gal.per ? 0 : e / gal.per;
-    moddown_final_body(Blk::hw(), out, acc, conv, tab, primes, add, add_mask, shared ? e - r * gal.per : e, gal.g[r], log_n);
+    const int e = blockIdx.z / 2, r = gridDim.z == 2 * gal.per ? 0 : e / gal.per, bi = e - r * gal.per;
+    moddown_final_body(Blk::hw(), out.p[r] + bi * out.bstride, out.cstride, acc, conv, tab, primes, add, add_mask,
+                       shared ? bi : e, gal.g[r], log_n);
 }
 
 // r_i = ([x + floor(q_t/2)]_{q_t} mod q_i - floor(q_t/2) mod q_i) for the lower limbs
@@ -1442,7 +1444,7 @@ __global__ void k_moddown_jobs(const ModDownJob *__restrict__ jobs, int n_jobs)
     after_previous_kernel();
     Blk b;
     const ModDownJob &J = job_of_block(jobs, n_jobs, blockIdx.x, b);
-    moddown_final_body(b, J.out, J.acc, J.conv, J.tab, J.primes, J.add, J.add_mask, b.z / 2, J.g, J.log_n);
+    moddown_final_body(b, J.out.p + (b.z / 2) * J.out.bstride, J.out.cstride, J.acc, J.conv, J.tab, J.primes, J.add, J.add_mask, b.z / 2, J.g, J.log_n);
 }
 
 } // namespace
@@ -1782,7 +1784,7 @@ void launch_moddown_final_mux(const LaunchCtx &c, View out, View acc, View conv,
     post(c);
 }
 
-void launch_moddown_final(const LaunchCtx &c, View out, View acc, View conv, const ModDownTable *tab, int B,
+void launch_moddown_final(const LaunchCtx &c, const OutTab &out, View acc, View conv, const ModDownTable *tab, int B,
                           int limbs, View add, int add_mask, const GaloisTab &gal, bool shared)
 {
     Timed tm_(c, K_MODDOWN, 8.0 * B * 2 * limbs * c.N * ((add_mask ? 4.0 : 3.0)));

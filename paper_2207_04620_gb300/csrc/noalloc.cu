@@ -123,7 +123,7 @@ extern "C" hx_status hx_rotate_noalloc(hx_context *ctx, const hx_keyset *ks, con
         r.n_rows = limbs;
         for (int l = 0; l < limbs; l++) r.src_off[l] = r.dst_off[l] = r.prime[l] = (int16_t)l;
         launch_ntt(lc, r, false);
-        launch_moddown_final(lc, View{out, 2 * limbs * n, limbs * n}, accv, View{conv, 2 * limbs * n, limbs * n},
+        launch_moddown_final(lc, batch_out(View{out, 2 * limbs * n, limbs * n}, 1), accv, View{conv, 2 * limbs * n, limbs * n},
                              ctx->t.moddown + limbs, 1, limbs, vin, 1, one_galois(g, 1));
         ctx->counters[C_ROT] += 1;
         ctx->counters[C_KS] += 1;

@@ -204,8 +204,13 @@ struct Eval {
     Cts rotate_hoisted(const Cts &a, const std::vector<int64_t> &steps, const hx_keyset &keys);
     // hoisting in two steps: the ModUp of c1 once, then any number of rotations
     BufPtr hoist(const Cts &a);
-    void rotate_hoisted_into(const Cts &out, const Cts &a, const BufPtr &D, const int64_t *steps, int R,
-                             const hx_keyset &keys);
+    // out[i]: where a's batch rotated by steps[i] goes, [a.B][2][a.limbs][N]
+    void rotate_hoisted_into(const std::vector<uint64_t *> &out, const Cts &a, const BufPtr &D,
+                             const std::vector<int64_t> &steps, const hx_keyset &keys);
+    // the ModUp of a that the steps need (none if they are all 0 mod N/2)
+    BufPtr hoist_for(const Cts &a, const std::vector<int64_t> &steps);
+    // the starts of c's R equal groups of entries
+    std::vector<uint64_t *> groups_of(const Cts &c, int R) const;
     // rotations of a batch of B at `limbs` limbs (or buffers of `words` each) to run in one launch per
     // stage, at most `most`
     int rot_chunk(int B, int limbs, int most, size_t words = 0);
@@ -229,7 +234,7 @@ struct Eval {
     // ModDown of extended-basis pairs accv ([B][2][limbs+K][N]): the converted special rows in NTT form
     // ([B][2][limbs][N]); and the epilogue with it, plus `add`
     void moddown_ntt(const View &accv, uint64_t *conv, int B, int limbs);
-    void moddown_add(const View &out, const View &accv, int B, int limbs, const View &add, int add_mask,
+    void moddown_add(const OutTab &out, const View &accv, int B, int limbs, const View &add, int add_mask,
                      const GaloisTab &gal, bool shared = false);
     // sum_i Rot(ct_i, k_i) with a single ModDown (terms with k = 0 are added unrotated), ct_i the i-th
     // of steps.size() equal groups of items' entries

@@ -542,7 +542,7 @@ Cts matmul_alg3(Eval &ev, const hx_keyset &ks, const hx_matmul_plan &p, const Ct
         }
         held[par] = evb.alloc(n * B0.B, 2, B0.limbs);
         held[par].scale = B0.scale;
-        evb.rotate_hoisted_into(held[par], B0, DB, bsteps.data(), n, ks);
+        evb.rotate_hoisted_into(evb.groups_of(held[par], n), B0, DB, bsteps, ks);
         HX_CUDA(cudaEventRecord(e[3 + par], ss.s));
         Eval &ec = par ? eva : ev;
         Cts Ak = ec.hoisted_mux(A0, DA, sel, sc, cm, ks);
@@ -608,7 +608,7 @@ Cts matmul_depth2(Eval &ev, const hx_keyset &ks, const hx_matmul_plan &p, const 
         XY = ev.rotate_each(ev.rescale(XY), rb, ks);
         Cts RA = ev.alloc(2 * c * n, 2, A0.limbs);
         RA.scale = A0.scale;
-        ev.rotate_hoisted_into(RA, A0, DA, ra.data(), 2 * c, ks);
+        ev.rotate_hoisted_into(ev.groups_of(RA, 2 * c), A0, DA, ra, ks);
         ev.tensor_sum(acc, RA, XY);
     }
     ev.from_mont(acc);
