@@ -694,14 +694,20 @@ hx_status hx_rotate_hoisted(hx_context *ctx, const hx_keyset *ks, const hx_ct *a
     mine(ctx, ks);
     mine(ctx, a);
     Eval ev(*ctx, S(stream));
-    const std::vector<int64_t> st(steps, steps + n);
-    // each handle owns its buffer, and the rotations write there
+    // each handle owns its buffer, and the rotations write there; an identity step copies the
+    // ciphertext whole (of three components too), as hx_rotate does
     std::vector<Cts> r(n);
-    std::vector<uint64_t *> at(n);
+    std::vector<int64_t> st;
+    std::vector<uint64_t *> at;
     for (int i = 0; i < n; i++) {
+        if (galois_for_step(steps[i], ctx->log_n) == 1) {
+            r[i] = ev.copy(a->c);
+            continue;
+        }
         r[i] = ev.alloc(1, 2, a->c.limbs);
         r[i].scale = a->c.scale;
-        at[i] = r[i].d;
+        st.push_back(steps[i]);
+        at.push_back(r[i].d);
     }
     ev.rotate_hoisted_into(at, a->c, ev.hoist_for(a->c, st), st, *ks);
     for (int i = 0; i < n; i++) outs[i] = wrap(ctx, r[i]);

@@ -63,3 +63,11 @@ def test_outputs_are_held_once(pair):
     assert mempool.peak() - before <= out + group + modup + (4 << 20)
     for h in got + [a]:
         hx.hx_ct_destroy(h)
+
+
+def test_identity_copies_three_components(pair):
+    """A step of 0 mod N/2 copies a product before its relinearisation whole, in hx_rotate and here."""
+    ct = _input(pair, 4, comps=3)
+    a = pair.to_lib(ct)
+    for h in [hx.hx_rotate(pair.ctx, pair.ks, a, 0)] + hx.hx_rotate_hoisted(pair.ctx, pair.ks, a, [0, pair.N // 2]):
+        assert pair.same(h, ct)
