@@ -475,10 +475,13 @@ hx_status hx_aggregate(hx_context *ctx, const hx_ct *const *grads, size_t n_part
  * pending requests of the same signature (context, keys, kind, level and h, or
  * d/k/relu) whenever one of n_lanes CUDA streams is idle and the batch's
  * estimated device memory fits in what hbm_budget_bytes leaves after the
- * registered keys; the lanes run concurrently.  Rotations are the exception to
- * the signature: pending rotations of every context and level form one batch,
- * run as one launch per key-switching stage over all of them (as
- * hx_rotate_jobs).  Each result equals the same request computed alone
+ * registered keys; the lanes run concurrently.  A product's rotations run in
+ * groups whose buffers come from what the budget leaves beside a batch for
+ * every other idle lane (as large as any so far); where that is little the
+ * groups are smaller, so admitted bytes stay within the budget and groups delay
+ * no such batch.  Rotations are the exception to the signature: pending
+ * rotations of every context and level form one batch, run as one launch per
+ * key-switching stage over all of them (as hx_rotate_jobs).  Each result equals the same request computed alone
  * (hx_matmul, hx_sign_approx with its refresh_seed, or hx_rotate).  Submitted
  * ciphertexts stay referenced until their request completes, so the caller
  * may destroy its handles at once. */

@@ -240,7 +240,7 @@ int Eval::rot_chunk(int B, int limbs, int most, size_t words)
 {
     const size_t per = words ? words : (size_t)B * 2 * (limbs + ctx.K) * ctx.N;
     const int grid = std::max(1, 16384 / (B * std::max(2, (limbs + ctx.alpha - 1) / ctx.alpha)));
-    return std::max(1, std::min({most, grid, (int)std::min<size_t>(MAX_ROT, kGroupBytes / 8 / per)}));
+    return std::max(1, std::min({most, grid, (int)std::min<size_t>(MAX_ROT, group / 8 / per)}));
 }
 
 Cts Eval::rotate_sum(const Cts &items, const std::vector<int64_t> &steps, const hx_keyset &keys)
@@ -253,7 +253,9 @@ Cts Eval::rotate_sum(const Cts &items, const std::vector<int64_t> &steps, const 
     HX_CUDA(cudaMemsetAsync(base.d, 0, sizeof(uint64_t) * base.bstride(N) * B, s));
     DevBuf acc((size_t)B * 2 * ext * N, s);
     View accv{acc.p, (size_t)2 * ext * N, (size_t)ext * N};
-    const int most = rot_chunk(B, limbs, MAX_ROT, (size_t)B * nd * ext * N / 2);  // the ModUp digits: up to 256 MB
+    // the ModUp digits take up to twice a group's bytes (sixteen 64x64 pairs 20.8 ms, 21.1 with half of
+    // that), a single digit's with its coefficients and source as much as it
+    const int most = rot_chunk(B, limbs, MAX_ROT, (size_t)B * std::max(nd, 2) * ext * N / 2);
     bool any = false;
     for (int r = 0; r < R;) {
         Cts first = items;

@@ -1,5 +1,6 @@
 // Host runtime: context, keys, batched ciphertext buffers and the evaluator.
 #pragma once
+#include <algorithm>
 #include <map>
 #include <tuple>
 #include <cstdint>
@@ -164,15 +165,23 @@ struct hx_matmul_plan {
 
 namespace hx {
 
+// Bytes of one buffer of a group of rotations or selections (see Eval::rot_chunk), and how many such
+// buffers a product holds at most: two groups of B^(k) and three chains' inner products, converted
+// rows and results in Step 2 (ten; the linear transforms' digits before it count eight), or the depth-2
+// form's two batches, their key switches and ModUp digits (half a buffer each)
+constexpr size_t kGroupBytes = (size_t)128 << 20;
+inline size_t group_buffers(int digits) { return std::max(10, 6 + (digits + 1) / 2); }
+
 // ---- evaluator (eval.cu) ----------------------------------------------------
 struct Eval {
     hx_context &ctx;
     cudaStream_t s;
+    size_t group;  // bytes of a group's buffer, at most; a group holds one rotation at least
     LaunchCtx lc()
     {
         return LaunchCtx{ctx.log_n, ctx.N, &ctx.t, s, &ctx.counters[C_LAUNCH], ctx.profiling ? &ctx.prof : nullptr};
     }
-    Eval(hx_context &c, cudaStream_t st) : ctx(c), s(st) {}
+    Eval(hx_context &c, cudaStream_t st, size_t group_bytes = kGroupBytes) : ctx(c), s(st), group(group_bytes) {}
 
     Cts alloc(int B, int comps, int limbs);
     Cts add(const Cts &a, const Cts &b, bool sub = false);
@@ -258,7 +267,6 @@ struct RotateJob {
 std::vector<Cts> rotate_jobs(const std::vector<RotateJob> &jobs, cudaStream_t s);
 
 Scalars scalars_for(const hx_context &ctx, int limbs, int64_t c);
-constexpr size_t kGroupBytes = (size_t)128 << 20;  // see Eval::rot_chunk
 int64_t const_int(double value, double scale);  // round(value * scale), refused beyond 64 bits
 void upload_plaintext(hx_context &ctx, cudaStream_t s, const int64_t *coeffs, int limbs, uint64_t *dst_mont);
 // the same over p_0..p_{K-1} then q_0..q_{limbs-1} (an extended mask's row order)
@@ -308,7 +316,8 @@ std::vector<int64_t> transpose_rotation_steps(int h, int beta);
 Cts transpose_batch(hx_context &ctx, const hx_keyset &ks, const hx_matmul_plan &plan, const Cts &x, cudaStream_t s);
 std::vector<int64_t> plan_rotation_steps(int h, int beta, int limbs, int t = 0);  // t = 0: t = h
 Cts matmul_batch(hx_context &ctx, const hx_keyset &ks, const hx_matmul_plan &plan, const Cts &A, const Cts &B,
-                 cudaStream_t s, int t = 0);  // t < h: the cut k-sum of the rectangular product
+                 cudaStream_t s, int t = 0,  // t < h: the cut k-sum of the rectangular product
+                 size_t group = kGroupBytes);
 // folds the Step 2 selection masks of plan into copies of the rotation keys of ks
 void bind_plan_keys(hx_context &ctx, hx_matmul_plan &plan, const hx_keyset &ks, cudaStream_t s);
 Cts rmatmul_batch(hx_context &ctx, const hx_keyset &ks, const hx_matmul_plan &plan, const Cts &At, const Cts &B, int t,

@@ -497,7 +497,7 @@ Cts matmul_alg3(Eval &ev, const hx_keyset &ks, const hx_matmul_plan &p, const Ct
     // buffer a stream reads from another is released on its own stream only after that stream
     // has waited for the read; everything is joined before the accumulators are summed.
     SideStream &ss = side_stream(ctx, ev.s);
-    Eval evb(ctx, ss.s), eva(ctx, ss.s2);
+    Eval evb(ctx, ss.s, ev.group), eva(ctx, ss.s2, ev.group);
     cudaEvent_t *e = ss.e;  // 0 fork, 1 B0 ready, 2 A0 ready, 3/4 B^(k) ready, 5/6 B^(k) used, 7 joins
     HX_CUDA(cudaEventRecord(e[0], ev.s));
     HX_CUDA(cudaStreamWaitEvent(ss.s, e[0], 0));
@@ -626,7 +626,7 @@ Cts transpose_batch(hx_context &ctx, const hx_keyset &ks, const hx_matmul_plan &
 }
 
 Cts matmul_batch(hx_context &ctx, const hx_keyset &ks, const hx_matmul_plan &plan, const Cts &A, const Cts &B,
-                 cudaStream_t s, int t)
+                 cudaStream_t s, int t, size_t group)
 {
     t = t ? t : plan.h;
     HX_CHECK(t >= 1 && t <= plan.h, HX_EINVAL, "t must be in [1, h]");
@@ -634,7 +634,7 @@ Cts matmul_batch(hx_context &ctx, const hx_keyset &ks, const hx_matmul_plan &pla
     HX_CHECK(A.comps == 2 && B.comps == 2 && A.B == B.B, HX_EINVAL, "matmul needs two batches of ciphertexts");
     HX_CHECK(A.limbs == plan.limbs && B.limbs == plan.limbs, HX_ELEVEL, "inputs are not at the plan's level");
     HX_CHECK(A.scale == B.scale, HX_ESCALE, "inputs must share the scale");
-    Eval ev(ctx, s);
+    Eval ev(ctx, s, group);
     return plan.alg3 ? matmul_alg3(ev, ks, plan, A, B, t) : matmul_depth2(ev, ks, plan, A, B, t);
 }
 

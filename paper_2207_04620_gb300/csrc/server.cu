@@ -55,7 +55,7 @@ bool same_batch(const Request &x, const Request &y)
                         : (x.d == y.d && x.k == y.k && x.relu == y.relu));
 }
 
-// conservative device-memory estimate of one batch entry (workspace included)
+// conservative device-memory estimate of one batch entry (workspace included, rotations one at a time)
 size_t estimate(const Request &r)
 {
     const size_t ct = (size_t)2 * r.a.limbs * r.ctx->N * 8;
@@ -66,12 +66,15 @@ size_t estimate(const Request &r)
     return r.kind == 0 ? 48 * ct : 24 * ct + (size_t)2 * r.ctx->n_q * r.ctx->N * 8;
 }
 
-// a product's grouped rotations and selections on top of that: some eight buffers over its three
-// streams, each of a group's size
+int digits(const Request &r) { return (r.a.limbs + r.ctx->alpha - 1) / r.ctx->alpha; }
+
+// what a product's groups of rotations take on top of that where nothing limits them
 size_t group_bytes(const Request &r, size_t entries)
 {
     if (r.kind != 0) return 0;
-    return 8 * std::min(kGroupBytes, entries * MAX_MUX * 2 * (r.a.limbs + r.ctx->K) * r.ctx->N * 8);
+    const size_t one = entries * 2 * (r.a.limbs + r.ctx->K) * r.ctx->N * 8, nd = digits(r);
+    const size_t most = std::min<size_t>(MAX_ROT, 2 * (size_t)r.h) * std::max<size_t>(4, nd) / 4;
+    return group_buffers((int)nd) * std::min(kGroupBytes, one * most);
 }
 
 size_t key_bytes(const hx_keyset &ks)
@@ -85,6 +88,7 @@ size_t key_bytes(const hx_keyset &ks)
 
 struct hx_server {
     size_t budget = 0, keys = 0, admitted = 0, peak = 0;
+    size_t largest = 0;  // estimate of the largest request or batch so far
     int max_batch = 16;
     std::mutex mu;
     std::condition_variable cv_dispatch, cv_done;
@@ -97,7 +101,7 @@ struct hx_server {
         cudaStream_t s = nullptr;
         std::thread th;
         std::vector<Request> batch;
-        size_t est = 0;
+        size_t est = 0, group = 0;  // group: bytes of a buffer of the batch's grouped rotations
         bool busy = false;
         std::condition_variable cv;
     };
@@ -148,11 +152,12 @@ void hx_server::run_dispatch()
             else cv_dispatch.wait_until(lk, next);
         };
         Lane *idle = nullptr;
-        for (auto &l : lanes)
-            if (!l->busy) {
-                idle = l.get();
-                break;
-            }
+        size_t others = 0;  // further idle lanes
+        for (auto &l : lanes) {
+            if (l->busy) continue;
+            if (idle) others++;
+            else idle = l.get();
+        }
         if (pending.empty() || !idle || paused) {
             sleep();
             continue;
@@ -165,8 +170,7 @@ void hx_server::run_dispatch()
                 ++it;
                 continue;
             }
-            // beside running batches a group's buffers have to fit too; a batch alone runs as before
-            if (admitted + est + it->est + (admitted ? group_bytes(*it, batch.size() + 1) : 0) > budget) break;
+            if (admitted + est + it->est > budget) break;
             est += it->est;
             batch.push_back(std::move(*it));
             it = pending.erase(it);
@@ -175,13 +179,20 @@ void hx_server::run_dispatch()
             sleep();
             continue;
         }
-        peak = std::max(peak, admitted + est);
-        est += group_bytes(batch[0], batch.size());
+        // Groups take what the budget leaves once every other idle lane could still run a batch as large
+        // as any so far; with less than that they shrink, down to one rotation at a time, which the
+        // estimate covers.  So grouping delays no batch that would fit without it.
+        largest = std::max(largest, est);
+        const size_t left = budget - admitted - est, reserved = others * largest;
+        const size_t groups = std::min(group_bytes(batch[0], batch.size()), left > reserved ? left - reserved : 0);
+        est += groups;
         admitted += est;
+        peak = std::max(peak, admitted);
         n_batches++;
         max_seen_batch = std::max<uint64_t>(max_seen_batch, batch.size());
         idle->batch = std::move(batch);
         idle->est = est;
+        idle->group = groups / group_buffers(digits(idle->batch[0]));
         idle->busy = true;
         n_inflight++;
         max_busy = std::max(max_busy, n_inflight);
@@ -197,6 +208,7 @@ void hx_server::run_lane(Lane &L)
         L.cv.wait(lk, [&] { return stop || L.busy; });
         if (stop && !L.busy) return;
         std::vector<Request> batch = std::move(L.batch);
+        const size_t group = L.group;
         lk.unlock();
         const Request &r0 = batch[0];
         hx_context &ctx = *r0.ctx;
@@ -231,7 +243,7 @@ void hx_server::run_lane(Lane &L)
                     for (int i = 0; i < B; i++) pack(Bc, i, batch[i].b);
                     launch_copies(ev.lc(), copies, Bc.limbs * N);
                     plan = cached_plan(ctx, r0.h, r0.a.limbs);  // held until the lane's stream is done
-                    out = matmul_batch(ctx, *r0.ks, *plan, A, Bc, L.s);
+                    out = matmul_batch(ctx, *r0.ks, *plan, A, Bc, L.s, 0, group);
                 } else {
                     std::vector<uint64_t> seeds;
                     for (auto &r : batch) seeds.push_back(r.seed);
@@ -328,6 +340,7 @@ static hx_status submit(hx_server *sv, Request &&r, uint64_t *id)
         set_error("request needs more device memory than the budget allows");
         return HX_ENOMEM;
     }
+    sv->largest = std::max(sv->largest, r.est);
     r.id = sv->next_id++;
     r.t0 = Clock::now();
     *id = r.id;

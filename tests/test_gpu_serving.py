@@ -118,6 +118,61 @@ def test_admission_by_budget_and_rejection(setup):
     hx.hx_server_destroy(tiny)
 
 
+@pytest.mark.parametrize("limbs,h", [(5, 8), (3, 16)])  # Alg. 3; the depth-2 form
+def test_groups_of_rotations_fit_the_budget(setup, limbs, h):
+    """A product's grouped rotations are part of what is admitted: none where the budget holds the
+    estimate alone, smaller ones where it leaves little, and the peak counts them.  The result is that
+    of the product alone at any of these."""
+    ctx, ks, s = setup
+    beta = s // (h * h)
+    a = hx.hx_encrypt(ctx, ks, workloads.pack(workloads.matrices(5, beta, h), h, beta), limbs, 6)
+    b = hx.hx_encrypt(ctx, ks, workloads.pack(workloads.matrices(6, beta, h), h, beta), limbs, 7)
+    alone = hx.hx_matmul(ctx, ks, a, b, h)
+    want = hx.hx_ct_export(ctx, alone)
+    one = 48 * 2 * limbs * (2 * s) * 8
+    for budget in (one, one + one // 2, 2 * one + one // 2, 64 << 30):
+        sv = hx.hx_server_create(budget, 1, 1)
+        rid = hx.hx_server_submit_matmul(sv, ctx, ks, a, b, h)
+        res, st, _ = _collect(sv, 1)[rid]
+        peak = hx.hx_server_stats(sv)["peak_admitted_bytes"]
+        hx.hx_server_destroy(sv)
+        assert st == 0 and np.array_equal(hx.hx_ct_export(ctx, res), want)
+        hx.hx_ct_destroy(res)
+        if budget < 3 * one:
+            assert peak == budget                  # what the estimate leaves is the groups'
+        else:
+            assert one < peak <= one + 20 * (128 << 20)
+    for x in (a, b, alone):
+        hx.hx_ct_destroy(x)
+    hx.hx_context_set_plan_cache(ctx, 1)  # the depth-2 plan is this test's own
+    hx.hx_context_set_plan_cache(ctx, 0)
+
+
+def test_groups_leave_room_for_the_other_lanes(setup):
+    """Two products of different size in a budget of two and a half estimates run side by side: the
+    first one's groups do not take the second one's room."""
+    ctx, ks, s = setup
+    one = 48 * 2 * 5 * (2 * s) * 8
+    cts = []
+    for i, h in enumerate((16, 8)):
+        beta = s // (h * h)
+        cts += [(hx.hx_encrypt(ctx, ks, workloads.pack(workloads.matrices(7 + i, beta, h), h, beta), 5, 8 + i),
+                 hx.hx_encrypt(ctx, ks, workloads.pack(workloads.matrices(9 + i, beta, h), h, beta), 5, 10 + i), h)]
+        hx.hx_ct_destroy(hx.hx_matmul(ctx, ks, *cts[-1]))  # its plan is built before the lanes need it
+    sv = hx.hx_server_create(2 * one + one // 2, 2, 4)
+    hx.hx_server_pause(sv, True)
+    ids = [hx.hx_server_submit_matmul(sv, ctx, ks, *c) for c in cts]
+    hx.hx_server_pause(sv, False)
+    got = _collect(sv, 2)
+    stats = hx.hx_server_stats(sv)
+    hx.hx_server_destroy(sv)
+    assert all(got[i][1] == 0 for i in ids)
+    assert stats["max_busy_lanes"] == 2 and 2 * one <= stats["peak_admitted_bytes"] <= 2 * one + one // 2
+    for i, (a, b, _) in zip(ids, cts):
+        for x in (a, b, got[i][0]):
+            hx.hx_ct_destroy(x)
+
+
 def test_deadline_expires_queued_requests_only(setup):
     ctx, ks, s = setup
     h, beta = 8, s // 64
