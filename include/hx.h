@@ -376,13 +376,16 @@ hx_status hx_transpose(hx_context *ctx, const hx_keyset *ks, const hx_matmul_pla
  * (its temporary allocations become graph memory nodes) over persistent input
  * and output buffers.  hx_matmul_exec_run copies the inputs in, launches the
  * graph on `stream` and returns fresh output handles; the residues equal
- * hx_matmul_batch's.  Runs of one executor must not overlap. */
+ * hx_matmul_batch's.  Runs of one executor must not overlap.  If the device has
+ * no room for the product's groups of rotations at the first run, the product is
+ * captured again with smaller ones (hx_matmul_batch, hx_transpose and
+ * hx_rotate_hoisted then run one rotation at a time). */
 typedef struct hx_matmul_exec hx_matmul_exec;
 hx_status hx_matmul_exec_create(hx_context *ctx, const hx_keyset *ks, const hx_matmul_plan *plan, size_t count,
                                 double scale, hx_matmul_exec **out);
 hx_status hx_matmul_exec_run(hx_matmul_exec *ex, const hx_ct *const *A, const hx_ct *const *B, hx_ct **out,
                              void *stream);
-/* kernel launches one replay contains */
+/* kernel launches one replay contains (more after a first run on a nearly full device) */
 int64_t hx_matmul_exec_launches(const hx_matmul_exec *ex);
 void hx_matmul_exec_destroy(hx_matmul_exec *ex);
 /* The same replay with host buffers: copies host_A and host_B

@@ -709,7 +709,8 @@ hx_status hx_rotate_hoisted(hx_context *ctx, const hx_keyset *ks, const hx_ct *a
         st.push_back(steps[i]);
         at.push_back(r[i].d);
     }
-    ev.rotate_hoisted_into(at, a->c, ev.hoist_for(a->c, st), st, *ks);
+    const BufPtr D = ev.hoist_for(a->c, st);
+    with_groups(ev.s, ev.group, [&](size_t group) { Eval(*ctx, ev.s, group).rotate_hoisted_into(at, a->c, D, st, *ks); });
     for (int i = 0; i < n; i++) outs[i] = wrap(ctx, r[i]);
     return HX_OK;
     HX_END
@@ -995,6 +996,66 @@ hx_status hx_transpose(hx_context *ctx, const hx_keyset *ks, const hx_matmul_pla
     HX_END
 }
 
+// captures ex's product with groups of at most `group` bytes a buffer
+static void capture_product(hx_matmul_exec &ex, size_t group)
+{
+    hx_context &ctx = *ex.ctx;
+    const size_t N = ctx.N;
+    const uint64_t l0 = ctx.counters[C_LAUNCH];
+    uint64_t saved[C_NUM];
+    for (int i = 0; i < C_NUM; i++) saved[i] = ctx.counters[i];
+    const bool prof = ctx.profiling;
+    ctx.profiling = false;
+    cudaGraph_t graph = nullptr;
+    HX_CUDA(cudaStreamBeginCapture(ex.cap, cudaStreamCaptureModeThreadLocal));
+    try {
+        Cts r = matmul_batch(ctx, *ex.ks, *ex.plan, ex.A, ex.B, ex.cap, 0, group);
+        HX_CHECK(r.limbs == ex.out.limbs, HX_EINVAL, "unexpected output level");
+        ex.out.scale = r.scale;
+        HX_CUDA(cudaMemcpyAsync(ex.out.d, r.d, sizeof(uint64_t) * r.bstride(N) * ex.count, cudaMemcpyDeviceToDevice,
+                                ex.cap));
+    } catch (...) {
+        cudaStreamEndCapture(ex.cap, &graph);
+        if (graph) cudaGraphDestroy(graph);
+        ctx.profiling = prof;
+        throw;
+    }
+    HX_CUDA(cudaStreamEndCapture(ex.cap, &graph));
+    ctx.profiling = prof;
+    ex.launches = (int64_t)(ctx.counters[C_LAUNCH] - l0);
+    for (int i = 0; i < C_NUM; i++) ctx.counters[i] = saved[i];  // a capture executes nothing
+    cudaGraphExec_t exec = nullptr;
+    cudaError_t e = cudaGraphInstantiate(&exec, graph, 0);
+    cudaGraphDestroy(graph);
+    HX_CUDA(e);
+    if (ex.exec) cudaGraphExecDestroy(ex.exec);
+    ex.exec = exec;
+    ex.group = group;
+}
+
+// One replay on s.  A graph's memory is mapped by its first launch, and a launch that fails for lack of
+// it leaves what it had mapped unusable.  So the groups are measured against what the device has left
+// before that launch, and captured again as large as fits: one rotation at a time needs what the
+// product needed without groups (five 32x32 products of N = 2^13: 224 MB, 864 in full groups).
+static void launch_product(hx_matmul_exec &ex, cudaStream_t s)
+{
+    if (!ex.launched) {
+        hx_context &ctx = *ex.ctx;
+        size_t free = 0, total = 0;
+        uint64_t reserved = 0, used = 0;
+        HX_CUDA(cudaMemGetInfo(&free, &total));
+        HX_CUDA(cudaDeviceGetGraphMemAttribute(ctx.device, cudaGraphMemAttrReservedMemCurrent, &reserved));
+        HX_CUDA(cudaDeviceGetGraphMemAttribute(ctx.device, cudaGraphMemAttrUsedMemCurrent, &used));
+        const size_t left = free + (size_t)(reserved - used), one = product_bytes(ctx, ex.plan->limbs, ex.count),
+                     buffers = group_buffers(product_digits(ctx, ex.plan->limbs));
+        const size_t group = left > one ? (left - one) / buffers : 0;
+        if (group < std::min(ex.group, group_most(ctx, ex.plan->limbs, ex.plan->h, ex.count))) capture_product(ex, group);
+        ex.launched = true;
+    }
+    HX_CUDA(cudaGraphLaunch(ex.exec, s));
+    ex.ctx->counters[C_LAUNCH] += ex.launches;
+}
+
 hx_status hx_matmul_exec_create(hx_context *ctx, const hx_keyset *ks, const hx_matmul_plan *plan, size_t count,
                                 double scale, hx_matmul_exec **out)
 {
@@ -1027,32 +1088,7 @@ hx_status hx_matmul_exec_create(hx_context *ctx, const hx_keyset *ks, const hx_m
     HX_CUDA(cudaDeviceSynchronize());
     HX_CUDA(cudaStreamCreateWithFlags(&ex->cap, cudaStreamNonBlocking));
     side_stream(*ctx, ex->cap);  // the schedule's side stream exists before the capture starts
-    const uint64_t l0 = ctx->counters[C_LAUNCH];
-    uint64_t saved[C_NUM];
-    for (int i = 0; i < C_NUM; i++) saved[i] = ctx->counters[i];
-    const bool prof = ctx->profiling;
-    ctx->profiling = false;
-    cudaGraph_t graph = nullptr;
-    HX_CUDA(cudaStreamBeginCapture(ex->cap, cudaStreamCaptureModeThreadLocal));
-    try {
-        Cts r = matmul_batch(*ctx, *ks, *plan, ex->A, ex->B, ex->cap);
-        HX_CHECK(r.limbs == ex->out.limbs, HX_EINVAL, "unexpected output level");
-        ex->out.scale = r.scale;
-        HX_CUDA(cudaMemcpyAsync(ex->out.d, r.d, sizeof(uint64_t) * r.bstride(N) * count, cudaMemcpyDeviceToDevice,
-                                ex->cap));
-    } catch (...) {
-        cudaStreamEndCapture(ex->cap, &graph);
-        if (graph) cudaGraphDestroy(graph);
-        ctx->profiling = prof;
-        throw;
-    }
-    HX_CUDA(cudaStreamEndCapture(ex->cap, &graph));
-    ctx->profiling = prof;
-    ex->launches = (int64_t)(ctx->counters[C_LAUNCH] - l0);
-    for (int i = 0; i < C_NUM; i++) ctx->counters[i] = saved[i];  // a capture executes nothing
-    cudaError_t e = cudaGraphInstantiate(&ex->exec, graph, 0);
-    cudaGraphDestroy(graph);
-    HX_CUDA(e);
+    capture_product(*ex, kGroupBytes);
     *out = ex.release();
     return HX_OK;
     HX_END
@@ -1083,8 +1119,7 @@ hx_status hx_matmul_exec_run(hx_matmul_exec *ex, const hx_ct *const *A, const hx
             copies.push_back({ex->B.d + i * ex->B.bstride(N) + c * ex->B.cstride(N), B[i]->c.d + c * B[i]->c.cstride(N)});
         }
     launch_copies(Eval(ctx, s).lc(), copies, ex->A.limbs * N);
-    HX_CUDA(cudaGraphLaunch(ex->exec, s));
-    ctx.counters[C_LAUNCH] += ex->launches;
+    launch_product(*ex, s);
     scatter(ctx, ex->out, out, s);
     return HX_OK;
     HX_END
@@ -1102,8 +1137,7 @@ hx_status hx_matmul_exec_run_host(hx_matmul_exec *ex, const uint64_t *host_A, co
                             s));
     HX_CUDA(cudaMemcpyAsync(ex->B.d, host_B, sizeof(uint64_t) * ex->B.bstride(N) * ex->count, cudaMemcpyHostToDevice,
                             s));
-    HX_CUDA(cudaGraphLaunch(ex->exec, s));
-    ex->ctx->counters[C_LAUNCH] += ex->launches;
+    launch_product(*ex, s);
     HX_CUDA(cudaMemcpyAsync(host_out, ex->out.d, sizeof(uint64_t) * ex->out.bstride(N) * ex->count,
                             cudaMemcpyDeviceToHost, s));
     return HX_OK;

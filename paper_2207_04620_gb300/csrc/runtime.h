@@ -133,6 +133,8 @@ struct hx_matmul_exec {
     size_t count = 0;
     hx::Cts A, B, out;
     cudaGraphExec_t exec = nullptr;
+    size_t group = 0;  // bytes of a group's buffer in the captured product
+    bool launched = false;
     cudaStream_t cap = nullptr;
     int64_t launches = 0;
 };
@@ -171,6 +173,15 @@ namespace hx {
 // form's two batches, their key switches and ModUp digits (half a buffer each)
 constexpr size_t kGroupBytes = (size_t)128 << 20;
 inline size_t group_buffers(int digits) { return std::max(10, 6 + (digits + 1) / 2); }
+// A product's device memory, by its inputs' limbs: conservatively that of `count` pairs with rotations
+// one at a time, and the bytes a group's buffer has at most where nothing limits it
+inline int product_digits(const hx_context &c, int limbs) { return (limbs + c.alpha - 1) / c.alpha; }
+inline size_t product_bytes(const hx_context &c, int limbs, size_t count) { return 96 * count * limbs * c.N * 8; }
+inline size_t group_most(const hx_context &c, int limbs, int h, size_t count)
+{
+    const size_t one = count * 2 * (limbs + c.K) * c.N * 8;
+    return std::min(kGroupBytes, one * std::min(MAX_ROT, 2 * h) * std::max(4, product_digits(c, limbs)) / 4);
+}
 
 // ---- evaluator (eval.cu) ----------------------------------------------------
 struct Eval {
@@ -255,6 +266,23 @@ struct Eval {
                  bool inverse);
     const SwitchKey &rot_key(const hx_keyset &ks, uint64_t g);
 };
+
+// f(group) on stream s; where the device has no room for groups of that size, again with one rotation
+// at a time, so that a nearly full device still runs what it held without groups.  f gives back what it
+// took and leaves no work on other streams when it throws; the operations it had run stay counted.
+template <class F> auto with_groups(cudaStream_t s, size_t group, F f) -> decltype(f(group))
+{
+    try {
+        return f(group);
+    } catch (const Error &e) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (e.code != HX_ENOMEM || group == 0 || cudaStreamIsCapturing(s, &capture) != cudaSuccess ||
+            capture != cudaStreamCaptureStatusNone)
+            throw;
+    }
+    HX_CUDA(cudaStreamSynchronize(s));  // what the attempt freed is free for every size again
+    return f(0);
+}
 
 // one rotation of a several-ring call: a ciphertext batch of its context, by `step` slots
 struct RotateJob {

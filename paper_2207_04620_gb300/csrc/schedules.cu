@@ -486,6 +486,18 @@ Cts lintrans(Eval &ev, const hx_keyset &ks, const Cts &ct, int lmin, int lmax, i
     return ev.rotate_sum(inner, giant, ks);
 }
 
+// Declared after the buffers that several streams use: when an exception is thrown, their work ends
+// before the buffers are released, each on its own stream only.
+struct JoinOnThrow {
+    cudaStream_t s[3];
+    int before = std::uncaught_exceptions();
+    ~JoinOnThrow()
+    {
+        if (std::uncaught_exceptions() > before)
+            for (cudaStream_t x : s) cudaStreamSynchronize(x);
+    }
+};
+
 // t < h: only the terms k < t of Steps 2-3 (the rectangular product, App. D)
 Cts matmul_alg3(Eval &ev, const hx_keyset &ks, const hx_matmul_plan &p, const Cts &A, const Cts &B, int t)
 {
@@ -498,32 +510,35 @@ Cts matmul_alg3(Eval &ev, const hx_keyset &ks, const hx_matmul_plan &p, const Ct
     // has waited for the read; everything is joined before the accumulators are summed.
     SideStream &ss = side_stream(ctx, ev.s);
     Eval evb(ctx, ss.s, ev.group), eva(ctx, ss.s2, ev.group);
+    Cts A0, B0, acc, acc_odd;
+    BufPtr DA, DB;
+    Cts held[2];  // B^(k) stays alive until its consumer's use is ordered before the release
+    const JoinOnThrow join{{ev.s, ss.s, ss.s2}};
     cudaEvent_t *e = ss.e;  // 0 fork, 1 B0 ready, 2 A0 ready, 3/4 B^(k) ready, 5/6 B^(k) used, 7 joins
     HX_CUDA(cudaEventRecord(e[0], ev.s));
     HX_CUDA(cudaStreamWaitEvent(ss.s, e[0], 0));
     HX_CUDA(cudaStreamWaitEvent(ss.s2, e[0], 0));
-    Cts B0 = evb.rescale(lintrans(evb, ks, B, 0, h - 1, h, p, 1));
-    BufPtr DB = evb.hoist(B0);  // one ModUp serves every B^(k)
+    B0 = evb.rescale(lintrans(evb, ks, B, 0, h - 1, h, p, 1));
+    DB = evb.hoist(B0);  // one ModUp serves every B^(k)
     HX_CUDA(cudaEventRecord(e[1], ss.s));
-    Cts A0 = ev.rescale(lintrans(ev, ks, A, -h + 1, h - 1, 1, p, 0));
-    BufPtr DA = ev.hoist(A0);
+    A0 = ev.rescale(lintrans(ev, ks, A, -h + 1, h - 1, 1, p, 0));
+    DA = ev.hoist(A0);
     // Step 2 (App. B multiplexer after hoisting): A^(k) = v_k . Rot(A0, k) + (1 - v_k) . Rot(A0, k-h),
     // all rotations of A0 from one ModUp, the selection before a single ModDown per k.  A^(k)
     // keeps the mask scale (no rescale per k); B^(k) = Rot(B0, h*k) stays at the same level.
     const uint64_t cm = mask_scale_int(ctx);  // the masks' scale as an integer: c of the multiplexer
-    Cts acc_odd = ev.alloc(A0.B, 3, A0.limbs);  // the odd-k accumulator, zero, owned by the main stream
+    acc_odd = ev.alloc(A0.B, 3, A0.limbs);  // the odd-k accumulator, zero, owned by the main stream
     HX_CUDA(cudaMemsetAsync(acc_odd.d, 0, sizeof(uint64_t) * acc_odd.bstride(ctx.N) * acc_odd.B, ev.s));
     HX_CUDA(cudaEventRecord(e[2], ev.s));
     HX_CUDA(cudaStreamWaitEvent(ss.s2, e[2], 0));
     HX_CUDA(cudaStreamWaitEvent(ev.s, e[1], 0));
     // Step 3's products are summed in Montgomery form (each times 2^-64) and scaled back once
-    Cts acc = ev.tensor(ev.mul_int(A0, (int64_t)cm, A0.scale * (double)cm), B0, true);
+    acc = ev.tensor(ev.mul_int(A0, (int64_t)cm, A0.scale * (double)cm), B0, true);
     acc_odd.scale = acc.scale;
     HX_CUDA(cudaEventRecord(e[5], ev.s));
     HX_CUDA(cudaStreamWaitEvent(ss.s, e[5], 0));  // B0's read by the main stream comes before its release
     // the k are taken in groups of C: a group's rotations, selections and products share a launch per
     // stage; groups alternate between the two streams and accumulators
-    Cts held[2];  // B^(k) stays alive until its consumer's use is ordered before the release
     const int C = ev.rot_chunk(A0.B, A0.limbs, MAX_MUX);
     for (int k0 = 1, grp = 1; k0 < t; k0 += C, grp++) {
         const int par = grp & 1, n = std::min(C, t - k0);
@@ -621,8 +636,10 @@ Cts transpose_batch(hx_context &ctx, const hx_keyset &ks, const hx_matmul_plan &
 {
     HX_CHECK(plan.kind == 1, HX_EINVAL, "not a transpose plan");
     HX_CHECK(x.comps == 2 && x.limbs == plan.limbs, HX_ELEVEL, "input is not at the plan's level");
-    Eval ev(ctx, s);
-    return ev.rescale(lintrans(ev, ks, x, -plan.h + 1, plan.h - 1, plan.h - 1, plan, 3));
+    return with_groups(s, kGroupBytes, [&](size_t group) {
+        Eval ev(ctx, s, group);
+        return ev.rescale(lintrans(ev, ks, x, -plan.h + 1, plan.h - 1, plan.h - 1, plan, 3));
+    });
 }
 
 Cts matmul_batch(hx_context &ctx, const hx_keyset &ks, const hx_matmul_plan &plan, const Cts &A, const Cts &B,
@@ -634,8 +651,10 @@ Cts matmul_batch(hx_context &ctx, const hx_keyset &ks, const hx_matmul_plan &pla
     HX_CHECK(A.comps == 2 && B.comps == 2 && A.B == B.B, HX_EINVAL, "matmul needs two batches of ciphertexts");
     HX_CHECK(A.limbs == plan.limbs && B.limbs == plan.limbs, HX_ELEVEL, "inputs are not at the plan's level");
     HX_CHECK(A.scale == B.scale, HX_ESCALE, "inputs must share the scale");
-    Eval ev(ctx, s, group);
-    return plan.alg3 ? matmul_alg3(ev, ks, plan, A, B, t) : matmul_depth2(ev, ks, plan, A, B, t);
+    return with_groups(s, group, [&](size_t bytes) {
+        Eval ev(ctx, s, bytes);
+        return plan.alg3 ? matmul_alg3(ev, ks, plan, A, B, t) : matmul_depth2(ev, ks, plan, A, B, t);
+    });
 }
 
 void bind_plan_keys(hx_context &ctx, hx_matmul_plan &plan, const hx_keyset &ks, cudaStream_t s)

@@ -63,18 +63,14 @@ size_t estimate(const Request &r)
         const size_t ext = (size_t)r.a.limbs + r.ctx->K, nd = ((size_t)r.a.limbs + r.ctx->alpha - 1) / r.ctx->alpha;
         return ((size_t)4 * r.a.limbs + (nd + 2) * ext + 2 * (size_t)r.a.limbs) * r.ctx->N * 8 + ct;
     }
-    return r.kind == 0 ? 48 * ct : 24 * ct + (size_t)2 * r.ctx->n_q * r.ctx->N * 8;
+    return r.kind == 0 ? product_bytes(*r.ctx, r.a.limbs, 1) : 24 * ct + (size_t)2 * r.ctx->n_q * r.ctx->N * 8;
 }
-
-int digits(const Request &r) { return (r.a.limbs + r.ctx->alpha - 1) / r.ctx->alpha; }
 
 // what a product's groups of rotations take on top of that where nothing limits them
 size_t group_bytes(const Request &r, size_t entries)
 {
-    if (r.kind != 0) return 0;
-    const size_t one = entries * 2 * (r.a.limbs + r.ctx->K) * r.ctx->N * 8, nd = digits(r);
-    const size_t most = std::min<size_t>(MAX_ROT, 2 * (size_t)r.h) * std::max<size_t>(4, nd) / 4;
-    return group_buffers((int)nd) * std::min(kGroupBytes, one * most);
+    if (r.kind != 0 || r.h < 1 || r.h > r.ctx->N) return 0;  // no such product: the lane says so
+    return group_buffers(product_digits(*r.ctx, r.a.limbs)) * group_most(*r.ctx, r.a.limbs, r.h, entries);
 }
 
 size_t key_bytes(const hx_keyset &ks)
@@ -192,7 +188,7 @@ void hx_server::run_dispatch()
         max_seen_batch = std::max<uint64_t>(max_seen_batch, batch.size());
         idle->batch = std::move(batch);
         idle->est = est;
-        idle->group = groups / group_buffers(digits(idle->batch[0]));
+        idle->group = groups / group_buffers(product_digits(*idle->batch[0].ctx, idle->batch[0].a.limbs));
         idle->busy = true;
         n_inflight++;
         max_busy = std::max(max_busy, n_inflight);
