@@ -98,7 +98,7 @@ Cts Eval::tensor(const Cts &a, const Cts &b, bool mont)
     HX_CHECK(a.B == b.B && a.limbs == b.limbs && a.comps == 2 && b.comps == 2, HX_ESCALE, "tensor operands differ");
     Cts o = alloc(a.B, 3, a.limbs);
     o.scale = a.scale * b.scale;
-    launch_tensor(lc(), o.view(ctx.N), a.view(ctx.N), b.view(ctx.N), a.B, a.limbs, false, mont);
+    launch_tensor(lc(), o.view(ctx.N), a.view(ctx.N), b.view(ctx.N), a.B, a.limbs, mont);
     ctx.counters[C_MULCT] += a.B;
     return o;
 }

@@ -228,8 +228,7 @@ void launch_mul_plain(const LaunchCtx &c, View out, View a, const uint64_t *pt_m
 void launch_mul_scalar(const LaunchCtx &c, View out, View a, const Scalars &sc, int B, int comps, int limbs);
 void launch_add_scalar_c0(const LaunchCtx &c, View out, View a, const Scalars &sc, int B, int limbs);
 // mont: the products left times 2^-64 (Montgomery reductions), to be scaled back once after summing
-void launch_tensor(const LaunchCtx &c, View out3, View a, View b, int B, int limbs, bool accumulate,
-                   bool mont = false);
+void launch_tensor(const LaunchCtx &c, View out3, View a, View b, int B, int limbs, bool mont = false);
 // Rotations of one launch, by their place in the batch: entry e of R * per entries belongs to
 // rotation e / per, so a schedule's rotations by different amounts share a launch per stage
 constexpr int MAX_ROT = 32;
@@ -293,7 +292,6 @@ struct AutomorphismJob {
     View out, in;
     uint64_t g;
     int comps, log_n;
-    const PrimeConst *primes;
     int gx, gy, gz;
     long long block0;
 };
@@ -382,7 +380,7 @@ void alu_calibrate(const LaunchCtx &c, uint64_t q, double *shoup_per_s, double *
 // their ModDown epilogue (v's chain rows start K rows in)
 void launch_moddown_final_mux(const LaunchCtx &c, View out, View acc, View conv, const ModDownTable *tab, int C, int B,
                               int K, int limbs, View src, const MuxTab &mux, const Scalars &cs);
-// out (+)= sum over i < C of a[i * B + b] x b[i * B + b] (3 components), each product times 2^-64
+// out += sum over i < C of a[i * B + b] x b[i * B + b] (3 components), each product times 2^-64
 void launch_tensor_sum(const LaunchCtx &c, View out3, View a, View b, int C, int B, int limbs);
 // prefix sums P_m = sum_{l < m} T_l (T_0 = mask_0 b, T_l = mask_l rb[(l-1) B + b]): out[(h - m) B + b] = P_m
 struct PrefixTab {

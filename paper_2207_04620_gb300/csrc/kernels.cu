@@ -238,7 +238,7 @@ __device__ __forceinline__ void tensor_one(uint64_t a0, uint64_t a1, uint64_t b0
     }
 }
 
-__global__ void k_tensor(View out, View a, View b, const PrimeConst *__restrict__ primes, int n, bool acc, bool mont)
+__global__ void k_tensor(View out, View a, View b, const PrimeConst *__restrict__ primes, int n, bool mont)
 {
     after_previous_kernel();
     const int l = blockIdx.y, bi = blockIdx.z;
@@ -253,23 +253,13 @@ __global__ void k_tensor(View out, View a, View b, const PrimeConst *__restrict_
         uint64_t x0, x1, x2, y0, y1, y2;
         tensor_one(a0.x, a1.x, b0.x, b1.x, P, mont, x0, x1, x2);
         tensor_one(a0.y, a1.y, b0.y, b1.y, P, mont, y0, y1, y2);
-        ulonglong2 r0 = make_ulonglong2(x0, y0), r1 = make_ulonglong2(x1, y1), r2 = make_ulonglong2(x2, y2);
-        ulonglong2 *o0 = reinterpret_cast<ulonglong2 *>(out.p + lo + j);
-        ulonglong2 *o1 = reinterpret_cast<ulonglong2 *>(out.p + lo + out.cstride + j);
-        ulonglong2 *o2 = reinterpret_cast<ulonglong2 *>(out.p + lo + 2 * out.cstride + j);
-        if (acc) {
-            const ulonglong2 x0 = *o0, x1 = *o1, x2 = *o2;
-            r0.x = addmod(r0.x, x0.x, P.q), r0.y = addmod(r0.y, x0.y, P.q);
-            r1.x = addmod(r1.x, x1.x, P.q), r1.y = addmod(r1.y, x1.y, P.q);
-            r2.x = addmod(r2.x, x2.x, P.q), r2.y = addmod(r2.y, x2.y, P.q);
-        }
-        *o0 = r0;
-        *o1 = r1;
-        *o2 = r2;
+        *reinterpret_cast<ulonglong2 *>(out.p + lo + j) = make_ulonglong2(x0, y0);
+        *reinterpret_cast<ulonglong2 *>(out.p + lo + out.cstride + j) = make_ulonglong2(x1, y1);
+        *reinterpret_cast<ulonglong2 *>(out.p + lo + 2 * out.cstride + j) = make_ulonglong2(x2, y2);
     }
 }
 
-// out (+)= sum_i a_i x b_i over C pairs of entries B apart, the products left times 2^-64
+// out += sum_i a_i x b_i over C pairs of entries B apart, the products left times 2^-64
 __global__ void k_tensor_sum(View out, View a, View b, const PrimeConst *__restrict__ primes, int C, int B, int n)
 {
     after_previous_kernel();
@@ -1537,11 +1527,11 @@ void launch_add_scalar_c0(const LaunchCtx &c, View out, View a, const Scalars &s
     post(c);
 }
 
-void launch_tensor(const LaunchCtx &c, View out3, View a, View b, int B, int limbs, bool accumulate, bool mont)
+void launch_tensor(const LaunchCtx &c, View out3, View a, View b, int B, int limbs, bool mont)
 {
-    Timed tm_(c, K_TENSOR, 8.0 * B * limbs * c.N * (accumulate ? 10 : 7));
+    Timed tm_(c, K_TENSOR, 8.0 * B * limbs * c.N * 7);
     dim3 grid(ew_blocks(c.N, 2), limbs, B);
-    launch(c.stream, k_tensor, grid, 256, 0, out3, a, b, c.t->primes, c.N, accumulate, mont);
+    launch(c.stream, k_tensor, grid, 256, 0, out3, a, b, c.t->primes, c.N, mont);
     post(c);
 }
 

@@ -122,7 +122,7 @@ std::vector<Cts> rotate_jobs(const std::vector<RotateJob> &in, cudaStream_t s)
         const View c1v{x.a->d + x.a->cstride(N), x.a->bstride(N), x.a->cstride(N)};
         const View accv{x.acc, (size_t)2 * ext * N, (size_t)ext * N};
         // sigma_g(c1)
-        aj.push_back(AutomorphismJob{tv, c1v, x.g, 1, ctx.log_n, ctx.t.primes, ew_blocks((int)N, 2), L, B, 0});
+        aj.push_back(AutomorphismJob{tv, c1v, x.g, 1, ctx.log_n, ew_blocks((int)N, 2), L, B, 0});
         // ModUp: inverse NTT, conversion of every digit, forward NTT of the extended rows
         std::vector<int> q_rows(L), ext_primes(ext), p_rows(K);
         for (int r = 0; r < L; r++) q_rows[r] = r;
