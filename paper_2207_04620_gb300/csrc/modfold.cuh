@@ -159,7 +159,8 @@ struct Sum30 {
         b &= kMask30;
         a &= (1ull << 60) - 1;
     }
-    // the sum times 2^-60 mod q, below 2^b + 2^(64-b) d (settle_rare() brings it below q)
+    // the sum times 2^-60 mod q.  Up to 14 products and the carries from below come to less than 18 2^b, so
+    // the fold leaves less than 2^b + 18 d < 2 q, which settle_rare() brings below q
     template <class P_> __device__ __forceinline__ uint64_t reduce(const P_ &P) const
     {
         const uint32_t m0 = ((uint32_t)a * P.minv) & kMask30;

@@ -1,5 +1,5 @@
 """Basis conversions on split sums: every source count up to the largest, full sums (60-bit primes),
-grids split over the destination rows, and overshoots that lie on an integer (where the FP64 sum
+sources and destinations of 33 to 60 bits in one conversion, grids split over the destination rows, and overshoots that lie on an integer (where the FP64 sum
 decides), bit-exact against the oracle."""
 import numpy as np
 import pytest
@@ -13,6 +13,10 @@ pytestmark = pytest.mark.gpu
 
 for a, k in ((1, 1), (2, 2), (3, 3), (4, 4), (5, 5), (7, 6)):
     PARAMS["conv%d" % a] = dict(log_n=11, q_bits=[60] * 9, p_bits=[60] * k, log2_scale=45, alpha=a)
+MIXED = [60, 33, 34, 60, 36, 33, 35, 60, 34]
+PARAMS["conv_mixed3"] = dict(log_n=11, q_bits=MIXED, p_bits=[60, 36, 33], log2_scale=33, alpha=3)
+PARAMS["conv_mixed7"] = dict(log_n=11, q_bits=MIXED, p_bits=[60, 33, 60, 36, 60, 34], log2_scale=33, alpha=7)
+PARAMS["conv_mixed14"] = dict(log_n=14, q_bits=MIXED, p_bits=[60, 34], log2_scale=33)
 PARAMS["conv40"] = dict(log_n=13, q_bits=[60] + [40] * 8, p_bits=[60] * 3, log2_scale=40, alpha=4)
 
 
@@ -26,7 +30,8 @@ def built():
         pytest.skip("no CUDA device")
 
 
-@pytest.mark.parametrize("name", ["conv1", "conv2", "conv3", "conv4", "conv5", "conv7", "conv40"])
+@pytest.mark.parametrize("name", ["conv1", "conv2", "conv3", "conv4", "conv5", "conv7", "conv40", "conv_mixed3", "conv_mixed7",
+                                  "conv_mixed14"])
 def test_switch_and_joint_division(name):
     pr = Pair(name, rot_steps=[3])
     try:

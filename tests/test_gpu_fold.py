@@ -1,6 +1,7 @@
 """Transforms on chains of primes just below powers of two (fold arithmetic): bit-exact against the
-oracle at the ends of the prime sizes it takes, on inputs that drive its signed, unreduced sums
-furthest.  Words are integers, so there is no tolerance."""
+oracle at the ends of the prime sizes it takes (33 and 60 bits), with final reductions of one fold and
+of two, on inputs that drive its signed, unreduced sums furthest.  Words are integers, so there is no
+tolerance."""
 import numpy as np
 import pytest
 
@@ -15,7 +16,33 @@ CHAINS = {
     "mixed": [60, 59, 55, 50, 45, 45, 45, 45, 45, 45],
     "40": [60] + [40] * 12,
     "small": [38, 38, 36, 36, 36, 35],
+    "33": [33, 33, 34, 34],
+    "60_33": [60, 33, 45, 34, 60, 36],
 }
+
+
+def folds(q):
+    """How many folds the final reduction of prime q takes; None if fold arithmetic does not hold for it:
+    on a unit u >= 2^b with folded values within 17/16 u and products within 25/16 u, sums up to
+    127/16 u have to stay inside 63 bits and end within 2^(b-1) of [0, 2^b)."""
+    b = q.bit_length()
+    one, d = 1 << b, (1 << b) - q
+    if not 33 <= b <= 60 or d >= 1 << 26:
+        return None
+
+    def folded(v):
+        return one + ((v >> b) + 1) * d
+
+    u = max(one, -(-16 * (one + one // 2 + (d << 31)) // 25))
+    for _ in range(3):
+        u = max(u, -(-16 * folded(u * 127 // 16 + 1) // 17))
+    limit = u * 127 // 16 + 1
+    if limit >= (1 << 63) - (1 << 32) or 16 * folded(limit) > 17 * u:
+        return None
+    once = folded(limit)
+    if once - one <= one // 2:
+        return 1
+    return 2 if folded(once) - one <= one // 2 else None
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -61,6 +88,9 @@ def test_extreme_inputs_bit_exact(chain, log_n):
     ctx = hx.hx_context_create(log_n, bits, [60], 40)
     try:
         primes = octx.q + octx.p
+        assert all(folds(q) for q in primes)
+        if chain in ("33", "60_33") and log_n >= 12:
+            assert 2 in [folds(q) for q in primes]
         x = inputs(log_n, primes, octx.N)
         flat = x.reshape(-1, octx.N)
         idx = list(range(len(primes)))

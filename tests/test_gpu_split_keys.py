@@ -1,6 +1,6 @@
 """Key inner products over keys split at bit 30: every digit count the kernels are built for and
 the general one, up to and past the counts at which their sums make room, with 60-bit primes (the
-fullest sums) and all words at q - 1, bit-exact against the oracle; batches that fill a block's
+fullest sums), with primes of 33 to 60 bits, and all words at q - 1, bit-exact against the oracle; batches that fill a block's
 entries partly."""
 import numpy as np
 import pytest
@@ -14,6 +14,7 @@ from hxpair import PARAMS, Pair
 pytestmark = pytest.mark.gpu
 
 PARAMS["split60"] = dict(log_n=11, q_bits=[60] * 16, p_bits=[60], log2_scale=45, alpha=1)
+PARAMS["split_mixed"] = dict(log_n=11, q_bits=[60, 33, 34, 60] + [36, 33, 60, 35] * 3, p_bits=[60], log2_scale=33, alpha=1)
 PARAMS["split60_mm"] = dict(log_n=11, q_bits=[60] * 9, p_bits=[60], log2_scale=45, alpha=1)
 PARAMS["split45_mm"] = dict(log_n=11, q_bits=[60] + [45] * 6, p_bits=[60, 60], log2_scale=45)
 
@@ -28,9 +29,9 @@ def built():
         pytest.skip("no CUDA device")
 
 
-@pytest.fixture(scope="module")
-def chain():
-    pr = Pair("split60", rot_steps=[1, 5, -3])
+@pytest.fixture(scope="module", params=["split60", "split_mixed"])
+def chain(request):
+    pr = Pair(request.param, rot_steps=[1, 5, -3])
     yield pr
     pr.close()
 
