@@ -230,12 +230,16 @@ void Eval::moddown_add(const OutTab &out, const View &accv, int B, int limbs, co
 }
 
 // Rotations (or selections) of a batch of B per launch: as many as keep the launch's buffer within
-// 128 MB, about L2's size, so that the stages that follow find most of it there (sixteen 64x64 pairs
-// 21.9 ms with 32 MB, 20.8 with 128; five 32x32 products 2.11 and 2.03, 2.33 with 16; a small dense layer
-// 8.66 and 7.85, 10.6 with 16).  One rotation of 16 entries of N = 2^14 (38 MB) already
+// 128 MB, about the size of GB300's L2, so that the stages that follow find most of it there.  Measured
+// with 16, 32, 64, 128 and 256 MB: sixteen 64x64 pairs 21.9, 21.9, 21.9, 20.8 and 20.5 ms; five 32x32
+// products 2.33, 2.11, 2.08, 2.03 and 2.03 ms; a small dense layer 10.6, 8.66, 8.07, 7.85 and 7.85 ms: past
+// 128 the last 1.5 % of one of them would cost twice the memory.  (kGroupBytes; the call's limit may
+// be lower, down to one rotation.)  One rotation of 16 entries of N = 2^14 (38 MB) already
 // fills the GPU; one of a single entry of N = 2^12 takes a few SMs, and with a launch per stage and
 // rotation the product of 16x16 matrices there waited on about 900 launches: 5.2 ms, 0.74 in groups
 // (five 32x32 products of N = 2^13: 4.0 ms, 2.6; a small dense layer of N = 2^14: 23.2 ms, 11.0).
+// A launch's entries times their digits, or their two components, lie in the z extent of a grid,
+// which ends at 65535: `grid` stays at a quarter of it.
 int Eval::rot_chunk(int B, int limbs, int most, size_t words)
 {
     const size_t per = words ? words : (size_t)B * 2 * (limbs + ctx.K) * ctx.N;

@@ -65,7 +65,7 @@ __global__ void k_copy(View out, View a, int comps, int n)
 }
 
 // Copies of equal length between ciphertexts' own buffers and a batch: a table of addresses in one
-// launch, where one device-to-device copy each took 2-4 us of the host and of the stream.  @C@
+// launch, where one device-to-device copy each took 2-4 us of the host and of the stream.
 // A block moves kCopyWords, 64 bytes a thread in flight.
 constexpr int kCopyWords = 2048;
 
@@ -476,9 +476,11 @@ __global__ void __launch_bounds__(256, MK <= 4 ? 4 : 2)
 // the reductions), the sign batch's (four sources, 16 limbs of N = 2^15) 2.27 ms and 1.6 per product.
 //
 // The shifted form's overshoot u = floor(sum of y_i / q_i rounded in FP64) comes from 32-bit
-// products (within 2^-29 of the sum) unless the sum lies within 2^-26 of an integer, where the
-// FP64 sum decides as in the form above: its pipe issues a sixteenth of a warp per cycle and
-// would take longer than the conversion.
+// products: y and 2^(31 + bits) / q are truncated, so a term is short by less than 2^-30 and the sum of
+// seven by less than 2^-27.  Where the estimate lies less than 2^-26 below an integer (the sum may have
+// reached it) or less than 2^-46 above one (the FP64 sum, within 2^-47, may have stayed below it), the
+// FP64 sum decides as in the form above: its pipe issues a sixteenth of a warp per cycle and would
+// take longer than the conversion.
 struct ConvShared {
     uint64_t w[MAXK * MAXP], prod[MAXP], sub[MAXP];  // w: a destination's sources together
     SumPrime dst[MAXP];
@@ -493,7 +495,7 @@ __device__ __forceinline__ void convert_split_pair(const ConvShared &S, const Co
 {
     const int nd = T.n_dst;
     uint32_t l0[NS], h0[NS], l1[NS], h1[NS];
-    uint64_t v0 = 0, v1 = 0;  // the overshoot's estimate in units of 2^-60, each term short by less than 2^31
+    uint64_t v0 = 0, v1 = 0;  // the overshoot's estimate in units of 2^-60, each term short by less than 2^30
 #pragma unroll
     for (int i = 0; i < NS; i++) {
         const FoldPrime &P = primes[T.src_prime[i]];

@@ -14,7 +14,7 @@
 // signed: |r| <= 1.5 2^b + 2^31 d.
 //
 // Values stay signed and unreduced through several butterflies; fold() brings one back to
-// about [0, 2^b) with one multiply-add: v = 2^b h + l = l + d h.  FoldBounds (host) proves for a
+// about [0, 2^b) with one multiply-add: v = 2^b h + l = l + d h.  fold_bounds (context.cu) proves for a
 // prime that no sum leaves 64 bits and how many folds the final reduction takes; chains with a
 // prime outside its range use the Shoup kernels.
 #pragma once

@@ -308,12 +308,12 @@ void keygen(hx_context &ctx, hx_keyset &ks, int n_parties, uint64_t seed, cudaSt
 void add_rotation_keys(hx_context &ctx, hx_keyset &ks, const std::vector<int64_t> &steps, cudaStream_t s);
 Cts encrypt_coeffs(hx_context &ctx, const hx_keyset &ks, const int64_t *m, double scale, int limbs, uint64_t seed,
                    uint32_t tag, uint32_t index, cudaStream_t s);
-// centered coefficients of c0 + c1 s mod q_0 for every batch entry: [B][N]
 // DDec and Dcd on the device: the shares' sum at q_0 (decrypt_coeffs's) and its first `count` slots
 void decrypt_slots(hx_context &ctx, const hx_keyset &ks, const Cts &c, double *slots, size_t count, cudaStream_t s);
 // the second half of it: slots of the sum of shares sh ([1 + n_parties][N], coefficient form mod q_0)
 void decode_shares(hx_context &ctx, const uint64_t *sh, int n_parties, double scale, double *slots_dev, int count,
                    cudaStream_t s);
+// centered coefficients of c0 + c1 s mod q_0 for every batch entry: [B][N]
 std::vector<int64_t> decrypt_coeffs(hx_context &ctx, const hx_keyset &ks, const Cts &c, cudaStream_t s);
 Cts dkeyswitch(hx_context &ctx, const hx_keyset &from, const hx_keyset &to, const Cts &ct, uint64_t seed,
                cudaStream_t s);
