@@ -548,13 +548,15 @@ void hx_counters_reset(hx_context *ctx);
  * 256, 768, more), and each bucket is timed on its own batch (48, 176, 512 and
  * 1024 limbs) on this device, each variant's time the best of three rounds.
  * Per (bucket, phase) the default (width 16, 8 for a phase of 256 points,
- * swapped radices off) is kept unless another variant is more than 2 % faster, in which case the fastest is
- * kept: alone the widths differ by about their timing noise, and blocks of the
- * default size share the SMs best with concurrently running kernels.  For an
- * odd log N both splits of the stages between the two phases are tuned this
- * way, and the other split replaces the default (the column phase takes the
- * larger half of the stages from log N = 13 on, the smaller one at 11) when the
- * sum of its phases' times is more than 2 % lower.  The table belongs to the context.  Every variant computes identical residues.
+ * swapped radices off) is kept unless another variant is more than 2 % faster,
+ * in which case the fastest is kept: alone the widths differ by about their
+ * timing noise, and blocks of the default size share the SMs best with
+ * concurrently running kernels.  For an odd log N both splits of the stages
+ * between the two phases are tuned this way, and the other split replaces the
+ * default (the column phase takes the larger half of the stages from log N = 13
+ * on, the smaller one at 11) when the sum of its phases' times is more than 2 %
+ * lower.  The table belongs to the context.  Every variant computes identical
+ * residues.
  * The call runs on `stream` and synchronizes it.  choice[4] (may be
  * NULL) receives the variants of the 256-limb bucket as signed widths
  * (negative: swapped radices). */
