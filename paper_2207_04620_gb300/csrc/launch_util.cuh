@@ -61,7 +61,9 @@ inline void launch(cudaStream_t s, void (*kernel)(P...), dim3 grid, dim3 block, 
     cfg.stream = s;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    HX_CUDA(cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...));
+    const cudaError_t launched = cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+    if (launched != cudaSuccess) cudaGetLastError();  // reported here, not by the next call as well
+    HX_CUDA(launched);
 }
 
 inline void post(const LaunchCtx &c, int k = 1)
