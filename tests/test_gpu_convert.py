@@ -1,5 +1,6 @@
 """Basis conversions on split sums: every source count up to the largest, full sums (60-bit primes),
-sources and destinations of 33 to 60 bits in one conversion, grids split over the destination rows, and overshoots that lie on an integer (where the FP64 sum
+sources and destinations of 33 to 60 bits in one conversion, chains outside fold arithmetic (Shoup
+products), grids split over the destination rows, and overshoots that lie on an integer (where the FP64 sum
 decides), bit-exact against the oracle."""
 import numpy as np
 import pytest
@@ -17,6 +18,7 @@ MIXED = [60, 33, 34, 60, 36, 33, 35, 60, 34]
 PARAMS["conv_mixed3"] = dict(log_n=11, q_bits=MIXED, p_bits=[60, 36, 33], log2_scale=33, alpha=3)
 PARAMS["conv_mixed7"] = dict(log_n=11, q_bits=MIXED, p_bits=[60, 33, 60, 36, 60, 34], log2_scale=33, alpha=7)
 PARAMS["conv_mixed14"] = dict(log_n=14, q_bits=MIXED, p_bits=[60, 34], log2_scale=33)
+PARAMS["conv_general"] = dict(log_n=11, q_bits=[60] * 9, p_bits=[61] * 3, log2_scale=45, alpha=4)
 PARAMS["conv40"] = dict(log_n=13, q_bits=[60] + [40] * 8, p_bits=[60] * 3, log2_scale=40, alpha=4)
 
 
@@ -31,7 +33,7 @@ def built():
 
 
 @pytest.mark.parametrize("name", ["conv1", "conv2", "conv3", "conv4", "conv5", "conv7", "conv40", "conv_mixed3", "conv_mixed7",
-                                  "conv_mixed14"])
+                                  "conv_mixed14", "conv_general"])
 def test_switch_and_joint_division(name):
     pr = Pair(name, rot_steps=[3])
     try:

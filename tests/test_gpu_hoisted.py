@@ -7,20 +7,23 @@ import mempool
 from oracle import ckks as C
 from paper_2207_04620_gb300 import hx, workloads
 
-from hxpair import Pair
+from hxpair import PARAMS, Pair
 
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def pair():
+PARAMS["hoisted_general"] = dict(log_n=12, q_bits=[60, 45, 45, 45, 45], p_bits=[61, 60], log2_scale=45)
+
+
+@pytest.fixture(scope="module", params=["alg3", "hoisted_general"])  # the second: outside fold arithmetic
+def pair(request):
     from paper_2207_04620_gb300 import build
 
     build.build()
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
-    pr = Pair("alg3", rot_steps=[1, -3])
+    pr = Pair(request.param, rot_steps=[1, -3])
     yield pr
     pr.close()
 

@@ -1,6 +1,7 @@
 """Key inner products over keys split at bit 30: every digit count the kernels are built for and
 the general one, up to and past the counts at which their sums make room, with 60-bit primes (the
-fullest sums), with primes of 33 to 60 bits, and all words at q - 1, bit-exact against the oracle; batches that fill a block's
+fullest sums), with primes of 33 to 60 bits, on a chain outside fold arithmetic (a 61-bit special prime:
+Montgomery keys, whole-word products, the same groups and schedules), and all words at q - 1, bit-exact against the oracle; batches that fill a block's
 entries partly."""
 import numpy as np
 import pytest
@@ -15,6 +16,8 @@ pytestmark = pytest.mark.gpu
 
 PARAMS["split60"] = dict(log_n=11, q_bits=[60] * 16, p_bits=[60], log2_scale=45, alpha=1)
 PARAMS["split_mixed"] = dict(log_n=11, q_bits=[60, 33, 34, 60] + [36, 33, 60, 35] * 3, p_bits=[60], log2_scale=33, alpha=1)
+PARAMS["general"] = dict(log_n=11, q_bits=[60] * 16, p_bits=[61], log2_scale=45, alpha=1)
+PARAMS["general_mm"] = dict(log_n=11, q_bits=[60] + [45] * 6, p_bits=[61, 60], log2_scale=45)
 PARAMS["split60_mm"] = dict(log_n=11, q_bits=[60] * 9, p_bits=[60], log2_scale=45, alpha=1)
 PARAMS["split45_mm"] = dict(log_n=11, q_bits=[60] + [45] * 6, p_bits=[60, 60], log2_scale=45)
 
@@ -29,7 +32,7 @@ def built():
         pytest.skip("no CUDA device")
 
 
-@pytest.fixture(scope="module", params=["split60", "split_mixed"])
+@pytest.fixture(scope="module", params=["split60", "split_mixed", "general"])
 def chain(request):
     pr = Pair(request.param, rot_steps=[1, 5, -3])
     yield pr
@@ -54,7 +57,8 @@ def test_rotations_by_digit_count(chain, limbs):
         assert chain.same(got, want)
 
 
-@pytest.mark.parametrize("name,h,limbs", [("split60_mm", 4, 9), ("split60_mm", 4, 5), ("split45_mm", 4, 7)])
+@pytest.mark.parametrize("name,h,limbs", [("split60_mm", 4, 9), ("split60_mm", 4, 5), ("split45_mm", 4, 7), ("general_mm", 4, 7),
+                                          ("general_mm", 4, 3)])
 @pytest.mark.parametrize("count", [1, 2, 3, 5])
 def test_products_bound_and_unbound(name, h, limbs, count):
     p = PARAMS[name]
@@ -66,7 +70,8 @@ def test_products_bound_and_unbound(name, h, limbs, count):
         la, lb = [pr.to_lib(x) for x in A], [pr.to_lib(x) for x in B]
         plan = hx.hx_matmul_plan_create(pr.ctx, h, limbs)
         plain = hx.hx_matmul_batch(pr.ctx, pr.ks, plan, la, lb, h)
-        hx.hx_matmul_plan_bind_keys(pr.ctx, plan, pr.ks)
+        if limbs > 3:  # Alg. 3; the depth-2 form has no selections to bind
+            hx.hx_matmul_plan_bind_keys(pr.ctx, plan, pr.ks)
         bound = hx.hx_matmul_batch(pr.ctx, pr.ks, plan, la, lb, h)
         masks, ev = Hc.MaskProvider(pr.octx, h, limbs), C.Evaluator(pr.octx, pr.oks)
         for i in sorted({0, count - 1}):
@@ -77,3 +82,29 @@ def test_products_bound_and_unbound(name, h, limbs, count):
         hx.hx_matmul_plan_destroy(plan)
     finally:
         pr.close()
+
+
+def test_rings_inside_and_outside_fold_arithmetic_in_one_call():
+    """hx_rotate_jobs and hx_ntt_multi over rings of both kinds: one arithmetic serves every transform,
+    keys and conversions keep their ring's."""
+    import torch
+
+    pairs = [Pair("split45_mm", rot_steps=[3]), Pair("general_mm", rot_steps=[3])]
+    try:
+        jobs, want, rows = [], [], []
+        for i, pr in enumerate(pairs):
+            limbs = 5 - i
+            x = workloads.residues(i, pr.octx.q[:limbs], 2, pr.N).reshape(2, limbs, pr.N)
+            ct = C.Ciphertext(x, 2.0 ** 45)
+            jobs.append((pr.ctx, pr.ks, pr.to_lib(ct), 3))
+            want.append(C.Evaluator(pr.octx, pr.oks).rotate(ct, 3))
+            t = torch.from_numpy(x.view(np.int64).copy()).cuda()
+            rows.append((t, pr.octx.ntt(x.reshape(-1, pr.N), pr.octx.q[:limbs] * 2)))
+        for pr, got, w in zip(pairs, hx.hx_rotate_jobs(jobs), want):
+            assert pr.same(got, w)
+        hx.hx_ntt_multi([(pr.ctx, t.data_ptr(), 2, list(range(t.shape[1]))) for pr, (t, _) in zip(pairs, rows)])
+        for t, w in rows:
+            assert np.array_equal(t.cpu().numpy().view(np.uint64).reshape(w.shape), w)
+    finally:
+        for pr in pairs:
+            pr.close()
