@@ -217,7 +217,8 @@ typedef struct {
  * fields, handles of another context, HX_EKEY for a missing Galois key) comes
  * before any device work; on an error no output is set.  count <= 65535. */
 hx_status hx_rotate_jobs(const hx_rotate_job *jobs, size_t count, hx_ct **out, void *stream);
-/* n rotations of one ciphertext sharing a single ModUp of c1 (hoisting). */
+/* n rotations of one ciphertext sharing a single ModUp of c1 (hoisting); a step
+ * of 0 mod N/2 copies it whole. */
 hx_status hx_rotate_hoisted(hx_context *ctx, const hx_keyset *ks, const hx_ct *a, const int32_t *steps, int n,
                             hx_ct **outs, void *stream);
 
