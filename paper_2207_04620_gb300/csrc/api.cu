@@ -1017,6 +1017,7 @@ static void capture_product(hx_matmul_exec &ex, size_t group)
     } catch (...) {
         cudaStreamEndCapture(ex.cap, &graph);
         if (graph) cudaGraphDestroy(graph);
+        cudaGetLastError();  // the capture's streams were not joined: not the next call's error
         ctx.profiling = prof;
         throw;
     }

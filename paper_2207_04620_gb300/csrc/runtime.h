@@ -267,6 +267,15 @@ struct Eval {
     const SwitchKey &rot_key(const hx_keyset &ks, uint64_t g);
 };
 
+// whether s is being captured (or cannot tell because another stream is)
+inline bool capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &c) == cudaSuccess) return c != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
 // f(group) on stream s; where the device has no room for groups of that size, again with one rotation
 // at a time, so that a nearly full device still runs what it held without groups.  f gives back what it
 // took and leaves no work on other streams when it throws; the operations it had run stay counted.
@@ -275,10 +284,7 @@ template <class F> auto with_groups(cudaStream_t s, size_t group, F f) -> declty
     try {
         return f(group);
     } catch (const Error &e) {
-        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-        if (e.code != HX_ENOMEM || group == 0 || cudaStreamIsCapturing(s, &capture) != cudaSuccess ||
-            capture != cudaStreamCaptureStatusNone)
-            throw;
+        if (e.code != HX_ENOMEM || group == 0 || capturing(s)) throw;
     }
     HX_CUDA(cudaStreamSynchronize(s));  // what the attempt freed is free for every size again
     return f(0);

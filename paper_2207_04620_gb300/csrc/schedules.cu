@@ -493,7 +493,7 @@ struct JoinOnThrow {
     int before = std::uncaught_exceptions();
     ~JoinOnThrow()
     {
-        if (std::uncaught_exceptions() > before)
+        if (std::uncaught_exceptions() > before && !capturing(s[0]))  // a capture has run nothing
             for (cudaStream_t x : s) cudaStreamSynchronize(x);
     }
 };
